@@ -317,14 +317,13 @@ rg_status lbvh_topology(TempAlloc& tmp, const float* lohi, uint32_t n, const int
                         uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges = nullptr) {
     const int key_bits = bits == 21 ? 64 : 32;
     const size_t kb = key_bits / 8;
-    void *codes, *sorted, *vals, *scratch;
+    void *codes, *sorted, *scratch;
     rg_status r;
     if ((r = tmp.get(&codes, n * kb, "morton codes"))) return r;
     if ((r = tmp.get(&sorted, n * kb, "sorted codes"))) return r;
-    if ((r = tmp.get(&vals, n * 4ull, "sort values"))) return r;
     if ((r = tmp.get(&scratch, radix_sort_scratch_bytes(n, key_bits), "sort scratch"))) return r;
-    RG_CK(launch_morton(lohi, n, cb_ord, bits, codes, static_cast<uint32_t*>(vals), nullptr, s));
-    RG_CK(radix_sort_pairs(codes, static_cast<uint32_t*>(vals), n, key_bits, sorted, perm, scratch, s));
+    RG_CK(launch_morton(lohi, n, cb_ord, bits, codes, nullptr, s));
+    RG_CK(radix_sort_pairs(codes, nullptr, n, key_bits, sorted, perm, scratch, s));
     RG_CK(launch_karras(sorted, n, key_bits, reinterpret_cast<uint32_t*>(nodes) + 12, 16, parents, s, ranges));
     return RG_OK;
 }
@@ -1043,7 +1042,7 @@ rg_status rg_morton_codes(const float* d_lohi, uint32_t n, uint32_t bits, void* 
     if ((r = tmp.get(&cb, 64, "centroid bounds"))) return r;
     RG_CK(launch_init_bounds(static_cast<int*>(cb), st));
     RG_CK(launch_centroid_bounds(d_lohi, n, static_cast<int*>(cb), st));
-    RG_CK(launch_morton(d_lohi, n, static_cast<int*>(cb), (int)bits, d_codes, nullptr, d_cbounds, st));
+    RG_CK(launch_morton(d_lohi, n, static_cast<int*>(cb), (int)bits, d_codes, d_cbounds, st));
     return RG_OK;
 }
 

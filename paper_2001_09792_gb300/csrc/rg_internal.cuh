@@ -168,15 +168,16 @@ cudaError_t launch_tri_bounds(const float* vtx, uint32_t nv, const uint32_t* idx
                               int* cb_ord, DevStatus* st, cudaStream_t s);
 cudaError_t launch_init_bounds(int* cb_ord, cudaStream_t s);
 cudaError_t launch_centroid_bounds(const float* lohi, uint32_t n, int* cb_ord, cudaStream_t s);
-cudaError_t launch_morton(const float* lohi, uint32_t n, const int* cb_ord, int bits, void* codes, uint32_t* vals,
-                          float* cb_out, cudaStream_t s);
+cudaError_t launch_morton(const float* lohi, uint32_t n, const int* cb_ord, int bits, void* codes, float* cb_out,
+                          cudaStream_t s);
 // Radix sort; scratch must hold radix_sort_scratch_bytes(n, key_bits) bytes:
-// ping-pong keys and values, and 256 digit counts per tile of kSortTilePairs
-// pairs, each part 256-byte aligned.
+// ping-pong keys and values, the digit counts and a tile counter of each pass,
+// and two passes' 256 look-back words per tile of kSortTilePairs pairs, each
+// part 256-byte aligned.  vals_in may be null: the values are 0 .. n - 1.
 constexpr uint32_t kSortTilePairs = 2048;
 constexpr size_t radix_sort_scratch_bytes(uint32_t n, int key_bits) {
     return ((((size_t)n * (key_bits == 64 ? 8 : 4)) + 255) & ~(size_t)255) + ((((size_t)n * 4) + 255) & ~(size_t)255) +
-           ((((size_t)256 * ((n + kSortTilePairs - 1) / kSortTilePairs) * 4) + 255) & ~(size_t)255);
+           (256 * 8 + 64) * 4 + (size_t)2 * 256 * (((size_t)n + kSortTilePairs - 1) / kSortTilePairs) * (n >= (1u << 30) ? 8 : 4);
 }
 cudaError_t radix_sort_pairs(const void* keys_in, const uint32_t* vals_in, uint32_t n, int key_bits, void* keys_out,
                              uint32_t* vals_out, void* scratch, cudaStream_t s);

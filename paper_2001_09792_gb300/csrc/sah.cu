@@ -1162,14 +1162,13 @@ rg_status sah_topology(const ScratchAlloc& tmp, const float* lohi, uint32_t n, c
                        uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges) {
     const int key_bits = bits == 21 ? 64 : 32;
     const size_t kb = key_bits / 8;
-    void *codes, *sorted, *vals, *scratch;
+    void *codes, *sorted, *scratch;
     rg_status r;
     if ((r = tmp.get(tmp.ctx, &codes, n * kb, "morton codes"))) return r;
     if ((r = tmp.get(tmp.ctx, &sorted, n * kb, "sorted codes"))) return r;
-    if ((r = tmp.get(tmp.ctx, &vals, n * 4ull, "sort values"))) return r;
     if ((r = tmp.get(tmp.ctx, &scratch, radix_sort_scratch_bytes(n, key_bits), "sort scratch"))) return r;
-    SAH_CK(launch_morton(lohi, n, cb_ord, bits, codes, static_cast<uint32_t*>(vals), nullptr, s));
-    SAH_CK(radix_sort_pairs(codes, static_cast<uint32_t*>(vals), n, key_bits, sorted, perm, scratch, s));
+    SAH_CK(launch_morton(lohi, n, cb_ord, bits, codes, nullptr, s));
+    SAH_CK(radix_sort_pairs(codes, nullptr, n, key_bits, sorted, perm, scratch, s));
     if (n <= kSahSmall) {
         SAH_CK(launch_karras(sorted, n, key_bits, reinterpret_cast<uint32_t*>(nodes) + 12, 16, parents, s, ranges));
         return RG_OK;
@@ -1274,7 +1273,7 @@ rg_status sah_one_topology(const ScratchAlloc& tmp, const float* lohi, uint32_t 
     if ((r = tmp.get(tmp.ctx, &n_pending, 16, "SAH pending count"))) return r;
     SahSmallScratch w{static_cast<uint32_t*>(keys), static_cast<uint32_t*>(perm0), static_cast<uint32_t*>(rank),
                       pending, static_cast<uint32_t*>(n_pending), boxes_done};
-    SAH_CK(launch_morton(lohi, n, cb_ord, bits, codes, nullptr, nullptr, s));
+    SAH_CK(launch_morton(lohi, n, cb_ord, bits, codes, nullptr, s));
     SAH_CK(launch_sah_small(lohi, n, static_cast<const uint32_t*>(codes), perm, nodes, parents, ranges, w, s));
     return RG_OK;
 }

@@ -90,6 +90,28 @@ def check_children(children, first, last, split):
     assert np.array_equal(ch[:, 1], want_r)
 
 
+@pytest.mark.parametrize("n", [1, 33, 4095, 4096, 4097, 6143, 6145, 2048 * 152 + 1])
+@pytest.mark.parametrize("key_bits", [32, 64])
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_radix_sort_edges(n, key_bits, noalloc):
+    """One block's limit, ends of tiles, and keys that share all but a few
+    digits, the largest key among them; exact, as every whole number is."""
+    if noalloc and n > 262144:
+        n = 262144
+    rng = np.random.default_rng(n)
+    keys = rng.integers(0, 3, n).astype(np.uint64) << np.uint64(key_bits - 2)
+    keys |= rng.integers(0, 5, n).astype(np.uint64) << np.uint64(7)
+    keys[rng.integers(0, n, max(1, n // 7))] = 2 ** key_bits - 1
+    keys = keys.astype(np.uint32 if key_bits == 32 else np.uint64)
+    signed = torch.from_numpy(keys.view(np.int32 if key_bits == 32 else np.int64)).cuda()
+    vals = torch.arange(n, dtype=torch.int32).cuda()
+    sort = rg.rg_radix_sort_pairs_noalloc if noalloc else rg.rg_radix_sort_pairs
+    ko, vo = sort(signed, vals)
+    order = np.argsort(keys, kind="stable")
+    assert np.array_equal(vo.cpu().numpy(), order)
+    assert np.array_equal(ko.cpu().numpy().view(keys.dtype), keys[order])
+
+
 @pytest.mark.parametrize("n,hi", [(2, 4), (3, 1), (17, 1), (1000, 8), (4097, 1 << 30), (50_000, 1 << 30), (9999, 64)])
 @pytest.mark.parametrize("key_bits", [32, 64])
 def test_karras_topology(n, hi, key_bits):
