@@ -47,6 +47,20 @@ def test_random_images(shape):
     assert_bitwise(gpu_fxaa(img2.astype(np.float32)), oracle.fxaa(img2.astype(np.float32)))
 
 
+@pytest.mark.parametrize("shape", [(31, 33), (352, 480), (353, 481), (417, 385)])
+def test_long_edges_across_tiles(shape):
+    """Both tile sizes, whole and ragged: edges of slope 0 to 1/40 both ways,
+    whose search runs past the tile and its halo, on a noisy ground."""
+    rng = np.random.default_rng(shape[0])
+    y, x = np.mgrid[:shape[0], :shape[1]]
+    lum = 0.2 + 0.02 * rng.uniform(0, 1, shape)
+    for k in range(1, 6):
+        lum += 0.25 * (y > shape[0] * k / 6 + x / (20.0 * k)) * (k % 2 * 2 - 1)
+        lum += 0.15 * (x > shape[1] * k / 6 - y / (25.0 * k)) * (k % 2 * 2 - 1)
+    img = (lum[..., None] * rng.uniform(0.5, 1, 4)).astype(np.float32)
+    assert_bitwise(gpu_fxaa(img), oracle.fxaa(img))
+
+
 @pytest.mark.parametrize("which", ["tiny", "medium"])
 def test_rendered_frames(which):
     s = g.tiny_scene() if which == "tiny" else g.medium_scene()
