@@ -526,7 +526,7 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
              RG_CK(cudaStreamSynchronize(st));  // hd lives on this stack frame
 
              TempAlloc tmp(st);
-             void *lohi, *cb, *perm, *parents, *fl, *ranges = nullptr, *tasks = nullptr;
+             void *lohi, *cb, *perm, *parents, *fl, *ranges = nullptr, *tasks = nullptr, *boxes_done = nullptr;
              rg_status q;
              if (wide) {
                  if ((q = tmp.get(&ranges, n_int * 8, "ranges"))) return q;
@@ -540,10 +540,13 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
              RG_CK(launch_init_bounds(static_cast<int*>(cb), st));
              RG_CK(launch_tri_bounds(d_vtx, nv, d_idx, nt, static_cast<float*>(lohi), static_cast<int*>(cb), s->st, st));
              if (nt > 1) {
-                 if (flags & RG_BLAS_SAH)
+                 if (flags & RG_BLAS_SAH) {
+                     boxes_done = static_cast<char*>(cb) + 32;  // (the bounds take 24 of the 64 bytes)
                      q = sah_topology(ScratchAlloc{temp_get, &tmp}, static_cast<float*>(lohi), nt,
                                       static_cast<int*>(cb), bits, b.nodes, static_cast<uint32_t*>(perm),
-                                      static_cast<uint32_t*>(parents), st, static_cast<uint32_t*>(ranges));
+                                      static_cast<uint32_t*>(parents), st, static_cast<uint32_t*>(ranges),
+                                      static_cast<uint32_t*>(boxes_done));
+                 }
                  else
                      q = lbvh_topology(tmp, static_cast<float*>(lohi), nt, static_cast<int*>(cb), bits, b.nodes,
                                        static_cast<uint32_t*>(perm), static_cast<uint32_t*>(parents), st,
@@ -555,7 +558,7 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
              }
              RG_CK(launch_blas_leaves_refit(d_vtx, d_idx, static_cast<uint32_t*>(perm), static_cast<float*>(lohi), nt,
                                             static_cast<uint32_t*>(parents), b.nodes, static_cast<uint32_t*>(fl), b.tris,
-                                            s->B->d_blas.p + id, s->st, st));
+                                            s->B->d_blas.p + id, s->st, st, static_cast<uint32_t*>(boxes_done)));
              RG_CK(launch_bound_sphere(d_vtx, nv, s->B->d_blas.p + id, st));
              RG_CK(launch_invert_perm(static_cast<uint32_t*>(perm), nt, b.leaf_of_prim, st));
              if (wide) {
@@ -613,9 +616,9 @@ static rg_status tlas_common(rg_scene* s, const rg_instance* d_inst, uint32_t n,
             if (s->wide && (r = tmp.get(&ranges, (size_t)(n - 1) * 8, "ranges"))) return r;
             if (sah && (r = tmp.get(&boxes_done, 16, "box flag"))) return r;
             if (sah)
-                r = sah_one_topology(ScratchAlloc{temp_get, &tmp}, s->wbox.p, n, static_cast<int*>(cb), 10,
-                                     s->tlas_nodes.p, s->perm.p, s->parents.p, st, static_cast<uint32_t*>(ranges),
-                                     static_cast<uint32_t*>(boxes_done));
+                r = sah_topology(ScratchAlloc{temp_get, &tmp}, s->wbox.p, n, static_cast<int*>(cb), 10,
+                                 s->tlas_nodes.p, s->perm.p, s->parents.p, st, static_cast<uint32_t*>(ranges),
+                                 static_cast<uint32_t*>(boxes_done));
             else
                 r = lbvh_topology(tmp, s->wbox.p, n, static_cast<int*>(cb), 10, s->tlas_nodes.p, s->perm.p,
                                   s->parents.p, st, static_cast<uint32_t*>(ranges));

@@ -508,7 +508,8 @@ __device__ void climb(uint32_t j, uint32_t n, float* box, const uint32_t* __rest
 __global__ void k_blas_leaves_refit(const float* __restrict__ vtx, const uint32_t* __restrict__ idx,
                                     const uint32_t* __restrict__ perm, const float* __restrict__ lohi, uint32_t n,
                                     const uint32_t* __restrict__ parents, float4* nodes, uint32_t* flags,
-                                    float4* __restrict__ tris, BlasDev* blas_out, DevStatus* st) {
+                                    float4* __restrict__ tris, BlasDev* blas_out, DevStatus* st,
+                                    const uint32_t* __restrict__ boxes_done) {
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     uint32_t prim = perm[j];
@@ -523,6 +524,17 @@ __global__ void k_blas_leaves_refit(const float* __restrict__ vtx, const uint32_
         t[c] = make_float4(x, y, z, w);
         t[3 + c] = make_float4(y, z, x, w);
         t[6 + c] = make_float4(z, x, y, w);
+    }
+    if (boxes_done && *boxes_done) {  // the build wrote every node's boxes
+        if (j == 0) {
+            const float* f = reinterpret_cast<const float*>(nodes);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                blas_out->lo[a] = fminf(f[a], f[6 + a]);
+                blas_out->hi[a] = fmaxf(f[3 + a], f[9 + a]);
+            }
+        }
+        return;
     }
     float box[6];
 #pragma unroll
@@ -893,9 +905,10 @@ cudaError_t launch_invert_perm(const uint32_t* perm, uint32_t n, uint32_t* inv, 
 
 cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, const uint32_t* perm, const float* lohi,
                                      uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
-                                     float4* tris, BlasDev* blas_out, DevStatus* st, cudaStream_t s) {
+                                     float4* tris, BlasDev* blas_out, DevStatus* st, cudaStream_t s,
+                                     const uint32_t* boxes_done) {
     k_blas_leaves_refit<<<grid_for(n), kBlock, 0, s>>>(vtx, idx, perm, lohi, n, parents, nodes, flags, tris, blas_out,
-                                                       st);
+                                                       st, boxes_done);
     count_launches(1);
     return cudaGetLastError();
 }

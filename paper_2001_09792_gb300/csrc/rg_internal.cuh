@@ -186,7 +186,8 @@ cudaError_t launch_karras(const void* keys, uint32_t n, int key_bits, uint32_t* 
                           uint32_t* parents, cudaStream_t s, uint32_t* ranges = nullptr);
 cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, const uint32_t* perm, const float* lohi,
                                      uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
-                                     float4* tris, BlasDev* blas_out, DevStatus* st, cudaStream_t s);
+                                     float4* tris, BlasDev* blas_out, DevStatus* st, cudaStream_t s,
+                                     const uint32_t* boxes_done = nullptr);
 // Bounding sphere of a mesh about its root box centre (after the BLAS refit
 // wrote the root box): blas->r2_bits = max over the vertices.
 cudaError_t launch_bound_sphere(const float* vtx, uint32_t nv, BlasDev* blas, cudaStream_t s);
@@ -221,78 +222,28 @@ cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasS
                                    uint32_t n_threads, uint32_t n_leaves, float4* nodes, uint32_t* parents,
                                    uint32_t* ranges, cudaStream_t s);
 
-// sah.cu: binned-SAH topology, one level of segments per launch sequence.
+// sah.cu: binned-SAH topology.
 constexpr int kSahBins = 16;            // bins per axis
-constexpr uint32_t kSahChunk = 2048;    // triangles per block of a level's kernels
-constexpr uint32_t kSahSmall = 2;       // segments of at most this many triangles get the Karras hierarchy
+constexpr uint32_t kSahChunk = 1024;    // positions per block of a level's kernels
+constexpr uint32_t kSahMid = 512;       // segments of at most this many items are built in a block
+constexpr uint32_t kSahTiny = 32;       // of at most this many, in a warp
 constexpr uint32_t kSahMaxLevels = 40;  // deeper segments get the Karras hierarchy whatever their size
-constexpr uint32_t kSahSliceTasks = 65536;  // segments per launch sequence (bounds the scratch)
-constexpr uint32_t kSahOneMax = 4096;       // items of the build without host round trips (launch_sah_small)
-constexpr uint32_t kSahAccInts = 6 + 3 * kSahBins * 7;  // per task: centroid bounds, then 7 values per bin and axis
-struct SahTask {                        // one segment split at this level
-    uint32_t begin, count, node;        // leaves begin .. begin + count - 1, internal node `node`
-    uint32_t first_block, n_blocks;     // its blocks in the level's block list
-    uint32_t pad[3];
-};
-struct SahParam {                       // per task: binning frame and the chosen split
-    float cmin[3], scale[3];
-    int axis, split;                    // axis -1: halved by position
-    uint32_t nl;                        // triangles on the left
-    uint32_t pad[3];
-};
-struct SahLevel {
-    const float* lohi;                  // triangle boxes (lo xyz, hi xyz)
-    uint32_t n_leaves, m, n_blocks;     // triangles of the mesh, tasks, blocks
-    const SahTask* tasks;
-    const uint2* blk;                   // per block: task, first position of its chunk
-    int* acc;                           // per task: centroid bounds and bins (scratch)
-    SahParam* par;
-    uint32_t* prim_at;                  // triangle at each position (updated)
-    void* key_at;                       // its Morton code (updated)
-    uint32_t* prim_out;                 // scratch, n
-    void* key_out;                      // scratch, n
-    uint32_t *blk_left, *blk_off;       // scratch, per block
-    uint32_t* out_nl;                   // per task: triangles on the left
-    float4* nodes;
-    uint32_t* parents;
-    uint32_t* ranges;                   // may be null
-};
-cudaError_t launch_sah_level(const SahLevel& L, int key_bits, cudaStream_t s);
-// The same binned-SAH hierarchy for 2 <= n <= kSahOneMax items from their
-// 30-bit Morton codes, in three launches without host round trips (the sort
-// and the top levels in one block, then the subtrees of at most 128 items in
-// a block each, then the leaf order): perm_out (the item of each leaf),
-// children, parents, (optional) leaf ranges, and the boxes of every node's
-// children where the splits give them; *boxes_done is 1 when every node's
-// boxes were written, 0 when the bottom-up refit must compute them.
-struct SahSmallScratch {
-    uint32_t* keys;       // n: the sorted codes
-    uint32_t* perm0;      // n: the Morton order
-    uint32_t* rank;       // n
-    void* pending;        // n / 3 + 1 entries of 16 B
-    uint32_t* n_pending;  // 1
-    uint32_t* boxes_done; // 1
-};
-cudaError_t launch_sah_small(const float* lohi, uint32_t n, const uint32_t* codes, uint32_t* perm_out, float4* nodes,
-                             uint32_t* parents, uint32_t* ranges, const SahSmallScratch& w, cudaStream_t s);
+constexpr uint32_t kSahOneMax = 4096;   // items of a build without host round trips
 // Device temporaries of one library call (stream-ordered, freed when the call
 // returns); get() reports its own failures.
 struct ScratchAlloc {
     rg_status (*get)(void* ctx, void** p, size_t bytes, const char* what);
     void* ctx;
 };
-// The binned-SAH topology over n triangle boxes: Morton sort into perm, then
-// the SAH levels (one host round trip each) and the Karras hierarchy inside
-// the remaining segments; children, parents and (optional) leaf ranges as the
-// LBVH emits them.
+// The binned-SAH topology over n >= 2 boxes: Morton sort into perm, then the
+// SAH splits; children, parents and (optional) leaf ranges as the LBVH emits
+// them, and the boxes of every node's children where the splits give them:
+// *boxes_done (device memory) is 1 when every node's boxes were written, 0
+// when the bottom-up refit must compute them.  Up to kSahOneMax items without
+// host round trips, above that usually with one.
 rg_status sah_topology(const ScratchAlloc& tmp, const float* lohi, uint32_t n, const int* cb_ord, int bits,
-                       float4* nodes, uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges);
-// The same, for 2 <= n <= kSahOneMax and bits 10, without host round trips
-// (launch_sah_small); it also writes the node boxes it can, and sets
-// *boxes_done (device memory) as launch_sah_small says.
-rg_status sah_one_topology(const ScratchAlloc& tmp, const float* lohi, uint32_t n, const int* cb_ord, int bits,
-                           float4* nodes, uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges,
-                           uint32_t* boxes_done);
+                       float4* nodes, uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges,
+                       uint32_t* boxes_done);
 
 // wide.cu
 // Collapse a binary LBVH (n leaves) into a compressed 8-wide BVH in one

@@ -1,20 +1,31 @@
-// Binned surface-area-heuristic (SAH) topology of a bottom-level BVH, the
-// build for trace speed (RG_BLAS_SAH).  The triangles start in Morton order
-// (the LBVH's sort); a segment of that order is one subtree.  Level by level,
-// every segment of more than kSahSmall triangles is split by the binned SAH
-// (kSahBins bins of the centroid bounds on each axis, the split of least
-// area(left) * count(left) + area(right) * count(right)), and partitioned
-// stably, so each side keeps its Morton order.  Segments of at most kSahSmall
-// triangles (a pair: one node), and every segment below kSahMaxLevels levels,
-// get the Karras hierarchy of their Morton codes.  (Stopping the SAH at
-// segments of 16 or 4 triangles measured 3-4 % and 1 % slower traversal.)  The internal
-// nodes of a segment of c triangles whose root is node d are d .. d + c - 2
-// (depth-first numbering: left subtree from d + 1, right from d + count(left)),
-// so no allocation is needed and the root is node 0, as in the LBVH.  Every
-// choice comes from atomic minima, maxima and counts, which do not depend on
-// the order of the atomics, and from one thread's fixed-order sweep, so the
-// build is deterministic.  The node boxes are computed afterwards by the
-// LBVH's bottom-up refit.
+// Binned surface-area-heuristic (SAH) topology: the trace-speed build of a
+// bottom-level BVH (RG_BLAS_SAH) and of a TLAS of up to kSahOneMax instances
+// (RG_SCENE_SAH_TLAS).  The items start in Morton order (the LBVH's sort); a
+// segment of that order is one subtree.  Level by level, every segment of more
+// than two items is split by the binned SAH (kSahBins bins of the centroid
+// bounds on each axis, the split of least area(left) * count(left) +
+// area(right) * count(right)), and partitioned stably, so each side keeps its
+// Morton order.  Every segment below kSahMaxLevels levels gets the Karras
+// hierarchy of its Morton codes.  (Stopping the SAH at segments of 16 or 4
+// triangles measured 3-4 % and 1 % slower traversal.)  The internal nodes of a
+// segment of c items whose root is node d are d .. d + c - 2 (depth-first
+// numbering: left subtree from d + 1, right from d + count(left)), so no
+// allocation is needed and the root is node 0, as in the LBVH.  Every choice
+// comes from atomic minima, maxima and counts, which do not depend on the
+// order of the atomics, so the build is deterministic.
+//
+// Three ways of splitting, by segment size, all on the device:
+//   more than kSahMid items: three launches per level over all such segments
+//     (bins, splits, partition), blocks of kSahChunk positions;
+//   kSahTiny + 1 .. kSahMid items: a block per segment builds its levels in
+//     shared memory (k_sah_block);
+//   at most kSahTiny items: a warp per segment builds it to the end
+//     (k_sah_tiny), an item a lane.
+// Bound by latency: the levels are a serial chain, and a level of one block
+// waits on its barriers and atomics, not on memory.  The splits' bins also
+// give the exact boxes of both children, which are written into the node; only
+// position halvings (no valid split), Karras segments and NaN boxes leave the
+// boxes to the bottom-up refit, which the build then asks for.
 #include <algorithm>
 #include <climits>
 #include <atomic>
@@ -31,8 +42,9 @@ namespace {
 constexpr int kBinVals = 7;  // per bin: count, box lo (3), box hi (3) as ordered ints
 constexpr int kTaskBins = 3 * kSahBins * kBinVals;
 constexpr int kTaskAcc = 6 + kTaskBins;  // centroid bounds (lo 3, hi 3), then the bins
-static_assert(kTaskAcc == (int)kSahAccInts, "per-task accumulator size");
+constexpr int kAcc = (kTaskAcc + 3) & ~3;  // a segment's accumulators, padded to 16 bytes
 constexpr int kSahBlock = 256;
+constexpr int kSahItems = (int)kSahChunk / kSahBlock;  // consecutive positions of a thread
 
 __device__ __forceinline__ float centroid_of(const float* __restrict__ lohi, uint32_t prim, int a) {
     return __fmul_rn(0.5f, __fadd_rn(lohi[6 * (size_t)prim + a], lohi[6 * (size_t)prim + 3 + a]));
@@ -49,412 +61,69 @@ __device__ __forceinline__ int bin_of(float c, float cmin, float scale) {
 __device__ __forceinline__ int ord_inf() { return f2ord(__int_as_float(0x7F800000)); }
 __device__ __forceinline__ int ord_ninf() { return f2ord(__int_as_float(0xFF800000)); }
 
-// The chunk of positions block b works on: [chunk begin, end).
-__device__ __forceinline__ void chunk_of(const SahTask* tasks, const uint2* blk, uint32_t b, uint32_t& t, uint32_t& p0,
-                                         uint32_t& p1) {
-    const uint2 e = blk[b];
-    t = e.x;
-    p0 = e.y;
-    const uint32_t end = tasks[t].begin + tasks[t].count;
-    p1 = min(p0 + kSahChunk, end);
+
+// A segment of more than kSahMid items at its level.
+struct SahTask {
+    uint32_t begin, count, node, first_block;
+};
+// What its split came to.
+struct SahSplit {
+    float cmin, scale;                   // the axis's binning frame
+    int axis, split;                     // axis -1: halved by position
+    uint32_t nl;                         // items on the left
+    uint32_t child[2];                   // next-level task of each side, or kNone
+    uint32_t pad;
+};
+// A segment left to a block or a warp; its items are in buffer `buf`.
+struct SahPending {
+    uint32_t begin, count, node;
+    uint16_t level, buf;
+};
+
+// Counters: per level {tasks, blocks}, then the pending lists' lengths.
+constexpr uint32_t kCntMid = 4 * (kSahMaxLevels + 1), kCntTiny = kCntMid + 1, kCntKarras = kCntMid + 2;
+constexpr uint32_t kCntAll = kCntMid + 4;
+
+// Everything the build's kernels share (device pointers).
+struct SahBuild {
+    const float* lohi;                   // item boxes (lo xyz, hi xyz)
+    uint32_t n;
+    uint32_t* prim[2];                   // item at each position; [0] is the result
+    void* key[2];                        // its Morton code
+    uint32_t* cnt;                       // kCntAll
+    SahTask* tasks[2];                   // of even and odd levels
+    uint2* blk[2];                       // per block of a level: task, first position
+    int* acc[2];                         // per task: centroid bounds and bins
+    SahSplit* split;                     // per task
+    uint32_t *blk_cnt, *blk_off;         // per block: 16 bin counts per axis; left items before it
+    SahPending *mid, *tiny;
+    KarrasSeg* karras;
+    float4* nodes;
+    uint32_t *parents, *ranges;          // ranges may be null
+    uint32_t* boxes_done;                // 1 until something leaves boxes to the refit
+};
+
+__device__ __forceinline__ int acc_init(int v) {
+    if (v < 6) return v < 3 ? ord_inf() : ord_ninf();
+    const int w = (v - 6) % kBinVals;
+    return w == 0 ? 0 : (w < 4 ? ord_inf() : ord_ninf());
 }
 
-__global__ void k_sah_init(int* __restrict__ acc, uint32_t m) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m * (uint32_t)kTaskAcc) return;
-    const uint32_t v = i % (uint32_t)kTaskAcc;
-    int x;
-    if (v < 6) {
-        x = v < 3 ? ord_inf() : ord_ninf();
-    } else {
-        const uint32_t w = (v - 6) % kBinVals;
-        x = w == 0 ? 0 : (w < 4 ? ord_inf() : ord_ninf());
-    }
-    acc[i] = x;
+// The binning frame of an axis with centroid bounds lo, hi (scale 0, every
+// centroid in bin 0, when they are a point).
+__device__ __forceinline__ float bin_scale(float lo, float hi) {
+    const float ext = __fsub_rn(hi, lo);
+    return ext > 0.0f ? fminf(__fdiv_rn((float)kSahBins, ext), 3.0e38f) : 0.0f;
 }
 
-// Centroid bounds of each task's segment: a block reduces its chunk, then one
-// atomic per bound.
-__global__ void __launch_bounds__(kSahBlock) k_sah_cbounds(const float* __restrict__ lohi,
-                                                           const uint32_t* __restrict__ prim_at,
-                                                           const SahTask* __restrict__ tasks,
-                                                           const uint2* __restrict__ blk, int* __restrict__ acc) {
-    __shared__ int s[6][kSahBlock / 32];
-    uint32_t t, p0, p1;
-    chunk_of(tasks, blk, blockIdx.x, t, p0, p1);
-    int mn[3] = {ord_inf(), ord_inf(), ord_inf()}, mx[3] = {ord_ninf(), ord_ninf(), ord_ninf()};
-    for (uint32_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        const uint32_t prim = prim_at[p];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const int c = f2ord(centroid_of(lohi, prim, a));
-            mn[a] = min(mn[a], c);
-            mx[a] = max(mx[a], c);
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            mn[a] = min(mn[a], __shfl_xor_sync(0xFFFFFFFFu, mn[a], off));
-            mx[a] = max(mx[a], __shfl_xor_sync(0xFFFFFFFFu, mx[a], off));
-        }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            s[a][warp] = mn[a];
-            s[3 + a][warp] = mx[a];
-        }
-    __syncthreads();
-    if (threadIdx.x < 6) {
-        const int q = threadIdx.x;
-        int v = s[q][0];
-        for (int w = 1; w < kSahBlock / 32; ++w) v = q < 3 ? min(v, s[q][w]) : max(v, s[q][w]);
-        int* dst = acc + (size_t)t * kTaskAcc + q;
-        if (q < 3)
-            atomicMin(dst, v);
-        else
-            atomicMax(dst, v);
-    }
-}
-
-// Per task: the binning frame of each axis from its centroid bounds (scale 0,
-// every centroid in bin 0, when the bounds are a point on that axis).
-__global__ void k_sah_prep(const int* __restrict__ acc, uint32_t m, SahParam* __restrict__ par) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= m) return;
-    const int* a = acc + (size_t)t * kTaskAcc;
-    SahParam P{};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float lo = ord2f(a[k]), hi = ord2f(a[3 + k]);
-        const float ext = __fsub_rn(hi, lo);
-        P.cmin[k] = lo;
-        P.scale[k] = ext > 0.0f ? fminf(__fdiv_rn((float)kSahBins, ext), 3.0e38f) : 0.0f;
-    }
-    P.axis = -1;
-    par[t] = P;
-}
-
-// Binning: per block in shared memory (count, box of the triangles per bin
-// and axis), then merged into the task's bins once per non-empty bin.
-__global__ void __launch_bounds__(kSahBlock) k_sah_bin(const float* __restrict__ lohi,
-                                                       const uint32_t* __restrict__ prim_at,
-                                                       const SahTask* __restrict__ tasks,
-                                                       const uint2* __restrict__ blk, const SahParam* __restrict__ par,
-                                                       int* __restrict__ acc) {
-    __shared__ int sb[kTaskBins];
-    for (int v = threadIdx.x; v < kTaskBins; v += blockDim.x) {
-        const int w = v % kBinVals;
-        sb[v] = w == 0 ? 0 : (w < 4 ? ord_inf() : ord_ninf());
-    }
-    __syncthreads();
-    uint32_t t, p0, p1;
-    chunk_of(tasks, blk, blockIdx.x, t, p0, p1);
-    const SahParam P = par[t];
-    for (uint32_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        const uint32_t prim = prim_at[p];
-        int lo[3], hi[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lo[k] = f2ord(lohi[6 * (size_t)prim + k]);
-            hi[k] = f2ord(lohi[6 * (size_t)prim + 3 + k]);
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const int b = bin_of(centroid_of(lohi, prim, a), P.cmin[a], P.scale[a]);
-            int* e = sb + (a * kSahBins + b) * kBinVals;
-            atomicAdd(e, 1);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                atomicMin(e + 1 + k, lo[k]);
-                atomicMax(e + 4 + k, hi[k]);
-            }
-        }
-    }
-    __syncthreads();
-    int* g = acc + (size_t)t * kTaskAcc + 6;
-    for (int v = threadIdx.x; v < kTaskBins; v += blockDim.x) {
-        const int w = v % kBinVals;
-        if (sb[v - w] == 0) continue;  // empty bin
-        if (w == 0)
-            atomicAdd(g + v, sb[v]);
-        else if (w < 4)
-            atomicMin(g + v, sb[v]);
-        else
-            atomicMax(g + v, sb[v]);
-    }
+__device__ __forceinline__ unsigned long long split_key(float cost, int a, int s) {
+    return ((unsigned long long)__float_as_uint(cost) << 32) | (uint32_t)(a * (kSahBins - 1) + s - 1);
 }
 
 __device__ __forceinline__ float half_area(const float* lo, const float* hi) {
     const float dx = __fsub_rn(hi[0], lo[0]), dy = __fsub_rn(hi[1], lo[1]), dz = __fsub_rn(hi[2], lo[2]);
     return __fadd_rn(__fadd_rn(__fmul_rn(dx, dy), __fmul_rn(dy, dz)), __fmul_rn(dz, dx));
 }
-
-// Per task (one thread): the split of least SAH cost over the kSahBins - 1
-// bin boundaries of each axis, in a fixed order (axis, then boundary; the
-// first of equal costs wins); without one (every axis' centroids in one bin)
-// the segment is halved by position.  Writes the task's node: its children
-// (a leaf when one side holds one triangle), their parent entries, its leaf
-// range (ranges may be null), and the left count for the host.
-__global__ void k_sah_split(const int* __restrict__ acc, const SahTask* __restrict__ tasks, uint32_t m,
-                            SahParam* __restrict__ par, uint32_t n_leaves, float4* __restrict__ nodes,
-                            uint32_t* __restrict__ parents, uint32_t* __restrict__ ranges,
-                            uint32_t* __restrict__ out_nl) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= m) return;
-    const SahTask T = tasks[t];
-    const int* g = acc + (size_t)t * kTaskAcc + 6;
-    float best = __int_as_float(0x7F800000);
-    int best_axis = -1, best_split = 0;
-    uint32_t best_nl = 0;
-    for (int a = 0; a < 3; ++a) {
-        float rlo[kSahBins][3], rhi[kSahBins][3];
-        uint32_t rc[kSahBins];
-        float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-        uint32_t c = 0;
-        for (int b = kSahBins - 1; b >= 1; --b) {
-            const int* e = g + (a * kSahBins + b) * kBinVals;
-            c += (uint32_t)e[0];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                lo[k] = fminf(lo[k], ord2f(e[1 + k]));
-                hi[k] = fmaxf(hi[k], ord2f(e[4 + k]));
-                rlo[b][k] = lo[k];
-                rhi[b][k] = hi[k];
-            }
-            rc[b] = c;
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lo[k] = INFINITY;
-            hi[k] = -INFINITY;
-        }
-        c = 0;
-        for (int s = 1; s < kSahBins; ++s) {
-            const int* e = g + (a * kSahBins + s - 1) * kBinVals;
-            c += (uint32_t)e[0];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                lo[k] = fminf(lo[k], ord2f(e[1 + k]));
-                hi[k] = fmaxf(hi[k], ord2f(e[4 + k]));
-            }
-            const uint32_t nl = c, nr = rc[s];
-            if (nl == 0 || nr == 0) continue;
-            const float cost = __fadd_rn(__fmul_rn(half_area(lo, hi), (float)nl),
-                                         __fmul_rn(half_area(rlo[s], rhi[s]), (float)nr));
-            if (cost < best) {
-                best = cost;
-                best_axis = a;
-                best_split = s;
-                best_nl = nl;
-            }
-        }
-    }
-    if (best_axis < 0) best_nl = T.count / 2;
-    par[t].axis = best_axis;
-    par[t].split = best_split;
-    par[t].nl = best_nl;
-    out_nl[t] = best_nl;
-    const uint32_t nl = best_nl, nr = T.count - best_nl;
-    const uint32_t left = nl == 1 ? (kLeaf | T.begin) : T.node + 1;
-    const uint32_t right = nr == 1 ? (kLeaf | (T.begin + nl)) : T.node + nl;
-    uint32_t* ch = reinterpret_cast<uint32_t*>(nodes + 4 * (size_t)T.node + 3);
-    ch[0] = left;
-    ch[1] = right;
-    parents[(left & kLeaf) ? (size_t)(n_leaves - 1) + (left & ~kLeaf) : left] = T.node;
-    parents[(right & kLeaf) ? (size_t)(n_leaves - 1) + (right & ~kLeaf) : right] = T.node;
-    if (T.node == 0) parents[0] = kNone;
-    if (ranges) {
-        ranges[2 * (size_t)T.node] = T.begin;
-        ranges[2 * (size_t)T.node + 1] = T.begin + T.count - 1;
-    }
-}
-
-__device__ __forceinline__ bool goes_left(const float* __restrict__ lohi, uint32_t prim, uint32_t p,
-                                          const SahTask& T, const SahParam& P) {
-    if (P.axis < 0) return p - T.begin < P.nl;
-    return bin_of(centroid_of(lohi, prim, P.axis), P.cmin[P.axis], P.scale[P.axis]) < P.split;
-}
-
-// Left-side count of each block's chunk.
-__global__ void __launch_bounds__(kSahBlock) k_sah_part_count(const float* __restrict__ lohi,
-                                                              const uint32_t* __restrict__ prim_at,
-                                                              const SahTask* __restrict__ tasks,
-                                                              const uint2* __restrict__ blk,
-                                                              const SahParam* __restrict__ par,
-                                                              uint32_t* __restrict__ blk_left) {
-    __shared__ uint32_t s[kSahBlock / 32];
-    uint32_t t, p0, p1;
-    chunk_of(tasks, blk, blockIdx.x, t, p0, p1);
-    const SahTask T = tasks[t];
-    const SahParam P = par[t];
-    uint32_t cnt = 0;
-    for (uint32_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) cnt += goes_left(lohi, prim_at[p], p, T, P);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, off);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t v = 0;
-        for (int w = 0; w < kSahBlock / 32; ++w) v += s[w];
-        blk_left[blockIdx.x] = v;
-    }
-}
-
-// Per task (one thread): the left-side count before each of its blocks.
-__global__ void k_sah_part_offsets(const SahTask* __restrict__ tasks, uint32_t m, const uint32_t* __restrict__ blk_left,
-                                   uint32_t* __restrict__ blk_off) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= m) return;
-    const SahTask T = tasks[t];
-    uint32_t off = 0;
-    for (uint32_t b = T.first_block; b < T.first_block + T.n_blocks; ++b) {
-        blk_off[b] = off;
-        off += blk_left[b];
-    }
-}
-
-// Stable partition: a block walks its chunk in order, tile by tile; a left
-// triangle goes to begin + (left triangles before it in the segment), a right
-// one to begin + count(left) + (right triangles before it).
-template <class K>
-__global__ void __launch_bounds__(kSahBlock) k_sah_part_scatter(const float* __restrict__ lohi,
-                                                                const uint32_t* __restrict__ prim_at,
-                                                                const K* __restrict__ key_at,
-                                                                const SahTask* __restrict__ tasks,
-                                                                const uint2* __restrict__ blk,
-                                                                const SahParam* __restrict__ par,
-                                                                const uint32_t* __restrict__ blk_off,
-                                                                uint32_t* __restrict__ prim_out, K* __restrict__ key_out) {
-    __shared__ uint32_t wc[kSahBlock / 32];
-    uint32_t t, p0, p1;
-    chunk_of(tasks, blk, blockIdx.x, t, p0, p1);
-    const SahTask T = tasks[t];
-    const SahParam P = par[t];
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint32_t run = blk_off[blockIdx.x];
-    for (uint32_t tile = p0; tile < p1; tile += kSahBlock) {
-        const uint32_t p = tile + threadIdx.x;
-        const bool valid = p < p1;
-        uint32_t prim = 0;
-        K key = 0;
-        bool left = false;
-        if (valid) {
-            prim = prim_at[p];
-            key = key_at[p];
-            left = goes_left(lohi, prim, p, T, P);
-        }
-        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, left);
-        if (lane == 0) wc[warp] = __popc(bal);
-        __syncthreads();
-        uint32_t before = 0, total = 0;
-        for (uint32_t w = 0; w < kSahBlock / 32; ++w) {
-            if (w < warp) before += wc[w];
-            total += wc[w];
-        }
-        if (valid) {
-            const uint32_t lrank = run + before + __popc(bal & ((1u << lane) - 1u));
-            const uint32_t dest = T.begin + (left ? lrank : P.nl + ((p - T.begin) - lrank));
-            prim_out[dest] = prim;
-            key_out[dest] = key;
-        }
-        run += total;
-        __syncthreads();
-    }
-}
-
-template <class K>
-__global__ void __launch_bounds__(kSahBlock) k_sah_copy_back(const SahTask* __restrict__ tasks,
-                                                             const uint2* __restrict__ blk,
-                                                             const uint32_t* __restrict__ prim_out,
-                                                             const K* __restrict__ key_out,
-                                                             uint32_t* __restrict__ prim_at, K* __restrict__ key_at) {
-    uint32_t t, p0, p1;
-    chunk_of(tasks, blk, blockIdx.x, t, p0, p1);
-    for (uint32_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        prim_at[p] = prim_out[p];
-        key_at[p] = key_out[p];
-    }
-}
-
-template <class K>
-cudaError_t sah_level_t(const SahLevel& L, cudaStream_t s) {
-    const uint32_t tg = (L.m + 127u) / 128u;
-    k_sah_init<<<(L.m * (uint32_t)kTaskAcc + 255u) / 256u, 256, 0, s>>>(L.acc, L.m);
-    k_sah_cbounds<<<L.n_blocks, kSahBlock, 0, s>>>(L.lohi, L.prim_at, L.tasks, L.blk, L.acc);
-    k_sah_prep<<<tg, 128, 0, s>>>(L.acc, L.m, L.par);
-    k_sah_bin<<<L.n_blocks, kSahBlock, 0, s>>>(L.lohi, L.prim_at, L.tasks, L.blk, L.par, L.acc);
-    k_sah_split<<<tg, 128, 0, s>>>(L.acc, L.tasks, L.m, L.par, L.n_leaves, L.nodes, L.parents, L.ranges, L.out_nl);
-    k_sah_part_count<<<L.n_blocks, kSahBlock, 0, s>>>(L.lohi, L.prim_at, L.tasks, L.blk, L.par, L.blk_left);
-    k_sah_part_offsets<<<tg, 128, 0, s>>>(L.tasks, L.m, L.blk_left, L.blk_off);
-    k_sah_part_scatter<K><<<L.n_blocks, kSahBlock, 0, s>>>(L.lohi, L.prim_at, static_cast<const K*>(L.key_at), L.tasks,
-                                                           L.blk, L.par, L.blk_off, L.prim_out,
-                                                           static_cast<K*>(L.key_out));
-    k_sah_copy_back<K><<<L.n_blocks, kSahBlock, 0, s>>>(L.tasks, L.blk, L.prim_out, static_cast<const K*>(L.key_out),
-                                                        L.prim_at, static_cast<K*>(L.key_at));
-    count_launches(9);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- small builds in blocks
-// The same hierarchy for at most kSahOneMax items (a TLAS rebuilt every
-// frame) in three launches after the Morton codes, without host round trips.
-// Phase 1, one block of 1024 threads: the stable Morton sort (an LSD radix
-// sort in shared memory), then levels of splits of the segments of more than
-// kSahSubMax items; the children of at most kSahSubMax
-// items go to a pending list.  Phase 2, a grid of blocks of kSahSubMax
-// threads: each block takes pending segments and builds them to the end.
-// Both keep every item's box in shared memory.  Every choice uses the
-// functions and the order of the level-by-level build above (centroid_of,
-// bin_of, the frames, the bins, the sweep), so the tree is the same.  The
-// split's bins also give the exact boxes of both children (the minima and
-// maxima of their items' boxes), which are written into the node; only
-// position halvings (no valid split) and Karras segments below the depth cap
-// leave boxes to the bottom-up refit, which the build then asks for.
-constexpr uint32_t kSahSubMax = 128;     // items of a phase-2 segment (= its block's threads)
-constexpr uint32_t kSahTopSegs = kSahOneMax / (kSahSubMax + 1) + 1;  // phase-1 segments of a level
-constexpr uint32_t kSahSubSegs = kSahSubMax / 3 + 1;                  // phase-2 segments of a level
-constexpr uint16_t kSegNone = 0xFFFF;
-constexpr int kAcc = (kTaskAcc + 3) & ~3;  // a segment's accumulators in a block, padded to 16 bytes
-
-struct OneSeg {
-    uint16_t begin, count, node, pad;    // block-local first position, items, internal node
-};
-struct OneRes {
-    uint16_t nl;                         // items on the left
-    int8_t axis, split;                  // the split (axis -1: halving by position)
-    float cmin, scale;                   // the axis's binning frame
-    uint16_t child[2];                   // next-level segment of each side, or kSegNone
-};
-struct SahPending {
-    uint32_t begin, count, node, level;  // a segment for phase 2 (global positions)
-};
-
-// Shared state of a block that builds the segments of NMAX items, at most SEGS
-// of them split per level.  Items are named by a block-local index: the box
-// of each, its Morton rank, and the local index at each position.
-template <int NMAX, int SEGS>
-struct BlockSah {
-    float box[NMAX][6];                  // (phase 1's sort uses it as scratch first)
-    uint16_t gr[NMAX];                   // Morton rank of each local index
-    uint16_t idx[2][NMAX];               // local index at each position (two buffers)
-    uint16_t seg_of[NMAX];               // this level's segment of each position, or kSegNone
-    uint16_t excl[NMAX];                 // left items before each position
-    OneSeg seg[2][SEGS];
-    OneRes res[SEGS];
-    alignas(16) int acc[SEGS * kAcc];    // per segment: centroid bounds and bins
-    float par[SEGS * 6];                 // per segment: cmin and scale of each axis
-    unsigned long long best[SEGS];       // per segment: least (cost, candidate)
-    alignas(16) int pat[kAcc];           // the accumulators' initial values of one segment
-    uint32_t m, mnext, npend, wsum[32];
-};
-using BlockTop = BlockSah<kSahOneMax, kSahTopSegs>;
-using BlockSub = BlockSah<kSahSubMax, kSahSubSegs>;
-static_assert(sizeof(BlockTop) <= 227 * 1024 && 3 * sizeof(BlockSub) <= 227 * 1024, "shared memory of the SAH blocks");
-static_assert(kSahOneMax <= 0xFFFFu && kSahOneMax % 1024 == 0, "16-bit positions and whole positions per thread");
-static_assert(kSahOneMax * 6 * sizeof(float) >= kSahOneMax * 6 + 32 * 65 * 4 + 32 * 4, "sort scratch fits the boxes");
 
 // Node `node` over leaves b .. b + c - 1 with nl on the left: its children
 // (a leaf when one side holds one item), their parent entries, its range.
@@ -484,166 +153,470 @@ __device__ __forceinline__ void put_child_boxes(float4* nodes, uint32_t node, co
     f[2] = make_float4(r[2], r[3], r[4], r[5]);
 }
 
-// Keys of a segment through its positions' local indices.
-template <class K>
-struct LocalKeys {
-    const K* keys;
-    const uint16_t* gr;
-    const uint16_t* idx;
-    __device__ __forceinline__ K operator[](int64_t i) const { return keys[gr[idx[i]]]; }
-};
 
-// Stable sort of n <= NMAX 30-bit Morton codes in shared memory: the sorted
-// codes, and the index of each, to keys_out and perm0.  An LSD radix sort, 6
-// bits a pass: a warp ranks its items of one digit by ballots, a block-wide
-// scan of the (digit, warp) counts places them.  The items are padded to NMAX
-// with the largest code (after every real item, which keeps them last).  Item
-// j of (warp w, lane l) is position 128 w + 32 j + l, so a warp's items in
-// (j, lane) order are in position order, and each pass is stable.
-template <int NT, int NMAX>
-__device__ void block_sort_codes(unsigned char* scratch, const uint32_t* __restrict__ codes, uint32_t n,
-                                 uint32_t* keys_out, uint32_t* perm0) {
-    static_assert(NMAX == 4 * NT && NT % 32 == 0, "four items per thread");
-    constexpr int D = 6, R = 1 << D, W = NT / 32, CS = R + 1;  // counters [warp][digit], padded rows
-    uint32_t* kbuf = reinterpret_cast<uint32_t*>(scratch);
-    uint16_t* vbuf = reinterpret_cast<uint16_t*>(kbuf + NMAX);
-    uint32_t* cnt = reinterpret_cast<uint32_t*>(vbuf + NMAX);
-    uint32_t* wtot = cnt + W * CS;
-    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
-    uint32_t k[4], v[4];
+// The least cost over the boundaries of one axis, by 16 lanes: lane s of the
+// group holds bin s (g: the axis's bins); the left side of boundary s is the
+// prefix of bins 0 .. s - 1, the right side the suffix s .. 15, both scanned
+// across the lanes.  All lanes of the warp call; every lane of a group gets its
+// least packed key (cost bits, then the candidate's index a * 15 + s - 1, so
+// the first of equal costs; -0 taken as +0), ~0 if no boundary is valid.  The
+// minima and maxima of each side are exact in any order.
+__device__ __forceinline__ unsigned long long sweep16(const int* g, int a, uint32_t s, bool valid) {
+    const int* e = g + (int)s * kBinVals;
+    int pc = valid ? e[0] : 0, sc = pc;
+    int pv[6], sv[6];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t p = 128u * warp + 32u * j + lane;
-        k[j] = p < n ? codes[p] : 0x3FFFFFFFu;
-        v[j] = p;
+    for (int k = 0; k < 6; ++k) pv[k] = sv[k] = valid ? e[1 + k] : (k < 3 ? ord_inf() : ord_ninf());
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) {
+        const int yc = __shfl_up_sync(0xFFFFFFFFu, pc, d, 16);
+        const int zc = __shfl_down_sync(0xFFFFFFFFu, sc, d, 16);
+        if ((int)s >= d) pc += yc;
+        if ((int)s + d < 16) sc += zc;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, pv[k], d, 16);
+            const int z = __shfl_down_sync(0xFFFFFFFFu, sv[k], d, 16);
+            if ((int)s >= d) pv[k] = k < 3 ? min(pv[k], y) : max(pv[k], y);
+            if ((int)s + d < 16) sv[k] = k < 3 ? min(sv[k], z) : max(sv[k], z);
+        }
     }
-    for (int shift = 0; shift < 30; shift += D) {
-        for (uint32_t i = lane; i < (uint32_t)R; i += 32) cnt[warp * CS + i] = 0;
-        __syncwarp();
-        uint32_t rank[4], dig[4];
+    const int lc = __shfl_up_sync(0xFFFFFFFFu, pc, 1, 16);
+    float lo[3], hi[3], rlo[3], rhi[3];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t d = (k[j] >> shift) & (R - 1);
-            uint32_t peers = 0xFFFFFFFFu;
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = ord2f(__shfl_up_sync(0xFFFFFFFFu, pv[k], 1, 16));
+        hi[k] = ord2f(__shfl_up_sync(0xFFFFFFFFu, pv[3 + k], 1, 16));
+        rlo[k] = ord2f(sv[k]);
+        rhi[k] = ord2f(sv[3 + k]);
+    }
+    unsigned long long key = ~0ull;
+    if (valid && s >= 1u && lc != 0 && sc != 0) {
+        const float cost = __fadd_rn(__fadd_rn(__fmul_rn(half_area(lo, hi), (float)(uint32_t)lc),
+                                               __fmul_rn(half_area(rlo, rhi), (float)(uint32_t)sc)),
+                                     0.0f);
+        if (cost < INFINITY) key = split_key(cost, a, (int)s);
+    }
 #pragma unroll
-            for (int bit = 0; bit < D; ++bit) {
-                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, (d >> bit) & 1u);
-                peers &= ((d >> bit) & 1u) ? bal : ~bal;
+    for (int d = 8; d > 0; d >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, key, d, 16);
+        key = y < key ? y : key;
+    }
+    return key;
+}
+
+// Both children's boxes from the bins of the winning axis; returns the left count.
+__device__ __forceinline__ uint32_t side_boxes(const int* g, int sp, float* l, float* r) {
+    int lb[6], rb[6];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        lb[k] = rb[k] = ord_inf();
+        lb[3 + k] = rb[3 + k] = ord_ninf();
+    }
+    uint32_t nl = 0;
+    for (int b = 0; b < kSahBins; ++b) {
+        const int* e = g + b * kBinVals;
+        int* d = b < sp ? lb : rb;
+        if (b < sp) nl += (uint32_t)e[0];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            d[k] = min(d[k], e[1 + k]);
+            d[3 + k] = max(d[3 + k], e[4 + k]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        l[k] = ord2f(lb[k]);
+        r[k] = ord2f(rb[k]);
+    }
+    return nl;
+}
+
+__device__ __forceinline__ bool has_nan(const float* b) {
+    return b[0] != b[0] || b[1] != b[1] || b[2] != b[2] || b[3] != b[3] || b[4] != b[4] || b[5] != b[5];
+}
+
+__device__ __forceinline__ void push_pending(const SahBuild& B, uint32_t begin, uint32_t count, uint32_t node,
+                                             uint32_t level, uint32_t buf) {
+    const SahPending T{begin, count, node, (uint16_t)level, (uint16_t)buf};
+    if (count <= kSahTiny)
+        B.tiny[atomicAdd(B.cnt + kCntTiny, 1u)] = T;
+    else
+        B.mid[atomicAdd(B.cnt + kCntMid, 1u)] = T;
+}
+
+// The root segment (its centroid bounds cb_ord are known); cnt is zeroed.
+__global__ void k_sah_start(SahBuild B, const int* __restrict__ cb_ord) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *B.boxes_done = 1u;
+    if (B.n <= kSahMid) {
+        if (i == 0) push_pending(B, 0, B.n, 0, 0, 0);
+        return;
+    }
+    const uint32_t chunks = (B.n + kSahChunk - 1) / kSahChunk;
+    if (i == 0) {
+        B.tasks[0][0] = SahTask{0u, B.n, 0u, 0u};
+        B.cnt[0] = 1u;
+        B.cnt[1] = chunks;
+    }
+    for (uint32_t b = i; b < chunks; b += gridDim.x * blockDim.x) B.blk[0][b] = make_uint2(0u, b * kSahChunk);
+    if (i < (uint32_t)kAcc) B.acc[0][i] = i < 6 ? cb_ord[i] : acc_init((int)i);
+}
+
+// Bins of a level: each block its chunk in shared memory (a thread merges its
+// consecutive positions, Morton neighbours, per run of one bin before the
+// atomics), then merged into the task's bins once per non-empty bin; the
+// chunk's counts are kept for the partition.
+__global__ void __launch_bounds__(kSahBlock) k_sah_bin(SahBuild B, uint32_t level) {
+    __shared__ int sb[kTaskBins];
+    __shared__ float s_cmin[3], s_scale[3];
+    const uint32_t cur = level & 1u;
+    if (blockIdx.x >= B.cnt[4 * level + 1]) return;
+    const uint2 e = B.blk[cur][blockIdx.x];
+    const SahTask T = B.tasks[cur][e.x];
+    int* acc = B.acc[cur] + (size_t)e.x * kAcc;
+    for (int v = threadIdx.x; v < kTaskBins; v += kSahBlock) sb[v] = acc_init(v + 6);
+    if (threadIdx.x < 3) {
+        const float lo = ord2f(acc[threadIdx.x]);
+        s_cmin[threadIdx.x] = lo;
+        s_scale[threadIdx.x] = bin_scale(lo, ord2f(acc[3 + threadIdx.x]));
+    }
+    __syncthreads();
+    const uint32_t p0 = e.y + threadIdx.x * kSahItems, p1 = min(e.y + kSahChunk, T.begin + T.count);
+    int rb[3] = {-1, -1, -1}, st[3][7] = {};
+    auto flush = [&](int a) {
+        int* d = sb + (a * kSahBins + rb[a]) * kBinVals;
+        atomicAdd(d, st[a][0]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            atomicMin(d + 1 + k, st[a][1 + k]);
+            atomicMax(d + 4 + k, st[a][4 + k]);
+        }
+    };
+    bool nan = false;
+#pragma unroll
+    for (int j = 0; j < kSahItems; ++j) {
+        if (p0 + j >= p1) break;
+        const uint32_t prim = B.prim[cur][p0 + j];
+        float bx[6];
+        int v[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            bx[k] = B.lohi[6 * (size_t)prim + k];
+            v[k] = f2ord(bx[k]);
+        }
+        nan |= has_nan(bx);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int b = bin_of(centroid_of(bx, 0, a), s_cmin[a], s_scale[a]);
+            if (b == rb[a]) {
+                st[a][0] += 1;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    st[a][1 + k] = min(st[a][1 + k], v[k]);
+                    st[a][4 + k] = max(st[a][4 + k], v[3 + k]);
+                }
+            } else {
+                if (rb[a] >= 0) flush(a);
+                rb[a] = b;
+                st[a][0] = 1;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    st[a][1 + k] = v[k];
+                    st[a][4 + k] = v[3 + k];
+                }
             }
-            const uint32_t before = cnt[warp * CS + d];
-            dig[j] = d;
-            rank[j] = before + __popc(peers & lt);
-            __syncwarp();
-            if ((peers & lt) == 0) cnt[warp * CS + d] = before + __popc(peers);
-            __syncwarp();
         }
-        __syncthreads();
-        // exclusive scan of the counters in (digit, warp) order, two a thread
-        uint32_t e[2], sum = 0;
+    }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t i = 2 * t + h, d = i / W, w = i % W;
-            e[h] = (i < (uint32_t)(R * W)) ? cnt[w * CS + d] : 0u;
-            sum += e[h];
+    for (int a = 0; a < 3; ++a)
+        if (rb[a] >= 0) flush(a);
+    if (nan) *B.boxes_done = 0u;
+    __syncthreads();
+    for (int v = threadIdx.x; v < kTaskBins; v += kSahBlock) {
+        const int w = v % kBinVals;
+        if (w == 0) B.blk_cnt[(size_t)blockIdx.x * (3 * kSahBins) + v / kBinVals] = (uint32_t)sb[v];
+        if (sb[v - w] == 0) continue;  // empty bin
+        if (w == 0)
+            atomicAdd(acc + 6 + v, sb[v]);
+        else if (w < 4)
+            atomicMin(acc + 6 + v, sb[v]);
+        else
+            atomicMax(acc + 6 + v, sb[v]);
+    }
+}
+
+// Splits of a level, a block per task: the split of least cost (axis, then
+// boundary; the first of equal costs), without one (every axis' centroids in
+// one bin) the halves by position; the node and its children's boxes; what
+// becomes of the children; and the left items before each block of the task.
+constexpr int kSplitBlock = 128;
+__global__ void __launch_bounds__(kSplitBlock) k_sah_split(SahBuild B, uint32_t level) {
+    __shared__ int sb[kTaskBins];
+    __shared__ unsigned long long s_best;
+    __shared__ SahSplit s_split;
+    __shared__ SahTask s_child[2];
+    __shared__ uint32_t s_warp[kSplitBlock / 32];
+    const uint32_t cur = level & 1u, nxt = cur ^ 1u, t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    if (blockIdx.x >= B.cnt[4 * level]) return;
+    const SahTask T = B.tasks[cur][blockIdx.x];
+    const int* acc = B.acc[cur] + (size_t)blockIdx.x * kAcc;
+    for (int v = t; v < kTaskBins; v += kSplitBlock) sb[v] = acc[6 + v];
+    if (t == 0) s_best = ~0ull;
+    __syncthreads();
+    if (t < 64) {
+        const int a = (int)(t >> 4);
+        const unsigned long long key = sweep16(sb + min(a, 2) * kSahBins * kBinVals, a, t & 15u, a < 3);
+        if ((t & 15u) == 0u && key != ~0ull) atomicMin(&s_best, key);
+    }
+    __syncthreads();
+    if (t == 0) {
+        SahSplit R{};
+        R.axis = -1;
+        R.nl = T.count / 2;
+        if (s_best != ~0ull) {
+            const uint32_t c = (uint32_t)s_best;
+            R.axis = (int)(c / (kSahBins - 1));
+            R.split = (int)(c % (kSahBins - 1)) + 1;
+            float l[6], r[6];
+            R.nl = side_boxes(sb + R.axis * kSahBins * kBinVals, R.split, l, r);
+            put_child_boxes(B.nodes, T.node, l, r);
+            R.cmin = ord2f(acc[R.axis]);
+            R.scale = bin_scale(R.cmin, ord2f(acc[3 + R.axis]));
+        } else {
+            *B.boxes_done = 0u;
         }
-        uint32_t inc = sum;
+        emit_sah_node(T.node, T.begin, T.count, R.nl, B.n, B.nodes, B.parents, B.ranges);
+        for (int side = 0; side < 2; ++side) {
+            const uint32_t b = side ? T.begin + R.nl : T.begin, c = side ? T.count - R.nl : R.nl;
+            const uint32_t nd = side ? T.node + R.nl : T.node + 1;
+            R.child[side] = kNone;
+            s_child[side] = SahTask{b, c, nd, 0u};
+            if (c >= 3 && level + 1 >= kSahMaxLevels) {  // (level kSahMaxLevels is even: its items are in buffer 0)
+                B.karras[atomicAdd(B.cnt + kCntKarras, 1u)] = KarrasSeg{b, c, nd, 0u};
+                *B.boxes_done = 0u;
+            } else if (c <= kSahMid) {
+                push_pending(B, b, c, nd, level + 1, nxt);
+            } else {
+                const uint32_t slot = atomicAdd(B.cnt + 4 * (level + 1), 1u);
+                s_child[side].first_block =
+                    atomicAdd(B.cnt + 4 * (level + 1) + 1, (c + kSahChunk - 1) / kSahChunk);
+                B.tasks[nxt][slot] = s_child[side];
+                R.child[side] = slot;
+            }
+        }
+        s_split = R;
+        B.split[blockIdx.x] = R;
+    }
+    __syncthreads();
+    const SahSplit R = s_split;
+    for (int side = 0; side < 2; ++side) {
+        if (R.child[side] == kNone) continue;
+        const SahTask C = s_child[side];
+        int* ca = B.acc[nxt] + (size_t)R.child[side] * kAcc;
+        for (int v = t; v < kAcc; v += kSplitBlock) ca[v] = acc_init(v);
+        const uint32_t chunks = (C.count + kSahChunk - 1) / kSahChunk;
+        for (uint32_t b = t; b < chunks; b += kSplitBlock)
+            B.blk[nxt][C.first_block + b] = make_uint2(R.child[side], C.begin + b * kSahChunk);
+    }
+    const uint32_t chunks = (T.count + kSahChunk - 1) / kSahChunk;
+    uint32_t carry = 0;
+    for (uint32_t b0 = 0; b0 < chunks; b0 += kSplitBlock) {
+        const uint32_t b = b0 + t;
+        uint32_t left = 0;
+        if (b < chunks) {
+            if (R.axis < 0) {
+                const uint32_t o = b * kSahChunk;
+                left = R.nl > o ? min(R.nl - o, kSahChunk) : 0u;
+            } else {
+                const uint32_t* c = B.blk_cnt + (size_t)(T.first_block + b) * (3 * kSahBins) + R.axis * kSahBins;
+                for (int q = 0; q < R.split; ++q) left += c[q];
+            }
+        }
+        uint32_t inc = left;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, off);
             if ((int)lane >= off) inc += y;
         }
-        if (lane == 31) wtot[warp] = inc;
+        if (lane == 31) s_warp[warp] = inc;
         __syncthreads();
-        if (warp == 0) {
-            const uint32_t x = lane < (uint32_t)W ? wtot[lane] : 0u;
-            uint32_t winc = x;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, winc, off);
-                if ((int)lane >= off) winc += y;
-            }
-            if (lane < (uint32_t)W) wtot[lane] = winc - x;
+        uint32_t before = carry, total = 0;
+        for (uint32_t w = 0; w < kSplitBlock / 32; ++w) {
+            if (w < warp) before += s_warp[w];
+            total += s_warp[w];
         }
-        __syncthreads();
-        uint32_t run = wtot[warp] + inc - sum;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t i = 2 * t + h, d = i / W, w = i % W;
-            if (i < (uint32_t)(R * W)) cnt[w * CS + d] = run;
-            run += e[h];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t dst = cnt[warp * CS + dig[j]] + rank[j];
-            kbuf[dst] = k[j];
-            vbuf[dst] = (uint16_t)v[j];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t p = 128u * warp + 32u * j + lane;
-            k[j] = kbuf[p];
-            v[j] = vbuf[p];
-        }
+        if (b < chunks) B.blk_off[T.first_block + b] = before + inc - left;
+        carry += total;
         __syncthreads();
     }
+}
+
+// Stable partition of a level into the other buffer; the centroid bounds of
+// the children that are split at the next level.
+template <class K>
+__global__ void __launch_bounds__(kSahBlock) k_sah_scatter(SahBuild B, uint32_t level) {
+    __shared__ uint32_t s_warp[kSahBlock / 32];
+    __shared__ int s_cb[2][6];
+    const uint32_t cur = level & 1u, nxt = cur ^ 1u, t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    if (blockIdx.x >= B.cnt[4 * level + 1]) return;
+    const uint2 e = B.blk[cur][blockIdx.x];
+    const SahTask T = B.tasks[cur][e.x];
+    const SahSplit R = B.split[e.x];
+    const K* key_in = static_cast<const K*>(B.key[cur]);
+    K* key_out = static_cast<K*>(B.key[nxt]);
+    if (t < 12) s_cb[t / 6][t % 6] = acc_init((int)(t % 6));
+    const uint32_t p0 = e.y + t * kSahItems, p1 = min(e.y + kSahChunk, T.begin + T.count);
+    uint32_t prim[kSahItems], mine = 0;
+    K key[kSahItems];
+    bool left[kSahItems];
+    int mn[2][3], mx[2][3];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t p = 128u * warp + 32u * j + lane;
-        if (p < n) {
-            keys_out[p] = k[j];
-            perm0[p] = v[j];
+    for (int k = 0; k < 3; ++k) {
+        mn[0][k] = mn[1][k] = ord_inf();
+        mx[0][k] = mx[1][k] = ord_ninf();
+    }
+#pragma unroll
+    for (int j = 0; j < kSahItems; ++j) {
+        left[j] = false;
+        if (p0 + j >= p1) continue;
+        prim[j] = B.prim[cur][p0 + j];
+        key[j] = key_in[p0 + j];
+        float c[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) c[k] = centroid_of(B.lohi, prim[j], k);
+        const float ca = R.axis == 0 ? c[0] : (R.axis == 1 ? c[1] : c[2]);
+        left[j] = R.axis < 0 ? (p0 + j - T.begin < R.nl) : bin_of(ca, R.cmin, R.scale) < R.split;
+        mine += left[j];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int v = f2ord(c[k]);
+            if (left[j]) {
+                mn[0][k] = min(mn[0][k], v);
+                mx[0][k] = max(mx[0][k], v);
+            } else {
+                mn[1][k] = min(mn[1][k], v);
+                mx[1][k] = max(mx[1][k], v);
+            }
+        }
+    }
+    uint32_t inc = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+        if ((int)lane >= off) inc += y;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    uint32_t run = B.blk_off[blockIdx.x] + inc - mine;
+    for (uint32_t w = 0; w < warp; ++w) run += s_warp[w];
+#pragma unroll
+    for (int j = 0; j < kSahItems; ++j) {
+        if (p0 + j >= p1) break;
+        const uint32_t dest = T.begin + (left[j] ? run : R.nl + ((p0 + j - T.begin) - run));
+        run += left[j];
+        B.prim[nxt][dest] = prim[j];
+        key_out[dest] = key[j];
+    }
+    if (R.child[0] == kNone && R.child[1] == kNone) return;
+#pragma unroll
+    for (int side = 0; side < 2; ++side)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int a = __reduce_min_sync(0xFFFFFFFFu, mn[side][k]);
+            const int b = __reduce_max_sync(0xFFFFFFFFu, mx[side][k]);
+            if (lane == 0) {
+                atomicMin(&s_cb[side][k], a);
+                atomicMax(&s_cb[side][3 + k], b);
+            }
+        }
+    __syncthreads();
+    if (t < 12) {
+        const int side = (int)t / 6, k = (int)t % 6;
+        if (R.child[side] != kNone) {
+            int* d = B.acc[nxt] + (size_t)R.child[side] * kAcc + k;
+            if (k < 3)
+                atomicMin(d, s_cb[side][k]);
+            else
+                atomicMax(d, s_cb[side][k]);
         }
     }
 }
 
-// Builds the segment of cnt items at global positions base .. base + cnt - 1,
-// rooted at internal node `node` at depth level0.  With stop > 0, children of
-// at most `stop` items go to the pending list instead of being split here.
-// The Morton rank at position base + i is base + i (phase 1) or rank_g's.
-// perm0 and keys may be written earlier in the same launch: no read-only
-// loads through them.
-template <int NT, int NMAX, int SEGS>
-__device__ void sah_block(BlockSah<NMAX, SEGS>& S, const float* __restrict__ lohi, uint32_t n_leaves,
-                          const uint32_t* keys, const uint32_t* perm0, uint32_t* rank_g, uint32_t base, uint32_t cnt,
-                          uint32_t node, uint32_t level0, uint32_t stop, bool ranks_identity, SahPending* pending,
-                          uint32_t* n_pending, float4* nodes, uint32_t* parents, uint32_t* ranges,
-                          uint32_t* boxes_done) {
+// ---------------------------------------------------------------- segments in a block
+constexpr uint16_t kSegNone = 0xFFFF;
+
+struct OneSeg {
+    uint16_t begin, count, node, pad;    // block-local first position, items, internal node past the segment's
+};
+struct OneRes {
+    uint16_t nl;                         // items on the left
+    int8_t axis, split;                  // the split (axis -1: halving by position)
+    float cmin, scale;                   // the axis's binning frame
+    uint16_t child[2];                   // next-level segment of each side, or kSegNone
+};
+
+// Shared state of a block that builds a segment of up to NMAX items, at most
+// SEGS subsegments split per level.  Items are named by their position in the
+// segment as it came: the box of each, and the item at each position now.
+template <int NMAX, int SEGS>
+struct BlockSah {
+    float box[NMAX][6];
+    uint16_t idx[2][NMAX];               // item at each position (two buffers)
+    uint16_t seg_of[NMAX];               // this level's segment of each position, or kSegNone
+    uint16_t excl[NMAX];                 // left items before each position
+    OneSeg seg[2][SEGS];
+    OneRes res[SEGS];
+    alignas(16) int acc[SEGS * kAcc];    // per segment: centroid bounds and bins
+    float par[SEGS * 6];                 // per segment: cmin and scale of each axis
+    unsigned long long best[SEGS];       // per segment: least (cost, candidate)
+    alignas(16) int pat[kAcc];           // the accumulators' initial values of one segment
+    uint32_t m, mnext, wsum[32];
+};
+constexpr int kMidThreads = 256, kTopThreads = 1024;
+using BlockMid = BlockSah<(int)kSahMid, (int)(kSahMid / (kSahTiny + 1) + 1)>;
+using BlockTop = BlockSah<(int)kSahOneMax, (int)(kSahOneMax / (kSahMid + 1) + 1)>;
+static_assert(sizeof(BlockTop) <= 227 * 1024 && 4 * (sizeof(BlockMid) + 1024) <= 227 * 1024, "shared memory of the SAH blocks");
+static_assert(kSahOneMax <= 0xFFFFu, "16-bit positions");
+
+// Keys of a segment through its positions' items.
+template <class K>
+struct LocalKeys {
+    const K* keys;
+    const uint16_t* idx;
+    __device__ __forceinline__ K operator[](int64_t i) const { return keys[idx[i]]; }
+};
+
+// Builds segment T to the end, or with subsegments of at most `stop` items left
+// to the pending lists; the final order of its items and codes goes to buffer 0
+// (the buffers' contents may be in place: every read comes before the writes).
+template <int NT, int NMAX, int SEGS, class K>
+__device__ void sah_block(BlockSah<NMAX, SEGS>& S, const SahBuild& B, const SahPending T, uint32_t stop) {
+    const uint32_t base = T.begin, cnt = T.count;
+    const uint32_t* src = B.prim[T.buf];
+    const K* skey = static_cast<const K*>(B.key[T.buf]);
+    float4* nodes = B.nodes;
     constexpr uint32_t P = (NMAX + NT - 1) / NT;  // positions per thread in the partition's scan
     constexpr int W = NT / 32;
-    constexpr bool kByShuffle = NT >= 512;       // the sweep: 16-lane groups, else a thread per axis
     const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+    bool nan = false;
     for (uint32_t i = t; i < cnt; i += NT) {
-        const uint32_t r = ranks_identity ? base + i : rank_g[base + i];
-        const uint32_t prim = perm0[r];
-        S.gr[i] = (uint16_t)r;
+        const uint32_t prim = src[base + i];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) S.box[i][k] = lohi[6 * (size_t)prim + k];
+        for (int k = 0; k < 6; ++k) S.box[i][k] = B.lohi[6 * (size_t)prim + k];
+        nan |= has_nan(S.box[i]);
         S.idx[0][i] = (uint16_t)i;
         S.seg_of[i] = 0;
     }
-    for (uint32_t w = t; w < (uint32_t)kAcc; w += NT) {
-        int x;
-        if (w >= (uint32_t)kTaskAcc) {
-            x = 0;
-        } else if (w < 6) {
-            x = w < 3 ? ord_inf() : ord_ninf();
-        } else {
-            const uint32_t u = (w - 6) % kBinVals;
-            x = u == 0 ? 0 : (u < 4 ? ord_inf() : ord_ninf());
-        }
-        S.pat[w] = x;
-    }
+    if (nan) *B.boxes_done = 0u;
+    for (uint32_t w = t; w < (uint32_t)kAcc; w += NT) S.pat[w] = w < (uint32_t)kTaskAcc ? acc_init((int)w) : 0;
     if (t == 0) {
-        S.seg[0][0] = OneSeg{0, (uint16_t)cnt, (uint16_t)node, 0};
+        S.seg[0][0] = OneSeg{0, (uint16_t)cnt, 0, 0};
         S.m = 1;
-        S.npend = 0;
     }
     __syncthreads();
     int cb = 0;
-    for (uint32_t level = level0;; ++level) {
+    for (uint32_t level = T.level;; ++level) {
         const uint32_t m = S.m;
         if (m == 0) break;
         OneSeg* cur = S.seg[cb];
@@ -726,9 +699,8 @@ __device__ void sah_block(BlockSah<NMAX, SEGS>& S, const float* __restrict__ loh
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const float lo = ord2f(a[k]), hi = ord2f(a[3 + k]);
-                const float ext = __fsub_rn(hi, lo);
                 S.par[6 * q + k] = lo;
-                S.par[6 * q + 3 + k] = ext > 0.0f ? fminf(__fdiv_rn((float)kSahBins, ext), 3.0e38f) : 0.0f;
+                S.par[6 * q + 3 + k] = bin_scale(lo, hi);
             }
             S.best[q] = ~0ull;
         }
@@ -793,115 +765,15 @@ __device__ void sah_block(BlockSah<NMAX, SEGS>& S, const float* __restrict__ loh
             }
         }
         __syncthreads();
-        // the least cost over the candidates (axis a, boundary s) of each
-        // segment, first in the candidates' order among equal costs: a packed
-        // key (cost bits, then the candidate's index a * 15 + s - 1; -0 taken
-        // as +0).  The minima and maxima of each side are exact in any order
-        // (a float and an ordered-int fold may differ only in the sign of a
-        // zero, which reaches the cost only as the sign of a zero cost), so
-        // the choice is the level-by-level sweep's.
-        if (kByShuffle) {
-            // 16-lane groups, one per (segment, axis): lane s holds bin s; the
-            // left side of boundary s is the prefix of bins 0 .. s - 1, the
-            // right side the suffix s .. 15, both scanned across the lanes
+        // the least cost of each segment, 16 lanes per (segment, axis)
         for (uint32_t v = t; v < ((m * 48u + 31u) & ~31u); v += NT) {
-            const uint32_t g = v >> 4, s = v & 15u;
+            const uint32_t g = v >> 4;
             const bool valid = g < m * 3u;
             const uint32_t q = valid ? g / 3u : 0u;
             const int a = valid ? (int)(g % 3u) : 0;
-            const int* e = S.acc + (size_t)q * kAcc + 6 + (a * kSahBins + (int)s) * kBinVals;
-            int pc = valid ? e[0] : 0, sc = pc;
-            int pv[6], sv[6];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) pv[k] = sv[k] = valid ? e[1 + k] : (k < 3 ? ord_inf() : ord_ninf());
-#pragma unroll
-            for (int d = 1; d < 16; d <<= 1) {
-                const int yc = __shfl_up_sync(0xFFFFFFFFu, pc, d, 16);
-                const int zc = __shfl_down_sync(0xFFFFFFFFu, sc, d, 16);
-                if ((int)s >= d) pc += yc;
-                if ((int)s + d < 16) sc += zc;
-#pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    const int y = __shfl_up_sync(0xFFFFFFFFu, pv[k], d, 16);
-                    const int z = __shfl_down_sync(0xFFFFFFFFu, sv[k], d, 16);
-                    if ((int)s >= d) pv[k] = k < 3 ? min(pv[k], y) : max(pv[k], y);
-                    if ((int)s + d < 16) sv[k] = k < 3 ? min(sv[k], z) : max(sv[k], z);
-                }
-            }
-            const int lc = __shfl_up_sync(0xFFFFFFFFu, pc, 1, 16);
-            float lo[3], hi[3], rlo[3], rhi[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                lo[k] = ord2f(__shfl_up_sync(0xFFFFFFFFu, pv[k], 1, 16));
-                hi[k] = ord2f(__shfl_up_sync(0xFFFFFFFFu, pv[3 + k], 1, 16));
-                rlo[k] = ord2f(sv[k]);
-                rhi[k] = ord2f(sv[3 + k]);
-            }
-            unsigned long long key = ~0ull;
-            if (valid && s >= 1u && lc != 0 && sc != 0) {
-                const float cost = __fadd_rn(__fadd_rn(__fmul_rn(half_area(lo, hi), (float)(uint32_t)lc),
-                                                       __fmul_rn(half_area(rlo, rhi), (float)(uint32_t)sc)),
-                                             0.0f);
-                if (cost < INFINITY)
-                    key = ((unsigned long long)__float_as_uint(cost) << 32) | (uint32_t)(a * (kSahBins - 1) + (int)s - 1);
-            }
-#pragma unroll
-            for (int d = 8; d > 0; d >>= 1) {
-                const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, key, d, 16);
-                key = y < key ? y : key;
-            }
-            if (valid && s == 0u && key != ~0ull) atomicMin(&S.best[q], key);
-        }
-        } else {
-            // a thread per (segment, axis): the sweep's suffix and prefix folds
-            for (uint32_t v = t; v < m * 3u; v += NT) {
-                const uint32_t q = v / 3u;
-                const int a = (int)(v % 3u);
-                const int* g = S.acc + (size_t)q * kAcc + 6 + a * kSahBins * kBinVals;
-                float rlo[kSahBins][3], rhi[kSahBins][3];
-                uint32_t rc[kSahBins];
-                float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-                uint32_t c = 0;
-#pragma unroll
-                for (int b = kSahBins - 1; b >= 1; --b) {
-                    const int* e = g + b * kBinVals;
-                    c += (uint32_t)e[0];
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        lo[k] = fminf(lo[k], ord2f(e[1 + k]));
-                        hi[k] = fmaxf(hi[k], ord2f(e[4 + k]));
-                        rlo[b][k] = lo[k];
-                        rhi[b][k] = hi[k];
-                    }
-                    rc[b] = c;
-                }
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    lo[k] = INFINITY;
-                    hi[k] = -INFINITY;
-                }
-                c = 0;
-                unsigned long long best = ~0ull;
-#pragma unroll
-                for (int s = 1; s < kSahBins; ++s) {
-                    const int* e = g + (s - 1) * kBinVals;
-                    c += (uint32_t)e[0];
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        lo[k] = fminf(lo[k], ord2f(e[1 + k]));
-                        hi[k] = fmaxf(hi[k], ord2f(e[4 + k]));
-                    }
-                    if (c == 0 || rc[s] == 0) continue;
-                    const float cost = __fadd_rn(__fadd_rn(__fmul_rn(half_area(lo, hi), (float)c),
-                                                           __fmul_rn(half_area(rlo[s], rhi[s]), (float)rc[s])),
-                                                 0.0f);
-                    if (!(cost < INFINITY)) continue;
-                    const unsigned long long key = ((unsigned long long)__float_as_uint(cost) << 32) |
-                                                   (uint32_t)(a * (kSahBins - 1) + s - 1);
-                    best = key < best ? key : best;
-                }
-                if (best != ~0ull) atomicMin(&S.best[q], best);
-            }
+            const unsigned long long key =
+                sweep16(S.acc + (size_t)q * kAcc + 6 + a * kSahBins * kBinVals, a, v & 15u, valid);
+            if (valid && (v & 15u) == 0u && key != ~0ull) atomicMin(&S.best[q], key);
         }
         __syncthreads();
         // the split of each segment, its node, and its children's boxes from
@@ -917,42 +789,20 @@ __device__ void sah_block(BlockSah<NMAX, SEGS>& S, const float* __restrict__ loh
             if (key != ~0ull) {
                 const uint32_t c = (uint32_t)key;
                 const int a = (int)(c / (kSahBins - 1)), sp = (int)(c % (kSahBins - 1)) + 1;
-                const int* g = S.acc + (size_t)q * kAcc + 6 + a * kSahBins * kBinVals;
-                int lb[6], rb[6];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    lb[k] = rb[k] = ord_inf();
-                    lb[3 + k] = rb[3 + k] = ord_ninf();
-                }
-                uint32_t nl = 0;
-                for (int b = 0; b < kSahBins; ++b) {
-                    const int* e = g + b * kBinVals;
-                    int* d = b < sp ? lb : rb;
-                    if (b < sp) nl += (uint32_t)e[0];
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        d[k] = min(d[k], e[1 + k]);
-                        d[3 + k] = max(d[3 + k], e[4 + k]);
-                    }
-                }
                 float l[6], r[6];
-#pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    l[k] = ord2f(lb[k]);
-                    r[k] = ord2f(rb[k]);
-                }
-                put_child_boxes(nodes, cur[q].node, l, r);
+                const uint32_t nl = side_boxes(S.acc + (size_t)q * kAcc + 6 + a * kSahBins * kBinVals, sp, l, r);
+                put_child_boxes(nodes, T.node + cur[q].node, l, r);
                 R.axis = (int8_t)a;
                 R.split = (int8_t)sp;
                 R.nl = (uint16_t)nl;
                 R.cmin = S.par[6 * q + a];
                 R.scale = S.par[6 * q + 3 + a];
             } else {
-                *boxes_done = 0u;  // halved by position: the children's boxes come from the refit
+                *B.boxes_done = 0u;  // halved by position: the children's boxes come from the refit
             }
             R.child[0] = R.child[1] = kSegNone;
             S.res[q] = R;
-            emit_sah_node(cur[q].node, base + cur[q].begin, count, R.nl, n_leaves, nodes, parents, ranges);
+            emit_sah_node(T.node + cur[q].node, base + cur[q].begin, count, R.nl, B.n, nodes, B.parents, B.ranges);
         }
         __syncthreads();
         // stable partition: exclusive left counts over the positions (thread t
@@ -1022,17 +872,16 @@ __device__ void sah_block(BlockSah<NMAX, SEGS>& S, const float* __restrict__ loh
                 const uint32_t c = side ? G.count - nl : nl;
                 const uint32_t nd = side ? G.node + nl : G.node + 1;
                 if (c == 2) {
-                    emit_sah_node(nd, base + b, 2, 1, n_leaves, nodes, parents, ranges);
-                    put_child_boxes(nodes, nd, S.box[ix2[b]], S.box[ix2[b + 1]]);
+                    emit_sah_node(T.node + nd, base + b, 2, 1, B.n, nodes, B.parents, B.ranges);
+                    put_child_boxes(nodes, T.node + nd, S.box[ix2[b]], S.box[ix2[b + 1]]);
                 } else if (c >= 3 && level + 1 >= kSahMaxLevels) {
-                    const LocalKeys<uint32_t> ks{keys, S.gr, ix2 + b};
+                    const LocalKeys<K> ks{skey + base, ix2 + b};
                     for (uint32_t i = 0; i + 1 < c; ++i)
-                        karras_node(ks, c, (int64_t)i, reinterpret_cast<uint32_t*>(nodes) + 12, 16, parents, ranges,
-                                    nd, base + b, n_leaves);
-                    *boxes_done = 0u;  // the Karras nodes' boxes come from the refit
-                } else if (c >= 3 && stop > 0 && c <= stop) {
-                    const uint32_t k = atomicAdd(&S.npend, 1u);
-                    pending[k] = SahPending{base + b, c, nd, level + 1};
+                        karras_node(ks, c, (int64_t)i, reinterpret_cast<uint32_t*>(nodes) + 12, 16, B.parents, B.ranges,
+                                    T.node + nd, base + b, B.n);
+                    *B.boxes_done = 0u;  // the Karras nodes' boxes come from the refit
+                } else if (c >= 3 && c <= stop) {
+                    push_pending(B, base + b, c, T.node + nd, level + 1, 0u);
                 } else if (c >= 3) {
                     const uint32_t slot = atomicAdd(&S.mnext, 1u);
                     nxt[slot] = OneSeg{(uint16_t)b, (uint16_t)c, (uint16_t)nd, 0};
@@ -1051,102 +900,253 @@ __device__ void sah_block(BlockSah<NMAX, SEGS>& S, const float* __restrict__ loh
         __syncthreads();
 
     }
-    for (uint32_t p = t; p < cnt; p += NT) rank_g[base + p] = S.gr[S.idx[cb][p]];
-    if (t == 0 && stop > 0) *n_pending = S.npend;
+    uint32_t prim[P];
+    K key[P];
+#pragma unroll
+    for (uint32_t j = 0; j < P; ++j) {
+        const uint32_t p = NT * j + t;
+        if (p >= cnt) continue;
+        const uint32_t i = base + S.idx[cb][p];
+        prim[j] = src[i];
+        key[j] = skey[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t j = 0; j < P; ++j) {
+        const uint32_t p = NT * j + t;
+        if (p >= cnt) continue;
+        B.prim[0][base + p] = prim[j];
+        static_cast<K*>(B.key[0])[base + p] = key[j];
+    }
     __syncthreads();
 }
 
-// Phase 1: the Morton sort, then the splits of the segments of more than
-// kSahSubMax items.
-__global__ void __launch_bounds__(1024, 1) k_sah_top(const float* __restrict__ lohi, uint32_t n,
-                                                     const uint32_t* __restrict__ codes, uint32_t* keys,
-                                                     uint32_t* perm0, uint32_t* rank_g, SahPending* pending,
-                                                     uint32_t* n_pending, float4* nodes, uint32_t* parents,
-                                                     uint32_t* ranges, uint32_t* boxes_done) {
+// A block per pending segment of kSahTiny + 1 .. kSahMid items.
+template <class K>
+__global__ void __launch_bounds__(kMidThreads) k_sah_block(SahBuild B) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    BlockMid& S = *reinterpret_cast<BlockMid*>(sm);
+    const uint32_t m = B.cnt[kCntMid];
+    for (uint32_t k = blockIdx.x; k < m; k += gridDim.x)
+        sah_block<kMidThreads, (int)kSahMid, (int)(kSahMid / (kSahTiny + 1) + 1), K>(S, B, B.mid[k], kSahTiny);
+}
+
+// The tasks left at `level` when the host does not look (n <= kSahOneMax):
+// usually none.
+template <class K>
+__global__ void __launch_bounds__(kTopThreads, 1) k_sah_rest(SahBuild B, uint32_t level) {
     extern __shared__ __align__(16) unsigned char sm[];
     BlockTop& S = *reinterpret_cast<BlockTop*>(sm);
-    block_sort_codes<1024, kSahOneMax>(reinterpret_cast<unsigned char*>(&S.box[0][0]), codes, n, keys, perm0);
-    for (uint32_t p = threadIdx.x; p < n; p += blockDim.x) rank_g[p] = p;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        *n_pending = 0;
-        *boxes_done = 1u;
-        if (n == 2) {
-            emit_sah_node(0, 0, 2, 1, n, nodes, parents, ranges);
-            put_child_boxes(nodes, 0, lohi + 6 * (size_t)perm0[0], lohi + 6 * (size_t)perm0[1]);
+    const uint32_t m = B.cnt[4 * level];
+    for (uint32_t k = blockIdx.x; k < m; k += gridDim.x) {
+        const SahTask T = B.tasks[level & 1u][k];
+        sah_block<kTopThreads, (int)kSahOneMax, (int)(kSahOneMax / (kSahMid + 1) + 1), K>(
+            S, B, SahPending{T.begin, T.count, T.node, (uint16_t)level, (uint16_t)(level & 1u)}, kSahMid);
+    }
+}
+
+// A warp per pending segment of at most kSahTiny items, an item a lane.  A
+// split of few items has few distinct partitions: each lane tries, on each
+// axis, the boundary above its item's bin (the first boundary of every
+// distinct partition is one of these), going over the items of its segment;
+// no bins are kept and the warp meets no block barrier.  Same costs, order of
+// candidates and results as the binned sweep.
+constexpr int kTinyBlock = 128;
+template <class K>
+__global__ void __launch_bounds__(kTinyBlock) k_sah_tiny(SahBuild B) {
+    struct Warp {
+        int box[32][6];                  // ordered ints of each position's box
+        unsigned long long key[32];
+        uint32_t prim[32], bins[32];
+        uint16_t item[32];               // its position in the segment as it came
+    };
+    __shared__ Warp sw[kTinyBlock / 32];
+    Warp& S = sw[threadIdx.x >> 5];
+    const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+    const uint32_t m = B.cnt[kCntTiny], n_warps = gridDim.x * (kTinyBlock / 32);
+    for (uint32_t w = blockIdx.x * (kTinyBlock / 32) + (threadIdx.x >> 5); w < m; w += n_warps) {
+        const SahPending T = B.tiny[w];
+        const uint32_t* src = B.prim[T.buf];
+        const bool valid = lane < T.count;
+        uint32_t prim = 0, item = lane;
+        int bx[6] = {0, 0, 0, 0, 0, 0};
+        if (valid) {
+            prim = src[T.begin + lane];
+            float f[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                f[k] = B.lohi[6 * (size_t)prim + k];
+                bx[k] = f2ord(f[k]);
+            }
+            if (has_nan(f)) *B.boxes_done = 0u;
         }
-        if (n >= 3 && n <= kSahSubMax) {
-            pending[0] = SahPending{0u, n, 0u, 0u};
-            *n_pending = 1;
+        // this lane's segment: positions sb .. sb + sc - 1, root node sn
+        uint32_t sb = 0, sc = valid && T.count > 1 ? T.count : 0u, sn = T.node;
+        for (uint32_t level = T.level;; ++level) {
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 6; ++k) S.box[lane][k] = bx[k];
+            S.item[lane] = (uint16_t)item;
+            __syncwarp();
+            if (sc == 2) {
+                if (lane == sb) {
+                    float l[6], r[6];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) {
+                        l[k] = ord2f(bx[k]);
+                        r[k] = ord2f(S.box[lane + 1][k]);
+                    }
+                    emit_sah_node(sn, T.begin + sb, 2, 1, B.n, B.nodes, B.parents, B.ranges);
+                    put_child_boxes(B.nodes, sn, l, r);
+                }
+                sc = 0;
+            }
+            if (sc >= 3 && level >= kSahMaxLevels) {
+                if (lane == sb) {
+                    const LocalKeys<K> ks{static_cast<const K*>(B.key[T.buf]) + T.begin, S.item + sb};
+                    for (uint32_t i = 0; i + 1 < sc; ++i)
+                        karras_node(ks, sc, (int64_t)i, reinterpret_cast<uint32_t*>(B.nodes) + 12, 16, B.parents,
+                                    B.ranges, sn, T.begin + sb, B.n);
+                    *B.boxes_done = 0u;
+                }
+                sc = 0;
+            }
+            const bool active = sc >= 3;
+            if (!__any_sync(0xFFFFFFFFu, active)) break;
+            // the frame of the segment, and this item's bins
+            int mn[3] = {ord_inf(), ord_inf(), ord_inf()}, mx[3] = {ord_ninf(), ord_ninf(), ord_ninf()};
+            for (uint32_t j = sb; j < sb + sc; ++j) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int c = f2ord(__fmul_rn(0.5f, __fadd_rn(ord2f(S.box[j][k]), ord2f(S.box[j][3 + k]))));
+                    mn[k] = min(mn[k], c);
+                    mx[k] = max(mx[k], c);
+                }
+            }
+            int bin[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float lo = ord2f(mn[k]);
+                bin[k] = bin_of(__fmul_rn(0.5f, __fadd_rn(ord2f(bx[k]), ord2f(bx[3 + k]))), lo,
+                                bin_scale(lo, ord2f(mx[k])));
+            }
+            S.bins[lane] = (uint32_t)(bin[0] | (bin[1] << 8) | (bin[2] << 16));
+            __syncwarp();
+            // both sides of this item's three boundaries
+            int lb[3][6], rb[3][6];
+            uint32_t nl[3] = {0, 0, 0};
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int k = 0; k < 6; ++k) lb[a][k] = rb[a][k] = k < 3 ? ord_inf() : ord_ninf();
+            for (uint32_t j = sb; j < sb + sc; ++j) {
+                int v[6];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) v[k] = S.box[j][k];
+                const uint32_t bj = S.bins[j];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const bool l = (int)((bj >> (8 * a)) & 0xFFu) <= bin[a];
+                    nl[a] += l;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        if (l) {
+                            lb[a][k] = min(lb[a][k], v[k]);
+                            lb[a][3 + k] = max(lb[a][3 + k], v[3 + k]);
+                        } else {
+                            rb[a][k] = min(rb[a][k], v[k]);
+                            rb[a][3 + k] = max(rb[a][3 + k], v[3 + k]);
+                        }
+                    }
+                }
+            }
+            unsigned long long mine = ~0ull;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                if (nl[a] == 0 || nl[a] >= sc) continue;
+                float l[6], r[6];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    l[k] = ord2f(lb[a][k]);
+                    r[k] = ord2f(rb[a][k]);
+                }
+                const float cost = __fadd_rn(__fadd_rn(__fmul_rn(half_area(l, l + 3), (float)nl[a]),
+                                                       __fmul_rn(half_area(r, r + 3), (float)(sc - nl[a]))),
+                                             0.0f);
+                if (!(cost < INFINITY)) continue;
+                const unsigned long long key = split_key(cost, a, bin[a] + 1);
+                mine = key < mine ? key : mine;
+            }
+            S.key[lane] = mine;
+            __syncwarp();
+            unsigned long long best = ~0ull;
+            for (uint32_t j = sb; j < sb + sc; ++j) best = S.key[j] < best ? S.key[j] : best;
+            const bool cut = active && best != ~0ull;
+            const int axis = cut ? (int)((uint32_t)best / (kSahBins - 1)) : -1;
+            const int split = (int)((uint32_t)best % (kSahBins - 1)) + 1;
+            const int ba = axis == 0 ? bin[0] : (axis == 1 ? bin[1] : bin[2]);
+            const bool left = active && (cut ? ba < split : lane - sb < sc / 2);
+            const uint32_t seg = active ? (0xFFFFFFFFu >> (32u - sc)) << sb : 0u;
+            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, left) & seg;
+            const uint32_t own = __ballot_sync(0xFFFFFFFFu, cut && mine == best) & seg;
+            const uint32_t nleft = (uint32_t)__popc(bal);
+            if (cut && (own & lt) == 0u && mine == best) {
+                float l[6], r[6];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    l[k] = ord2f(axis == 0 ? lb[0][k] : (axis == 1 ? lb[1][k] : lb[2][k]));
+                    r[k] = ord2f(axis == 0 ? rb[0][k] : (axis == 1 ? rb[1][k] : rb[2][k]));
+                }
+                put_child_boxes(B.nodes, sn, l, r);
+            }
+            uint32_t dest = lane;
+            if (active) {
+                if (lane == sb) {
+                    emit_sah_node(sn, T.begin + sb, sc, nleft, B.n, B.nodes, B.parents, B.ranges);
+                    if (!cut) *B.boxes_done = 0u;
+                }
+                const uint32_t lr = (uint32_t)__popc(bal & lt);
+                dest = left ? sb + lr : sb + nleft + ((lane - sb) - lr);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 6; ++k) S.box[dest][k] = bx[k];
+            S.prim[dest] = prim;
+            S.item[dest] = (uint16_t)item;
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 6; ++k) bx[k] = S.box[lane][k];
+            prim = S.prim[lane];
+            item = S.item[lane];
+            if (active) {
+                if (lane - sb < nleft) {
+                    sc = nleft;
+                    sn = sn + 1;
+                } else {
+                    sb += nleft;
+                    sc -= nleft;
+                    sn += nleft;
+                }
+                if (sc < 2) sc = 0;
+            }
         }
-    }
-    __syncthreads();
-    if (n <= kSahSubMax) return;
-    sah_block<1024, kSahOneMax, kSahTopSegs>(S, lohi, n, keys, perm0, rank_g, 0, n, 0, 0, kSahSubMax, true, pending,
-                                             n_pending, nodes, parents, ranges, boxes_done);
-}
-
-// Phase 2: each block builds pending segments to the end.
-__global__ void __launch_bounds__(kSahSubMax) k_sah_sub(const float* __restrict__ lohi, uint32_t n,
-                                                        const uint32_t* __restrict__ keys,
-                                                        const uint32_t* __restrict__ perm0, uint32_t* rank_g,
-                                                        const SahPending* __restrict__ pending,
-                                                        const uint32_t* __restrict__ n_pending, float4* nodes,
-                                                        uint32_t* parents, uint32_t* ranges, uint32_t* boxes_done) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    BlockSub& S = *reinterpret_cast<BlockSub*>(sm);
-    const uint32_t np = *n_pending;
-    for (uint32_t k = blockIdx.x; k < np; k += gridDim.x) {
-        const SahPending T = pending[k];
-        sah_block<kSahSubMax, kSahSubMax, kSahSubSegs>(S, lohi, n, keys, perm0, rank_g, T.begin, T.count, T.node,
-                                                       T.level, 0, false, nullptr, nullptr, nodes, parents, ranges,
-                                                       boxes_done);
+        if (valid) B.prim[0][T.begin + lane] = prim;
     }
 }
 
-__global__ void k_sah_gather(const uint32_t* __restrict__ perm0, const uint32_t* __restrict__ rank_g, uint32_t n,
-                             uint32_t* __restrict__ perm_out) {
-    const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) perm_out[p] = perm0[rank_g[p]];
+template <class K>
+cudaError_t set_block_smem() {
+    cudaError_t e = cudaFuncSetAttribute(k_sah_block<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockMid));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_sah_rest<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockTop));
+    return e;
 }
 
-}  // namespace
-
-cudaError_t launch_sah_small(const float* lohi, uint32_t n, const uint32_t* codes, uint32_t* perm_out, float4* nodes,
-                             uint32_t* parents, uint32_t* ranges, const SahSmallScratch& w, cudaStream_t s) {
-    if (n < 2 || n > kSahOneMax) return cudaErrorInvalidValue;
-    static std::atomic<int> attr_set{0};  // per process; concurrent first callers set the same values
-    if (!attr_set.load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(k_sah_top, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sizeof(BlockTop));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_sah_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockSub));
-        if (e != cudaSuccess) return e;
-        attr_set.store(1, std::memory_order_release);
-    }
-    SahPending* pending = static_cast<SahPending*>(w.pending);
-    k_sah_top<<<1, 1024, sizeof(BlockTop), s>>>(lohi, n, codes, w.keys, w.perm0, w.rank, pending, w.n_pending, nodes,
-                                                parents, ranges, w.boxes_done);
-    const uint32_t grid = std::min<uint32_t>((uint32_t)device_sm_count(), n / 3 + 1);
-    k_sah_sub<<<grid, kSahSubMax, sizeof(BlockSub), s>>>(lohi, n, w.keys, w.perm0, w.rank, pending, w.n_pending,
-                                                         nodes, parents, ranges, w.boxes_done);
-    k_sah_gather<<<(n + 255) / 256, 256, 0, s>>>(w.perm0, w.rank, n, perm_out);
-    count_launches(3);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sah_level(const SahLevel& L, int key_bits, cudaStream_t s) {
-    if (L.m == 0) return cudaSuccess;
-    return key_bits == 64 ? sah_level_t<uint64_t>(L, s) : sah_level_t<uint32_t>(L, s);
-}
-
-namespace {
 rg_status sah_cuda_fail(cudaError_t e, const char* what) {
     cudaGetLastError();  // clear a sticky launch error
     return report_error(e == cudaErrorMemoryAllocation ? RG_ERR_OOM : RG_ERR_CUDA,
                         (std::string(what) + ": " + cudaGetErrorString(e)).c_str());
 }
-}  // namespace
 
 #define SAH_CK(call)                                             \
     do {                                                         \
@@ -1154,128 +1154,125 @@ rg_status sah_cuda_fail(cudaError_t e, const char* what) {
         if (e_ != cudaSuccess) return sah_cuda_fail(e_, #call);  \
     } while (0)
 
-// Binned-SAH topology (RG_BLAS_SAH): the LBVH's Morton sort, then
-// levels of SAH splits over the segments of more than kSahSmall triangles
-// (one host round trip per level for the left counts), then the Karras
-// hierarchy inside every remaining segment.  Same outputs as lbvh_topology.
-rg_status sah_topology(const ScratchAlloc& tmp, const float* lohi, uint32_t n, const int* cb_ord, int bits, float4* nodes,
-                       uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges) {
-    const int key_bits = bits == 21 ? 64 : 32;
-    const size_t kb = key_bits / 8;
-    void *codes, *sorted, *scratch;
-    rg_status r;
-    if ((r = tmp.get(tmp.ctx, &codes, n * kb, "morton codes"))) return r;
-    if ((r = tmp.get(tmp.ctx, &sorted, n * kb, "sorted codes"))) return r;
-    if ((r = tmp.get(tmp.ctx, &scratch, radix_sort_scratch_bytes(n, key_bits), "sort scratch"))) return r;
-    SAH_CK(launch_morton(lohi, n, cb_ord, bits, codes, nullptr, s));
-    SAH_CK(radix_sort_pairs(codes, nullptr, n, key_bits, sorted, perm, scratch, s));
-    if (n <= kSahSmall) {
-        SAH_CK(launch_karras(sorted, n, key_bits, reinterpret_cast<uint32_t*>(nodes) + 12, 16, parents, s, ranges));
-        return RG_OK;
+template <class K>
+rg_status sah_build(SahBuild B, const int* cb_ord, cudaStream_t s) {
+    static std::atomic<int> attr_set{0};  // per process; concurrent first callers set the same values
+    if (!attr_set.load(std::memory_order_acquire)) {
+        SAH_CK(set_block_smem<K>());
+        attr_set.store(1, std::memory_order_release);
     }
-    // a level's segments go through the kernels in slices of at most
-    // kSahSliceTasks, which bounds the bins' scratch (1,368 B per segment)
-    const uint32_t max_tasks = std::min(n / (kSahSmall + 1) + 1, kSahSliceTasks);
-    const uint32_t max_blocks = n / kSahChunk + max_tasks;
-    void *prim_out, *key_out, *d_tasks, *d_blk, *acc, *par, *blk_left, *blk_off, *out_nl;
-    if ((r = tmp.get(tmp.ctx, &prim_out, n * 4ull, "SAH positions")) || (r = tmp.get(tmp.ctx, &key_out, n * kb, "SAH keys")) ||
-        (r = tmp.get(tmp.ctx, &d_tasks, (size_t)max_tasks * sizeof(SahTask), "SAH tasks")) ||
-        (r = tmp.get(tmp.ctx, &d_blk, (size_t)max_blocks * sizeof(uint2), "SAH blocks")) ||
-        (r = tmp.get(tmp.ctx, &acc, (size_t)max_tasks * kSahAccInts * 4, "SAH bins")) ||
-        (r = tmp.get(tmp.ctx, &par, (size_t)max_tasks * sizeof(SahParam), "SAH splits")) ||
-        (r = tmp.get(tmp.ctx, &blk_left, (size_t)max_blocks * 4, "SAH block counts")) ||
-        (r = tmp.get(tmp.ctx, &blk_off, (size_t)max_blocks * 4, "SAH block offsets")) ||
-        (r = tmp.get(tmp.ctx, &out_nl, (size_t)max_tasks * 4, "SAH left counts")))
-        return r;
-    std::vector<SahTask> tasks(1);
-    tasks[0] = SahTask{0u, n, 0u, 0u, 0u, {0u, 0u, 0u}};
-    std::vector<KarrasSeg> segs;
-    uint32_t seg_threads = 0;
-    std::vector<uint2> blk;
-    std::vector<uint32_t> nl;
-    std::vector<SahTask> next;
-    for (uint32_t level = 0; !tasks.empty(); ++level) {
-        next.clear();
-        for (size_t t0 = 0; t0 < tasks.size(); t0 += kSahSliceTasks) {
-            const uint32_t m = (uint32_t)std::min(tasks.size() - t0, (size_t)kSahSliceTasks);
-            SahTask* slice = tasks.data() + t0;
-            blk.clear();
-            for (uint32_t t = 0; t < m; ++t) {
-                slice[t].first_block = (uint32_t)blk.size();
-                for (uint32_t p = slice[t].begin; p < slice[t].begin + slice[t].count; p += kSahChunk)
-                    blk.push_back(make_uint2(t, p));
-                slice[t].n_blocks = (uint32_t)blk.size() - slice[t].first_block;
-            }
-            SAH_CK(cudaMemcpyAsync(d_tasks, slice, m * sizeof(SahTask), cudaMemcpyHostToDevice, s));
-            SAH_CK(cudaMemcpyAsync(d_blk, blk.data(), blk.size() * sizeof(uint2), cudaMemcpyHostToDevice, s));
-            SahLevel L{};
-            L.lohi = lohi;
-            L.n_leaves = n;
-            L.m = m;
-            L.n_blocks = (uint32_t)blk.size();
-            L.tasks = static_cast<const SahTask*>(d_tasks);
-            L.blk = static_cast<const uint2*>(d_blk);
-            L.acc = static_cast<int*>(acc);
-            L.par = static_cast<SahParam*>(par);
-            L.prim_at = perm;
-            L.key_at = sorted;
-            L.prim_out = static_cast<uint32_t*>(prim_out);
-            L.key_out = key_out;
-            L.blk_left = static_cast<uint32_t*>(blk_left);
-            L.blk_off = static_cast<uint32_t*>(blk_off);
-            L.out_nl = static_cast<uint32_t*>(out_nl);
-            L.nodes = nodes;
-            L.parents = parents;
-            L.ranges = ranges;
-            SAH_CK(launch_sah_level(L, key_bits, s));
-            nl.resize(m);
-            SAH_CK(cudaMemcpyAsync(nl.data(), out_nl, m * 4ull, cudaMemcpyDeviceToHost, s));
+    const uint32_t n = B.n, sms = (uint32_t)device_sm_count();
+    SAH_CK(cudaMemsetAsync(B.cnt, 0, kCntAll * 4, s));
+    const uint32_t chunks = (n + kSahChunk - 1) / kSahChunk;
+    k_sah_start<<<std::min(chunks / 512u + 1u, 1024u), 512, 0, s>>>(B, cb_ord);
+    count_launches(1);
+    const uint32_t max_tasks = n / (kSahMid + 1) + 1;
+    auto run_level = [&](uint32_t level) {
+        const uint32_t tasks = level < 31 ? std::min(1u << level, max_tasks) : max_tasks;
+        const uint32_t blocks = n / kSahChunk + tasks;
+        k_sah_bin<<<blocks, kSahBlock, 0, s>>>(B, level);
+        k_sah_split<<<tasks, kSplitBlock, 0, s>>>(B, level);
+        k_sah_scatter<K><<<blocks, kSahBlock, 0, s>>>(B, level);
+        count_launches(3);
+    };
+    // levels for a balanced tree and one more; then the host looks whether
+    // large segments are left (small builds leave that to the device)
+    uint32_t levels = 0;
+    if (n > kSahMid) {
+        for (uint32_t c = n; c > kSahMid; c = (c + 1) / 2) ++levels;
+        ++levels;
+        for (uint32_t l = 0; l < levels; ++l) run_level(l);
+    }
+    if (n > kSahOneMax) {
+        uint32_t h[kCntAll];
+        for (;;) {
+            SAH_CK(cudaMemcpyAsync(h, B.cnt, sizeof h, cudaMemcpyDeviceToHost, s));
             SAH_CK(cudaStreamSynchronize(s));
-            auto child = [&](uint32_t b, uint32_t c, uint32_t node) {
-                if (c <= 1) return;
-                if (c <= kSahSmall || level + 1 >= kSahMaxLevels) {
-                    segs.push_back(KarrasSeg{b, c, node, seg_threads});
-                    seg_threads += c - 1;
-                } else {
-                    next.push_back(SahTask{b, c, node, 0u, 0u, {0u, 0u, 0u}});
-                }
-            };
-            for (uint32_t t = 0; t < m; ++t) {
-                const SahTask& T = slice[t];
-                child(T.begin, nl[t], T.node + 1);
-                child(T.begin + nl[t], T.count - nl[t], T.node + nl[t]);
-            }
+            if (levels >= kSahMaxLevels || h[4 * levels] == 0) break;
+            const uint32_t more = std::min(levels + 4, kSahMaxLevels);
+            for (; levels < more; ++levels) run_level(levels);
         }
-        tasks.swap(next);
+        if (h[kCntKarras]) {  // segments of more than kSahMid items at the depth cap
+            std::vector<KarrasSeg> segs(h[kCntKarras]);
+            SAH_CK(cudaMemcpyAsync(segs.data(), B.karras, segs.size() * sizeof(KarrasSeg), cudaMemcpyDeviceToHost, s));
+            SAH_CK(cudaStreamSynchronize(s));
+            uint32_t threads = 0;
+            for (KarrasSeg& g : segs) {
+                g.first = threads;
+                threads += g.count - 1;
+            }
+            SAH_CK(cudaMemcpyAsync(B.karras, segs.data(), segs.size() * sizeof(KarrasSeg), cudaMemcpyHostToDevice, s));
+            SAH_CK(launch_karras_segments(B.key[0], 8 * (int)sizeof(K), B.karras, (uint32_t)segs.size(), threads, n,
+                                          B.nodes, B.parents, B.ranges, s));
+            SAH_CK(cudaStreamSynchronize(s));  // segs is this frame's
+        }
+    } else if (n > kSahMid) {
+        k_sah_rest<K><<<std::min(max_tasks, sms), kTopThreads, sizeof(BlockTop), s>>>(B, levels);
+        count_launches(1);
     }
-    if (!segs.empty()) {
-        void* d_segs;
-        if ((r = tmp.get(tmp.ctx, &d_segs, segs.size() * sizeof(KarrasSeg), "Karras segments"))) return r;
-        SAH_CK(cudaMemcpyAsync(d_segs, segs.data(), segs.size() * sizeof(KarrasSeg), cudaMemcpyHostToDevice, s));
-        SAH_CK(launch_karras_segments(sorted, key_bits, static_cast<const KarrasSeg*>(d_segs), (uint32_t)segs.size(),
-                                     seg_threads, n, nodes, parents, ranges, s));
+    if (n > kSahTiny) {
+        k_sah_block<K><<<std::min(n / (kSahTiny + 1) + 1, 4 * sms), kMidThreads, sizeof(BlockMid), s>>>(B);
+        count_launches(1);
     }
+    k_sah_tiny<K><<<std::min(n / 128u + 1u, 8 * sms), kTinyBlock, 0, s>>>(B);
+    count_launches(1);
+    SAH_CK(cudaGetLastError());
     return RG_OK;
 }
 
+}  // namespace
 
-rg_status sah_one_topology(const ScratchAlloc& tmp, const float* lohi, uint32_t n, const int* cb_ord, int bits,
-                           float4* nodes, uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges,
-                           uint32_t* boxes_done) {
-    if (bits != 10) return report_error(RG_ERR_INVALID_ARG, "the small SAH build takes 30-bit Morton codes");
-    void *codes, *keys, *perm0, *rank, *pending, *n_pending;
+rg_status sah_topology(const ScratchAlloc& tmp, const float* lohi, uint32_t n, const int* cb_ord, int bits, float4* nodes,
+                       uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges, uint32_t* boxes_done) {
+    const int key_bits = bits == 21 ? 64 : 32;
+    const size_t kb = key_bits / 8;
+    const size_t max_tasks = n > kSahMid ? n / (kSahMid + 1) + 1 : 1, max_blocks = n / kSahChunk + max_tasks;
+    // every split leaves at most two pending segments, each of its own items
+    const size_t max_tiny = n, max_mid = n / (kSahTiny + 1) + 1;
+    // one allocation, its parts 256-byte aligned
+    size_t total = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t o_codes = part(n * kb), o_sorted = part(n * kb), o_sort = part(radix_sort_scratch_bytes(n, key_bits));
+    const size_t o_prim = part(n * 4ull), o_key = part(n * kb), o_cnt = part(kCntAll * 4);
+    const size_t o_tasks = part(2 * max_tasks * sizeof(SahTask)), o_blk = part(2 * max_blocks * sizeof(uint2));
+    const size_t o_acc = part(2 * max_tasks * kAcc * 4), o_split = part(max_tasks * sizeof(SahSplit));
+    const size_t o_bc = part(max_blocks * 3 * kSahBins * 4), o_bo = part(max_blocks * 4);
+    const size_t o_mid = part(max_mid * sizeof(SahPending)), o_tiny = part(max_tiny * sizeof(SahPending));
+    const size_t o_karras = part(2 * max_tasks * sizeof(KarrasSeg));
+    void* mem;
     rg_status r;
-    if ((r = tmp.get(tmp.ctx, &codes, n * 4ull, "morton codes"))) return r;
-    if ((r = tmp.get(tmp.ctx, &keys, n * 4ull, "sorted codes"))) return r;
-    if ((r = tmp.get(tmp.ctx, &perm0, n * 4ull, "Morton order"))) return r;
-    if ((r = tmp.get(tmp.ctx, &rank, n * 4ull, "SAH ranks"))) return r;
-    if ((r = tmp.get(tmp.ctx, &pending, (size_t)(n / 3 + 1) * 16, "SAH pending segments"))) return r;
-    if ((r = tmp.get(tmp.ctx, &n_pending, 16, "SAH pending count"))) return r;
-    SahSmallScratch w{static_cast<uint32_t*>(keys), static_cast<uint32_t*>(perm0), static_cast<uint32_t*>(rank),
-                      pending, static_cast<uint32_t*>(n_pending), boxes_done};
-    SAH_CK(launch_morton(lohi, n, cb_ord, bits, codes, nullptr, s));
-    SAH_CK(launch_sah_small(lohi, n, static_cast<const uint32_t*>(codes), perm, nodes, parents, ranges, w, s));
-    return RG_OK;
+    if ((r = tmp.get(tmp.ctx, &mem, total, "SAH build scratch"))) return r;
+    char* m = static_cast<char*>(mem);
+    SAH_CK(launch_morton(lohi, n, cb_ord, bits, m + o_codes, nullptr, s));
+    SAH_CK(radix_sort_pairs(m + o_codes, nullptr, n, key_bits, m + o_sorted, perm, m + o_sort, s));
+    SahBuild B{};
+    B.lohi = lohi;
+    B.n = n;
+    B.prim[0] = perm;
+    B.prim[1] = reinterpret_cast<uint32_t*>(m + o_prim);
+    B.key[0] = m + o_sorted;
+    B.key[1] = m + o_key;
+    B.cnt = reinterpret_cast<uint32_t*>(m + o_cnt);
+    for (int k = 0; k < 2; ++k) {
+        B.tasks[k] = reinterpret_cast<SahTask*>(m + o_tasks) + k * max_tasks;
+        B.blk[k] = reinterpret_cast<uint2*>(m + o_blk) + k * max_blocks;
+        B.acc[k] = reinterpret_cast<int*>(m + o_acc) + k * max_tasks * kAcc;
+    }
+    B.split = reinterpret_cast<SahSplit*>(m + o_split);
+    B.blk_cnt = reinterpret_cast<uint32_t*>(m + o_bc);
+    B.blk_off = reinterpret_cast<uint32_t*>(m + o_bo);
+    B.mid = reinterpret_cast<SahPending*>(m + o_mid);
+    B.tiny = reinterpret_cast<SahPending*>(m + o_tiny);
+    B.karras = reinterpret_cast<KarrasSeg*>(m + o_karras);
+    B.nodes = nodes;
+    B.parents = parents;
+    B.ranges = ranges;
+    B.boxes_done = boxes_done;
+    return key_bits == 64 ? sah_build<uint64_t>(B, cb_ord, s) : sah_build<uint32_t>(B, cb_ord, s);
 }
 
 }  // namespace rg

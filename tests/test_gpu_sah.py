@@ -108,6 +108,47 @@ def test_sah_sizes_around_the_thresholds(nt):
     assert np.array_equal(np.sort(ex["tris"].reshape(nt, 12)[:, 3].view(np.uint32)), np.arange(nt, dtype=np.uint32))
 
 
+def clusters(n, seed):
+    """n small boxes: a third coincident at one point (halved by position), the
+    rest in clusters whose sizes and places span six orders of magnitude."""
+    rng = np.random.default_rng(seed)
+    c = (10.0 ** rng.uniform(-3, 3, (12, 3)))[rng.integers(0, 12, n)]
+    lo = (c * (1 + 0.1 * rng.standard_normal((n, 3)))).astype(np.float32)
+    lo[rng.permutation(n)[:n // 3]] = np.float32(0.25)
+    return boxes_mesh(lo, (lo + np.abs(lo) * np.float32(0.01)).astype(np.float32))
+
+
+@pytest.mark.parametrize("mesh,n", [("ico", k) for k in (31, 32, 33, 511, 512, 513, 1025, 4095, 4096, 4097)] +
+                         [("clusters", k) for k in (32, 512, 700, 4096, 9001)] +
+                         [("chain", k) for k in (600, 5000)])
+@pytest.mark.parametrize("morton", [rg.RG_MORTON30, rg.RG_MORTON63])
+def test_sah_ranges_of_the_build(mesh, n, morton):
+    """Both sides of the sizes at which the build goes over from levels of all
+    segments to a block and to a warp per segment, and to a look by the host;
+    halvings by position; and more than a block's items at level 40.  Order,
+    topology and every box as the oracle has them."""
+    if mesh == "ico":
+        v, i = g.make_mesh("ico", 4)
+        i = i[np.random.default_rng(n).permutation(len(i))[:n]]
+    else:
+        v, i = clusters(n, n) if mesh == "clusters" else chain_to_level_40(42, n)
+    nt = i.shape[0]
+    ex = build(v, i, morton | rg.RG_BLAS_SAH)
+    ref = oracle.sah_reference(v, i, 21 if morton else 10)
+    perm = ex["tris"].reshape(nt, 12)[:, 3].view(np.uint32)
+    assert np.array_equal(perm, ref["perm"])
+    lo0, hi0, lo1, hi1, ch = node_fields(ex["nodes"])
+    assert np.array_equal(ch, ref["child"])
+    first, last = walk(ex, nt)
+    lohi = oracle.tri_bounds(v, i)[perm]
+    for k in range(nt - 1):
+        c0 = int(ch[k][0])
+        split = (c0 & ~LEAF) if c0 & LEAF else last[c0]
+        a, b = lohi[first[k]:split + 1], lohi[split + 1:last[k] + 1]
+        assert np.array_equal(np.r_[lo0[k], hi0[k]], np.r_[a[:, :3].min(0), a[:, 3:].max(0)]), k
+        assert np.array_equal(np.r_[lo1[k], hi1[k]], np.r_[b[:, :3].min(0), b[:, 3:].max(0)]), k
+
+
 def test_sah_cost_below_lbvh_and_deterministic():
     s = g.large_scene()
     v, i = s.meshes[2]                       # 102,400 triangles
