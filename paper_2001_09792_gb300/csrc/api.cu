@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -61,18 +62,73 @@ uint32_t test_limit(const char* name) {
     return x > 0 && x < (1l << 30) ? (uint32_t)x : 0u;
 }
 
+// The pool of the calls' stream-ordered temporaries, one per device, made on
+// first use.  It keeps up to kPoolKeep bytes across synchronisations: the
+// device's default pool keeps none, so that the first temporary after each wait
+// for the GPU cost about 110 us of mapping.  What it keeps is given back
+// when a device allocation of the library runs out of memory.  (Null: the
+// default pool serves.)
+constexpr uint64_t kPoolKeep = 64ull << 20;
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[kMaxDevices] = {};
+
+cudaMemPool_t temp_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pools[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = kPoolKeep;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+        g_pools[dev] = pool;
+    }
+    return g_pools[dev];
+}
+
+// Gives back what the current device's pool holds unused; true if there is one.
+bool trim_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    return g_pools[dev] && cudaMemPoolTrimTo(g_pools[dev], 0) == cudaSuccess;
+}
+
 rg_status dev_alloc(void** p, size_t bytes, const char* what) {
     *p = nullptr;
     long k = ++g_alloc_count;
     if (fault_alloc_index() == k) return fail(RG_ERR_OOM, std::string("injected allocation failure: ") + what);
     if (bytes == 0) bytes = 16;
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && trim_pool()) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         return cuda_fail(e, what);
     }
     return RG_OK;
 }
+
+// Parts of one allocation, each 256-byte aligned: the offset of the next part.
+struct Parts {
+    size_t total = 0;
+    size_t add(size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) & ~(size_t)255;
+        return at;
+    }
+};
 
 struct TempAlloc {
     // stream-ordered temporaries, freed on the stream when the call ends
@@ -86,7 +142,12 @@ struct TempAlloc {
         *p = nullptr;
         long k = ++g_alloc_count;
         if (fault_alloc_index() == k) return fail(RG_ERR_OOM, std::string("injected allocation failure: ") + what);
-        cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 16, s);
+        // (a capture's allocations belong to the graph, and no pool is made during one)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+        cudaMemPool_t pool = cap == cudaStreamCaptureStatusNone ? temp_pool() : nullptr;
+        if (bytes == 0) bytes = 16;
+        cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
         if (e != cudaSuccess) {
             *p = nullptr;
             return cuda_fail(e, what);
@@ -118,6 +179,7 @@ struct DevBuf {
 };
 
 struct BlasHost {
+    void* mem = nullptr;               // the one allocation that the arrays are parts of
     float4* nodes = nullptr;
     float4* tris = nullptr;
     uint32_t nt = 0;
@@ -132,14 +194,7 @@ struct BlasHost {
 };
 
 void free_blas(BlasHost& b) {
-    cudaFree(b.nodes);
-    cudaFree(b.tris);
-    if (b.leaf_of_prim) cudaFree(b.leaf_of_prim);
-    if (b.nodes8) cudaFree(b.nodes8);
-    if (b.tris8) cudaFree(b.tris8);
-    if (b.src8) cudaFree(b.src8);
-    if (b.item_src8) cudaFree(b.item_src8);
-    if (b.counts8) cudaFree(b.counts8);
+    if (b.mem) cudaFree(b.mem);
     b = BlasHost();
 }
 
@@ -184,11 +239,13 @@ struct rg_scene {
     bool tlas_built = false;
     uint32_t n_inst = 0;
     uint32_t tlas_root = 0;
-    DevBuf<float4> tlas_nodes;
-    DevBuf<InstDev> inst, inst_tmp;
-    DevBuf<float> wbox;
-    DevBuf<uint32_t> perm, parents, flags;
-    DevBuf<uint32_t> leaf_of_inst;  // TLAS leaf of each instance index (made on first need after a build)
+    DevBuf<char> tlas_mem;          // the arrays of a TLAS of up to tlas_cap instances
+    uint32_t tlas_cap = 0;
+    float4* tlas_nodes = nullptr;
+    InstDev *inst = nullptr, *inst_tmp = nullptr;
+    float* wbox = nullptr;
+    uint32_t *perm = nullptr, *parents = nullptr, *flags = nullptr;
+    uint32_t* leaf_of_inst = nullptr;  // TLAS leaf of each instance index (made on first need after a build)
     bool leaf_of_inst_valid = false;
     // compressed 8-wide TLAS
     bool wide = false;
@@ -208,9 +265,9 @@ struct rg_scene {
     DevBuf<uint32_t> seg_count;    // per shadow ray of a split launch: segments finished / occluded (kept zero)
     DevBuf<uint32_t> counters;     // [0] closest work, [1] next count, [2] shadow work, [3] unused,
                                    // [4 + l] shadow rays toward light l
-    DevBuf<uint32_t> trace_ctr;    // rg_trace_rays work counters: kTraceSlots slots, 128 B apart
+    uint32_t* trace_ctr = nullptr; // rg_trace_rays work counters: kTraceSlots slots, 128 B apart (after the status word)
     uint32_t trace_slot = 0;       // the next call's slot
-    uint32_t* h_counts = nullptr;  // pinned, 16 entries
+    uint32_t* h_counts = nullptr;  // pinned, 16 entries (made by the first render that waits for counts)
     cudaEvent_t count_ev = nullptr;  // the next level's ray count has reached h_counts
     // statistics and timing
     uint64_t closest_rays = 0, shadow_rays_host = 0;
@@ -296,9 +353,9 @@ uint32_t iter_cap_for(const rg_scene* s, bool brute) {
 
 TraceArgs base_trace_args(rg_scene* s, bool wide) {
     TraceArgs a{};
-    a.tlas_nodes = s->tlas_nodes.p;
+    a.tlas_nodes = s->tlas_nodes;
     a.tlas_root = s->tlas_root;
-    a.inst = s->inst.p;
+    a.inst = s->inst;
     a.n_inst = s->n_inst;
     a.st = s->st;
     a.iter_cap = iter_cap_for(s, false);
@@ -317,11 +374,13 @@ rg_status lbvh_topology(TempAlloc& tmp, const float* lohi, uint32_t n, const int
                         uint32_t* perm, uint32_t* parents, cudaStream_t s, uint32_t* ranges = nullptr) {
     const int key_bits = bits == 21 ? 64 : 32;
     const size_t kb = key_bits / 8;
-    void *codes, *sorted, *scratch;
+    Parts P;
+    const size_t o_codes = P.add(n * kb), o_sorted = P.add(n * kb), o_sort = P.add(radix_sort_scratch_bytes(n, key_bits));
+    void* mem;
     rg_status r;
-    if ((r = tmp.get(&codes, n * kb, "morton codes"))) return r;
-    if ((r = tmp.get(&sorted, n * kb, "sorted codes"))) return r;
-    if ((r = tmp.get(&scratch, radix_sort_scratch_bytes(n, key_bits), "sort scratch"))) return r;
+    if ((r = tmp.get(&mem, P.total, "Morton codes and sort scratch"))) return r;
+    void *codes = static_cast<char*>(mem) + o_codes, *sorted = static_cast<char*>(mem) + o_sorted;
+    void* scratch = static_cast<char*>(mem) + o_sort;
     RG_CK(launch_morton(lohi, n, cb_ord, bits, codes, nullptr, s));
     RG_CK(radix_sort_pairs(codes, nullptr, n, key_bits, sorted, perm, scratch, s));
     RG_CK(launch_karras(sorted, n, key_bits, reinterpret_cast<uint32_t*>(nodes) + 12, 16, parents, s, ranges));
@@ -353,25 +412,16 @@ rg_status rg_scene_create(rg_scene** out, const rg_scene_desc* desc) {
         s->desc.ambient = 0.1f;
         s->desc.flags = 0;
     }
-    rg_status r = dev_alloc(reinterpret_cast<void**>(&s->st), sizeof(DevStatus), "status");
+    constexpr size_t kCtrAt = (sizeof(DevStatus) + 255) & ~(size_t)255;
+    rg_status r = dev_alloc(reinterpret_cast<void**>(&s->st), kCtrAt + (size_t)kTraceSlots * 128, "status");
     if (r) {
         delete s;
         return r;
     }
-    if ((r = s->counters.ensure(4 + kMaxLights, "counters")) ||
-        (r = s->trace_ctr.ensure((size_t)kTraceSlots * 32, "trace counters"))) {
-        cudaFree(s->st);
-        s->counters.release();
-        delete s;
-        return r;
-    }
+    s->trace_ctr = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(s->st) + kCtrAt);
     cudaError_t e = cudaMemset(s->st, 0, sizeof(DevStatus));
-    if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&s->h_counts), 16 * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->count_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         cudaFree(s->st);
-        s->counters.release();
-        s->trace_ctr.release();
         delete s;
         return cuda_fail(e, "scene setup");
     }
@@ -427,14 +477,7 @@ rg_status rg_scene_destroy(rg_scene* s) {
     s->item_src8.release();
     s->counts8.release();
     s->tasks8.release();
-    s->tlas_nodes.release();
-    s->inst.release();
-    s->leaf_of_inst.release();
-    s->inst_tmp.release();
-    s->wbox.release();
-    s->perm.release();
-    s->parents.release();
-    s->flags.release();
+    s->tlas_mem.release();
     s->mats.release();
     s->lights.release();
     for (int k = 0; k < 2; ++k) {
@@ -446,7 +489,6 @@ rg_status rg_scene_destroy(rg_scene* s) {
     s->hits.release();
     s->seg_count.release();
     s->counters.release();
-    s->trace_ctr.release();
     if (s->st) cudaFree(s->st);
     if (s->h_counts) cudaFreeHost(s->h_counts);
     if (s->count_ev) cudaEventDestroy(s->count_ev);
@@ -482,21 +524,28 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
     BlasHost b;
     b.nt = nt;
     b.root = nt == 1 ? kLeaf : 0u;
-    if ((r = dev_alloc(reinterpret_cast<void**>(&b.nodes), n_int * 64, "BLAS nodes"))) return r;
-    if ((r = dev_alloc(reinterpret_cast<void**>(&b.tris), (size_t)nt * kTriRecord, "BLAS triangles")) ||
-        (r = dev_alloc(reinterpret_cast<void**>(&b.leaf_of_prim), (size_t)nt * 4, "BLAS leaf map"))) {
-        free_blas(b);
-        return r;
-    }
+    Parts P;
+    const size_t o_nodes = P.add(n_int * 64), o_tris = P.add((size_t)nt * kTriRecord), o_map = P.add((size_t)nt * 4);
+    const size_t o_nodes8 = P.total;
+    size_t o_tris8 = 0, o_src8 = 0, o_item8 = 0, o_counts8 = 0;
     if (wide) {
-        if ((r = dev_alloc(reinterpret_cast<void**>(&b.nodes8), n_int * 80, "wide BLAS nodes")) ||
-            (r = dev_alloc(reinterpret_cast<void**>(&b.tris8), (size_t)nt * kTriRecord, "wide BLAS triangles")) ||
-            (r = dev_alloc(reinterpret_cast<void**>(&b.src8), n_int * 32, "wide BLAS slot sources")) ||
-            (r = dev_alloc(reinterpret_cast<void**>(&b.item_src8), (size_t)nt * 4, "wide BLAS item sources")) ||
-            (r = dev_alloc(reinterpret_cast<void**>(&b.counts8), 16, "wide BLAS counts"))) {
-            free_blas(b);
-            return r;
-        }
+        P.add(n_int * 80);
+        o_tris8 = P.add((size_t)nt * kTriRecord);
+        o_src8 = P.add(n_int * 32);
+        o_item8 = P.add((size_t)nt * 4);
+        o_counts8 = P.add(16);
+    }
+    if ((r = dev_alloc(&b.mem, P.total, "BLAS"))) return r;
+    char* bm = static_cast<char*>(b.mem);
+    b.nodes = reinterpret_cast<float4*>(bm + o_nodes);
+    b.tris = reinterpret_cast<float4*>(bm + o_tris);
+    b.leaf_of_prim = reinterpret_cast<uint32_t*>(bm + o_map);
+    if (wide) {
+        b.nodes8 = reinterpret_cast<float4*>(bm + o_nodes8);
+        b.tris8 = reinterpret_cast<float4*>(bm + o_tris8);
+        b.src8 = reinterpret_cast<uint32_t*>(bm + o_src8);
+        b.item_src8 = reinterpret_cast<uint32_t*>(bm + o_item8);
+        b.counts8 = reinterpret_cast<uint32_t*>(bm + o_counts8);
     }
     uint32_t id = (uint32_t)s->B->blas.size();
     if ((r = [&]() -> rg_status {
@@ -522,22 +571,18 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
              hd.nodes8 = b.nodes8;
              hd.tris8 = b.tris8;
              hd.leaf_of_prim = b.leaf_of_prim;
-             RG_CK(cudaMemcpyAsync(s->B->d_blas.p + id, &hd, sizeof hd, cudaMemcpyHostToDevice, st));
-             RG_CK(cudaStreamSynchronize(st));  // hd lives on this stack frame
-
              TempAlloc tmp(st);
-             void *lohi, *cb, *perm, *parents, *fl, *ranges = nullptr, *tasks = nullptr, *boxes_done = nullptr;
              rg_status q;
-             if (wide) {
-                 if ((q = tmp.get(&ranges, n_int * 8, "ranges"))) return q;
-                 if ((q = tmp.get(&tasks, (size_t)nt * 16, "collapse tasks"))) return q;
-             }
-             if ((q = tmp.get(&lohi, (size_t)nt * 24, "triangle boxes"))) return q;
-             if ((q = tmp.get(&cb, 64, "centroid bounds"))) return q;
-             if ((q = tmp.get(&perm, (size_t)nt * 4, "permutation"))) return q;
-             if ((q = tmp.get(&parents, (size_t)(2 * (size_t)nt - 1) * 4, "parents"))) return q;
-             if ((q = tmp.get(&fl, (size_t)(nt > 1 ? nt - 1 : 1) * 4, "refit flags"))) return q;
-             RG_CK(launch_init_bounds(static_cast<int*>(cb), st));
+             Parts T;
+             const size_t t_lohi = T.add((size_t)nt * 24), t_cb = T.add(64), t_perm = T.add((size_t)nt * 4);
+             const size_t t_parents = T.add((2 * (size_t)nt - 1) * 4), t_fl = T.add(n_int * 4);
+             const size_t t_ranges = wide ? T.add(n_int * 8) : 0, t_tasks = wide ? T.add((size_t)nt * 16) : 0;
+             void* mem;
+             if ((q = tmp.get(&mem, T.total, "BLAS build scratch"))) return q;
+             char* tm = static_cast<char*>(mem);
+             void *lohi = tm + t_lohi, *cb = tm + t_cb, *perm = tm + t_perm, *parents = tm + t_parents, *fl = tm + t_fl;
+             void *ranges = wide ? tm + t_ranges : nullptr, *tasks = wide ? tm + t_tasks : nullptr, *boxes_done = nullptr;
+             RG_CK(launch_blas_begin(static_cast<int*>(cb), s->B->d_blas.p + id, hd, st));
              RG_CK(launch_tri_bounds(d_vtx, nv, d_idx, nt, static_cast<float*>(lohi), static_cast<int*>(cb), s->st, st));
              if (nt > 1) {
                  if (flags & RG_BLAS_SAH) {
@@ -590,24 +635,24 @@ static rg_status tlas_common(rg_scene* s, const rg_instance* d_inst, uint32_t n,
         // one single-block launch for the whole build or refit
         void* ranges = nullptr;
         if (!refit && s->wide && n > 1 && (r = tmp.get(&ranges, (size_t)(n - 1) * 8, "ranges"))) return r;
-        RG_CK(launch_tlas_small(d_inst, n, s->B->d_blas.p, (uint32_t)s->B->blas.size(), s->inst_tmp.p, s->wbox.p, refit,
-                                s->tlas_nodes.p, s->perm.p, s->parents.p, s->flags.p, static_cast<uint32_t*>(ranges),
-                                s->inst.p, s->st, st));
+        RG_CK(launch_tlas_small(d_inst, n, s->B->d_blas.p, (uint32_t)s->B->blas.size(), s->inst_tmp, s->wbox, refit,
+                                s->tlas_nodes, s->perm, s->parents, s->flags, static_cast<uint32_t*>(ranges),
+                                s->inst, s->st, st));
         if (s->wide) {
             WideOut out{s->tlas8.p, s->src8.p, s->item_src8.p, s->counts8.p, s->tasks8.p};
             if (refit)
-                RG_CK(launch_wide_refit(s->tlas_nodes.p, s->wbox.p, s->perm.p, n, s->inst.p, s->inst8.p, s->B->d_blas.p,
+                RG_CK(launch_wide_refit(s->tlas_nodes, s->wbox, s->perm, n, s->inst, s->inst8.p, s->B->d_blas.p,
                                         out, s->st, st));
             else
-                RG_CK(launch_collapse(s->tlas_nodes.p, static_cast<uint32_t*>(ranges), n, s->wbox.p, nullptr, nullptr,
-                                      s->inst.p, s->inst8.p, s->B->d_blas.p, out, s->st, st, 1u));
+                RG_CK(launch_collapse(s->tlas_nodes, static_cast<uint32_t*>(ranges), n, s->wbox, nullptr, nullptr,
+                                      s->inst, s->inst8.p, s->B->d_blas.p, out, s->st, st, 1u));
         }
         return RG_OK;
     }
     void* cb;
     if ((r = tmp.get(&cb, 64, "centroid bounds"))) return r;
     if (!refit) RG_CK(launch_init_bounds(static_cast<int*>(cb), st));
-    RG_CK(launch_instance_prep(d_inst, n, s->B->d_blas.p, (uint32_t)s->B->blas.size(), s->inst_tmp.p, s->wbox.p,
+    RG_CK(launch_instance_prep(d_inst, n, s->B->d_blas.p, (uint32_t)s->B->blas.size(), s->inst_tmp, s->wbox,
                                refit ? nullptr : static_cast<int*>(cb), refit, s->st, st));
     void* ranges = nullptr;
     void* boxes_done = nullptr;  // set by the SAH build when it wrote every node's boxes
@@ -616,28 +661,28 @@ static rg_status tlas_common(rg_scene* s, const rg_instance* d_inst, uint32_t n,
             if (s->wide && (r = tmp.get(&ranges, (size_t)(n - 1) * 8, "ranges"))) return r;
             if (sah && (r = tmp.get(&boxes_done, 16, "box flag"))) return r;
             if (sah)
-                r = sah_topology(ScratchAlloc{temp_get, &tmp}, s->wbox.p, n, static_cast<int*>(cb), 10,
-                                 s->tlas_nodes.p, s->perm.p, s->parents.p, st, static_cast<uint32_t*>(ranges),
+                r = sah_topology(ScratchAlloc{temp_get, &tmp}, s->wbox, n, static_cast<int*>(cb), 10,
+                                 s->tlas_nodes, s->perm, s->parents, st, static_cast<uint32_t*>(ranges),
                                  static_cast<uint32_t*>(boxes_done));
             else
-                r = lbvh_topology(tmp, s->wbox.p, n, static_cast<int*>(cb), 10, s->tlas_nodes.p, s->perm.p,
-                                  s->parents.p, st, static_cast<uint32_t*>(ranges));
+                r = lbvh_topology(tmp, s->wbox, n, static_cast<int*>(cb), 10, s->tlas_nodes, s->perm,
+                                  s->parents, st, static_cast<uint32_t*>(ranges));
             if (r) return r;
         } else {
-            RG_CK(cudaMemsetAsync(s->perm.p, 0, 4, st));
+            RG_CK(cudaMemsetAsync(s->perm, 0, 4, st));
         }
     }
-    if (n > 1) RG_CK(cudaMemsetAsync(s->flags.p, 0, (size_t)(n - 1) * 4, st));
-    RG_CK(launch_tlas_leaves_refit(s->inst_tmp.p, s->wbox.p, s->perm.p, n, s->parents.p, s->tlas_nodes.p, s->flags.p,
-                                   s->inst.p, s->st, st, static_cast<const uint32_t*>(boxes_done)));
+    if (n > 1) RG_CK(cudaMemsetAsync(s->flags, 0, (size_t)(n - 1) * 4, st));
+    RG_CK(launch_tlas_leaves_refit(s->inst_tmp, s->wbox, s->perm, n, s->parents, s->tlas_nodes, s->flags,
+                                   s->inst, s->st, st, static_cast<const uint32_t*>(boxes_done)));
     if (s->wide) {
         WideOut out{s->tlas8.p, s->src8.p, s->item_src8.p, s->counts8.p, s->tasks8.p};
         if (refit)
-            RG_CK(launch_wide_refit(s->tlas_nodes.p, s->wbox.p, s->perm.p, n, s->inst.p, s->inst8.p, s->B->d_blas.p, out,
+            RG_CK(launch_wide_refit(s->tlas_nodes, s->wbox, s->perm, n, s->inst, s->inst8.p, s->B->d_blas.p, out,
                                     s->st, st));
         else
-            RG_CK(launch_collapse(s->tlas_nodes.p, static_cast<uint32_t*>(ranges), n, s->wbox.p, nullptr, nullptr,
-                                  s->inst.p, s->inst8.p, s->B->d_blas.p, out, s->st, st, 1u));
+            RG_CK(launch_collapse(s->tlas_nodes, static_cast<uint32_t*>(ranges), n, s->wbox, nullptr, nullptr,
+                                  s->inst, s->inst8.p, s->B->d_blas.p, out, s->st, st, 1u));
     }
     return RG_OK;
 }
@@ -652,13 +697,25 @@ rg_status rg_tlas_build(rg_scene* s, const rg_instance* d_inst, uint32_t n, void
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     s->tlas_built = false;
     s->leaf_of_inst_valid = false;
-    if ((r = s->tlas_nodes.ensure((size_t)(n > 1 ? n - 1 : 1) * 4, "TLAS nodes"))) return r;
-    if ((r = s->inst.ensure(n, "instances"))) return r;
-    if ((r = s->inst_tmp.ensure(n, "instance staging"))) return r;
-    if ((r = s->wbox.ensure((size_t)n * 6, "instance boxes"))) return r;
-    if ((r = s->perm.ensure(n, "TLAS order"))) return r;
-    if ((r = s->parents.ensure(2 * (size_t)n, "TLAS parents"))) return r;
-    if ((r = s->flags.ensure(n, "TLAS flags"))) return r;
+    if (n > s->tlas_cap) {
+        const size_t m = n < 16 ? 16 : n;
+        Parts P;
+        const size_t o_nodes = P.add((m - 1) * 64), o_inst = P.add(m * sizeof(InstDev)), o_tmp = P.add(m * sizeof(InstDev));
+        const size_t o_box = P.add(m * 24), o_perm = P.add(m * 4), o_parents = P.add(2 * m * 4), o_flags = P.add(m * 4);
+        const size_t o_leaf = P.add(m * 4);
+        s->tlas_cap = 0;
+        if ((r = s->tlas_mem.ensure(P.total, "TLAS"))) return r;
+        char* p = s->tlas_mem.p;
+        s->tlas_nodes = reinterpret_cast<float4*>(p + o_nodes);
+        s->inst = reinterpret_cast<InstDev*>(p + o_inst);
+        s->inst_tmp = reinterpret_cast<InstDev*>(p + o_tmp);
+        s->wbox = reinterpret_cast<float*>(p + o_box);
+        s->perm = reinterpret_cast<uint32_t*>(p + o_perm);
+        s->parents = reinterpret_cast<uint32_t*>(p + o_parents);
+        s->flags = reinterpret_cast<uint32_t*>(p + o_flags);
+        s->leaf_of_inst = reinterpret_cast<uint32_t*>(p + o_leaf);
+        s->tlas_cap = (uint32_t)m;
+    }
     s->wide = false;
     if (s->desc.flags & RG_SCENE_COMPRESSED) {
         for (const BlasHost& b : s->B->blas)
@@ -731,7 +788,7 @@ rg_status rg_trace_rays(rg_scene* s, const rg_ray* d_rays, uint32_t n, uint32_t 
     a.n = n;
     a.hits_abi = d_hits;
     // a work counter of its own, so calls on other streams may run at the same time
-    uint32_t* ctr = s->trace_ctr.p + 32 * (size_t)(s->trace_slot++ % kTraceSlots);
+    uint32_t* ctr = s->trace_ctr + 32 * (size_t)(s->trace_slot++ % kTraceSlots);
     a.work_counter = ctr;
     a.iter_cap = iter_cap_for(s, flags & RG_TRACE_BRUTE);
     RG_CK(cudaMemsetAsync(ctr, 0, 4, st));
@@ -745,12 +802,11 @@ rg_status rg_trace_rays(rg_scene* s, const rg_ray* d_rays, uint32_t n, uint32_t 
     // walked)
     if (!any) {
         if (!s->leaf_of_inst_valid) {
-            if ((r = s->leaf_of_inst.ensure(s->n_inst, "instance leaf map"))) return r;
-            RG_CK(launch_invert_perm(s->perm.p, s->n_inst, s->leaf_of_inst.p, st));
+            RG_CK(launch_invert_perm(s->perm, s->n_inst, s->leaf_of_inst, st));
             s->leaf_of_inst_valid = true;
         }
         if ((r = event_begin(s, 3, st, &ev))) return r;
-        RG_CK(launch_refine_hits(a.rays, d_hits, n, s->inst.p, s->leaf_of_inst.p, s->B->d_blas.p, st));
+        RG_CK(launch_refine_hits(a.rays, d_hits, n, s->inst, s->leaf_of_inst, s->B->d_blas.p, st));
         if ((r = event_end(s, st))) return r;
     }
     if (any)
@@ -828,7 +884,7 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         sa.rays = s->q_rays[q].p;
         sa.payload = s->q_pay[q].p;
         sa.hits = s->hits.p;
-        sa.inst = s->wide ? s->inst8.p : s->inst.p;
+        sa.inst = s->wide ? s->inst8.p : s->inst;
         sa.mats = s->mats.p;
         sa.n_mats = s->n_mats;
         sa.lights = s->lights.p;
@@ -865,6 +921,12 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         RG_CK(launch_trace(kModeClosestRender, false, s->desc.flags & RG_SCENE_COUNT, a, st));
         return event_end(s, st);
     };
+
+    if (!async) {
+        if (!s->h_counts)
+            RG_CK(cudaMallocHost(reinterpret_cast<void**>(&s->h_counts), 16 * sizeof(uint32_t)));
+        if (!s->count_ev) RG_CK(cudaEventCreateWithFlags(&s->count_ev, cudaEventDisableTiming));
+    }
 
     uint32_t n = N;  // this level's rays (a bound on them when async)
     int cur = 0;
@@ -1123,12 +1185,12 @@ rg_status rg_tlas_export(rg_scene* s, void* h_nodes, float* h_wbox, float* h_inv
     if ((r = set_device(s))) return r;
     RG_CK(cudaDeviceSynchronize());
     const uint32_t n = s->n_inst;
-    if (h_nodes && n > 1) RG_CK(cudaMemcpy(h_nodes, s->tlas_nodes.p, (size_t)(n - 1) * 64, cudaMemcpyDeviceToHost));
-    if (h_wbox) RG_CK(cudaMemcpy(h_wbox, s->wbox.p, (size_t)n * 24, cudaMemcpyDeviceToHost));
-    if (h_order) RG_CK(cudaMemcpy(h_order, s->perm.p, (size_t)n * 4, cudaMemcpyDeviceToHost));
+    if (h_nodes && n > 1) RG_CK(cudaMemcpy(h_nodes, s->tlas_nodes, (size_t)(n - 1) * 64, cudaMemcpyDeviceToHost));
+    if (h_wbox) RG_CK(cudaMemcpy(h_wbox, s->wbox, (size_t)n * 24, cudaMemcpyDeviceToHost));
+    if (h_order) RG_CK(cudaMemcpy(h_order, s->perm, (size_t)n * 4, cudaMemcpyDeviceToHost));
     if (h_inv) {
         std::vector<InstDev> v(n);
-        RG_CK(cudaMemcpy(v.data(), s->inst.p, (size_t)n * sizeof(InstDev), cudaMemcpyDeviceToHost));
+        RG_CK(cudaMemcpy(v.data(), s->inst, (size_t)n * sizeof(InstDev), cudaMemcpyDeviceToHost));
         for (uint32_t j = 0; j < n; ++j) {
             uint32_t k = v[j].id;
             if (k >= n) return fail(RG_ERR_CUDA, "corrupt instance table");
@@ -1155,10 +1217,10 @@ rg_status scene_view(rg_scene* s, SceneView* v) {
     v->device = s->device;
     v->d_blas = s->B->d_blas.p;
     v->n_blas = (uint32_t)s->B->blas.size();
-    v->tlas_nodes = s->tlas_nodes.p;
-    v->perm = s->perm.p;
-    v->parents = s->parents.p;
-    v->inst = s->inst.p;
+    v->tlas_nodes = s->tlas_nodes;
+    v->perm = s->perm;
+    v->parents = s->parents;
+    v->inst = s->inst;
     v->n_inst = s->n_inst;
     v->tlas_root = s->tlas_root;
     v->mats = s->mats.p;

@@ -69,6 +69,14 @@ __global__ void k_init_bounds(int* cb_ord) {
     else if (t < 6) cb_ord[t] = f2ord(__int_as_float(0xFF800000));   // -inf
 }
 
+// The same, and a BLAS's descriptor (its boxes come later).
+__global__ void k_blas_begin(int* cb_ord, BlasDev* out, BlasDev desc) {
+    const int t = threadIdx.x;
+    if (t < 3) cb_ord[t] = f2ord(__int_as_float(0x7F800000));
+    else if (t < 6) cb_ord[t] = f2ord(__int_as_float(0xFF800000));
+    else if (t == 6) *out = desc;
+}
+
 __global__ void k_tri_bounds(const float* __restrict__ vtx, uint32_t nv, const uint32_t* __restrict__ idx,
                              uint32_t nt, float* __restrict__ lohi, int* cb_ord, DevStatus* st) {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -779,6 +787,12 @@ inline unsigned grid_for(size_t n, int block = kBlock) { return (unsigned)((n + 
 
 cudaError_t launch_init_bounds(int* cb_ord, cudaStream_t s) {
     k_init_bounds<<<1, 32, 0, s>>>(cb_ord);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_blas_begin(int* cb_ord, BlasDev* out, const BlasDev& desc, cudaStream_t s) {
+    k_blas_begin<<<1, 32, 0, s>>>(cb_ord, out, desc);
     count_launches(1);
     return cudaGetLastError();
 }

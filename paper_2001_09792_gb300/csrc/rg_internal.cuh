@@ -167,6 +167,7 @@ __device__ __forceinline__ float ord2f(int i) { return __int_as_float(i >= 0 ? i
 cudaError_t launch_tri_bounds(const float* vtx, uint32_t nv, const uint32_t* idx, uint32_t nt, float* lohi,
                               int* cb_ord, DevStatus* st, cudaStream_t s);
 cudaError_t launch_init_bounds(int* cb_ord, cudaStream_t s);
+cudaError_t launch_blas_begin(int* cb_ord, BlasDev* out, const BlasDev& desc, cudaStream_t s);
 cudaError_t launch_centroid_bounds(const float* lohi, uint32_t n, int* cb_ord, cudaStream_t s);
 cudaError_t launch_morton(const float* lohi, uint32_t n, const int* cb_ord, int bits, void* codes, float* cb_out,
                           cudaStream_t s);
