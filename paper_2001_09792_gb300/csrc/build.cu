@@ -187,9 +187,9 @@ __global__ void k_morton(const float* __restrict__ lohi, uint32_t n, const int* 
 // Garland 2016, in the one-pass-per-digit form of Adinets & Merrill 2022) and
 // writes its pairs grouped by digit, so that the stores are runs.  Bound by
 // memory (12 B read and written per pair and pass) where the launch is large,
-// by the launches where it is small.  1,000,003 pairs of 32-bit keys: 95.6 us,
+// by the launches where it is small.  1,000,003 pairs of 32-bit keys: 78.7 us,
 // 304.7 us with a count, a one-block scan (50 us a pass) and a scatter per
-// pass; 2,048 pairs a tile keep every SM busy from 311,296 pairs on.
+// pass.
 //
 // The look-back waits on nothing: a tile takes its number from a counter, so
 // the tiles before it have started, and a count that has not appeared after
@@ -197,6 +197,10 @@ __global__ void k_morton(const float* __restrict__ lohi, uint32_t n, const int* 
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSpinMax = 1 << 14;
+constexpr uint32_t kLook = 8, kSortLargeTiles = 200;
+// Items per thread: 8 (tiles of kSortTilePairs), or 16 from kSortLargeTiles tiles
+// of those on: 1,000,003 pairs take 78.7 us with 16 and 88.9 with 8, 16M 615 and
+// 667, but 100,001 pairs 51.6 and 43.7 (few tiles, each longer).
 constexpr int kSortItems = (int)kSortTilePairs / kSortThreads;
 
 // Ranks of a warp's ITEMS x 32 digits among its own: cnt (256 entries, this
@@ -312,19 +316,34 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_pass(const K* __restrict__ 
     const uint32_t off = scan256(total, s_wsum);
     const uint32_t first = scan256(hist[t], s_wsum);  // the digit's place over all tiles
     // the pairs of this digit in the tiles before
+    // (kLook tiles are read at a time, for the chain of reads is what a pass waits
+    // on: 95.6 -> 88.9 us at 1,000,003 pairs; 16 and 32 at a time 86.0 and 98.4
+    // against 78.7 with the larger tiles)
     uint32_t before = 0;
-    for (uint32_t q = tile; q-- > 0;) {
-        const volatile W* st = status + (size_t)q * 256 + t;
-        W v = *st;
-        for (int spin = 0; !(v >> kFlag) && spin < kSpinMax; ++spin) v = *st;
-        if (!(v >> kFlag)) {
-            uint32_t c = 0;
-            for (uint32_t p = 0; p < (uint32_t)kTile; ++p)
-                c += ((uint32_t)(keys[(size_t)q * kTile + p] >> shift) & 0xFFu) == t;
-            v = kOwn | (W)c;
+    for (uint32_t q = tile;; q -= kLook) {
+        W v[kLook];
+#pragma unroll
+        for (uint32_t k = 0; k < kLook; ++k)
+            v[k] = q > k ? *reinterpret_cast<const volatile W*>(status + (size_t)(q - 1 - k) * 256 + t) : kAll;
+        bool done = false;
+#pragma unroll
+        for (uint32_t k = 0; k < kLook; ++k) {
+            if (done) continue;
+            if (!(v[k] >> kFlag)) {
+                const size_t p = q - 1 - k;
+                for (int spin = 0; !(v[k] >> kFlag) && spin < kSpinMax; ++spin)
+                    v[k] = *reinterpret_cast<const volatile W*>(status + p * 256 + t);
+                if (!(v[k] >> kFlag)) {
+                    uint32_t c = 0;
+                    for (uint32_t i = 0; i < (uint32_t)kTile; ++i)
+                        c += ((uint32_t)(keys[p * kTile + i] >> shift) & 0xFFu) == t;
+                    v[k] = kOwn | (W)c;
+                }
+            }
+            before += (uint32_t)(v[k] & kCount);
+            done = (v[k] & kAll) != 0;
         }
-        before += (uint32_t)(v & kCount);
-        if (v & kAll) break;
+        if (done) break;
     }
     if (tile) *reinterpret_cast<volatile W*>(mine) = kAll | (W)(before + total);
     s_off[t] = off;
@@ -833,7 +852,9 @@ static cudaError_t radix_sort_impl(const K* keys_in, const uint32_t* vals_in, ui
         return cudaGetLastError();
     }
     constexpr int passes = (int)sizeof(K);
-    const uint32_t nb = (uint32_t)(((size_t)n + kSortTilePairs - 1) / kSortTilePairs);
+    const bool large = n / (2 * kSortTilePairs) >= kSortLargeTiles;
+    const uint32_t tile = large ? 2 * kSortTilePairs : kSortTilePairs;
+    const uint32_t nb = (uint32_t)(((size_t)n + tile - 1) / tile);
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     char* p = static_cast<char*>(scratch);
     K* kt = reinterpret_cast<K*>(p);
@@ -855,7 +876,8 @@ static cudaError_t radix_sort_impl(const K* keys_in, const uint32_t* vals_in, ui
         const bool to_out = (pass & 1) != 0;
         K* kdst = to_out ? keys_out : kt;
         uint32_t* vdst = to_out ? vals_out : vt;
-        k_rs_pass<K, W, kSortItems><<<nb, kSortThreads, 0, s>>>(
+        auto* pass_kernel = large ? k_rs_pass<K, W, 2 * kSortItems> : k_rs_pass<K, W, kSortItems>;
+        pass_kernel<<<nb, kSortThreads, 0, s>>>(
             ksrc, vsrc, n, 8 * pass, hist + 256 * pass, status[pass & 1],
             pass + 1 < passes ? status[(pass + 1) & 1] : nullptr, ticket + pass, kdst, vdst);
         ksrc = kdst;
