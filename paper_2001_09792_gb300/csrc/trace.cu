@@ -1,7 +1,8 @@
 // Ray traversal kernels of the two-level BVH (the per-ray code is in
 // traverse.cuh): persistent warps pull rays from a global counter, 32 at a
 // time (k_trace_warp), as lanes fall idle (k_trace_lane), or from two queues
-// in one launch (k_trace_pair); k_trace8 walks the compressed 8-wide BVH.
+// in one launch (k_trace_pair); k_trace8 and k_trace8_lane walk the compressed
+// 8-wide BVH.
 #include <atomic>
 
 #include "traverse.cuh"
@@ -374,6 +375,81 @@ __device__ __forceinline__ float plane_err(float S, float B) {
     return fmaf(kQuantErr, fmaf(255.0f, fabsf(S), fabsf(B)), kPlaneErr * fabsf(S));
 }
 
+// A ray's place in the wide tree: the node group (children of one node still
+// to visit: base index, hit bits in visiting order, the node's internal-slot
+// mask) and the item group (base index, one bit per item).
+struct Groups {
+    uint32_t base, hits, imask, ibase, ibits;
+};
+
+// Tests the eight children of the node at nd: the groups of those the ray meets.
+__device__ __forceinline__ void visit8(const float4* nd, const SpaceRay& cr, uint32_t oct, float tmin, float tlim,
+                                       Groups& G) {
+        const float4 w0 = __ldg(nd);
+    const uint4 w1 = __ldg(reinterpret_cast<const uint4*>(nd + 1));
+    const uint4 w2 = __ldg(reinterpret_cast<const uint4*>(nd + 2));
+    const uint4 w3 = __ldg(reinterpret_cast<const uint4*>(nd + 3));
+    const uint4 w4 = __ldg(reinterpret_cast<const uint4*>(nd + 4));
+    const uint32_t bits = __float_as_uint(w0.w);
+    const uint32_t imask = bits >> 24;
+    const float sx = __int_as_float((((int)(int8_t)(bits & 0xFF)) + 127) << 23);
+    const float sy = __int_as_float((((int)(int8_t)((bits >> 8) & 0xFF)) + 127) << 23);
+    const float sz = __int_as_float((((int)(int8_t)((bits >> 16) & 0xFF)) + 127) << 23);
+    const float Sx = sx * cr.ix, Sy = sy * cr.iy, Sz = sz * cr.iz;  // exact: powers of two
+    const float Bx = __fmul_rn(__fsub_rn(w0.x, cr.ox), cr.ix);
+    const float By = __fmul_rn(__fsub_rn(w0.y, cr.oy), cr.iy);
+    const float Bz = __fmul_rn(__fsub_rn(w0.z, cr.oz), cr.iz);
+    const float Ux = Sx * kBias, Uy = Sy * kBias, Uz = Sz * kBias;  // exact (or inf)
+    const float Cx = plane_offset(Sx, Bx), Cy = plane_offset(Sy, By), Cz = plane_offset(Sz, Bz);
+    const float Ex = plane_err(Sx, Bx), Ey = plane_err(Sy, By), Ez = plane_err(Sz, Bz);
+    // near planes shifted down by E, far planes up by E
+    const float Bxn = Cx - Ex, Byn = Cy - Ey, Bzn = Cz - Ez;
+    const float Bxf = Cx + Ex, Byf = Cy + Ey, Bzf = Cz + Ez;
+    // near/far planes per axis from the direction signs
+    const bool nx = oct & 1, ny = oct & 2, nz = oct & 4;
+    const uint32_t nx0 = nx ? w3.z : w2.x, nx1 = nx ? w3.w : w2.y, fx0 = nx ? w2.x : w3.z, fx1 = nx ? w2.y : w3.w;
+    const uint32_t ny0 = ny ? w4.x : w2.z, ny1 = ny ? w4.y : w2.w, fy0 = ny ? w2.z : w4.x, fy1 = ny ? w2.w : w4.y;
+    const uint32_t nz0 = nz ? w4.z : w3.x, nz1 = nz ? w4.w : w3.y, fz0 = nz ? w3.x : w4.z, fz1 = nz ? w3.y : w4.w;
+        const uint32_t meta_lo = w1.z, meta_hi = w1.w;
+    uint32_t hitmask = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const int k = c & 3;
+        const float tnx = fmaf(byte_v(c < 4 ? nx0 : nx1, k), Ux, Bxn);
+        const float tfx = fmaf(byte_v(c < 4 ? fx0 : fx1, k), Ux, Bxf);
+        const float tny = fmaf(byte_v(c < 4 ? ny0 : ny1, k), Uy, Byn);
+        const float tfy = fmaf(byte_v(c < 4 ? fy0 : fy1, k), Uy, Byf);
+        const float tnz = fmaf(byte_v(c < 4 ? nz0 : nz1, k), Uz, Bzn);
+        const float tfz = fmaf(byte_v(c < 4 ? fz0 : fz1, k), Uz, Bzf);
+        const float tn = fmaxf(fmaxf(tnx, tny), fmaxf(tnz, tmin));
+        const float tf = fminf(fminf(tfx, tfy), fminf(tfz, tlim));
+        if (tn <= tf) hitmask |= 1u << c;
+    }
+    // keep occupied slots only: internal ones and leaves (meta != 0)
+    const uint32_t occ_lo = __vcmpne4(meta_lo, 0u) & 0x08040201u;
+    const uint32_t occ_hi = __vcmpne4(meta_hi, 0u) & 0x80402010u;
+    uint32_t occ = occ_lo | occ_hi;
+    occ = (occ | (occ >> 8) | (occ >> 16) | (occ >> 24)) & 0xFFu;
+    hitmask &= occ | imask;
+    // internal hits, bit positions permuted to visiting order (slot ^ oct)
+    uint32_t hits = hitmask & imask;
+    if (oct & 1u) hits = ((hits & 0x55u) << 1) | ((hits >> 1) & 0x55u);
+    if (oct & 2u) hits = ((hits & 0x33u) << 2) | ((hits >> 2) & 0x33u);
+    if (oct & 4u) hits = ((hits & 0x0Fu) << 4) | ((hits >> 4) & 0x0Fu);
+    uint32_t items = 0;
+    for (uint32_t lm = hitmask & ~imask; lm; lm &= lm - 1) {
+        const int c = __ffs(lm) - 1;
+        const uint32_t meta = ((c < 4 ? meta_lo : meta_hi) >> (8 * (c & 3))) & 0xFFu;
+        items |= ((1u << (meta >> 5)) - 1u) << (meta & 31u);
+    }
+    G.base = w1.x;
+    G.hits = hits;
+    G.imask = imask;
+    G.ibase = w1.y;
+    G.ibits = items;
+}
+
+// Wide traversal, whole-warp refill (the renderer's rays).
 template <int MODE, bool STATS>
 __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
     const uint32_t iter_cap = a.iter_cap;
@@ -443,71 +519,14 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
                         }
                         stack[sp++] = make_uint2(g_base, g_hits | (g_imask << 8) | kKindNode);
                     }
-                    const float4* nd = nodes + 5 * (size_t)node;
-                    const float4 w0 = __ldg(nd);
-                    const uint4 w1 = __ldg(reinterpret_cast<const uint4*>(nd + 1));
-                    const uint4 w2 = __ldg(reinterpret_cast<const uint4*>(nd + 2));
-                    const uint4 w3 = __ldg(reinterpret_cast<const uint4*>(nd + 3));
-                    const uint4 w4 = __ldg(reinterpret_cast<const uint4*>(nd + 4));
                     if (STATS) ++c_nodes;
-                    const uint32_t bits = __float_as_uint(w0.w);
-                    const uint32_t imask = bits >> 24;
-                    const float sx = __int_as_float((((int)(int8_t)(bits & 0xFF)) + 127) << 23);
-                    const float sy = __int_as_float((((int)(int8_t)((bits >> 8) & 0xFF)) + 127) << 23);
-                    const float sz = __int_as_float((((int)(int8_t)((bits >> 16) & 0xFF)) + 127) << 23);
-                    const float Sx = sx * cr.ix, Sy = sy * cr.iy, Sz = sz * cr.iz;  // exact: powers of two
-                    const float Bx = __fmul_rn(__fsub_rn(w0.x, cr.ox), cr.ix);
-                    const float By = __fmul_rn(__fsub_rn(w0.y, cr.oy), cr.iy);
-                    const float Bz = __fmul_rn(__fsub_rn(w0.z, cr.oz), cr.iz);
-                    const float Ux = Sx * kBias, Uy = Sy * kBias, Uz = Sz * kBias;  // exact (or inf)
-                    const float Cx = plane_offset(Sx, Bx), Cy = plane_offset(Sy, By), Cz = plane_offset(Sz, Bz);
-                    const float Ex = plane_err(Sx, Bx), Ey = plane_err(Sy, By), Ez = plane_err(Sz, Bz);
-                    // near planes shifted down by E, far planes up by E
-                    const float Bxn = Cx - Ex, Byn = Cy - Ey, Bzn = Cz - Ez;
-                    const float Bxf = Cx + Ex, Byf = Cy + Ey, Bzf = Cz + Ez;
-                    // near/far planes per axis from the direction signs
-                    const bool nx = oct & 1, ny = oct & 2, nz = oct & 4;
-                    const uint32_t nx0 = nx ? w3.z : w2.x, nx1 = nx ? w3.w : w2.y, fx0 = nx ? w2.x : w3.z, fx1 = nx ? w2.y : w3.w;
-                    const uint32_t ny0 = ny ? w4.x : w2.z, ny1 = ny ? w4.y : w2.w, fy0 = ny ? w2.z : w4.x, fy1 = ny ? w2.w : w4.y;
-                    const uint32_t nz0 = nz ? w4.z : w3.x, nz1 = nz ? w4.w : w3.y, fz0 = nz ? w3.x : w4.z, fz1 = nz ? w3.y : w4.w;
-                    const float tlim = kAny ? __fmul_rn(tmax, kCullSlack) : __fmul_rn(best.t, kCullSlack);
-                    const uint32_t meta_lo = w1.z, meta_hi = w1.w;
-                    uint32_t hitmask = 0;
-    #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const int k = c & 3;
-                        const float tnx = fmaf(byte_v(c < 4 ? nx0 : nx1, k), Ux, Bxn);
-                        const float tfx = fmaf(byte_v(c < 4 ? fx0 : fx1, k), Ux, Bxf);
-                        const float tny = fmaf(byte_v(c < 4 ? ny0 : ny1, k), Uy, Byn);
-                        const float tfy = fmaf(byte_v(c < 4 ? fy0 : fy1, k), Uy, Byf);
-                        const float tnz = fmaf(byte_v(c < 4 ? nz0 : nz1, k), Uz, Bzn);
-                        const float tfz = fmaf(byte_v(c < 4 ? fz0 : fz1, k), Uz, Bzf);
-                        const float tn = fmaxf(fmaxf(tnx, tny), fmaxf(tnz, tmin));
-                        const float tf = fminf(fminf(tfx, tfy), fminf(tfz, tlim));
-                        if (tn <= tf) hitmask |= 1u << c;
-                    }
-                    // keep occupied slots only: internal ones and leaves (meta != 0)
-                    const uint32_t occ_lo = __vcmpne4(meta_lo, 0u) & 0x08040201u;
-                    const uint32_t occ_hi = __vcmpne4(meta_hi, 0u) & 0x80402010u;
-                    uint32_t occ = occ_lo | occ_hi;
-                    occ = (occ | (occ >> 8) | (occ >> 16) | (occ >> 24)) & 0xFFu;
-                    hitmask &= occ | imask;
-                    // internal hits, bit positions permuted to visiting order (slot ^ oct)
-                    uint32_t hits = hitmask & imask;
-                    if (oct & 1u) hits = ((hits & 0x55u) << 1) | ((hits >> 1) & 0x55u);
-                    if (oct & 2u) hits = ((hits & 0x33u) << 2) | ((hits >> 2) & 0x33u);
-                    if (oct & 4u) hits = ((hits & 0x0Fu) << 4) | ((hits >> 4) & 0x0Fu);
-                    uint32_t items = 0;
-                    for (uint32_t lm = hitmask & ~imask; lm; lm &= lm - 1) {
-                        const int c = __ffs(lm) - 1;
-                        const uint32_t meta = ((c < 4 ? meta_lo : meta_hi) >> (8 * (c & 3))) & 0xFFu;
-                        items |= ((1u << (meta >> 5)) - 1u) << (meta & 31u);
-                    }
-                    g_base = w1.x;
-                    g_hits = hits;
-                    g_imask = imask;
-                    i_base = w1.y;
-                    i_bits = items;
+                    Groups G;
+                    visit8(nodes + 5 * (size_t)node, cr, oct, tmin, __fmul_rn(kAny ? tmax : best.t, kCullSlack), G);
+                    g_base = G.base;
+                    g_hits = G.hits;
+                    g_imask = G.imask;
+                    i_base = G.ibase;
+                    i_bits = G.ibits;
             }
             if (done) break;
             while (i_bits) {
@@ -613,18 +632,225 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
     flush_counts<kAny, STATS>(a, c_nodes, c_tris, c_inst);
 }
 
+// Wide traversal, per-lane refill, as k_trace_lane: each lane holds a ray, and a
+// warp takes new rays for its idle lanes once a.refill of them are idle.  A
+// lane with items (triangles or an instance) waits until kLeafBatch8 lanes hold
+// the same kind or fewer than kLeafNodesMin8 are left on nodes.  Each ray takes
+// the steps that it takes alone, so the records do not depend on either.
+// Bound by ALU issue (eight child tests a node); with whole-warp refill a warp
+// waited for its slowest ray.  2^21 closest and 2^21 any hits of the medium
+// scene, us: 1,960 (6 blocks of 128 per SM, 80 registers), 1,998 with 7 blocks,
+// 2,009 with 8; 2,141 and 2,622 with runs of 2 and 4 nodes an iteration; 2,090
+// and 2,036 with a batch of 1 and 8; 2,156 with refill at 16 idle lanes.
+constexpr int kLeafBatch8 = 4, kLeafNodesMin8 = 8, kRefill8 = 8;
 template <int MODE, bool STATS>
-cudaError_t launch_mode8(const TraceArgs& a, cudaStream_t s) {
+__global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(TraceArgs a) {
+    const uint32_t iter_cap = a.iter_cap;
+    constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender);
+    constexpr bool kTies = MODE == kModeClosestAbi;
+    __shared__ uint32_t pre[kMaxLights + 1];
+    const uint32_t n = ray_count<MODE == kModeShadowRender>(a, pre);
+    count_closest<MODE>(a, n);
+    const uint32_t lane = threadIdx.x & 31u, refill = a.refill;
+    unsigned long long c_nodes = 0, c_tris = 0, c_inst = 0;
+
+    bool active = false, exhausted = false;
+    uint32_t i = 0, j = 0, iter = 0;
+    float tmin = 0.f, tmax = 0.f;
+    SpaceRay wr, cr;
+    uint32_t oct = 0;
+    Shear sh;
+    Best2 best;
+    best.reset(0.f);
+    float any_V = 0.f, any_W = 0.f, any_det = 1.f;
+    bool found = false, ok = true, in_blas = false;
+    uint2 stack[kStack8];
+    int sp = 0;
+    const float4* nodes = nullptr;
+    const float4* tris = nullptr;
+    uint32_t cur_id = 0, cur_leaf = 0;
+    Groups G{0, 0, 0, 0, 0};
+
+    for (;;) {
+        const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
+        if (!exhausted && idle != 0u && (__popc(idle) >= (int)refill || idle == 0xFFFFFFFFu)) {
+            const uint32_t k = (uint32_t)__popc(idle);
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(a.work_counter, k);
+            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            if (base + k >= n) exhausted = true;
+            const uint32_t idx = base + (uint32_t)__popc(idle & ((1u << lane) - 1u));
+            if (!active && idx < n) {
+                i = idx;
+                j = sub_entry(a, pre, i);
+                const float4 r0 = __ldg(a.rays + 2 * (size_t)j), r1 = __ldg(a.rays + 2 * (size_t)j + 1);
+                tmin = r0.w;
+                tmax = r1.w;
+                wr.ox = r0.x; wr.oy = r0.y; wr.oz = r0.z;
+                wr.ix = safe_rcp(r1.x); wr.iy = safe_rcp(r1.y); wr.iz = safe_rcp(r1.z);
+                cr = wr;
+                oct = oct_of(wr);
+                best.reset(tmax);
+                found = false;
+                ok = true;
+                in_blas = false;
+                sp = 0;
+                nodes = a.tlas_nodes8;
+                // the root as the only internal child (slot 0) of a virtual node
+                G = Groups{0u, 1u << oct, 1u, 0u, 0u};
+                iter = 0;
+                active = true;
+            }
+        }
+        const uint32_t act = __ballot_sync(0xFFFFFFFFu, active);
+        if (act == 0u) break;
+        const uint32_t bt = __ballot_sync(0xFFFFFFFFu, active && G.ibits && in_blas);
+        const uint32_t bi = __ballot_sync(0xFFFFFFFFu, active && G.ibits && !in_blas);
+        const bool few_nodes = __popc(act & ~bt & ~bi) < kLeafNodesMin8;
+        if (!active) continue;
+        if (G.ibits && !few_nodes && __popc(in_blas ? bt : bi) < kLeafBatch8) continue;
+
+        bool finished = false;
+        if (!G.ibits) {
+            const uint32_t b = 31 - __clz(G.hits);
+            const uint32_t s = b ^ oct;
+            const uint32_t node = G.base + __popc(G.imask & ((1u << s) - 1u));
+            G.hits &= ~(1u << b);
+            if (++iter > iter_cap) {
+                record_error(a.st, RG_ERR_TIMEOUT);
+                ok = false;
+                finished = true;
+            } else if (G.hits && sp >= kStack8) {
+                record_error(a.st, RG_ERR_STACK);
+                ok = false;
+                finished = true;
+            } else {
+                if (G.hits) stack[sp++] = make_uint2(G.base, G.hits | (G.imask << 8) | kKindNode);
+                if (STATS) ++c_nodes;
+                visit8(nodes + 5 * (size_t)node, cr, oct, tmin, __fmul_rn(kAny ? tmax : best.t, kCullSlack), G);
+            }
+        } else if (++iter > iter_cap) {
+            record_error(a.st, RG_ERR_TIMEOUT);
+            ok = false;
+            finished = true;
+        } else if (!in_blas) {
+            // instance: save the TLAS groups, enter its BLAS
+            const uint32_t k = __ffs(G.ibits) - 1;
+            G.ibits &= G.ibits - 1;
+            const uint32_t item = G.ibase + k;
+            if (sp + 3 > kStack8) {
+                record_error(a.st, RG_ERR_STACK);
+                ok = false;
+                finished = true;
+            } else {
+                if (G.hits) stack[sp++] = make_uint2(G.base, G.hits | (G.imask << 8) | kKindNode);
+                if (G.ibits) stack[sp++] = make_uint2(G.ibase, G.ibits | kKindItem);
+                stack[sp++] = make_uint2(0u, kKindMarker);
+                const InstDev* I = a.inst8 + item;
+                const float4 m0 = __ldg(&I->inv[0]), m1 = __ldg(&I->inv[1]), m2 = __ldg(&I->inv[2]);
+                const float4 meta0 = __ldg(reinterpret_cast<const float4*>(&I->nodes));
+                const uint4 meta1 = __ldg(reinterpret_cast<const uint4*>(&I->root));
+                if (STATS) ++c_inst;
+                const float4 r1w = __ldg(a.rays + 2 * (size_t)j + 1);  // the world direction, read again
+                const float dx = r1w.x, dy = r1w.y, dz = r1w.z;
+                const float ox = fmaf(m0.x, wr.ox, fmaf(m0.y, wr.oy, fmaf(m0.z, wr.oz, m0.w)));
+                const float oy = fmaf(m1.x, wr.ox, fmaf(m1.y, wr.oy, fmaf(m1.z, wr.oz, m1.w)));
+                const float oz = fmaf(m2.x, wr.ox, fmaf(m2.y, wr.oy, fmaf(m2.z, wr.oz, m2.w)));
+                const float ddx = fmaf(m0.x, dx, fmaf(m0.y, dy, __fmul_rn(m0.z, dz)));
+                const float ddy = fmaf(m1.x, dx, fmaf(m1.y, dy, __fmul_rn(m1.z, dz)));
+                const float ddz = fmaf(m2.x, dx, fmaf(m2.y, dy, __fmul_rn(m2.z, dz)));
+                cr.ox = ox; cr.oy = oy; cr.oz = oz;
+                cr.ix = safe_rcp(ddx); cr.iy = safe_rcp(ddy); cr.iz = safe_rcp(ddz);
+                oct = oct_of(cr);
+                sh = make_shear(ox, oy, oz, ddx, ddy, ddz);
+                nodes = reinterpret_cast<const float4*>(
+                    ((unsigned long long)__float_as_uint(meta0.y) << 32) | __float_as_uint(meta0.x));
+                tris = reinterpret_cast<const float4*>(
+                           ((unsigned long long)__float_as_uint(meta0.w) << 32) | __float_as_uint(meta0.z)) +
+                       3 * sh.order;  // the ray's axis order
+                cur_id = meta1.y;
+                cur_leaf = item;
+                in_blas = true;
+                G = Groups{0u, 1u << oct, 1u, 0u, 0u};
+            }
+        } else {
+            const uint32_t k = __ffs(G.ibits) - 1;
+            G.ibits &= G.ibits - 1;
+            const uint32_t item = G.ibase + k;
+            const float4* tp = tri_rec(tris, item);
+            const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
+            if (STATS) ++c_tris;
+            const float tlo = kAny ? tmax : (kTies && found ? fminf(__fmul_rn(best.t, kTieBand), tmax) : best.t);
+            const TriResult h = tri_test(sh, v0, v1, v2, tmin, tlo);
+            if (h.hit) {
+                const uint32_t prim = __float_as_uint(v0.w);
+                if (kTies) {
+                    if (best.offer(h.t, cur_id, prim)) found = true;
+                } else if (kAny || h.t < best.t || cur_id < best.id || (cur_id == best.id && prim < best.prim)) {
+                    best.t = h.t; best.id = cur_id; best.prim = prim;
+                    best.il = cur_leaf; best.tl = item;
+                    any_V = h.V; any_W = h.W; any_det = h.det;
+                    found = true;
+                }
+                if (kAny) finished = true;
+            }
+        }
+        // pop what the step left (the marker brings back the world-space ray)
+        while (!finished && !G.ibits && !G.hits) {
+            if (sp == 0) {
+                finished = true;
+                break;
+            }
+            const uint2 e = stack[--sp];
+            const uint32_t kind = e.y & (3u << 30);
+            if (kind == kKindMarker) {
+                in_blas = false;
+                nodes = a.tlas_nodes8;
+                cr = wr;
+                oct = oct_of(wr);
+            } else if (kind == kKindItem) {
+                G.ibase = e.x;
+                G.ibits = e.y & 0xFFFFFFu;
+            } else {
+                G.base = e.x;
+                G.hits = e.y & 0xFFu;
+                G.imask = (e.y >> 8) & 0xFFu;
+            }
+        }
+        if (finished) {
+            emit<MODE>(a, i, j, found && ok, ok, best.t, best.id, best.prim, best.il, best.tl,
+                       kTies ? best.tie_id() : kMiss, best.prim2, any_V, any_W, any_det);
+            active = false;
+        }
+    }
+    flush_counts<kAny, STATS>(a, c_nodes, c_tris, c_inst);
+}
+
+// The queries of rg_trace_rays, whose rays are often incoherent, take the
+// per-lane kernel (2^21 closest and as many any hits of the medium scene: 1,960
+// us, whole-warp 3,549), the renderer's rays the whole-warp one (the medium
+// frame at 1080p: 3,516 us, per-lane 4,145).
+template <int MODE, bool STATS>
+cudaError_t launch_mode8(const TraceArgs& a0, cudaStream_t s) {
+    constexpr bool kLane = MODE == kModeClosestAbi || MODE == kModeAnyAbi;
+    TraceArgs a = a0;
+    a.refill = kRefill8;
+    auto kernel = [] {
+        if constexpr (kLane)
+            return k_trace8_lane<MODE, STATS>;
+        else
+            return k_trace8<MODE, STATS>;
+    }();
     static std::atomic<int> cached{0};  // per process; concurrent first callers store the same value
     int blocks = cached.load(std::memory_order_relaxed);
     if (blocks == 0) {
         int per_sm = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace8<MODE, STATS>, kTraceBlock, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kTraceBlock, 0);
         if (e != cudaSuccess) return e;
         blocks = device_sm_count() * (per_sm > 0 ? per_sm : 1);
         cached.store(blocks, std::memory_order_relaxed);
     }
-    k_trace8<MODE, STATS><<<blocks, kTraceBlock, 0, s>>>(a);
+    kernel<<<blocks, kTraceBlock, 0, s>>>(a);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -171,6 +171,18 @@ def test_identical_hits_large_full_launch():
         assert torch.equal(a[:, 0] == -1, b[:, 0] == -1)
 
 
+@pytest.mark.parametrize("n", [1, 7, 31, 33, 4097, 120_001])
+def test_identical_hits_any_number_of_rays(n):
+    """Fewer rays than a warp's lanes, than the resident lanes, and more, a
+    third of them sharing an origin on a cube's corner: the records of closest
+    hits bit for bit, the occlusion of any hits, as the binary BVH gives them."""
+    s = _random_scene(83, 200)
+    lo, hi = s.world_aabb()
+    rays = g.random_rays(n, lo - 5, hi + 5, seed=n)
+    rays[::3, :3] = s.M[0][:, 3] + s.M[0][:, :3] @ np.full(3, 0.5, np.float32)
+    compare_paths(s, rays, any_tmax=np.random.default_rng(n).uniform(1, 60, n))
+
+
 def test_compressed_render_matches_plain_render():
     s = g.medium_scene()
     with rg.GpuScene(s, flags=rg.RG_SCENE_COMPRESSED) as gw:
