@@ -226,7 +226,7 @@ cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasS
 // sah.cu: binned-SAH topology.
 constexpr int kSahBins = 16;            // bins per axis
 constexpr uint32_t kSahChunk = 1024;    // positions per block of a level's kernels
-constexpr uint32_t kSahMid = 512;       // segments of at most this many items are built in a block
+constexpr uint32_t kSahMid = 1024;      // segments of at most this many items are built in a block
 constexpr uint32_t kSahTiny = 32;       // of at most this many, in a warp
 constexpr uint32_t kSahMaxLevels = 40;  // deeper segments get the Karras hierarchy whatever their size
 constexpr uint32_t kSahOneMax = 4096;   // items of a build without host round trips

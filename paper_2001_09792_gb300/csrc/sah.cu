@@ -19,7 +19,7 @@
 //     (bins, splits, partition), blocks of kSahChunk positions;
 //   kSahTiny + 1 .. kSahMid items: a block per segment builds its levels in
 //     shared memory (k_sah_block);
-//   at most kSahTiny items: a warp per segment builds it to the end
+//   at most kSahTiny items: a warp or three per segment build it to the end
 //     (k_sah_tiny), an item a lane.
 // Bound by latency: the levels are a serial chain, and a level of one block
 // waits on its barriers and atomics, not on memory.  The splits' bins also
@@ -573,10 +573,10 @@ struct BlockSah {
     alignas(16) int pat[kAcc];           // the accumulators' initial values of one segment
     uint32_t m, mnext, wsum[32];
 };
-constexpr int kMidThreads = 256, kTopThreads = 1024;
+constexpr int kMidThreads = 512, kTopThreads = 1024;
 using BlockMid = BlockSah<(int)kSahMid, (int)(kSahMid / (kSahTiny + 1) + 1)>;
 using BlockTop = BlockSah<(int)kSahOneMax, (int)(kSahOneMax / (kSahMid + 1) + 1)>;
-static_assert(sizeof(BlockTop) <= 227 * 1024 && 4 * (sizeof(BlockMid) + 1024) <= 227 * 1024, "shared memory of the SAH blocks");
+static_assert(sizeof(BlockTop) <= 227 * 1024 && 2 * (sizeof(BlockMid) + 1024) <= 227 * 1024, "shared memory of the SAH blocks");
 static_assert(kSahOneMax <= 0xFFFFu, "16-bit positions");
 
 // Keys of a segment through its positions' items.
@@ -945,56 +945,70 @@ __global__ void __launch_bounds__(kTopThreads, 1) k_sah_rest(SahBuild B, uint32_
     }
 }
 
-// A warp per pending segment of at most kSahTiny items, an item a lane.  A
-// split of few items has few distinct partitions: each lane tries, on each
-// axis, the boundary above its item's bin (the first boundary of every
-// distinct partition is one of these), going over the items of its segment;
-// no bins are kept and the warp meets no block barrier.  Same costs, order of
-// candidates and results as the binned sweep.
-constexpr int kTinyBlock = 128;
-template <class K>
+// A warp (W = 1), or three with an axis each (W = 3), per pending segment of at
+// most kSahTiny items, an item a lane.  A split of few items has few distinct
+// partitions: each lane tries, on each axis, the boundary above its item's bin
+// (the first boundary of every distinct partition is one of these), going over
+// the items of its subsegment; no bins are kept, and no barrier is wider than the
+// segment's warps.  Same costs, order of candidates and results as the binned
+// sweep.  Bound by the latency of the lanes' loops in a small build, where
+// three warps shorten them (a tick of 4,096 instances 286 -> 264 us, the four
+// medium meshes 1,733 -> 1,721), by issue in a large one, where they repeat
+// the rest (400,000 triangles 1,254 -> 1,321 us): see the launch.
+constexpr int kTinyBlock = 96;
+constexpr uint32_t kSahWideMax = 65536;
+template <class K, int W>
 __global__ void __launch_bounds__(kTinyBlock) k_sah_tiny(SahBuild B) {
-    struct Warp {
-        int box[32][6];                  // ordered ints of each position's box
-        unsigned long long key[32];
-        uint32_t prim[32], bins[32];
-        uint16_t item[32];               // its position in the segment as it came
+    constexpr int A = 3 / W, GROUPS = kTinyBlock / (32 * W);  // axes of a warp, segments of a block
+    struct Group {
+        int box[2][32][6];               // ordered ints of each position's box (two buffers)
+        unsigned long long key[W][32], best[W][32];
+        uint32_t prim[2][32];
+        uint16_t item[2][32];            // its position in the segment as it came
+        uint8_t bin[3][32];
     };
-    __shared__ Warp sw[kTinyBlock / 32];
-    Warp& S = sw[threadIdx.x >> 5];
+    __shared__ Group sg[GROUPS];
     const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
-    const uint32_t m = B.cnt[kCntTiny], n_warps = gridDim.x * (kTinyBlock / 32);
-    for (uint32_t w = blockIdx.x * (kTinyBlock / 32) + (threadIdx.x >> 5); w < m; w += n_warps) {
+    const int warp = (int)(threadIdx.x >> 5), part = W == 1 ? 0 : warp, axis0 = part * A;
+    Group& S = sg[W == 1 ? warp : 0];
+    const auto sync = [] {
+        if (W == 1)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
+    const uint32_t m = B.cnt[kCntTiny];
+    for (uint32_t w = blockIdx.x * GROUPS + (W == 1 ? warp : 0); w < m; w += gridDim.x * GROUPS) {
         const SahPending T = B.tiny[w];
-        const uint32_t* src = B.prim[T.buf];
         const bool valid = lane < T.count;
-        uint32_t prim = 0, item = lane;
-        int bx[6] = {0, 0, 0, 0, 0, 0};
-        if (valid) {
-            prim = src[T.begin + lane];
-            float f[6];
+        int cb = 0;
+        sync();
+        if (part == 0) {
+            S.item[0][lane] = (uint16_t)lane;
+            if (valid) {
+                const uint32_t prim = B.prim[T.buf][T.begin + lane];
+                float f[6];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                f[k] = B.lohi[6 * (size_t)prim + k];
-                bx[k] = f2ord(f[k]);
+                for (int k = 0; k < 6; ++k) {
+                    f[k] = B.lohi[6 * (size_t)prim + k];
+                    S.box[0][lane][k] = f2ord(f[k]);
+                }
+                S.prim[0][lane] = prim;
+                if (has_nan(f)) *B.boxes_done = 0u;
             }
-            if (has_nan(f)) *B.boxes_done = 0u;
         }
-        // this lane's segment: positions sb .. sb + sc - 1, root node sn
+        sync();
+        // this lane's subsegment: positions sb .. sb + sc - 1, root node sn
         uint32_t sb = 0, sc = valid && T.count > 1 ? T.count : 0u, sn = T.node;
         for (uint32_t level = T.level;; ++level) {
-            __syncwarp();
-#pragma unroll
-            for (int k = 0; k < 6; ++k) S.box[lane][k] = bx[k];
-            S.item[lane] = (uint16_t)item;
-            __syncwarp();
+            const int(*box)[6] = S.box[cb];
             if (sc == 2) {
-                if (lane == sb) {
+                if (part == 0 && lane == sb) {
                     float l[6], r[6];
 #pragma unroll
                     for (int k = 0; k < 6; ++k) {
-                        l[k] = ord2f(bx[k]);
-                        r[k] = ord2f(S.box[lane + 1][k]);
+                        l[k] = ord2f(box[lane][k]);
+                        r[k] = ord2f(box[lane + 1][k]);
                     }
                     emit_sah_node(sn, T.begin + sb, 2, 1, B.n, B.nodes, B.parents, B.ranges);
                     put_child_boxes(B.nodes, sn, l, r);
@@ -1002,8 +1016,8 @@ __global__ void __launch_bounds__(kTinyBlock) k_sah_tiny(SahBuild B) {
                 sc = 0;
             }
             if (sc >= 3 && level >= kSahMaxLevels) {
-                if (lane == sb) {
-                    const LocalKeys<K> ks{static_cast<const K*>(B.key[T.buf]) + T.begin, S.item + sb};
+                if (part == 0 && lane == sb) {
+                    const LocalKeys<K> ks{static_cast<const K*>(B.key[T.buf]) + T.begin, S.item[cb] + sb};
                     for (uint32_t i = 0; i + 1 < sc; ++i)
                         karras_node(ks, sc, (int64_t)i, reinterpret_cast<uint32_t*>(B.nodes) + 12, 16, B.parents,
                                     B.ranges, sn, T.begin + sb, B.n);
@@ -1012,112 +1026,119 @@ __global__ void __launch_bounds__(kTinyBlock) k_sah_tiny(SahBuild B) {
                 sc = 0;
             }
             const bool active = sc >= 3;
-            if (!__any_sync(0xFFFFFFFFu, active)) break;
-            // the frame of the segment, and this item's bins
-            int mn[3] = {ord_inf(), ord_inf(), ord_inf()}, mx[3] = {ord_ninf(), ord_ninf(), ord_ninf()};
-            for (uint32_t j = sb; j < sb + sc; ++j) {
+            if (!__any_sync(0xFFFFFFFFu, active)) break;  // (the same in all the segment's warps)
+            // per axis: the frame of the subsegment, and this item's bin
+            int bin[A];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const int c = f2ord(__fmul_rn(0.5f, __fadd_rn(ord2f(S.box[j][k]), ord2f(S.box[j][3 + k]))));
-                    mn[k] = min(mn[k], c);
-                    mx[k] = max(mx[k], c);
+            for (int q = 0; q < A; ++q) {
+                const int axis = axis0 + q;
+                int mn = ord_inf(), mx = ord_ninf();
+                for (uint32_t j = sb; j < sb + sc; ++j) {
+                    const int c = f2ord(__fmul_rn(0.5f, __fadd_rn(ord2f(box[j][axis]), ord2f(box[j][3 + axis]))));
+                    mn = min(mn, c);
+                    mx = max(mx, c);
                 }
+                const float cmin = ord2f(mn);
+                bin[q] = 0;
+                if (active)
+                    bin[q] = bin_of(__fmul_rn(0.5f, __fadd_rn(ord2f(box[lane][axis]), ord2f(box[lane][3 + axis]))),
+                                    cmin, bin_scale(cmin, ord2f(mx)));
+                S.bin[axis][lane] = (uint8_t)bin[q];
             }
-            int bin[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const float lo = ord2f(mn[k]);
-                bin[k] = bin_of(__fmul_rn(0.5f, __fadd_rn(ord2f(bx[k]), ord2f(bx[3 + k]))), lo,
-                                bin_scale(lo, ord2f(mx[k])));
-            }
-            S.bins[lane] = (uint32_t)(bin[0] | (bin[1] << 8) | (bin[2] << 16));
             __syncwarp();
-            // both sides of this item's three boundaries
-            int lb[3][6], rb[3][6];
-            uint32_t nl[3] = {0, 0, 0};
+            // both sides of this item's boundary on each axis
+            int lb[A][6], rb[A][6];
+            uint32_t nl[A];
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
+            for (int q = 0; q < A; ++q) {
+                nl[q] = 0;
 #pragma unroll
-                for (int k = 0; k < 6; ++k) lb[a][k] = rb[a][k] = k < 3 ? ord_inf() : ord_ninf();
+                for (int k = 0; k < 6; ++k) lb[q][k] = rb[q][k] = k < 3 ? ord_inf() : ord_ninf();
+            }
             for (uint32_t j = sb; j < sb + sc; ++j) {
                 int v[6];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) v[k] = S.box[j][k];
-                const uint32_t bj = S.bins[j];
+                for (int k = 0; k < 6; ++k) v[k] = box[j][k];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const bool l = (int)((bj >> (8 * a)) & 0xFFu) <= bin[a];
-                    nl[a] += l;
+                for (int q = 0; q < A; ++q) {
+                    const bool l = (int)S.bin[axis0 + q][j] <= bin[q];
+                    nl[q] += l;
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         if (l) {
-                            lb[a][k] = min(lb[a][k], v[k]);
-                            lb[a][3 + k] = max(lb[a][3 + k], v[3 + k]);
+                            lb[q][k] = min(lb[q][k], v[k]);
+                            lb[q][3 + k] = max(lb[q][3 + k], v[3 + k]);
                         } else {
-                            rb[a][k] = min(rb[a][k], v[k]);
-                            rb[a][3 + k] = max(rb[a][3 + k], v[3 + k]);
+                            rb[q][k] = min(rb[q][k], v[k]);
+                            rb[q][3 + k] = max(rb[q][3 + k], v[3 + k]);
                         }
                     }
                 }
             }
             unsigned long long mine = ~0ull;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (nl[a] == 0 || nl[a] >= sc) continue;
+            for (int q = 0; q < A; ++q) {
+                if (nl[q] == 0 || nl[q] >= sc) continue;
                 float l[6], r[6];
 #pragma unroll
                 for (int k = 0; k < 6; ++k) {
-                    l[k] = ord2f(lb[a][k]);
-                    r[k] = ord2f(rb[a][k]);
+                    l[k] = ord2f(lb[q][k]);
+                    r[k] = ord2f(rb[q][k]);
                 }
-                const float cost = __fadd_rn(__fadd_rn(__fmul_rn(half_area(l, l + 3), (float)nl[a]),
-                                                       __fmul_rn(half_area(r, r + 3), (float)(sc - nl[a]))),
+                const float cost = __fadd_rn(__fadd_rn(__fmul_rn(half_area(l, l + 3), (float)nl[q]),
+                                                       __fmul_rn(half_area(r, r + 3), (float)(sc - nl[q]))),
                                              0.0f);
                 if (!(cost < INFINITY)) continue;
-                const unsigned long long key = split_key(cost, a, bin[a] + 1);
+                const unsigned long long key = split_key(cost, axis0 + q, bin[q] + 1);
                 mine = key < mine ? key : mine;
             }
-            S.key[lane] = mine;
+            S.key[part][lane] = mine;
             __syncwarp();
             unsigned long long best = ~0ull;
-            for (uint32_t j = sb; j < sb + sc; ++j) best = S.key[j] < best ? S.key[j] : best;
+            for (uint32_t j = sb; j < sb + sc; ++j) best = S.key[part][j] < best ? S.key[part][j] : best;
+            S.best[part][lane] = best;
+            sync();
+#pragma unroll
+            for (int a = 0; a < W; ++a) best = S.best[a][lane] < best ? S.best[a][lane] : best;
             const bool cut = active && best != ~0ull;
-            const int axis = cut ? (int)((uint32_t)best / (kSahBins - 1)) : -1;
+            const int ax = cut ? (int)((uint32_t)best / (kSahBins - 1)) : 0;
             const int split = (int)((uint32_t)best % (kSahBins - 1)) + 1;
-            const int ba = axis == 0 ? bin[0] : (axis == 1 ? bin[1] : bin[2]);
-            const bool left = active && (cut ? ba < split : lane - sb < sc / 2);
+            const bool left = active && (cut ? (int)S.bin[ax][lane] < split : lane - sb < sc / 2);
             const uint32_t seg = active ? (0xFFFFFFFFu >> (32u - sc)) << sb : 0u;
             const uint32_t bal = __ballot_sync(0xFFFFFFFFu, left) & seg;
             const uint32_t own = __ballot_sync(0xFFFFFFFFu, cut && mine == best) & seg;
             const uint32_t nleft = (uint32_t)__popc(bal);
-            if (cut && (own & lt) == 0u && mine == best) {
+            if (cut && mine == best && (own & lt) == 0u) {  // (a key names its axis: one warp has it)
                 float l[6], r[6];
 #pragma unroll
                 for (int k = 0; k < 6; ++k) {
-                    l[k] = ord2f(axis == 0 ? lb[0][k] : (axis == 1 ? lb[1][k] : lb[2][k]));
-                    r[k] = ord2f(axis == 0 ? rb[0][k] : (axis == 1 ? rb[1][k] : rb[2][k]));
+                    int x = lb[0][k], y = rb[0][k];
+#pragma unroll
+                    for (int q = 1; q < A; ++q)
+                        if (ax == q) {
+                            x = lb[q][k];
+                            y = rb[q][k];
+                        }
+                    l[k] = ord2f(x);
+                    r[k] = ord2f(y);
                 }
                 put_child_boxes(B.nodes, sn, l, r);
             }
             uint32_t dest = lane;
             if (active) {
-                if (lane == sb) {
+                if (part == 0 && lane == sb) {
                     emit_sah_node(sn, T.begin + sb, sc, nleft, B.n, B.nodes, B.parents, B.ranges);
                     if (!cut) *B.boxes_done = 0u;
                 }
                 const uint32_t lr = (uint32_t)__popc(bal & lt);
                 dest = left ? sb + lr : sb + nleft + ((lane - sb) - lr);
             }
-            __syncwarp();
 #pragma unroll
-            for (int k = 0; k < 6; ++k) S.box[dest][k] = bx[k];
-            S.prim[dest] = prim;
-            S.item[dest] = (uint16_t)item;
-            __syncwarp();
-#pragma unroll
-            for (int k = 0; k < 6; ++k) bx[k] = S.box[lane][k];
-            prim = S.prim[lane];
-            item = S.item[lane];
+            for (int c = 0; c < 2 * A; ++c) S.box[cb ^ 1][dest][2 * axis0 + c] = box[lane][2 * axis0 + c];
+            if (part == 0) S.prim[cb ^ 1][dest] = S.prim[cb][lane];
+            if (part == W - 1) S.item[cb ^ 1][dest] = S.item[cb][lane];
+            cb ^= 1;
+            sync();
             if (active) {
                 if (lane - sb < nleft) {
                     sc = nleft;
@@ -1130,7 +1151,7 @@ __global__ void __launch_bounds__(kTinyBlock) k_sah_tiny(SahBuild B) {
                 if (sc < 2) sc = 0;
             }
         }
-        if (valid) B.prim[0][T.begin + lane] = prim;
+        if (valid && part == 0) B.prim[0][T.begin + lane] = S.prim[cb][lane];
     }
 }
 
@@ -1214,7 +1235,11 @@ rg_status sah_build(SahBuild B, const int* cb_ord, cudaStream_t s) {
         k_sah_block<K><<<std::min(n / (kSahTiny + 1) + 1, 4 * sms), kMidThreads, sizeof(BlockMid), s>>>(B);
         count_launches(1);
     }
-    k_sah_tiny<K><<<std::min(n / 128u + 1u, 8 * sms), kTinyBlock, 0, s>>>(B);
+    // three warps per segment while the chip holds all segments at once that way
+    if (n <= kSahWideMax)
+        k_sah_tiny<K, 3><<<std::min(n / 16u + 1u, 16 * sms), kTinyBlock, 0, s>>>(B);
+    else
+        k_sah_tiny<K, 1><<<8 * sms, kTinyBlock, 0, s>>>(B);
     count_launches(1);
     SAH_CK(cudaGetLastError());
     return RG_OK;

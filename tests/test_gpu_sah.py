@@ -118,9 +118,9 @@ def clusters(n, seed):
     return boxes_mesh(lo, (lo + np.abs(lo) * np.float32(0.01)).astype(np.float32))
 
 
-@pytest.mark.parametrize("mesh,n", [("ico", k) for k in (31, 32, 33, 511, 512, 513, 1025, 4095, 4096, 4097)] +
+@pytest.mark.parametrize("mesh,n", [("ico", k) for k in (31, 32, 33, 511, 512, 513, 1023, 1024, 1025, 4095, 4096, 4097)] +
                          [("clusters", k) for k in (32, 512, 700, 4096, 9001)] +
-                         [("chain", k) for k in (600, 5000)])
+                         [("chain", k) for k in (600, 2000, 5000)])
 @pytest.mark.parametrize("morton", [rg.RG_MORTON30, rg.RG_MORTON63])
 def test_sah_ranges_of_the_build(mesh, n, morton):
     """Both sides of the sizes at which the build goes over from levels of all
