@@ -64,6 +64,7 @@ __device__ __forceinline__ void reduce_bounds(int* cb_ord, int c0, int c1, int c
 __device__ __forceinline__ float centroid(float lo, float hi) { return __fmul_rn(__fadd_rn(lo, hi), 0.5f); }
 
 __global__ void k_init_bounds(int* cb_ord) {
+    chain_wait();
     int t = threadIdx.x;
     if (t < 3) cb_ord[t] = f2ord(__int_as_float(0x7F800000));        // +inf
     else if (t < 6) cb_ord[t] = f2ord(__int_as_float(0xFF800000));   // -inf
@@ -71,6 +72,7 @@ __global__ void k_init_bounds(int* cb_ord) {
 
 // The same, and a BLAS's descriptor (its boxes come later).
 __global__ void k_blas_begin(int* cb_ord, BlasDev* out, BlasDev desc) {
+    chain_wait();
     const int t = threadIdx.x;
     if (t < 3) cb_ord[t] = f2ord(__int_as_float(0x7F800000));
     else if (t < 6) cb_ord[t] = f2ord(__int_as_float(0xFF800000));
@@ -79,6 +81,7 @@ __global__ void k_blas_begin(int* cb_ord, BlasDev* out, BlasDev desc) {
 
 __global__ void k_tri_bounds(const float* __restrict__ vtx, uint32_t nv, const uint32_t* __restrict__ idx,
                              uint32_t nt, float* __restrict__ lohi, int* cb_ord, DevStatus* st) {
+    chain_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     bool valid = i < nt;
     int c[3] = {0, 0, 0};
@@ -103,6 +106,7 @@ __global__ void k_tri_bounds(const float* __restrict__ vtx, uint32_t nv, const u
 }
 
 __global__ void k_centroid_bounds(const float* __restrict__ lohi, uint32_t n, int* cb_ord) {
+    chain_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     bool valid = i < n;
     int c[3] = {0, 0, 0};
@@ -160,6 +164,7 @@ __device__ __forceinline__ uint32_t morton30(const MortonGrid& g, const float* b
 template <int BITS>
 __global__ void k_morton(const float* __restrict__ lohi, uint32_t n, const int* __restrict__ cb_ord,
                          void* __restrict__ codes, float* cb_out) {
+    chain_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     const MortonGrid g = morton_grid(cb_ord, BITS);
     if (cb_out && i == 0) {
@@ -250,6 +255,7 @@ __device__ __forceinline__ uint32_t scan256(uint32_t v, uint32_t* wsum) {
 template <class K>
 __global__ void __launch_bounds__(kSortThreads) k_rs_hist(const K* __restrict__ keys, uint32_t n,
                                                            uint32_t* __restrict__ hist) {
+    chain_wait();
     constexpr int P = (int)sizeof(K);
     __shared__ uint32_t cnt[P][256];
 #pragma unroll
@@ -277,6 +283,7 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_pass(const K* __restrict__ 
                                                            uint32_t n, int shift, const uint32_t* __restrict__ hist,
                                                            W* status, W* __restrict__ next, uint32_t* ticket,
                                                            K* __restrict__ keys_out, uint32_t* __restrict__ vals_out) {
+    chain_wait();
     constexpr int kTile = kSortThreads * ITEMS;
     constexpr int kFlag = (int)sizeof(W) * 8 - 2;
     constexpr W kOwn = W(1) << kFlag, kAll = W(2) << kFlag, kCount = kOwn - 1;
@@ -384,6 +391,7 @@ constexpr uint32_t kSortOneMax = kSortOneThreads * kSortOneItems;
 template <class K>
 __global__ void __launch_bounds__(kSortOneThreads) k_rs_one(const K* keys, const uint32_t* vals, uint32_t n,
                                                              K* keys_out, uint32_t* vals_out) {
+    chain_wait();
     constexpr int ITEMS = kSortOneItems, kW = kSortOneThreads / 32;
     __shared__ uint16_t s_cnt[kW][256];
     __shared__ K s_pair[kSortOneMax];
@@ -449,6 +457,7 @@ template <class K>
 __global__ void k_karras_segments(const K* __restrict__ keys, const KarrasSeg* __restrict__ segs, uint32_t n_segs,
                                   uint32_t n_threads, uint32_t n_leaves, uint32_t* __restrict__ child_base,
                                   uint32_t* __restrict__ parents, uint32_t* __restrict__ ranges) {
+    chain_wait();
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n_threads) return;
     uint32_t lo = 0, hi = n_segs - 1;
@@ -467,6 +476,7 @@ __global__ void k_karras_segments(const K* __restrict__ keys, const KarrasSeg* _
 template <class K>
 __global__ void k_karras(const K* __restrict__ keys, uint32_t n, uint32_t* __restrict__ child_base, int stride,
                          uint32_t* __restrict__ parents, uint32_t* __restrict__ ranges) {
+    chain_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)n - 1) return;
     karras_node(keys, n, i, child_base, stride, parents, ranges);
@@ -537,6 +547,7 @@ __global__ void k_blas_leaves_refit(const float* __restrict__ vtx, const uint32_
                                     const uint32_t* __restrict__ parents, float4* nodes, uint32_t* flags,
                                     float4* __restrict__ tris, BlasDev* blas_out, DevStatus* st,
                                     const uint32_t* __restrict__ boxes_done) {
+    chain_wait();
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     uint32_t prim = perm[j];
@@ -574,6 +585,7 @@ __global__ void k_blas_leaves_refit(const float* __restrict__ vtx, const uint32_
 // Bounding sphere: the largest upward-rounded squared distance of a vertex
 // from the root box centre, reduced per warp, one atomicMax per warp.
 __global__ void k_bound_sphere(const float* __restrict__ vtx, uint32_t nv, BlasDev* blas) {
+    chain_wait();
     float c[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) c[q] = __fmul_rn(__fadd_rn(blas->lo[q], blas->hi[q]), 0.5f);
@@ -684,6 +696,7 @@ __device__ __forceinline__ void instance_prep_one(const rg_instance* __restrict_
 __global__ void k_instance_prep(const rg_instance* __restrict__ in, uint32_t n, const BlasDev* __restrict__ blas,
                                 uint32_t nblas, InstDev* tmp, float* __restrict__ wbox, int* cb_ord, bool check_blas,
                                 DevStatus* st) {
+    chain_wait();
     uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     bool valid = k < n;
     int c[3] = {0, 0, 0};
@@ -695,6 +708,7 @@ __global__ void k_tlas_leaves_refit(const InstDev* __restrict__ tmp, const float
                                     const uint32_t* __restrict__ perm, uint32_t n, const uint32_t* __restrict__ parents,
                                     float4* nodes, uint32_t* flags, InstDev* __restrict__ inst_out, DevStatus* st,
                                     const uint32_t* __restrict__ boxes_done) {
+    chain_wait();
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     uint32_t k = perm[j];
@@ -719,6 +733,7 @@ __global__ void __launch_bounds__(kTlasSmallMax) k_tlas_small(const rg_instance*
                                                               InstDev* tmp, float* wbox, bool refit, float4* nodes,
                                                               uint32_t* perm, uint32_t* parents, uint32_t* flags,
                                                               uint32_t* ranges, InstDev* inst_out, DevStatus* st) {
+    chain_wait();
     __shared__ int s_cb[6];
     __shared__ uint32_t s_key[kTlasSmallMax], s_val[kTlasSmallMax];
     __shared__ uint32_t s_warp[32], s_total;
@@ -805,13 +820,13 @@ inline unsigned grid_for(size_t n, int block = kBlock) { return (unsigned)((n + 
 }  // namespace
 
 cudaError_t launch_init_bounds(int* cb_ord, cudaStream_t s) {
-    k_init_bounds<<<1, 32, 0, s>>>(cb_ord);
+    launch_chain(k_init_bounds, 1, 32, 0, s, cb_ord);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_blas_begin(int* cb_ord, BlasDev* out, const BlasDev& desc, cudaStream_t s) {
-    k_blas_begin<<<1, 32, 0, s>>>(cb_ord, out, desc);
+    launch_chain(k_blas_begin, 1, 32, 0, s, cb_ord, out, desc);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -819,14 +834,14 @@ cudaError_t launch_blas_begin(int* cb_ord, BlasDev* out, const BlasDev& desc, cu
 cudaError_t launch_tri_bounds(const float* vtx, uint32_t nv, const uint32_t* idx, uint32_t nt, float* lohi,
                               int* cb_ord, DevStatus* st, cudaStream_t s) {
     if (nt == 0) return cudaSuccess;
-    k_tri_bounds<<<grid_for(nt), kBlock, 0, s>>>(vtx, nv, idx, nt, lohi, cb_ord, st);
+    launch_chain(k_tri_bounds, grid_for(nt), kBlock, 0, s, vtx, nv, idx, nt, lohi, cb_ord, st);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_centroid_bounds(const float* lohi, uint32_t n, int* cb_ord, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    k_centroid_bounds<<<grid_for(n), kBlock, 0, s>>>(lohi, n, cb_ord);
+    launch_chain(k_centroid_bounds, grid_for(n), kBlock, 0, s, lohi, n, cb_ord);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -835,9 +850,9 @@ cudaError_t launch_morton(const float* lohi, uint32_t n, const int* cb_ord, int 
                           cudaStream_t s) {
     unsigned g = grid_for(n > 0 ? n : 1);
     if (bits == 10)
-        k_morton<10><<<g, kBlock, 0, s>>>(lohi, n, cb_ord, codes, cb_out);
+        launch_chain(k_morton<10>, g, kBlock, 0, s, lohi, n, cb_ord, codes, cb_out);
     else
-        k_morton<21><<<g, kBlock, 0, s>>>(lohi, n, cb_ord, codes, cb_out);
+        launch_chain(k_morton<21>, g, kBlock, 0, s, lohi, n, cb_ord, codes, cb_out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -847,7 +862,7 @@ static cudaError_t radix_sort_impl(const K* keys_in, const uint32_t* vals_in, ui
                                    uint32_t* vals_out, void* scratch, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     if (n <= kSortOneMax) {
-        k_rs_one<K><<<1, kSortOneThreads, 0, s>>>(keys_in, vals_in, n, keys_out, vals_out);
+        launch_chain(k_rs_one<K>, 1, kSortOneThreads, 0, s, keys_in, vals_in, n, keys_out, vals_out);
         count_launches(1);
         return cudaGetLastError();
     }
@@ -868,7 +883,7 @@ static cudaError_t radix_sort_impl(const K* keys_in, const uint32_t* vals_in, ui
     status[1] = status[0] + (size_t)256 * nb;
     cudaError_t e = cudaMemsetAsync(hist, 0, (256 * 8 + 64) * 4 + (size_t)256 * nb * sizeof(W), s);
     if (e != cudaSuccess) return e;
-    k_rs_hist<K><<<std::min(nb, (uint32_t)device_sm_count() * 4u), kSortThreads, 0, s>>>(keys_in, n, hist);
+    launch_chain(k_rs_hist<K>, std::min(nb, (uint32_t)device_sm_count() * 4u), kSortThreads, 0, s, keys_in, n, hist);
     // even pass count: in -> tmp -> out -> tmp ... ends in `out`
     const K* ksrc = keys_in;
     const uint32_t* vsrc = vals_in;
@@ -877,7 +892,7 @@ static cudaError_t radix_sort_impl(const K* keys_in, const uint32_t* vals_in, ui
         K* kdst = to_out ? keys_out : kt;
         uint32_t* vdst = to_out ? vals_out : vt;
         auto* pass_kernel = large ? k_rs_pass<K, W, 2 * kSortItems> : k_rs_pass<K, W, kSortItems>;
-        pass_kernel<<<nb, kSortThreads, 0, s>>>(
+        launch_chain(pass_kernel, nb, kSortThreads, 0, s, 
             ksrc, vsrc, n, 8 * pass, hist + 256 * pass, status[pass & 1],
             pass + 1 < passes ? status[(pass + 1) & 1] : nullptr, ticket + pass, kdst, vdst);
         ksrc = kdst;
@@ -902,10 +917,10 @@ cudaError_t launch_karras(const void* keys, uint32_t n, int key_bits, uint32_t* 
                           uint32_t* parents, cudaStream_t s, uint32_t* ranges) {
     if (n < 2) return cudaSuccess;
     if (key_bits == 64)
-        k_karras<uint64_t><<<grid_for(n - 1), kBlock, 0, s>>>(static_cast<const uint64_t*>(keys), n, child_base, stride,
+        launch_chain(k_karras<uint64_t>, grid_for(n - 1), kBlock, 0, s, static_cast<const uint64_t*>(keys), n, child_base, stride,
                                                               parents, ranges);
     else
-        k_karras<uint32_t><<<grid_for(n - 1), kBlock, 0, s>>>(static_cast<const uint32_t*>(keys), n, child_base, stride,
+        launch_chain(k_karras<uint32_t>, grid_for(n - 1), kBlock, 0, s, static_cast<const uint32_t*>(keys), n, child_base, stride,
                                                               parents, ranges);
     count_launches(1);
     return cudaGetLastError();
@@ -913,6 +928,7 @@ cudaError_t launch_karras(const void* keys, uint32_t n, int key_bits, uint32_t* 
 
 namespace {
 __global__ void k_invert_perm(const uint32_t* __restrict__ perm, uint32_t n, uint32_t* __restrict__ inv) {
+    chain_wait();
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) inv[perm[j]] = j;
 }
 }  // namespace
@@ -923,10 +939,10 @@ cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasS
     if (n_segs == 0 || n_threads == 0) return cudaSuccess;
     uint32_t* child_base = reinterpret_cast<uint32_t*>(nodes) + 12;
     if (key_bits == 64)
-        k_karras_segments<uint64_t><<<grid_for(n_threads), kBlock, 0, s>>>(
+        launch_chain(k_karras_segments<uint64_t>, grid_for(n_threads), kBlock, 0, s, 
             static_cast<const uint64_t*>(keys), segs, n_segs, n_threads, n_leaves, child_base, parents, ranges);
     else
-        k_karras_segments<uint32_t><<<grid_for(n_threads), kBlock, 0, s>>>(
+        launch_chain(k_karras_segments<uint32_t>, grid_for(n_threads), kBlock, 0, s, 
             static_cast<const uint32_t*>(keys), segs, n_segs, n_threads, n_leaves, child_base, parents, ranges);
     count_launches(1);
     return cudaGetLastError();
@@ -934,7 +950,7 @@ cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasS
 
 cudaError_t launch_invert_perm(const uint32_t* perm, uint32_t n, uint32_t* inv, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    k_invert_perm<<<min(grid_for(n), 4096u), kBlock, 0, s>>>(perm, n, inv);
+    launch_chain(k_invert_perm, min(grid_for(n), 4096u), kBlock, 0, s, perm, n, inv);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -943,7 +959,7 @@ cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, cons
                                      uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
                                      float4* tris, BlasDev* blas_out, DevStatus* st, cudaStream_t s,
                                      const uint32_t* boxes_done) {
-    k_blas_leaves_refit<<<grid_for(n), kBlock, 0, s>>>(vtx, idx, perm, lohi, n, parents, nodes, flags, tris, blas_out,
+    launch_chain(k_blas_leaves_refit, grid_for(n), kBlock, 0, s, vtx, idx, perm, lohi, n, parents, nodes, flags, tris, blas_out,
                                                        st, boxes_done);
     count_launches(1);
     return cudaGetLastError();
@@ -952,7 +968,7 @@ cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, cons
 cudaError_t launch_bound_sphere(const float* vtx, uint32_t nv, BlasDev* blas, cudaStream_t s) {
     if (nv == 0) return cudaSuccess;
     const uint32_t blocks = (uint32_t)min((nv + 255u) / 256u, (uint32_t)device_sm_count() * 4u);
-    k_bound_sphere<<<blocks, 256, 0, s>>>(vtx, nv, blas);
+    launch_chain(k_bound_sphere, blocks, 256, 0, s, vtx, nv, blas);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -960,7 +976,7 @@ cudaError_t launch_bound_sphere(const float* vtx, uint32_t nv, BlasDev* blas, cu
 cudaError_t launch_instance_prep(const rg_instance* in, uint32_t n, const BlasDev* blas, uint32_t nblas,
                                  InstDev* tmp, float* wbox, int* cb_ord, bool check_blas, DevStatus* st,
                                  cudaStream_t s) {
-    k_instance_prep<<<grid_for(n), kBlock, 0, s>>>(in, n, blas, nblas, tmp, wbox, cb_ord, check_blas, st);
+    launch_chain(k_instance_prep, grid_for(n), kBlock, 0, s, in, n, blas, nblas, tmp, wbox, cb_ord, check_blas, st);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -968,7 +984,7 @@ cudaError_t launch_instance_prep(const rg_instance* in, uint32_t n, const BlasDe
 cudaError_t launch_tlas_leaves_refit(const InstDev* tmp, const float* wbox, const uint32_t* perm, uint32_t n,
                                      const uint32_t* parents, float4* nodes, uint32_t* flags, InstDev* inst_out,
                                      DevStatus* st, cudaStream_t s, const uint32_t* boxes_done) {
-    k_tlas_leaves_refit<<<grid_for(n), kBlock, 0, s>>>(tmp, wbox, perm, n, parents, nodes, flags, inst_out, st,
+    launch_chain(k_tlas_leaves_refit, grid_for(n), kBlock, 0, s, tmp, wbox, perm, n, parents, nodes, flags, inst_out, st,
                                                        boxes_done);
     count_launches(1);
     return cudaGetLastError();
@@ -979,7 +995,7 @@ cudaError_t launch_tlas_small(const rg_instance* in, uint32_t n, const BlasDev* 
                               uint32_t* flags, uint32_t* ranges, InstDev* inst_out, DevStatus* st, cudaStream_t s) {
     if (n == 0 || n > kTlasSmallMax) return cudaErrorInvalidValue;
     const uint32_t threads = (n + 31u) & ~31u;
-    k_tlas_small<<<1, threads, 0, s>>>(in, n, blas, nblas, tmp, wbox, refit, nodes, perm, parents, flags, ranges,
+    launch_chain(k_tlas_small, 1, threads, 0, s, in, n, blas, nblas, tmp, wbox, refit, nodes, perm, parents, flags, ranges,
                                        inst_out, st);
     count_launches(1);
     return cudaGetLastError();

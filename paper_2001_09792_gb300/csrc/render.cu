@@ -77,6 +77,7 @@ __device__ __forceinline__ void tile_pixel(uint32_t i, uint32_t w, uint32_t h, u
 
 __global__ void k_raygen(CameraDev cam, uint32_t w, uint32_t h, float4* __restrict__ rays,
                          Payload* __restrict__ payload) {
+    chain_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= w * h) return;
     uint32_t x, y;
@@ -395,6 +396,7 @@ __device__ __forceinline__ void shade_one(const ShadeArgs& a, uint32_t head, uin
 // only on the device; whole blocks step together through the queue so that
 // every thread takes part in the block claims.
 __global__ void __launch_bounds__(kShadeBlock) k_shade(ShadeArgs a, uint32_t n_host) {
+    chain_wait();
     __shared__ ClaimSmem cs;
     claim_init(&cs);
     __syncthreads();
@@ -408,6 +410,7 @@ __global__ void __launch_bounds__(kShadeBlock) k_shade(ShadeArgs a, uint32_t n_h
 // Mixed queue: the count is read on the device; whole blocks step together so
 // that every thread takes part in the block claims.
 __global__ void __launch_bounds__(kShadeBlock) k_shade_batch(ShadeArgs a) {
+    chain_wait();
     __shared__ int live_delta[kMaxSlots];
     __shared__ ClaimSmem cs;
     static_assert(kShadeBlock >= kMaxSlots, "one thread per slot flushes the block's sums");
@@ -430,6 +433,7 @@ __global__ void __launch_bounds__(kShadeBlock) k_shade_batch(ShadeArgs a) {
 __global__ void k_raygen_batch(const RaygenReq* __restrict__ reqs, const uint32_t* __restrict__ n_reqs_p,
                                const uint32_t* __restrict__ n_rays_p, const uint32_t* __restrict__ gen_base_p,
                                uint32_t ring_mask, float4* __restrict__ rays, Payload* __restrict__ payload) {
+    chain_wait();
     __shared__ RaygenReq sr[kMaxSlots];
     const uint32_t n_reqs = min(*n_reqs_p, kMaxSlots);
     const uint32_t n_rays = *n_rays_p, gen_base = *gen_base_p;
@@ -599,6 +603,7 @@ __device__ __forceinline__ float3 fxaa_edge(const FxaaTile<T>& I, int x, int y) 
 template <int T>
 __global__ void __launch_bounds__(kFxaaThreads, 4) k_fxaa(const float4* __restrict__ in, int w, int h,
                                                        float4* __restrict__ out) {
+    chain_wait();
     constexpr int S = FxaaTile<T>::S, kPix = T * T / kFxaaThreads, H = kFxaaHalo;
     constexpr int kRing = S * S - T * T;  // halo pixels: H rows above and below, then H columns left and right
     __shared__ float s[S * S];
@@ -664,7 +669,7 @@ __global__ void __launch_bounds__(kFxaaThreads, 4) k_fxaa(const float4* __restri
 cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, float4* rays, Payload* payload,
                           cudaStream_t s) {
     size_t n = (size_t)w * h;
-    k_raygen<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(cam, w, h, rays, payload);
+    launch_chain(k_raygen, (unsigned)((n + 255) / 256), 256, 0, s, cam, w, h, rays, payload);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -673,7 +678,7 @@ cudaError_t launch_shade(const ShadeArgs& a, uint32_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     // n: the rays (a.d_count null) or a bound on them; blocks loop over the queue
     const uint32_t blocks = min((n + kShadeBlock - 1) / kShadeBlock, (uint32_t)device_sm_count() * 8u);
-    k_shade<<<blocks, kShadeBlock, 0, s>>>(a, n);
+    launch_chain(k_shade, blocks, kShadeBlock, 0, s, a, n);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -682,13 +687,13 @@ cudaError_t launch_raygen_batch(const RaygenReq* reqs, const uint32_t* n_reqs, u
                                 const uint32_t* n_rays, const uint32_t* gen_base, uint32_t ring_mask, float4* rays,
                                 Payload* payload, cudaStream_t s) {
     const uint32_t blocks = (uint32_t)min((max_rays + 255u) / 256u, (uint32_t)device_sm_count() * 8u);
-    k_raygen_batch<<<blocks > 0 ? blocks : 1, 256, 0, s>>>(reqs, n_reqs, n_rays, gen_base, ring_mask, rays, payload);
+    launch_chain(k_raygen_batch, blocks > 0 ? blocks : 1, 256, 0, s, reqs, n_reqs, n_rays, gen_base, ring_mask, rays, payload);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_shade_batch(const ShadeArgs& a, cudaStream_t s) {
-    k_shade_batch<<<device_sm_count() * 8, kShadeBlock, 0, s>>>(a);
+    launch_chain(k_shade_batch, device_sm_count() * 8, kShadeBlock, 0, s, a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -699,9 +704,9 @@ cudaError_t launch_fxaa(const float4* in, uint32_t w, uint32_t h, float4* out, c
     // tiles 4; the small ones where the large would not give every SM a block
     const uint64_t tiles = (uint64_t)((w + 31) / 32) * ((h + 31) / 32);
     if (tiles >= (uint64_t)device_sm_count() && (h + 15) / 16 <= 65535)
-        k_fxaa<32><<<dim3((w + 31) / 32, (h + 31) / 32), kFxaaThreads, 0, s>>>(in, (int)w, (int)h, out);
+        launch_chain(k_fxaa<32>, dim3((w + 31) / 32, (h + 31) / 32), kFxaaThreads, 0, s, in, (int)w, (int)h, out);
     else
-        k_fxaa<16><<<dim3((w + 15) / 16, (h + 15) / 16), kFxaaThreads, 0, s>>>(in, (int)w, (int)h, out);
+        launch_chain(k_fxaa<16>, dim3((w + 15) / 16, (h + 15) / 16), kFxaaThreads, 0, s, in, (int)w, (int)h, out);
     count_launches(1);
     return cudaGetLastError();
 }

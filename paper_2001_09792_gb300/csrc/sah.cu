@@ -247,6 +247,7 @@ __device__ __forceinline__ void push_pending(const SahBuild& B, uint32_t begin, 
 
 // The root segment (its centroid bounds cb_ord are known); cnt is zeroed.
 __global__ void k_sah_start(SahBuild B, const int* __restrict__ cb_ord) {
+    chain_wait();
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) *B.boxes_done = 1u;
     if (B.n <= kSahMid) {
@@ -268,6 +269,7 @@ __global__ void k_sah_start(SahBuild B, const int* __restrict__ cb_ord) {
 // atomics), then merged into the task's bins once per non-empty bin; the
 // chunk's counts are kept for the partition.
 __global__ void __launch_bounds__(kSahBlock) k_sah_bin(SahBuild B, uint32_t level) {
+    chain_wait();
     __shared__ int sb[kTaskBins];
     __shared__ float s_cmin[3], s_scale[3];
     const uint32_t cur = level & 1u;
@@ -352,6 +354,7 @@ __global__ void __launch_bounds__(kSahBlock) k_sah_bin(SahBuild B, uint32_t leve
 // becomes of the children; and the left items before each block of the task.
 constexpr int kSplitBlock = 128;
 __global__ void __launch_bounds__(kSplitBlock) k_sah_split(SahBuild B, uint32_t level) {
+    chain_wait();
     __shared__ int sb[kTaskBins];
     __shared__ unsigned long long s_best;
     __shared__ SahSplit s_split;
@@ -456,6 +459,7 @@ __global__ void __launch_bounds__(kSplitBlock) k_sah_split(SahBuild B, uint32_t 
 // the children that are split at the next level.
 template <class K>
 __global__ void __launch_bounds__(kSahBlock) k_sah_scatter(SahBuild B, uint32_t level) {
+    chain_wait();
     __shared__ uint32_t s_warp[kSahBlock / 32];
     __shared__ int s_cb[2][6];
     const uint32_t cur = level & 1u, nxt = cur ^ 1u, t = threadIdx.x, lane = t & 31u, warp = t >> 5;
@@ -924,6 +928,7 @@ __device__ void sah_block(BlockSah<NMAX, SEGS>& S, const SahBuild& B, const SahP
 // A block per pending segment of kSahTiny + 1 .. kSahMid items.
 template <class K>
 __global__ void __launch_bounds__(kMidThreads) k_sah_block(SahBuild B) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char sm[];
     BlockMid& S = *reinterpret_cast<BlockMid*>(sm);
     const uint32_t m = B.cnt[kCntMid];
@@ -935,6 +940,7 @@ __global__ void __launch_bounds__(kMidThreads) k_sah_block(SahBuild B) {
 // usually none.
 template <class K>
 __global__ void __launch_bounds__(kTopThreads, 1) k_sah_rest(SahBuild B, uint32_t level) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char sm[];
     BlockTop& S = *reinterpret_cast<BlockTop*>(sm);
     const uint32_t m = B.cnt[4 * level];
@@ -959,6 +965,7 @@ constexpr int kTinyBlock = 96;
 constexpr uint32_t kSahWideMax = 65536;
 template <class K, int W>
 __global__ void __launch_bounds__(kTinyBlock) k_sah_tiny(SahBuild B) {
+    chain_wait();
     constexpr int A = 3 / W, GROUPS = kTinyBlock / (32 * W);  // axes of a warp, segments of a block
     struct Group {
         int box[2][32][6];               // ordered ints of each position's box (two buffers)
@@ -1185,15 +1192,15 @@ rg_status sah_build(SahBuild B, const int* cb_ord, cudaStream_t s) {
     const uint32_t n = B.n, sms = (uint32_t)device_sm_count();
     SAH_CK(cudaMemsetAsync(B.cnt, 0, kCntAll * 4, s));
     const uint32_t chunks = (n + kSahChunk - 1) / kSahChunk;
-    k_sah_start<<<std::min(chunks / 512u + 1u, 1024u), 512, 0, s>>>(B, cb_ord);
+    launch_chain(k_sah_start, std::min(chunks / 512u + 1u, 1024u), 512, 0, s, B, cb_ord);
     count_launches(1);
     const uint32_t max_tasks = n / (kSahMid + 1) + 1;
     auto run_level = [&](uint32_t level) {
         const uint32_t tasks = level < 31 ? std::min(1u << level, max_tasks) : max_tasks;
         const uint32_t blocks = n / kSahChunk + tasks;
-        k_sah_bin<<<blocks, kSahBlock, 0, s>>>(B, level);
-        k_sah_split<<<tasks, kSplitBlock, 0, s>>>(B, level);
-        k_sah_scatter<K><<<blocks, kSahBlock, 0, s>>>(B, level);
+        launch_chain(k_sah_bin, blocks, kSahBlock, 0, s, B, level);
+        launch_chain(k_sah_split, tasks, kSplitBlock, 0, s, B, level);
+        launch_chain(k_sah_scatter<K>, blocks, kSahBlock, 0, s, B, level);
         count_launches(3);
     };
     // levels for a balanced tree and one more; then the host looks whether
@@ -1228,18 +1235,18 @@ rg_status sah_build(SahBuild B, const int* cb_ord, cudaStream_t s) {
             SAH_CK(cudaStreamSynchronize(s));  // segs is this frame's
         }
     } else if (n > kSahMid) {
-        k_sah_rest<K><<<std::min(max_tasks, sms), kTopThreads, sizeof(BlockTop), s>>>(B, levels);
+        launch_chain(k_sah_rest<K>, std::min(max_tasks, sms), kTopThreads, sizeof(BlockTop), s, B, levels);
         count_launches(1);
     }
     if (n > kSahTiny) {
-        k_sah_block<K><<<std::min(n / (kSahTiny + 1) + 1, 4 * sms), kMidThreads, sizeof(BlockMid), s>>>(B);
+        launch_chain(k_sah_block<K>, std::min(n / (kSahTiny + 1) + 1, 4 * sms), kMidThreads, sizeof(BlockMid), s, B);
         count_launches(1);
     }
     // three warps per segment while the chip holds all segments at once that way
     if (n <= kSahWideMax)
-        k_sah_tiny<K, 3><<<std::min(n / 16u + 1u, 16 * sms), kTinyBlock, 0, s>>>(B);
+        launch_chain(k_sah_tiny<K, 3>, std::min(n / 16u + 1u, 16 * sms), kTinyBlock, 0, s, B);
     else
-        k_sah_tiny<K, 1><<<8 * sms, kTinyBlock, 0, s>>>(B);
+        launch_chain(k_sah_tiny<K, 1>, 8 * sms, kTinyBlock, 0, s, B);
     count_launches(1);
     SAH_CK(cudaGetLastError());
     return RG_OK;

@@ -17,6 +17,7 @@ namespace {
 // work (camera and secondary rays).
 template <int MODE, bool BRUTE, bool STATS, int BLOCK, int SD>
 __global__ void __launch_bounds__(BLOCK) k_trace_warp(TraceArgs a) {
+    chain_wait();
     constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender || MODE == kModeShadowBatch);
     __shared__ uint32_t pre[kMaxLights + 1];
     const uint32_t n = ray_count<MODE == kModeShadowRender>(a, pre);
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(BLOCK) k_trace_warp(TraceArgs a) {
 // at a time the same, and 768 threads slower than both.
 template <int SMODE, int CMODE, bool STATS, int BLOCK, int SD>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_trace_pair(TraceArgs sa, TraceArgs ca) {
+    chain_wait();
     __shared__ uint32_t pre[kMaxLights + 1];
     const uint32_t ns_rays = ray_count<SMODE == kModeShadowRender>(sa, pre);
     const uint32_t k = shadow_split<SMODE>(sa, ns_rays);
@@ -121,6 +123,7 @@ constexpr int kLeafBatch = 4, kLeafNodesMin = 8, kNodeRun = 4;
 template <int MODE, bool BRUTE, bool STATS, int BLOCK, int SD>
 __global__ void __launch_bounds__(BLOCK, (BRUTE || STATS) ? 1 : (MODE == kModeClosestBatch ? 896 : 1024) / BLOCK)
     k_trace_lane(TraceArgs a) {
+    chain_wait();
     const uint32_t iter_cap = a.iter_cap;
     constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender || MODE == kModeShadowBatch);
     constexpr bool kBatch = (MODE == kModeClosestBatch || MODE == kModeShadowBatch);
@@ -452,6 +455,7 @@ __device__ __forceinline__ void visit8(const float4* nd, const SpaceRay& cr, uin
 // Wide traversal, whole-warp refill (the renderer's rays).
 template <int MODE, bool STATS>
 __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
+    chain_wait();
     const uint32_t iter_cap = a.iter_cap;
     constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender);
     __shared__ uint32_t pre[kMaxLights + 1];
@@ -645,6 +649,7 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
 constexpr int kLeafBatch8 = 4, kLeafNodesMin8 = 8, kRefill8 = 8;
 template <int MODE, bool STATS>
 __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(TraceArgs a) {
+    chain_wait();
     const uint32_t iter_cap = a.iter_cap;
     constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender);
     constexpr bool kTies = MODE == kModeClosestAbi;
@@ -850,7 +855,7 @@ cudaError_t launch_mode8(const TraceArgs& a0, cudaStream_t s) {
         blocks = device_sm_count() * (per_sm > 0 ? per_sm : 1);
         cached.store(blocks, std::memory_order_relaxed);
     }
-    kernel<<<blocks, kTraceBlock, 0, s>>>(a);
+    launch_chain(kernel, blocks, kTraceBlock, 0, s, a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -881,9 +886,9 @@ cudaError_t launch_block(const TraceArgs& a, int blocks_per_sm, cudaStream_t s) 
     if (e != cudaSuccess) return e;
     const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
     if (LANE)
-        k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD><<<device_sm_count() * b, BLOCK, smem, s>>>(a);
+        launch_chain(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD>, device_sm_count() * b, BLOCK, smem, s, a);
     else
-        k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD><<<device_sm_count() * b, BLOCK, smem, s>>>(a);
+        launch_chain(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, device_sm_count() * b, BLOCK, smem, s, a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -896,7 +901,7 @@ cudaError_t launch_pair_t(const TraceArgs& sa, const TraceArgs& ca, int blocks_p
     cudaError_t e = resident_blocks(k_trace_pair<SMODE, CMODE, STATS, BLOCK, SD>, BLOCK, smem, cached, &per_sm);
     if (e != cudaSuccess) return e;
     const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
-    k_trace_pair<SMODE, CMODE, STATS, BLOCK, SD><<<device_sm_count() * b, BLOCK, smem, s>>>(sa, ca);
+    launch_chain(k_trace_pair<SMODE, CMODE, STATS, BLOCK, SD>, device_sm_count() * b, BLOCK, smem, s, sa, ca);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1006,6 +1011,7 @@ __global__ void __launch_bounds__(kRefineBlock, 4) k_refine_hits(const float4* _
                                                               const InstDev* __restrict__ inst,
                                                               const uint32_t* __restrict__ leaf_of_inst,
                                                               const BlasDev* __restrict__ blas) {
+    chain_wait();
     __shared__ uint32_t queue[kRefineBlock / 32][64];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint32_t* q = queue[warp];
@@ -1035,7 +1041,7 @@ cudaError_t launch_refine_hits(const float4* rays, rg_hit* hits, uint32_t n, con
                                const uint32_t* leaf_of_inst, const BlasDev* blas, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     const uint32_t blocks = min((n + kRefineBlock - 1u) / kRefineBlock, (uint32_t)device_sm_count() * 8u);
-    k_refine_hits<<<blocks, kRefineBlock, 0, s>>>(rays, hits, n, inst, leaf_of_inst, blas);
+    launch_chain(k_refine_hits, blocks, kRefineBlock, 0, s, rays, hits, n, inst, leaf_of_inst, blas);
     count_launches(1);
     return cudaGetLastError();
 }
