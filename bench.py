@@ -577,7 +577,7 @@ def run_medium(args, world, rank, local, embedded=False):
                        "blas_build_ms": round(blas_build_ms, 2), "blas_build": blas_build,
                        "l2": "flushed before each frame (256 MiB write on the frame's stream, inside the timed region)",
                        "fxaa": {"ms": round(fxaa_ms, 4), "gbs": round(W * H * 32 / (fxaa_ms / 1e3) / 1e9, 1),
-                                "bytes_per_pixel": 32, "note": "k_fxaa_luma + k_fxaa on the frame, timed alone, not in the step"},
+                                "bytes_per_pixel": 32, "note": "k_fxaa on the frame, timed alone, not in the step"},
                        "parallelism": f"replicas x{world}", "bvh": bvh_label(args)},
             "roofline": roofline,
             "gpu_launches": int(stats_f[0]["kernel_launches"]),

@@ -243,8 +243,7 @@ rg_status rg_render(rg_scene* scene, const rg_camera* h_cam, uint32_t w, uint32_
  * to 26.5 pixels each way) give an offset across the edge, at least the
  * sub-pixel offset 0.75 s^2 of the 3x3 contrast, and the colour is
  * resampled bilinearly there (clamp-to-edge); alpha is copied.  Needs no
- * scene; w or h = 0 does nothing.  Takes w*h*4 bytes of stream-ordered
- * temporary device memory (the luma image) for the duration of the call. */
+ * scene; w or h = 0 does nothing. */
 rg_status rg_fxaa(const float* d_in, uint32_t w, uint32_t h, float* d_out, void* stream);
 
 /* rg_sync waits for all of the device's work and returns the first error a
@@ -319,7 +318,7 @@ rg_status rg_wide_export(rg_scene* scene, uint32_t blas_id, void* h_nodes, uint3
  * Same result as rg_radix_sort_pairs (same arguments and order), but the call
  * makes no device allocation: its temporaries live in one fixed array inside
  * librg.so, sized for RG_NOALLOC_SORT_MAX_PAIRS pairs of 64-bit keys (about
- * 3.2 MB, held on every GPU that loads the library until the process exits).
+ * 3.4 MB, held on every GPU that loads the library until the process exits).
  * It is meant for callers that cannot allocate device memory: code whose
  * device memory is owned by a caching allocator that has already reserved
  * what the GPU has free, and frame loops that must not stall on an

@@ -245,8 +245,7 @@ struct rg_scene {
     InstDev *inst = nullptr, *inst_tmp = nullptr;
     float* wbox = nullptr;
     uint32_t *perm = nullptr, *parents = nullptr, *flags = nullptr;
-    uint32_t* leaf_of_inst = nullptr;  // TLAS leaf of each instance index (made on first need after a build)
-    bool leaf_of_inst_valid = false;
+    uint32_t* leaf_of_inst = nullptr;  // TLAS leaf of each instance index
     // compressed 8-wide TLAS
     bool wide = false;
     DevBuf<float4> tlas8;
@@ -583,7 +582,8 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
              void *lohi = tm + t_lohi, *cb = tm + t_cb, *perm = tm + t_perm, *parents = tm + t_parents, *fl = tm + t_fl;
              void *ranges = wide ? tm + t_ranges : nullptr, *tasks = wide ? tm + t_tasks : nullptr, *boxes_done = nullptr;
              RG_CK(launch_blas_begin(static_cast<int*>(cb), s->B->d_blas.p + id, hd, st));
-             RG_CK(launch_tri_bounds(d_vtx, nv, d_idx, nt, static_cast<float*>(lohi), static_cast<int*>(cb), s->st, st));
+             RG_CK(launch_tri_bounds(d_vtx, nv, d_idx, nt, static_cast<float*>(lohi), static_cast<int*>(cb), s->st, st,
+                                     static_cast<uint32_t*>(fl)));
              if (nt > 1) {
                  if (flags & RG_BLAS_SAH) {
                      boxes_done = static_cast<char*>(cb) + 32;  // (the bounds take 24 of the 64 bytes)
@@ -597,15 +597,14 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
                                        static_cast<uint32_t*>(perm), static_cast<uint32_t*>(parents), st,
                                        static_cast<uint32_t*>(ranges));
                  if (q) return q;
-                 RG_CK(cudaMemsetAsync(fl, 0, (size_t)(nt - 1) * 4, st));
              } else {
                  RG_CK(cudaMemsetAsync(perm, 0, 4, st));
              }
              RG_CK(launch_blas_leaves_refit(d_vtx, d_idx, static_cast<uint32_t*>(perm), static_cast<float*>(lohi), nt,
                                             static_cast<uint32_t*>(parents), b.nodes, static_cast<uint32_t*>(fl), b.tris,
+                                            b.leaf_of_prim,
                                             s->B->d_blas.p + id, s->st, st, static_cast<uint32_t*>(boxes_done)));
              RG_CK(launch_bound_sphere(d_vtx, nv, s->B->d_blas.p + id, st));
-             RG_CK(launch_invert_perm(static_cast<uint32_t*>(perm), nt, b.leaf_of_prim, st));
              if (wide) {
                  WideOut out{b.nodes8, b.src8, b.item_src8, b.counts8, static_cast<uint2*>(tasks)};
                  const float* leaf_box = reinterpret_cast<const float*>(reinterpret_cast<const char*>(s->B->d_blas.p + id) +
@@ -637,7 +636,7 @@ static rg_status tlas_common(rg_scene* s, const rg_instance* d_inst, uint32_t n,
         if (!refit && s->wide && n > 1 && (r = tmp.get(&ranges, (size_t)(n - 1) * 8, "ranges"))) return r;
         RG_CK(launch_tlas_small(d_inst, n, s->B->d_blas.p, (uint32_t)s->B->blas.size(), s->inst_tmp, s->wbox, refit,
                                 s->tlas_nodes, s->perm, s->parents, s->flags, static_cast<uint32_t*>(ranges),
-                                s->inst, s->st, st));
+                                s->inst, s->leaf_of_inst, s->st, st));
         if (s->wide) {
             WideOut out{s->tlas8.p, s->src8.p, s->item_src8.p, s->counts8.p, s->tasks8.p};
             if (refit)
@@ -653,7 +652,7 @@ static rg_status tlas_common(rg_scene* s, const rg_instance* d_inst, uint32_t n,
     if ((r = tmp.get(&cb, 64, "centroid bounds"))) return r;
     if (!refit) RG_CK(launch_init_bounds(static_cast<int*>(cb), st));
     RG_CK(launch_instance_prep(d_inst, n, s->B->d_blas.p, (uint32_t)s->B->blas.size(), s->inst_tmp, s->wbox,
-                               refit ? nullptr : static_cast<int*>(cb), refit, s->st, st));
+                               refit ? nullptr : static_cast<int*>(cb), refit, s->flags, s->st, st));
     void* ranges = nullptr;
     void* boxes_done = nullptr;  // set by the SAH build when it wrote every node's boxes
     if (!refit) {
@@ -672,9 +671,8 @@ static rg_status tlas_common(rg_scene* s, const rg_instance* d_inst, uint32_t n,
             RG_CK(cudaMemsetAsync(s->perm, 0, 4, st));
         }
     }
-    if (n > 1) RG_CK(cudaMemsetAsync(s->flags, 0, (size_t)(n - 1) * 4, st));
     RG_CK(launch_tlas_leaves_refit(s->inst_tmp, s->wbox, s->perm, n, s->parents, s->tlas_nodes, s->flags,
-                                   s->inst, s->st, st, static_cast<const uint32_t*>(boxes_done)));
+                                   s->inst, s->leaf_of_inst, s->st, st, static_cast<const uint32_t*>(boxes_done)));
     if (s->wide) {
         WideOut out{s->tlas8.p, s->src8.p, s->item_src8.p, s->counts8.p, s->tasks8.p};
         if (refit)
@@ -696,7 +694,6 @@ rg_status rg_tlas_build(rg_scene* s, const rg_instance* d_inst, uint32_t n, void
     if ((r = set_device(s))) return r;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     s->tlas_built = false;
-    s->leaf_of_inst_valid = false;
     if (n > s->tlas_cap) {
         const size_t m = n < 16 ? 16 : n;
         Parts P;
@@ -787,11 +784,11 @@ rg_status rg_trace_rays(rg_scene* s, const rg_ray* d_rays, uint32_t n, uint32_t 
     a.rays = reinterpret_cast<const float4*>(d_rays);
     a.n = n;
     a.hits_abi = d_hits;
-    // a work counter of its own, so calls on other streams may run at the same time
+    // a work counter of its own, so calls on other streams may run at the same
+    // time (cleared by the launch where it is used)
     uint32_t* ctr = s->trace_ctr + 32 * (size_t)(s->trace_slot++ % kTraceSlots);
     a.work_counter = ctr;
     a.iter_cap = iter_cap_for(s, flags & RG_TRACE_BRUTE);
-    RG_CK(cudaMemsetAsync(ctr, 0, 4, st));
     const bool any = flags & RG_ANY;
     EventPair* ev;
     if ((r = event_begin(s, any ? 1 : 0, st, &ev))) return r;
@@ -801,10 +798,6 @@ rg_status rg_trace_rays(rg_scene* s, const rg_ray* d_rays, uint32_t n, uint32_t 
     // traversal wrote provisional records that refer to the instance array it
     // walked)
     if (!any) {
-        if (!s->leaf_of_inst_valid) {
-            RG_CK(launch_invert_perm(s->perm, s->n_inst, s->leaf_of_inst, st));
-            s->leaf_of_inst_valid = true;
-        }
         if ((r = event_begin(s, 3, st, &ev))) return r;
         RG_CK(launch_refine_hits(a.rays, d_hits, n, s->inst, s->leaf_of_inst, s->B->d_blas.p, st));
         if ((r = event_end(s, st))) return r;
@@ -872,11 +865,13 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         if ((r = s->seg_count.ensure(kShadowSplitMax, "shadow segment counts"))) return r;
         RG_CK(cudaMemsetAsync(s->seg_count.p, 0, (size_t)kShadowSplitMax * sizeof(uint32_t), st));
     }
-    RG_CK(cudaMemsetAsync(s->counters.p, 0, CB * ((size_t)max_depth + 1) * sizeof(uint32_t), st));
-    RG_CK(cudaMemsetAsync(d_rgba, 0, (size_t)N * 16, st));
+    const bool aligned = reinterpret_cast<uintptr_t>(d_rgba) % 16 == 0;
+    if (!aligned) RG_CK(cudaMemsetAsync(d_rgba, 0, (size_t)N * 16, st));
     CameraDev cd;
     std::memcpy(&cd, cam, sizeof cd);
-    RG_CK(launch_raygen(cd, w, h, s->q_rays[0].p, s->q_pay[0].p, st));
+    RG_CK(launch_raygen(cd, w, h, s->q_rays[0].p, s->q_pay[0].p,
+                        aligned ? reinterpret_cast<float4*>(d_rgba) : nullptr, s->counters.p,
+                        (uint32_t)(CB * ((size_t)max_depth + 1)), st));
 
     // shading of depth level `depth` (its rays in queue q, spawns into 1 - q)
     auto shade_args = [&](uint32_t depth, int q, uint32_t* c, bool last, uint32_t n_stride) {

@@ -80,11 +80,13 @@ __global__ void k_blas_begin(int* cb_ord, BlasDev* out, BlasDev desc) {
 }
 
 __global__ void k_tri_bounds(const float* __restrict__ vtx, uint32_t nv, const uint32_t* __restrict__ idx,
-                             uint32_t nt, float* __restrict__ lohi, int* cb_ord, DevStatus* st) {
+                             uint32_t nt, float* __restrict__ lohi, int* cb_ord, DevStatus* st,
+                             uint32_t* __restrict__ flags) {
     chain_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     bool valid = i < nt;
     int c[3] = {0, 0, 0};
+    if (flags && i + 1 < nt) flags[i] = 0u;
     if (valid) {
         uint32_t a = idx[3 * (size_t)i], b = idx[3 * (size_t)i + 1], cc = idx[3 * (size_t)i + 2];
         if (a >= nv || b >= nv || cc >= nv) {
@@ -545,12 +547,13 @@ __device__ void climb(uint32_t j, uint32_t n, float* box, const uint32_t* __rest
 __global__ void k_blas_leaves_refit(const float* __restrict__ vtx, const uint32_t* __restrict__ idx,
                                     const uint32_t* __restrict__ perm, const float* __restrict__ lohi, uint32_t n,
                                     const uint32_t* __restrict__ parents, float4* nodes, uint32_t* flags,
-                                    float4* __restrict__ tris, BlasDev* blas_out, DevStatus* st,
-                                    const uint32_t* __restrict__ boxes_done) {
+                                    float4* __restrict__ tris, uint32_t* __restrict__ leaf_of_prim, BlasDev* blas_out,
+                                    DevStatus* st, const uint32_t* __restrict__ boxes_done) {
     chain_wait();
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     uint32_t prim = perm[j];
+    leaf_of_prim[prim] = j;
     uint32_t vi[3] = {idx[3 * (size_t)prim], idx[3 * (size_t)prim + 1], idx[3 * (size_t)prim + 2]};
     // the triangle record: its vertices in the axis orders (x, y, z), (y, z, x)
     // and (z, x, y), prim in the first vertex's w of each
@@ -695,24 +698,27 @@ __device__ __forceinline__ void instance_prep_one(const rg_instance* __restrict_
 
 __global__ void k_instance_prep(const rg_instance* __restrict__ in, uint32_t n, const BlasDev* __restrict__ blas,
                                 uint32_t nblas, InstDev* tmp, float* __restrict__ wbox, int* cb_ord, bool check_blas,
-                                DevStatus* st) {
+                                uint32_t* __restrict__ flags, DevStatus* st) {
     chain_wait();
     uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     bool valid = k < n;
     int c[3] = {0, 0, 0};
+    if (k + 1 < n) flags[k] = 0u;
     if (valid) instance_prep_one(in, k, blas, nblas, tmp, wbox, check_blas, st, c);
     if (cb_ord) reduce_bounds(cb_ord, c[0], c[1], c[2], valid);
 }
 
 __global__ void k_tlas_leaves_refit(const InstDev* __restrict__ tmp, const float* __restrict__ wbox,
                                     const uint32_t* __restrict__ perm, uint32_t n, const uint32_t* __restrict__ parents,
-                                    float4* nodes, uint32_t* flags, InstDev* __restrict__ inst_out, DevStatus* st,
+                                    float4* nodes, uint32_t* flags, InstDev* __restrict__ inst_out,
+                                    uint32_t* __restrict__ leaf_of_inst, DevStatus* st,
                                     const uint32_t* __restrict__ boxes_done) {
     chain_wait();
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     uint32_t k = perm[j];
     inst_out[j] = tmp[k];
+    if (leaf_of_inst) leaf_of_inst[k] = j;
     if (boxes_done && *boxes_done) return;
     float box[6];
 #pragma unroll
@@ -732,7 +738,8 @@ __global__ void __launch_bounds__(kTlasSmallMax) k_tlas_small(const rg_instance*
                                                               const BlasDev* __restrict__ blas, uint32_t nblas,
                                                               InstDev* tmp, float* wbox, bool refit, float4* nodes,
                                                               uint32_t* perm, uint32_t* parents, uint32_t* flags,
-                                                              uint32_t* ranges, InstDev* inst_out, DevStatus* st) {
+                                                              uint32_t* ranges, InstDev* inst_out,
+                                                              uint32_t* leaf_of_inst, DevStatus* st) {
     chain_wait();
     __shared__ int s_cb[6];
     __shared__ uint32_t s_key[kTlasSmallMax], s_val[kTlasSmallMax];
@@ -807,6 +814,7 @@ __global__ void __launch_bounds__(kTlasSmallMax) k_tlas_small(const rg_instance*
     if (valid) {
         const uint32_t k = perm[t];
         inst_out[t] = tmp[k];
+        leaf_of_inst[k] = t;
         float box[6];
 #pragma unroll
         for (int a = 0; a < 6; ++a) box[a] = wbox[6 * (size_t)k + a];
@@ -832,9 +840,9 @@ cudaError_t launch_blas_begin(int* cb_ord, BlasDev* out, const BlasDev& desc, cu
 }
 
 cudaError_t launch_tri_bounds(const float* vtx, uint32_t nv, const uint32_t* idx, uint32_t nt, float* lohi,
-                              int* cb_ord, DevStatus* st, cudaStream_t s) {
+                              int* cb_ord, DevStatus* st, cudaStream_t s, uint32_t* flags) {
     if (nt == 0) return cudaSuccess;
-    launch_chain(k_tri_bounds, grid_for(nt), kBlock, 0, s, vtx, nv, idx, nt, lohi, cb_ord, st);
+    launch_chain(k_tri_bounds, grid_for(nt), kBlock, 0, s, vtx, nv, idx, nt, lohi, cb_ord, st, flags);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -926,13 +934,6 @@ cudaError_t launch_karras(const void* keys, uint32_t n, int key_bits, uint32_t* 
     return cudaGetLastError();
 }
 
-namespace {
-__global__ void k_invert_perm(const uint32_t* __restrict__ perm, uint32_t n, uint32_t* __restrict__ inv) {
-    chain_wait();
-    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) inv[perm[j]] = j;
-}
-}  // namespace
-
 cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasSeg* segs, uint32_t n_segs,
                                    uint32_t n_threads, uint32_t n_leaves, float4* nodes, uint32_t* parents,
                                    uint32_t* ranges, cudaStream_t s) {
@@ -948,18 +949,11 @@ cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasS
     return cudaGetLastError();
 }
 
-cudaError_t launch_invert_perm(const uint32_t* perm, uint32_t n, uint32_t* inv, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    launch_chain(k_invert_perm, min(grid_for(n), 4096u), kBlock, 0, s, perm, n, inv);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, const uint32_t* perm, const float* lohi,
                                      uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
-                                     float4* tris, BlasDev* blas_out, DevStatus* st, cudaStream_t s,
-                                     const uint32_t* boxes_done) {
-    launch_chain(k_blas_leaves_refit, grid_for(n), kBlock, 0, s, vtx, idx, perm, lohi, n, parents, nodes, flags, tris, blas_out,
+                                     float4* tris, uint32_t* leaf_of_prim, BlasDev* blas_out, DevStatus* st,
+                                     cudaStream_t s, const uint32_t* boxes_done) {
+    launch_chain(k_blas_leaves_refit, grid_for(n), kBlock, 0, s, vtx, idx, perm, lohi, n, parents, nodes, flags, tris, leaf_of_prim, blas_out,
                                                        st, boxes_done);
     count_launches(1);
     return cudaGetLastError();
@@ -974,17 +968,18 @@ cudaError_t launch_bound_sphere(const float* vtx, uint32_t nv, BlasDev* blas, cu
 }
 
 cudaError_t launch_instance_prep(const rg_instance* in, uint32_t n, const BlasDev* blas, uint32_t nblas,
-                                 InstDev* tmp, float* wbox, int* cb_ord, bool check_blas, DevStatus* st,
-                                 cudaStream_t s) {
-    launch_chain(k_instance_prep, grid_for(n), kBlock, 0, s, in, n, blas, nblas, tmp, wbox, cb_ord, check_blas, st);
+                                 InstDev* tmp, float* wbox, int* cb_ord, bool check_blas, uint32_t* flags,
+                                 DevStatus* st, cudaStream_t s) {
+    launch_chain(k_instance_prep, grid_for(n), kBlock, 0, s, in, n, blas, nblas, tmp, wbox, cb_ord, check_blas, flags, st);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tlas_leaves_refit(const InstDev* tmp, const float* wbox, const uint32_t* perm, uint32_t n,
                                      const uint32_t* parents, float4* nodes, uint32_t* flags, InstDev* inst_out,
-                                     DevStatus* st, cudaStream_t s, const uint32_t* boxes_done) {
-    launch_chain(k_tlas_leaves_refit, grid_for(n), kBlock, 0, s, tmp, wbox, perm, n, parents, nodes, flags, inst_out, st,
+                                     uint32_t* leaf_of_inst, DevStatus* st, cudaStream_t s,
+                                     const uint32_t* boxes_done) {
+    launch_chain(k_tlas_leaves_refit, grid_for(n), kBlock, 0, s, tmp, wbox, perm, n, parents, nodes, flags, inst_out, leaf_of_inst, st,
                                                        boxes_done);
     count_launches(1);
     return cudaGetLastError();
@@ -992,11 +987,12 @@ cudaError_t launch_tlas_leaves_refit(const InstDev* tmp, const float* wbox, cons
 
 cudaError_t launch_tlas_small(const rg_instance* in, uint32_t n, const BlasDev* blas, uint32_t nblas, InstDev* tmp,
                               float* wbox, bool refit, float4* nodes, uint32_t* perm, uint32_t* parents,
-                              uint32_t* flags, uint32_t* ranges, InstDev* inst_out, DevStatus* st, cudaStream_t s) {
+                              uint32_t* flags, uint32_t* ranges, InstDev* inst_out, uint32_t* leaf_of_inst,
+                              DevStatus* st, cudaStream_t s) {
     if (n == 0 || n > kTlasSmallMax) return cudaErrorInvalidValue;
     const uint32_t threads = (n + 31u) & ~31u;
     launch_chain(k_tlas_small, 1, threads, 0, s, in, n, blas, nblas, tmp, wbox, refit, nodes, perm, parents, flags, ranges,
-                                       inst_out, st);
+inst_out, leaf_of_inst, st);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -75,11 +75,16 @@ __device__ __forceinline__ void tile_pixel(uint32_t i, uint32_t w, uint32_t h, u
     x = 8u * blk + rem % bw;
 }
 
+// The primary rays; clears the image (null: already clear) and the frame's
+// counters on the way, which were two launches of their own.
 __global__ void k_raygen(CameraDev cam, uint32_t w, uint32_t h, float4* __restrict__ rays,
-                         Payload* __restrict__ payload) {
+                         Payload* __restrict__ payload, float4* __restrict__ image, uint32_t* __restrict__ counters,
+                         uint32_t n_counters) {
     chain_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    for (uint32_t k = i; k < n_counters; k += gridDim.x * blockDim.x) counters[k] = 0u;
     if (i >= w * h) return;
+    if (image) image[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     uint32_t x, y;
     tile_pixel(i, w, h, x, y);
     float4 o, d;
@@ -666,10 +671,10 @@ __global__ void __launch_bounds__(kFxaaThreads, 4) k_fxaa(const float4* __restri
 
 }  // namespace
 
-cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, float4* rays, Payload* payload,
-                          cudaStream_t s) {
+cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, float4* rays, Payload* payload, float4* image,
+                          uint32_t* counters, uint32_t n_counters, cudaStream_t s) {
     size_t n = (size_t)w * h;
-    launch_chain(k_raygen, (unsigned)((n + 255) / 256), 256, 0, s, cam, w, h, rays, payload);
+    launch_chain(k_raygen, (unsigned)((n + 255) / 256), 256, 0, s, cam, w, h, rays, payload, image, counters, n_counters);
     count_launches(1);
     return cudaGetLastError();
 }

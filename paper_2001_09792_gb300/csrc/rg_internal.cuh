@@ -195,7 +195,7 @@ __device__ __forceinline__ float ord2f(int i) { return __int_as_float(i >= 0 ? i
 // ---------------------------------------------------------------- launchers
 // build.cu
 cudaError_t launch_tri_bounds(const float* vtx, uint32_t nv, const uint32_t* idx, uint32_t nt, float* lohi,
-                              int* cb_ord, DevStatus* st, cudaStream_t s);
+                              int* cb_ord, DevStatus* st, cudaStream_t s, uint32_t* flags = nullptr);
 cudaError_t launch_init_bounds(int* cb_ord, cudaStream_t s);
 cudaError_t launch_blas_begin(int* cb_ord, BlasDev* out, const BlasDev& desc, cudaStream_t s);
 cudaError_t launch_centroid_bounds(const float* lohi, uint32_t n, int* cb_ord, cudaStream_t s);
@@ -217,29 +217,29 @@ cudaError_t launch_karras(const void* keys, uint32_t n, int key_bits, uint32_t* 
                           uint32_t* parents, cudaStream_t s, uint32_t* ranges = nullptr);
 cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, const uint32_t* perm, const float* lohi,
                                      uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
-                                     float4* tris, BlasDev* blas_out, DevStatus* st, cudaStream_t s,
-                                     const uint32_t* boxes_done = nullptr);
+                                     float4* tris, uint32_t* leaf_of_prim, BlasDev* blas_out, DevStatus* st,
+                                     cudaStream_t s, const uint32_t* boxes_done = nullptr);
 // Bounding sphere of a mesh about its root box centre (after the BLAS refit
 // wrote the root box): blas->r2_bits = max over the vertices.
 cudaError_t launch_bound_sphere(const float* vtx, uint32_t nv, BlasDev* blas, cudaStream_t s);
-// inv[perm[j]] = j for j < n (perm a permutation of 0..n-1).
-cudaError_t launch_invert_perm(const uint32_t* perm, uint32_t n, uint32_t* inv, cudaStream_t s);
 cudaError_t launch_instance_prep(const rg_instance* in, uint32_t n, const BlasDev* blas, uint32_t nblas,
-                                 InstDev* tmp, float* wbox, int* cb_ord, bool check_blas, DevStatus* st,
-                                 cudaStream_t s);
+                                 InstDev* tmp, float* wbox, int* cb_ord, bool check_blas, uint32_t* flags,
+                                 DevStatus* st, cudaStream_t s);
 // The whole TLAS build (refit = false) or refit of n <= kTlasSmallMax
 // instances in one single-block launch; same results as instance prep +
 // bounds + Morton + sort + Karras + leaves refit.  ranges may be NULL.
 constexpr uint32_t kTlasSmallMax = 1024;
 cudaError_t launch_tlas_small(const rg_instance* in, uint32_t n, const BlasDev* blas, uint32_t nblas, InstDev* tmp,
                               float* wbox, bool refit, float4* nodes, uint32_t* perm, uint32_t* parents,
-                              uint32_t* flags, uint32_t* ranges, InstDev* inst_out, DevStatus* st, cudaStream_t s);
+                              uint32_t* flags, uint32_t* ranges, InstDev* inst_out, uint32_t* leaf_of_inst,
+                              DevStatus* st, cudaStream_t s);
 // The instances in leaf order and the bottom-up refit of the node boxes; with
 // boxes_done set (device memory, may be null) the boxes are already in place
 // and only the instances are copied.
 cudaError_t launch_tlas_leaves_refit(const InstDev* tmp, const float* wbox, const uint32_t* perm, uint32_t n,
                                      const uint32_t* parents, float4* nodes, uint32_t* flags, InstDev* inst_out,
-                                     DevStatus* st, cudaStream_t s, const uint32_t* boxes_done = nullptr);
+                                     uint32_t* leaf_of_inst, DevStatus* st, cudaStream_t s,
+                                     const uint32_t* boxes_done = nullptr);
 
 // Karras hierarchies over segments of the sorted keys (the bottom of the SAH
 // build): segment k spans leaves begin .. begin + count - 1 and its internal
@@ -321,7 +321,7 @@ struct TraceArgs {
     HitDev* hits_render;         // kModeClosestRender
     const Payload* payload;      // kModeShadowRender
     float* image;                // kModeShadowRender: RGBA32F accumulation
-    uint32_t* work_counter;      // persistent-thread work queue head (zeroed before launch)
+    uint32_t* work_counter;      // persistent-thread work queue head (zeroed before launch; null for small queries)
     DevStatus* st;
     uint32_t iter_cap;           // bound on the loop steps of one ray (a valid traversal needs fewer)
     const float4* tlas_nodes8;   // compressed 8-wide TLAS (null: binary path)
@@ -401,7 +401,9 @@ struct ShadeArgs {
     const uint32_t* next_base;
     uint32_t ring_mask;
 };
-cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, float4* rays, Payload* payload,
+// image (may be null) and counters are cleared.
+cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, float4* rays, Payload* payload, float4* image,
+                          uint32_t* counters, uint32_t n_counters,
                           cudaStream_t s);
 cudaError_t launch_shade(const ShadeArgs& a, uint32_t n_max, cudaStream_t s);
 // Batched wavefront: primary rays of newly admitted requests, written to ring

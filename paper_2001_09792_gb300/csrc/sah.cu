@@ -245,10 +245,12 @@ __device__ __forceinline__ void push_pending(const SahBuild& B, uint32_t begin, 
         B.mid[atomicAdd(B.cnt + kCntMid, 1u)] = T;
 }
 
-// The root segment (its centroid bounds cb_ord are known); cnt is zeroed.
+// The counters, and the root segment (its centroid bounds cb_ord are known).
 __global__ void k_sah_start(SahBuild B, const int* __restrict__ cb_ord) {
     chain_wait();
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    for (uint32_t k = i; blockIdx.x == 0 && k < kCntAll; k += blockDim.x) B.cnt[k] = 0u;
+    __syncthreads();
     if (i == 0) *B.boxes_done = 1u;
     if (B.n <= kSahMid) {
         if (i == 0) push_pending(B, 0, B.n, 0, 0, 0);
@@ -1190,7 +1192,6 @@ rg_status sah_build(SahBuild B, const int* cb_ord, cudaStream_t s) {
         attr_set.store(1, std::memory_order_release);
     }
     const uint32_t n = B.n, sms = (uint32_t)device_sm_count();
-    SAH_CK(cudaMemsetAsync(B.cnt, 0, kCntAll * 4, s));
     const uint32_t chunks = (n + kSahChunk - 1) / kSahChunk;
     launch_chain(k_sah_start, std::min(chunks / 512u + 1u, 1024u), 512, 0, s, B, cb_ord);
     count_launches(1);

@@ -326,12 +326,11 @@ rg_status enqueue_refit(rg_server* s, Lane& L, uint32_t k, uint32_t e) {
     SlotBufs& b = L.slots[k];
     const uint32_t n = v.n_inst;
     SV_CK(cudaMemcpyAsync(b.d_inst, b.h_inst, (size_t)n * sizeof(rg_instance), cudaMemcpyHostToDevice, L.stream));
-    SV_CK(launch_instance_prep(b.d_inst, n, v.d_blas, v.n_blas, b.inst_tmp, b.wbox, nullptr, false, L.st, L.stream));
-    if (n > 1) {
+    SV_CK(launch_instance_prep(b.d_inst, n, v.d_blas, v.n_blas, b.inst_tmp, b.wbox, nullptr, false, b.flags, L.st,
+                               L.stream));
+    if (n > 1)
         SV_CK(cudaMemcpyAsync(b.tlas_nodes, v.tlas_nodes, (size_t)(n - 1) * 64, cudaMemcpyDeviceToDevice, L.stream));
-        SV_CK(cudaMemsetAsync(b.flags, 0, (size_t)(n - 1) * 4, L.stream));
-    }
-    SV_CK(launch_tlas_leaves_refit(b.inst_tmp, b.wbox, v.perm, n, v.parents, b.tlas_nodes, b.flags, b.inst, L.st,
+    SV_CK(launch_tlas_leaves_refit(b.inst_tmp, b.wbox, v.perm, n, v.parents, b.tlas_nodes, b.flags, b.inst, nullptr, L.st,
                                    L.stream));
     return RG_OK;
 }

@@ -11,6 +11,22 @@ namespace rg {
 
 namespace {
 
+// The next k rays for this warp's idle lanes.  A query of no more rays than
+// the launch has threads has no work counter (and no launch that clears one):
+// each warp takes its own 32, once.
+template <int MODE>
+__device__ __forceinline__ uint32_t claim_rays(const TraceArgs& a, uint32_t k, bool& exhausted) {
+    uint32_t base = 0;
+    if ((MODE == kModeClosestAbi || MODE == kModeAnyAbi) && !a.work_counter) {
+        base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u;
+        exhausted = true;
+    } else {
+        if ((threadIdx.x & 31u) == 0u) base = atomicAdd(a.work_counter, k);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    }
+    return base;
+}
+
 // Binary traversal, whole-warp refill: a warp takes 32 rays from the work
 // counter, each lane runs its ray to completion, and the warp takes the next
 // 32 when all its lanes are done.  Best when the rays of a warp take similar
@@ -162,9 +178,7 @@ __global__ void __launch_bounds__(BLOCK, (BRUTE || STATS) ? 1 : (MODE == kModeCl
         const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
         if (!exhausted && idle != 0u && (__popc(idle) >= (int)refill || idle == 0xFFFFFFFFu)) {
             const uint32_t k = (uint32_t)__popc(idle);
-            uint32_t base = 0;
-            if (lane == 0) base = atomicAdd(a.work_counter, k);
-            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            const uint32_t base = claim_rays<MODE>(a, k, exhausted);
             if (base + k >= n) exhausted = true;
             if (!active) {
                 const uint32_t idx = base + (uint32_t)__popc(idle & ((1u << lane) - 1u));
@@ -680,9 +694,7 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
         const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
         if (!exhausted && idle != 0u && (__popc(idle) >= (int)refill || idle == 0xFFFFFFFFu)) {
             const uint32_t k = (uint32_t)__popc(idle);
-            uint32_t base = 0;
-            if (lane == 0) base = atomicAdd(a.work_counter, k);
-            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            const uint32_t base = claim_rays<MODE>(a, k, exhausted);
             if (base + k >= n) exhausted = true;
             const uint32_t idx = base + (uint32_t)__popc(idle & ((1u << lane) - 1u));
             if (!active && idx < n) {
@@ -831,6 +843,17 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
     flush_counts<kAny, STATS>(a, c_nodes, c_tris, c_inst);
 }
 
+// Grid of a query on the per-lane kernels: as many blocks as its rays fill, up to
+// the resident ones; beyond those the warps share the work counter, cleared
+// here.
+cudaError_t query_grid(TraceArgs& a, int block, int& blocks, cudaStream_t s) {
+    const uint64_t need = ((uint64_t)a.n + block - 1) / block;
+    if (need > (uint64_t)blocks) return cudaMemsetAsync(a.work_counter, 0, 4, s);
+    a.work_counter = nullptr;
+    blocks = (int)need;
+    return cudaSuccess;
+}
+
 // The queries of rg_trace_rays, whose rays are often incoherent, take the
 // per-lane kernel (2^21 closest and as many any hits of the medium scene: 1,960
 // us, whole-warp 3,549), the renderer's rays the whole-warp one (the medium
@@ -855,6 +878,10 @@ cudaError_t launch_mode8(const TraceArgs& a0, cudaStream_t s) {
         blocks = device_sm_count() * (per_sm > 0 ? per_sm : 1);
         cached.store(blocks, std::memory_order_relaxed);
     }
+    if (kLane) {
+        const cudaError_t e = query_grid(a, kTraceBlock, blocks, s);
+        if (e != cudaSuccess) return e;
+    }
     launch_chain(kernel, blocks, kTraceBlock, 0, s, a);
     count_launches(1);
     return cudaGetLastError();
@@ -877,7 +904,8 @@ cudaError_t resident_blocks(K kernel, int block, size_t smem, std::atomic<int>& 
 }
 
 template <int MODE, bool BRUTE, bool STATS, int BLOCK, bool LANE, int SD>
-cudaError_t launch_block(const TraceArgs& a, int blocks_per_sm, cudaStream_t s) {
+cudaError_t launch_block(const TraceArgs& a0, int blocks_per_sm, cudaStream_t s) {
+    TraceArgs a = a0;
     static std::atomic<int> cached{0};
     constexpr size_t smem = (size_t)SD * BLOCK * sizeof(uint32_t);
     int per_sm = 0;
@@ -885,10 +913,13 @@ cudaError_t launch_block(const TraceArgs& a, int blocks_per_sm, cudaStream_t s) 
                          : resident_blocks(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, BLOCK, smem, cached, &per_sm);
     if (e != cudaSuccess) return e;
     const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
+    int blocks = device_sm_count() * b;
+    if (LANE && (MODE == kModeClosestAbi || MODE == kModeAnyAbi) && (e = query_grid(a, BLOCK, blocks, s)) != cudaSuccess)
+        return e;
     if (LANE)
-        launch_chain(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD>, device_sm_count() * b, BLOCK, smem, s, a);
+        launch_chain(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD>, blocks, BLOCK, smem, s, a);
     else
-        launch_chain(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, device_sm_count() * b, BLOCK, smem, s, a);
+        launch_chain(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, blocks, BLOCK, smem, s, a);
     count_launches(1);
     return cudaGetLastError();
 }

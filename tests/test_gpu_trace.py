@@ -299,6 +299,27 @@ def test_refit_equals_fresh_build():
         assert np.array_equal(a[k].view(np.uint32), b[k].view(np.uint32)), k
 
 
+@pytest.mark.parametrize("n", [1, 31, 33, 127, 129, 152 * 8 * 128, 152 * 8 * 128 + 1])
+def test_small_and_large_queries_agree(n):
+    """A query of no more rays than the launch has threads has no work counter:
+    both sides of that line give each ray the record it has in a query of
+    twice the rays and of a third of them, call after call."""
+    s = _random_scene(91, 40)
+    lo, hi = s.world_aabb()
+    rays = g.random_rays(2 * n, lo - 5, hi + 5, seed=n)
+    with rg.GpuScene(s) as gs:
+        all_hits = trace(gs, rays)
+        for _ in range(2):
+            a, b = trace(gs, rays[:n]), trace(gs, rays[:(n + 2) // 3])
+            for k in ("inst", "prim", "t", "u", "v"):
+                x = np.ascontiguousarray(all_hits[k]).view(np.uint32)
+                assert np.array_equal(np.ascontiguousarray(a[k]).view(np.uint32), x[:n]), k
+                assert np.array_equal(np.ascontiguousarray(b[k]).view(np.uint32), x[:(n + 2) // 3]), k
+        rays[:, 7] = np.random.default_rng(n).uniform(1, 60, len(rays))
+        occ = trace(gs, rays, rg.RG_ANY)["inst"] != MISS
+        assert np.array_equal(trace(gs, rays[:n], rg.RG_ANY)["inst"] != MISS, occ[:n])
+
+
 def test_injected_allocation_failure_is_reported():
     """RG_FAULT=alloc:N makes the N-th library allocation fail (host side);
     the call returns RG_ERR_OOM and the library stays usable."""
