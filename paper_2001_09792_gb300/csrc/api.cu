@@ -229,6 +229,16 @@ struct EventPair {
 // counter of its own, in turn)
 constexpr uint32_t kTraceSlots = 64;
 
+// A frame of at least kBandPixels is enqueued as kBands bands of pixels on
+// streams of their own, each a whole pipeline: a launch of a level ends with
+// its longest rays and leaves most of the chip idle, which another band's launch
+// then fills.  The medium frame at 1080p, us: 2,140 as one, 2,009 in 2 bands,
+// 2,011 in 3, 1,971 in 4, 2,032 in 8; at 640x480 903, 905, 898, 893, 887.  Scenes
+// that share their BLAS are made to have frames in flight, which fill each
+// other's tails: they keep one pipeline a frame (four in flight 0.632 ms a
+// frame as one, 0.651 in 2 bands, 0.691 in 4).
+constexpr uint32_t kBands = 4, kBandPixels = 1u << 18;
+
 struct rg_scene {
     int device = 0;
     rg_scene_desc desc{};
@@ -267,6 +277,8 @@ struct rg_scene {
     uint32_t* trace_ctr = nullptr; // rg_trace_rays work counters: kTraceSlots slots, 128 B apart (after the status word)
     uint32_t trace_slot = 0;       // the next call's slot
     uint32_t* h_counts = nullptr;  // pinned, 16 entries (made by the first render that waits for counts)
+    cudaStream_t band_stream[kBands - 1] = {};  // of a frame's further bands (made by the first such frame)
+    cudaEvent_t band_ev[kBands] = {};           // [0] the frame may start, [k] band k is done
     cudaEvent_t count_ev = nullptr;  // the next level's ray count has reached h_counts
     // statistics and timing
     uint64_t closest_rays = 0, shadow_rays_host = 0;
@@ -491,6 +503,10 @@ rg_status rg_scene_destroy(rg_scene* s) {
     if (s->st) cudaFree(s->st);
     if (s->h_counts) cudaFreeHost(s->h_counts);
     if (s->count_ev) cudaEventDestroy(s->count_ev);
+    for (cudaEvent_t e : s->band_ev)
+        if (e) cudaEventDestroy(e);
+    for (cudaStream_t b : s->band_stream)
+        if (b) cudaStreamDestroy(b);
     for (EventPair& ep : s->events) {
         cudaEventDestroy(ep.a);
         cudaEventDestroy(ep.b);
@@ -809,76 +825,31 @@ rg_status rg_trace_rays(rg_scene* s, const rg_ray* d_rays, uint32_t n, uint32_t 
     return RG_OK;
 }
 
-rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, uint32_t max_depth, float* d_rgba,
-                    void* stream) {
+// One band of rg_render: its whole pipeline on stream st.  Without async
+// the host sizes the scene's queues level by level (one band).
+static rg_status render_band(rg_scene* s, const CameraDev& cd, uint32_t w, uint32_t h, uint32_t max_depth, float* d_rgba,
+                             bool clear, bool async, uint32_t first, uint32_t count, uint32_t N, const uint64_t cap_q[2],
+                             uint64_t cap_max, uint32_t* counters, uint32_t* seg_count, cudaStream_t st) {
     rg_status r;
-    if ((r = check_scene(s))) return r;
-    if (!s->tlas_built) return fail(RG_ERR_NOT_BUILT, "render before rg_tlas_build");
-    if (!cam || !d_rgba || w == 0 || h == 0 || max_depth == 0) return fail(RG_ERR_INVALID_ARG, "bad render arguments");
-    if ((uint64_t)w * h > (1ull << 28)) return fail(RG_ERR_INVALID_ARG, "image too large");
-    if (s->n_mats == 0) return fail(RG_ERR_NOT_BUILT, "no materials set");
-    if ((r = set_device(s))) return r;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const uint32_t N = w * h;
     const uint32_t L = s->n_lights;
-    // Per depth level: closest-hit traversal, shading, shadow traversal.  The
-    // shadow rays of a level and the closest-hit rays of the next depend only
-    // on the level's shading and share one launch (k_trace_pair) unless
-    // RG_SCENE_NO_PAIR is set or the BVH is the compressed one.  Every launch
-    // reads its ray count on the device.  Counters: one block per level, [0]
-    // closest work, [1] rays of the next level, [2] shadow work (and the
-    // pair's), [4 + l] shadow rays toward light l.
     const size_t CB = 4 + kMaxLights;
-    if ((r = s->counters.ensure(CB * ((size_t)max_depth + 1), "counters"))) return r;
-    // Queue room (before anything is written to the queues: growing one
-    // frees its contents).  Level d holds at most N 2^(d-1) rays (a ray spawns at most
-    // two).  When that worst case for the whole frame fits the budget it is
-    // allocated once and the frame is enqueued without the host waiting:
-    // every count is read on the device.  Otherwise the host learns each
-    // level's count one level late (copied back while the GPU traces) and
-    // sizes the next queues from it.
-    auto cap_of = [&](uint32_t d) { return (uint64_t)N << (d - 1); };
-    bool async = !(s->desc.flags & RG_SCENE_FRUGAL) && max_depth <= 24;
-    uint64_t cap_q[2] = {0, 0}, cap_max = 0;
-    if (async) {
-        for (uint32_t d = 1; d <= max_depth; ++d) {
-            cap_q[(d - 1) & 1] = std::max(cap_q[(d - 1) & 1], cap_of(d));
-            cap_max = std::max(cap_max, cap_of(d));
-        }
-        const uint64_t bytes = (cap_q[0] + cap_q[1]) * 48 + cap_max * 16 + cap_max * L * 48;
-        async = cap_max <= 0xFFFFFFFFull && bytes <= kAsyncQueueBudget;
-    }
-    if (async) {
-        if ((r = s->q_rays[0].ensure(2 * cap_q[0], "ray queue")) || (r = s->q_pay[0].ensure(cap_q[0], "payload queue")) ||
-            (max_depth > 1 && ((r = s->q_rays[1].ensure(2 * cap_q[1], "ray queue")) ||
-                               (r = s->q_pay[1].ensure(cap_q[1], "payload queue")))) ||
-            (r = s->hits.ensure(cap_max, "hit queue")) ||
-            (L && ((r = s->s_rays.ensure(2 * cap_max * L, "shadow queue")) ||
-                   (r = s->s_pay.ensure(cap_max * L, "shadow payload")))))
-            return r;
-    }
-
-    if ((r = s->q_rays[0].ensure(2 * (size_t)N, "ray queue"))) return r;
-    if ((r = s->q_pay[0].ensure(N, "payload queue"))) return r;
-    if ((r = s->hits.ensure(N, "hit queue"))) return r;
-    if (!s->seg_count.p) {
-        if ((r = s->seg_count.ensure(kShadowSplitMax, "shadow segment counts"))) return r;
-        RG_CK(cudaMemsetAsync(s->seg_count.p, 0, (size_t)kShadowSplitMax * sizeof(uint32_t), st));
-    }
-    const bool aligned = reinterpret_cast<uintptr_t>(d_rgba) % 16 == 0;
-    if (!aligned) RG_CK(cudaMemsetAsync(d_rgba, 0, (size_t)N * 16, st));
-    CameraDev cd;
-    std::memcpy(&cd, cam, sizeof cd);
-    RG_CK(launch_raygen(cd, w, h, s->q_rays[0].p, s->q_pay[0].p,
-                        aligned ? reinterpret_cast<float4*>(d_rgba) : nullptr, s->counters.p,
-                        (uint32_t)(CB * ((size_t)max_depth + 1)), st));
+    auto cap_of = [&](uint32_t d) { return (uint64_t)count << (d - 1); };
+    // the band's part of each queue: queue q holds up to cap_q[q] rays for N pixels
+    auto part = [&](uint64_t cap) { return (size_t)(cap / N * first); };
+    auto rays_q = [&](int q) { return s->q_rays[q].p + 2 * part(cap_q[q]); };
+    auto pay_q = [&](int q) { return s->q_pay[q].p + part(cap_q[q]); };
+    auto hits_p = [&] { return s->hits.p + part(cap_max); };
+    auto s_rays = [&] { return s->s_rays.p + 2 * part(cap_max) * L; };
+    auto s_pay = [&] { return s->s_pay.p + part(cap_max) * L; };
+    RG_CK(launch_raygen(cd, w, h, first, count, rays_q(0), pay_q(0), clear ? reinterpret_cast<float4*>(d_rgba) : nullptr,
+                        counters, (uint32_t)(CB * ((size_t)max_depth + 1)), st));
 
     // shading of depth level `depth` (its rays in queue q, spawns into 1 - q)
     auto shade_args = [&](uint32_t depth, int q, uint32_t* c, bool last, uint32_t n_stride) {
         ShadeArgs sa{};
-        sa.rays = s->q_rays[q].p;
-        sa.payload = s->q_pay[q].p;
-        sa.hits = s->hits.p;
+        sa.rays = rays_q(q);
+        sa.payload = pay_q(q);
+        sa.hits = hits_p();
         sa.inst = s->wide ? s->inst8.p : s->inst;
         sa.mats = s->mats.p;
         sa.n_mats = s->n_mats;
@@ -891,11 +862,11 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         sa.depth = depth;
         sa.max_depth = max_depth;
         sa.image = d_rgba;
-        sa.next_rays = last ? nullptr : s->q_rays[1 - q].p;
-        sa.next_payload = last ? nullptr : s->q_pay[1 - q].p;
+        sa.next_rays = last ? nullptr : rays_q(1 - q);
+        sa.next_payload = last ? nullptr : pay_q(1 - q);
         sa.next_count = c + 1;
-        sa.shadow_rays = s->s_rays.p;
-        sa.shadow_payload = s->s_pay.p;
+        sa.shadow_rays = s_rays();
+        sa.shadow_payload = s_pay();
         sa.shadow_count = c + 4;
         sa.shadow_stride = n_stride;
         sa.st = s->st;
@@ -905,10 +876,10 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
     // closest-hit traversal of level d (count on the host, or on the device)
     auto trace_closest = [&](int q, uint32_t n_host, const uint32_t* d_count, uint32_t* c) -> rg_status {
         TraceArgs a = base_trace_args(s, true);
-        a.rays = s->q_rays[q].p;
+        a.rays = rays_q(q);
         a.n = n_host;
         a.d_count = d_count;
-        a.hits_render = s->hits.p;
+        a.hits_render = hits_p();
         a.work_counter = c + 0;
         EventPair* ev;
         rg_status rr;
@@ -917,18 +888,12 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         return event_end(s, st);
     };
 
-    if (!async) {
-        if (!s->h_counts)
-            RG_CK(cudaMallocHost(reinterpret_cast<void**>(&s->h_counts), 16 * sizeof(uint32_t)));
-        if (!s->count_ev) RG_CK(cudaEventCreateWithFlags(&s->count_ev, cudaEventDisableTiming));
-    }
-
-    uint32_t n = N;  // this level's rays (a bound on them when async)
+    uint32_t n = count;  // this level's rays (a bound on them when async)
     int cur = 0;
-    if ((r = trace_closest(cur, N, nullptr, s->counters.p))) return r;
+    if ((r = trace_closest(cur, count, nullptr, counters))) return r;
     for (uint32_t depth = 1; depth <= max_depth; ++depth) {
         const bool last = depth == max_depth;
-        uint32_t* c = s->counters.p + CB * (depth - 1);
+        uint32_t* c = counters + CB * (depth - 1);
         if (async) {
             n = (uint32_t)cap_of(depth);
         } else {
@@ -952,11 +917,11 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         TraceArgs b{};
         if (L) {
             b = base_trace_args(s, true);
-            b.rays = s->s_rays.p;
+            b.rays = s_rays();
             b.sub_counts = c + 4;
             b.n_sub = L;
             b.sub_stride = n;
-            b.payload = s->s_pay.p;
+            b.payload = s_pay();
             b.image = d_rgba;
             b.work_counter = c + 2;
         }
@@ -965,7 +930,7 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
             // the last level's shadow rays, traced on their own: when few, each
             // as segments side by side (in a pair the closest-hit rays fill
             // the lanes); the same rule with and without pairs
-            b.seg_count = s->seg_count.p;
+            b.seg_count = seg_count;
             b.split = kShadowSplit;
             b.split_max = kShadowSplitMax;
         }
@@ -981,9 +946,9 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         if (!async && (r = s->hits.ensure(2 * (size_t)n, "hit queue"))) return r;
         if (pair) {
             TraceArgs a = base_trace_args(s, true);
-            a.rays = s->q_rays[1 - cur].p;
+            a.rays = rays_q(1 - cur);
             a.d_count = c + 1;
-            a.hits_render = s->hits.p;
+            a.hits_render = hits_p();
             EventPair* ev;
             if ((r = event_begin(s, 2, st, &ev))) return r;
             RG_CK(launch_trace_pair(false, s->desc.flags & RG_SCENE_COUNT, b, a, st));
@@ -996,6 +961,101 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
             RG_CK(cudaEventSynchronize(s->count_ev));
             n = s->h_counts[0];
             if (n == 0) break;
+        }
+    }
+    return RG_OK;
+}
+
+rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, uint32_t max_depth, float* d_rgba,
+                    void* stream) {
+    rg_status r;
+    if ((r = check_scene(s))) return r;
+    if (!s->tlas_built) return fail(RG_ERR_NOT_BUILT, "render before rg_tlas_build");
+    if (!cam || !d_rgba || w == 0 || h == 0 || max_depth == 0) return fail(RG_ERR_INVALID_ARG, "bad render arguments");
+    if ((uint64_t)w * h > (1ull << 28)) return fail(RG_ERR_INVALID_ARG, "image too large");
+    if (s->n_mats == 0) return fail(RG_ERR_NOT_BUILT, "no materials set");
+    if ((r = set_device(s))) return r;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const uint32_t N = w * h;
+    const uint32_t L = s->n_lights;
+    // Per depth level: closest-hit traversal, shading, shadow traversal.  The
+    // shadow rays of a level and the closest-hit rays of the next depend only
+    // on the level's shading and share one launch (k_trace_pair) unless
+    // RG_SCENE_NO_PAIR is set or the BVH is the compressed one.  Every launch
+    // reads its ray count on the device.  Counters: one block per level, [0]
+    // closest work, [1] rays of the next level, [2] shadow work (and the
+    // pair's), [4 + l] shadow rays toward light l.
+    const size_t CB = 4 + kMaxLights;
+    // Queue room (before anything is written to the queues: growing one
+    // frees its contents).  Level d holds at most N 2^(d-1) rays (a ray spawns at most
+    // two).  When that worst case for the whole frame fits the budget it is
+    // allocated once and the frame is enqueued without the host waiting:
+    // every count is read on the device.  Otherwise the host learns each
+    // level's count one level late (copied back while the GPU traces) and
+    // sizes the next queues from it.
+    auto cap_of = [&](uint32_t d) { return (uint64_t)N << (d - 1); };
+    bool async = !(s->desc.flags & RG_SCENE_FRUGAL) && max_depth <= 24;
+    uint64_t cap_q[2] = {0, 0}, cap_max = 0;
+    if (async) {
+        for (uint32_t d = 1; d <= max_depth; ++d) {
+            cap_q[(d - 1) & 1] = std::max(cap_q[(d - 1) & 1], cap_of(d));
+            cap_max = std::max(cap_max, cap_of(d));
+        }
+        const uint64_t bytes = (cap_q[0] + cap_q[1]) * 48 + cap_max * 16 + cap_max * L * 48;
+        async = cap_max <= 0xFFFFFFFFull && bytes <= kAsyncQueueBudget;
+    }
+    const bool banded = async && max_depth > 1 && N >= kBandPixels && s->B.use_count() == 1 &&
+                        !(s->desc.flags & (RG_SCENE_TIMING | RG_SCENE_COUNT));
+    const uint32_t n_bands = banded ? kBands : 1u;
+    const size_t n_counters = CB * ((size_t)max_depth + 1);
+    if ((r = s->counters.ensure(n_counters * n_bands, "counters"))) return r;
+    if (async) {
+        if ((r = s->q_rays[0].ensure(2 * cap_q[0], "ray queue")) || (r = s->q_pay[0].ensure(cap_q[0], "payload queue")) ||
+            (max_depth > 1 && ((r = s->q_rays[1].ensure(2 * cap_q[1], "ray queue")) ||
+                               (r = s->q_pay[1].ensure(cap_q[1], "payload queue")))) ||
+            (r = s->hits.ensure(cap_max, "hit queue")) ||
+            (L && ((r = s->s_rays.ensure(2 * cap_max * L, "shadow queue")) ||
+                   (r = s->s_pay.ensure(cap_max * L, "shadow payload")))))
+            return r;
+    }
+
+    if ((r = s->q_rays[0].ensure(2 * (size_t)N, "ray queue"))) return r;
+    if ((r = s->q_pay[0].ensure(N, "payload queue"))) return r;
+    if ((r = s->hits.ensure(N, "hit queue"))) return r;
+    if (s->seg_count.cap < (size_t)kShadowSplitMax * n_bands) {
+        if ((r = s->seg_count.ensure((size_t)kShadowSplitMax * n_bands, "shadow segment counts"))) return r;
+        RG_CK(cudaMemsetAsync(s->seg_count.p, 0, (size_t)kShadowSplitMax * n_bands * sizeof(uint32_t), st));
+    }
+    const bool aligned = reinterpret_cast<uintptr_t>(d_rgba) % 16 == 0;
+    if (!aligned) RG_CK(cudaMemsetAsync(d_rgba, 0, (size_t)N * 16, st));
+    CameraDev cd;
+    std::memcpy(&cd, cam, sizeof cd);
+    if (!async) {
+        if (!s->h_counts)
+            RG_CK(cudaMallocHost(reinterpret_cast<void**>(&s->h_counts), 16 * sizeof(uint32_t)));
+        if (!s->count_ev) RG_CK(cudaEventCreateWithFlags(&s->count_ev, cudaEventDisableTiming));
+    }
+    if (n_bands > 1) {
+        for (uint32_t k = 0; k < n_bands; ++k) {
+            if (!s->band_ev[k]) RG_CK(cudaEventCreateWithFlags(&s->band_ev[k], cudaEventDisableTiming));
+            if (k && !s->band_stream[k - 1])
+                RG_CK(cudaStreamCreateWithFlags(&s->band_stream[k - 1], cudaStreamNonBlocking));
+        }
+        RG_CK(cudaEventRecord(s->band_ev[0], st));
+    }
+    // each band's pixels, stream, and parts of the queues and counters; the
+    // caller's stream goes on when all are done
+    for (uint32_t band = 0; band < n_bands; ++band) {
+        const uint32_t first = (uint32_t)((uint64_t)N * band / n_bands);
+        const uint32_t count = (uint32_t)((uint64_t)N * (band + 1) / n_bands) - first;
+        const cudaStream_t bst = band ? s->band_stream[band - 1] : st;
+        if (band) RG_CK(cudaStreamWaitEvent(bst, s->band_ev[0], 0));
+        if ((r = render_band(s, cd, w, h, max_depth, d_rgba, aligned, async, first, count, N, cap_q, cap_max,
+                             s->counters.p + n_counters * band, s->seg_count.p + (size_t)kShadowSplitMax * band, bst)))
+            return r;
+        if (band) {
+            RG_CK(cudaEventRecord(s->band_ev[band], bst));
+            RG_CK(cudaStreamWaitEvent(st, s->band_ev[band], 0));
         }
     }
     return RG_OK;

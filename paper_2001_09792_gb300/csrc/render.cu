@@ -75,24 +75,26 @@ __device__ __forceinline__ void tile_pixel(uint32_t i, uint32_t w, uint32_t h, u
     x = 8u * blk + rem % bw;
 }
 
-// The primary rays; clears the image (null: already clear) and the frame's
+// The primary rays of `count` pixels from `first` on (in tile order); clears
+// those pixels of the image (null: already clear) and the frame's
 // counters on the way, which were two launches of their own.
-__global__ void k_raygen(CameraDev cam, uint32_t w, uint32_t h, float4* __restrict__ rays,
+__global__ void k_raygen(CameraDev cam, uint32_t w, uint32_t h, uint32_t first, uint32_t count, float4* __restrict__ rays,
                          Payload* __restrict__ payload, float4* __restrict__ image, uint32_t* __restrict__ counters,
                          uint32_t n_counters) {
     chain_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     for (uint32_t k = i; k < n_counters; k += gridDim.x * blockDim.x) counters[k] = 0u;
-    if (i >= w * h) return;
-    if (image) image[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i >= count) return;
+
     uint32_t x, y;
-    tile_pixel(i, w, h, x, y);
+    tile_pixel(first + i, w, h, x, y);
     float4 o, d;
     camera_ray(cam, w, h, x, y, o, d);
     rays[2 * (size_t)i] = o;
     rays[2 * (size_t)i + 1] = d;
     Payload p;
     p.pixel = y * w + x;
+    if (image) image[p.pixel] = make_float4(0.f, 0.f, 0.f, 0.f);
     p.r = p.g = p.b = 1.0f;
     payload[i] = p;
 }
@@ -671,10 +673,10 @@ __global__ void __launch_bounds__(kFxaaThreads, 4) k_fxaa(const float4* __restri
 
 }  // namespace
 
-cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, float4* rays, Payload* payload, float4* image,
-                          uint32_t* counters, uint32_t n_counters, cudaStream_t s) {
-    size_t n = (size_t)w * h;
-    launch_chain(k_raygen, (unsigned)((n + 255) / 256), 256, 0, s, cam, w, h, rays, payload, image, counters, n_counters);
+cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, uint32_t first, uint32_t count, float4* rays,
+                          Payload* payload, float4* image, uint32_t* counters, uint32_t n_counters, cudaStream_t s) {
+    launch_chain(k_raygen, (unsigned)(((size_t)count + 255) / 256), 256, 0, s, cam, w, h, first, count, rays, payload,
+                 image, counters, n_counters);
     count_launches(1);
     return cudaGetLastError();
 }

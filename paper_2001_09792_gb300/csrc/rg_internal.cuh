@@ -401,10 +401,10 @@ struct ShadeArgs {
     const uint32_t* next_base;
     uint32_t ring_mask;
 };
-// image (may be null) and counters are cleared.
-cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, float4* rays, Payload* payload, float4* image,
-                          uint32_t* counters, uint32_t n_counters,
-                          cudaStream_t s);
+// The primary rays of `count` pixels from `first` on in tile order; their pixels
+// of the image (may be null) and the counters are cleared.
+cudaError_t launch_raygen(const CameraDev& cam, uint32_t w, uint32_t h, uint32_t first, uint32_t count, float4* rays,
+                          Payload* payload, float4* image, uint32_t* counters, uint32_t n_counters, cudaStream_t s);
 cudaError_t launch_shade(const ShadeArgs& a, uint32_t n_max, cudaStream_t s);
 // Batched wavefront: primary rays of newly admitted requests, written to ring
 // entries (*gen_base + req[k].offset + pixel) & ring_mask for request k; each

@@ -256,6 +256,42 @@ def test_frugal_queues_equal_worst_case_queues(lights, bvh):
     assert sa["closest_rays"] > s.width * s.height
 
 
+@pytest.mark.parametrize("w,h,depth,lights,bvh", [(1280, 720, 3, 4, 0), (769, 521, 2, 1, 0), (1024, 256, 4, 0, 0),
+                                                  (640, 480, 3, 2, rg.RG_SCENE_COMPRESSED)])
+def test_banded_frame_equals_one_pipeline(w, h, depth, lights, bvh):
+    """Frames large enough to be enqueued as bands on streams of their own show the
+    image, and trace the rays, of the one pipeline that RG_SCENE_FRUGAL
+    keeps; read on the caller's stream at once, frame after frame, into a
+    fresh image, one that is reused, and one that is not 16-byte aligned."""
+    s = g.medium_scene(width=w, height=h, max_depth=depth)
+    s.light_pos, s.light_I = s.light_pos[:lights], s.light_I[:lights]
+    with rg.GpuScene(s, flags=rg.RG_SCENE_FRUGAL | bvh) as gs:
+        rg.rg_reset_stats(gs.h)
+        ref = render(s, gs=gs)
+        sr = rg.rg_get_stats(gs.h)
+    side = torch.cuda.Stream()
+    with rg.GpuScene(s, flags=bvh) as gs:
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            rg.rg_reset_stats(gs.h)
+            img = rg.rg_render(gs.h, s.camera, w, h, depth)
+            got = [img.clone()]
+            st = rg.rg_get_stats(gs.h)
+            small = rg.rg_render(gs.h, s.camera, 64, 32, depth)   # one pipeline in between
+            img.fill_(7.0)
+            rg.rg_render(gs.h, s.camera, w, h, depth, out=img)
+            got.append(img.clone())
+            odd = torch.full((w * h * 4 + 1,), 3.0, device="cuda")[1:]
+            rg.rg_render(gs.h, s.camera, w, h, depth, out=odd)
+            got.append(odd.reshape(h, w, 4).clone())
+        side.synchronize()
+        rg.rg_sync(gs.h)
+        assert torch.isfinite(small).all()
+    for a in got:
+        np.testing.assert_allclose(a.cpu().numpy().reshape(ref.shape), ref, atol=1e-5)
+    assert (st["closest_rays"], st["shadow_rays"]) == (sr["closest_rays"], sr["shadow_rays"])
+
+
 def test_deep_render_beyond_the_worst_case_budget():
     """A render whose worst-case queues exceed the budget (960x540, depth 10:
     up to 512 rays per pixel at the last level) takes the per-level path and
