@@ -499,20 +499,20 @@ __device__ __forceinline__ float fxaa_luma(float4 c) {
 }
 
 // A block filters a T x T tile of pixels in one pass over the image: the lumas
-// of the tile and kFxaaHalo pixels around it go to shared memory (an edge pixel
+// of the tile and H pixels around it go to shared memory (an edge pixel
 // looks up about a hundred), each thread keeps the colours of its own pixels in
 // registers and writes those that step 2 copies, and the edge pixels, queued
 // in shared memory, are shared out over the block's threads, so that a few of
 // them do not hold the other lanes of their warps.  The edge search leaves
 // the halo only on long edges; there the luma comes from the colour.  Bound by
-// memory (32 B a pixel); 3840x2160: 57 us, 4.6 TB/s, against 101 us for a luma
+// memory (32 B a pixel); 3840x2160: 50.3 us, 5.3 TB/s, against 101 us for a luma
 // image written by one kernel and read with the colours again by another.
-constexpr int kFxaaHalo = 8;
 constexpr int kFxaaThreads = 256;
+constexpr uint64_t kFxaaManyTiles = 4800;
 
-template <int T>
+template <int T, int H>
 struct FxaaTile {
-    static constexpr int S = T + 2 * kFxaaHalo;
+    static constexpr int S = T + 2 * H;
     const float4* p;
     const float* s;  // S x S lumas from (x0, y0) on, clamped to the image's edge
     int w, h, x0, y0;
@@ -557,8 +557,8 @@ __device__ __forceinline__ float second_diff(float a, float m, float b) { return
 __constant__ float kFxaaStep[12] = {1.0f, 1.0f, 1.0f, 1.0f, 1.0f, 1.5f, 2.0f, 2.0f, 2.0f, 2.0f, 4.0f, 8.0f};
 
 // Steps 3 to 7 for an edge pixel (x, y): its filtered colour.
-template <int T>
-__device__ __forceinline__ float3 fxaa_edge(const FxaaTile<T>& I, int x, int y) {
+template <int T, int H>
+__device__ __forceinline__ float3 fxaa_edge(const FxaaTile<T, H>& I, int x, int y) {
     const float lM = I.luma(x, y), lN = I.luma(x, y - 1), lS = I.luma(x, y + 1);
     const float lW = I.luma(x - 1, y), lE = I.luma(x + 1, y);
     const float lo = fminf(lM, fminf(fminf(lN, lS), fminf(lW, lE)));
@@ -607,17 +607,17 @@ __device__ __forceinline__ float3 fxaa_edge(const FxaaTile<T>& I, int x, int y) 
             return I.color_at(horiz ? fx : fx + f * sgn, horiz ? fy + f * sgn : fy);
 }
 
-template <int T>
-__global__ void __launch_bounds__(kFxaaThreads, 4) k_fxaa(const float4* __restrict__ in, int w, int h,
+template <int T, int H, int BLOCKS>
+__global__ void __launch_bounds__(kFxaaThreads, BLOCKS) k_fxaa(const float4* __restrict__ in, int w, int h,
                                                        float4* __restrict__ out) {
     chain_wait();
-    constexpr int S = FxaaTile<T>::S, kPix = T * T / kFxaaThreads, H = kFxaaHalo;
+    constexpr int S = FxaaTile<T, H>::S, kPix = T * T / kFxaaThreads;
     constexpr int kRing = S * S - T * T;  // halo pixels: H rows above and below, then H columns left and right
     __shared__ float s[S * S];
     __shared__ uint16_t list[T * T];
     __shared__ int n_list;
     const int t = threadIdx.x;
-    FxaaTile<T> I{in, s, w, h, (int)blockIdx.x * T - H, (int)blockIdx.y * T - H};
+    FxaaTile<T, H> I{in, s, w, h, (int)blockIdx.x * T - H, (int)blockIdx.y * T - H};
     if (t == 0) n_list = 0;
     float4 c[kPix];
 #pragma unroll
@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(kFxaaThreads, 4) k_fxaa(const float4* __restri
     for (int q = t; q < n_list; q += kFxaaThreads) {
         const int i = list[q];
         const int x = I.x0 + H + i % T, y = I.y0 + H + i / T;
-        const float3 r = fxaa_edge<T>(I, x, y);
+        const float3 r = fxaa_edge(I, x, y);
         out[(size_t)y * (size_t)w + (size_t)x] = make_float4(r.x, r.y, r.z, I.at(x, y).w);
     }
 }
@@ -707,13 +707,21 @@ cudaError_t launch_shade_batch(const ShadeArgs& a, cudaStream_t s) {
 
 cudaError_t launch_fxaa(const float4* in, uint32_t w, uint32_t h, float4* out, cudaStream_t s) {
     if (w == 0 || h == 0) return cudaSuccess;
-    // 32 x 32 tiles read 2.25 pixels per pixel (the halo's from L2), 16 x 16
-    // tiles 4; the small ones where the large would not give every SM a block
+    // 32 x 32 tiles with a halo of 8 read 2.25 pixels per pixel (the halo's from
+    // L2), 16 x 16 tiles 4; the small ones where the large would not give every
+    // SM a block.  An image of many waves of tiles is bound by the reads rather
+    // than by the searches' chains, and takes a halo of 4 (1.56 pixels), which
+    // the searches leave sooner, and a fifth block per SM: 3840x2160 50.3 us
+    // against 58.5, 3200x1800 40.1 against 43.0, but 2880x1620 (4,590 tiles) 37.2
+    // both and 1920x1080 23.6 against 21.9.
     const uint64_t tiles = (uint64_t)((w + 31) / 32) * ((h + 31) / 32);
-    if (tiles >= (uint64_t)device_sm_count() && (h + 15) / 16 <= 65535)
-        launch_chain(k_fxaa<32>, dim3((w + 31) / 32, (h + 31) / 32), kFxaaThreads, 0, s, in, (int)w, (int)h, out);
+    const dim3 big((w + 31) / 32, (h + 31) / 32), small((w + 15) / 16, (h + 15) / 16);
+    if (tiles < (uint64_t)device_sm_count() || (h + 15) / 16 > 65535)
+        launch_chain(k_fxaa<16, 8, 4>, small, kFxaaThreads, 0, s, in, (int)w, (int)h, out);
+    else if (tiles < kFxaaManyTiles)
+        launch_chain(k_fxaa<32, 8, 4>, big, kFxaaThreads, 0, s, in, (int)w, (int)h, out);
     else
-        launch_chain(k_fxaa<16>, dim3((w + 15) / 16, (h + 15) / 16), kFxaaThreads, 0, s, in, (int)w, (int)h, out);
+        launch_chain(k_fxaa<32, 4, 5>, big, kFxaaThreads, 0, s, in, (int)w, (int)h, out);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -47,9 +47,9 @@ def test_random_images(shape):
     assert_bitwise(gpu_fxaa(img2.astype(np.float32)), oracle.fxaa(img2.astype(np.float32)))
 
 
-@pytest.mark.parametrize("shape", [(31, 33), (352, 480), (353, 481), (417, 385)])
+@pytest.mark.parametrize("shape", [(31, 33), (352, 480), (353, 481), (417, 385), (2209, 2241)])
 def test_long_edges_across_tiles(shape):
-    """Both tile sizes, whole and ragged: edges of slope 0 to 1/40 both ways,
+    """Both tile sizes and both halos, whole and ragged: edges of slope 0 to 1/40 both ways,
     whose search runs past the tile and its halo, on a noisy ground."""
     rng = np.random.default_rng(shape[0])
     y, x = np.mgrid[:shape[0], :shape[1]]
