@@ -616,7 +616,7 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
              } else {
                  RG_CK(cudaMemsetAsync(perm, 0, 4, st));
              }
-             RG_CK(launch_blas_leaves_refit(d_vtx, d_idx, static_cast<uint32_t*>(perm), static_cast<float*>(lohi), nt,
+             RG_CK(launch_blas_leaves_refit(d_vtx, nv, d_idx, static_cast<uint32_t*>(perm), static_cast<float*>(lohi), nt,
                                             static_cast<uint32_t*>(parents), b.nodes, static_cast<uint32_t*>(fl), b.tris,
                                             b.leaf_of_prim,
                                             s->B->d_blas.p + id, s->st, st, static_cast<uint32_t*>(boxes_done)));

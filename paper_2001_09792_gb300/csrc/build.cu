@@ -544,7 +544,7 @@ __device__ void climb(uint32_t j, uint32_t n, float* box, const uint32_t* __rest
     record_error(st, RG_ERR_TIMEOUT);
 }
 
-__global__ void k_blas_leaves_refit(const float* __restrict__ vtx, const uint32_t* __restrict__ idx,
+__global__ void k_blas_leaves_refit(const float* __restrict__ vtx, uint32_t nv, const uint32_t* __restrict__ idx,
                                     const uint32_t* __restrict__ perm, const float* __restrict__ lohi, uint32_t n,
                                     const uint32_t* __restrict__ parents, float4* nodes, uint32_t* flags,
                                     float4* __restrict__ tris, uint32_t* __restrict__ leaf_of_prim, BlasDev* blas_out,
@@ -555,6 +555,8 @@ __global__ void k_blas_leaves_refit(const float* __restrict__ vtx, const uint32_
     uint32_t prim = perm[j];
     leaf_of_prim[prim] = j;
     uint32_t vi[3] = {idx[3 * (size_t)prim], idx[3 * (size_t)prim + 1], idx[3 * (size_t)prim + 2]};
+    // (a bad index was reported by k_tri_bounds, which boxed vertex 0 in its place)
+    if (vi[0] >= nv || vi[1] >= nv || vi[2] >= nv) vi[0] = vi[1] = vi[2] = 0u;
     // the triangle record: its vertices in the axis orders (x, y, z), (y, z, x)
     // and (z, x, y), prim in the first vertex's w of each
     float4* t = tris + 9 * (size_t)j;
@@ -949,12 +951,12 @@ cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasS
     return cudaGetLastError();
 }
 
-cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, const uint32_t* perm, const float* lohi,
-                                     uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
+cudaError_t launch_blas_leaves_refit(const float* vtx, uint32_t nv, const uint32_t* idx, const uint32_t* perm,
+                                     const float* lohi, uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
                                      float4* tris, uint32_t* leaf_of_prim, BlasDev* blas_out, DevStatus* st,
                                      cudaStream_t s, const uint32_t* boxes_done) {
-    launch_chain(k_blas_leaves_refit, grid_for(n), kBlock, 0, s, vtx, idx, perm, lohi, n, parents, nodes, flags, tris, leaf_of_prim, blas_out,
-                                                       st, boxes_done);
+    launch_chain(k_blas_leaves_refit, grid_for(n), kBlock, 0, s, vtx, nv, idx, perm, lohi, n, parents, nodes, flags,
+                 tris, leaf_of_prim, blas_out, st, boxes_done);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -215,8 +215,9 @@ cudaError_t radix_sort_pairs(const void* keys_in, const uint32_t* vals_in, uint3
 // ranges (optional, 2 per internal node): first and last leaf of node i.
 cudaError_t launch_karras(const void* keys, uint32_t n, int key_bits, uint32_t* child_base, int child_stride_words,
                           uint32_t* parents, cudaStream_t s, uint32_t* ranges = nullptr);
-cudaError_t launch_blas_leaves_refit(const float* vtx, const uint32_t* idx, const uint32_t* perm, const float* lohi,
-                                     uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
+// (an index of nv or more is read as vertex 0 throughout its triangle, as the box is)
+cudaError_t launch_blas_leaves_refit(const float* vtx, uint32_t nv, const uint32_t* idx, const uint32_t* perm,
+                                     const float* lohi, uint32_t n, const uint32_t* parents, float4* nodes, uint32_t* flags,
                                      float4* tris, uint32_t* leaf_of_prim, BlasDev* blas_out, DevStatus* st,
                                      cudaStream_t s, const uint32_t* boxes_done = nullptr);
 // Bounding sphere of a mesh about its root box centre (after the BLAS refit

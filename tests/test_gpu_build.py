@@ -290,6 +290,34 @@ def test_build_errors_reported():
         rg.rg_scene_destroy(h)
 
 
+@pytest.mark.parametrize("flags", [rg.RG_MORTON30, rg.RG_BLAS_SAH])
+def test_bad_index_reads_no_vertex_past_the_mesh(flags):
+    """A triangle with an index of nv or more is reported, and its record holds
+    vertex 0 in place of whatever lies behind the mesh (here memory that
+    the test owns: the call is told of fewer vertices than the tensor has)."""
+    import ctypes
+    v, i = g.make_mesh("uv", 16, 8)
+    nv = v.shape[0]
+    vt = cu(np.r_[v, np.full((8, 3), 777.0, np.float32)], np.float32)
+    bad = i.astype(np.uint32).copy()
+    rows = [0, 5, len(bad) - 1]
+    for k, r in enumerate(rows):
+        bad[r, k] = nv + k
+    it = cu(bad, np.int32)
+    h = rg.rg_scene_create()
+    try:
+        bid = ctypes.c_uint32()
+        assert rg.lib().rg_blas_build(h, vt.data_ptr(), nv, it.data_ptr(), len(bad), flags, ctypes.byref(bid), None) == 0
+        with pytest.raises(rg.RgError) as e:
+            rg.rg_sync(h)
+        assert e.value.status == rg.RG_ERR_INVALID_ARG
+        tris = rg.rg_blas_export(h, bid.value, len(bad))["tris"].reshape(-1, 3, 4)
+    finally:
+        rg.rg_scene_destroy(h)
+    want = v[np.where(np.isin(np.arange(len(bad)), rows)[:, None], 0, bad)]
+    assert np.array_equal(tris[:, :, :3], want[tris[:, 0, 3].view(np.uint32)])
+
+
 def test_not_built_errors():
     h = rg.rg_scene_create()
     try:
