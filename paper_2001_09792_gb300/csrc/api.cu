@@ -570,8 +570,10 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
                  BlasDev* np = nullptr;
                  rg_status rr = dev_alloc(reinterpret_cast<void**>(&np), ncap * sizeof(BlasDev), "BLAS table");
                  if (rr) return rr;
-                 if (s->B->d_blas.p && id) RG_CK(cudaMemcpyAsync(np, s->B->d_blas.p, id * sizeof(BlasDev), cudaMemcpyDeviceToDevice, st));
                  if (s->B->d_blas.p) {
+                     // (builds on other streams may still be writing their entries)
+                     RG_CK(cudaDeviceSynchronize());
+                     if (id) RG_CK(cudaMemcpyAsync(np, s->B->d_blas.p, id * sizeof(BlasDev), cudaMemcpyDeviceToDevice, st));
                      RG_CK(cudaStreamSynchronize(st));
                      cudaFree(s->B->d_blas.p);
                  }

@@ -1,0 +1,88 @@
+"""The library's host code on a fake CUDA runtime (fake_cudart.cpp), without a
+GPU: the order of what it puts on its streams, and what it does when a call
+fails or another device is current.  Kernels do not run here."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_2001_09792_gb300 as rg
+from paper_2001_09792_gb300 import _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    _build.build()
+    objs = [os.path.join(_build.OUT, s.replace(".cu", ".o")) for s in _build.SOURCES]
+    if not all(os.path.exists(o) for o in objs):
+        _build.build(force=True)
+    out = str(tmp_path_factory.mktemp("fake") / "librg_fake.so")
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build.nvcc()))), "include")
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-w", "-fno-gnu-unique", f"-I{inc}",
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs, "-o", out, "-Wl,-Bsymbolic", "-Wl,--no-undefined",
+                    "-lpthread"], check=True)
+    L = ctypes.CDLL(out)
+    L.fake_log.restype = ctypes.c_char_p
+    L.fake_stream.restype = ctypes.c_void_p
+    L.rg_last_error.restype = ctypes.c_char_p
+    return L
+
+
+class Host:
+    """The library on the fake runtime, with meshes in host memory."""
+
+    def __init__(self, L):
+        self.L = L
+        self.scenes = []
+
+    def stream(self, prio=0):
+        return ctypes.c_void_p(self.L.fake_stream(prio))
+
+    def log(self):
+        return self.L.fake_log().decode().splitlines()
+
+    def scene(self, flags=0):
+        h = ctypes.c_void_p()
+        desc = rg.rg_scene_desc((ctypes.c_float * 3)(0, 0, 0), 0.1, flags)
+        assert self.L.rg_scene_create(ctypes.byref(h), ctypes.byref(desc)) == 0
+        self.scenes.append(h)
+        return h
+
+    def destroy(self, h):
+        self.scenes.remove(h)
+        assert self.L.rg_scene_destroy(h) == 0
+
+    def blas(self, h, nt=12, flags=0, stream=None):
+        v, i = np.zeros((8, 3), np.float32), np.zeros((nt, 3), np.uint32)
+        bid = ctypes.c_uint32()
+        return self.L.rg_blas_build(h, v.ctypes.data_as(ctypes.c_void_p), 8, i.ctypes.data_as(ctypes.c_void_p), nt, flags,
+                                    ctypes.byref(bid), stream)
+
+
+@pytest.fixture
+def host(fake_lib):
+    fake_lib.cudaSetDevice(0)
+    fake_lib.fake_reset()
+    H = Host(fake_lib)
+    yield H
+    for h in list(H.scenes):
+        H.destroy(h)
+    fake_lib.fake_finish()
+    fake_lib.cudaSetDevice(0)
+
+
+def test_growing_the_blas_table_waits_for_builds_on_other_streams(host):
+    """The table of BLAS descriptors is copied when it grows; a build on another
+    stream writes its descriptor and root box there, so the copy comes after
+    it."""
+    h, a, b = host.scene(), host.stream(), host.stream()
+    assert host.blas(h, stream=a) == 0 and host.blas(h, stream=a) == 0
+    at = len(host.log())
+    assert host.blas(h, stream=b) == 0
+    new = host.log()[at:]
+    copy = next(k for k, line in enumerate(new) if line.startswith(f"copy s{b.value // 16} "))
+    assert "devsync" in new[:copy]
