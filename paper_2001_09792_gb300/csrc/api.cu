@@ -430,7 +430,9 @@ rg_status rg_scene_create(rg_scene** out, const rg_scene_desc* desc) {
         return r;
     }
     s->trace_ctr = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(s->st) + kCtrAt);
+    // (the clear goes to the default stream, which the streams of later calls may not wait for)
     cudaError_t e = cudaMemset(s->st, 0, sizeof(DevStatus));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         cudaFree(s->st);
         delete s;
@@ -472,6 +474,11 @@ rg_status rg_scene_create_shared(rg_scene** out, rg_scene* src) {
             rg_scene_destroy(s);
             return cuda_fail(e, "copying lights");
         }
+    }
+    // (copies between device buffers do not wait on the host)
+    if (cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy); e != cudaSuccess) {
+        rg_scene_destroy(s);
+        return cuda_fail(e, "copying materials and lights");
     }
     s->n_lights = src->n_lights;
     *out = s;

@@ -35,7 +35,7 @@ void log(const char* fmt, ...) {
 }
 cudaError_t ret(cudaError_t e) { return e == cudaSuccess ? e : g_last = e; }
 void* handle() { return reinterpret_cast<void*>((size_t)g_next++ * 16); }
-int id(const void* h) { return (int)((size_t)h / 16); }
+int id(const void* h) { return (int)((size_t)h / 16); }  // (the legacy stream has the handle 1)
 
 cudaError_t launch(const void* f, dim3 g, size_t smem, cudaStream_t s) {
     if (++g_launches == g_fail_launch) return ret(cudaErrorLaunchOutOfResources);
@@ -95,7 +95,9 @@ cudaError_t cudaMemset(void* p, int v, size_t n) { return log("memset s0"), mems
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) {
     return log("memset s%d", id(s)), memset(p, v, n), cudaSuccess;
 }
-cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return memcpy(d, s, n), cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+    return log("copy s0"), memcpy(d, s, n), cudaSuccess;
+}
 cudaError_t cudaMemcpyAsync(void* d, const void* p, size_t n, cudaMemcpyKind, cudaStream_t s) {
     return log("copy s%d %zu", id(s), n), memcpy(d, p, n), cudaSuccess;
 }

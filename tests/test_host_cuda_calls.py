@@ -86,3 +86,24 @@ def test_growing_the_blas_table_waits_for_builds_on_other_streams(host):
     new = host.log()[at:]
     copy = next(k for k, line in enumerate(new) if line.startswith(f"copy s{b.value // 16} "))
     assert "devsync" in new[:copy]
+
+
+def test_scene_creation_waits_for_its_clear(host):
+    """The clear of the status word is queued on the default stream; calls on
+    streams that do not wait for that one come after it all the same."""
+    host.scene()
+    log = host.log()
+    assert "streamsync s0" in log[log.index("memset s0"):]
+
+
+def test_shared_scene_creation_waits_for_its_copies(host):
+    h = host.scene()
+    light = rg.rg_light((ctypes.c_float * 3)(0, 1, 0), (ctypes.c_float * 3)(1, 1, 1))
+    assert host.L.rg_scene_set_lights(h, ctypes.byref(light), 1) == 0
+    at = len(host.log())
+    out = ctypes.c_void_p()
+    assert host.L.rg_scene_create_shared(ctypes.byref(out), h) == 0
+    host.scenes.append(out)
+    new = host.log()[at:]
+    last_copy = max(k for k, line in enumerate(new) if line == "copy s0")
+    assert "streamsync s0" in new[last_copy:]
