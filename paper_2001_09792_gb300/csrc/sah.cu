@@ -1186,10 +1186,15 @@ rg_status sah_cuda_fail(cudaError_t e, const char* what) {
 
 template <class K>
 rg_status sah_build(SahBuild B, const int* cb_ord, cudaStream_t s) {
-    static std::atomic<int> attr_set{0};  // per process; concurrent first callers set the same values
-    if (!attr_set.load(std::memory_order_acquire)) {
+    // a bit per device, for the attribute holds for the current one only
+    // (concurrent first callers set the same values; devices past 63 set them each time)
+    static std::atomic<uint64_t> attr_set{0};
+    int dev = 0;
+    SAH_CK(cudaGetDevice(&dev));
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+    if (!(attr_set.load(std::memory_order_acquire) & bit)) {
         SAH_CK(set_block_smem<K>());
-        attr_set.store(1, std::memory_order_release);
+        attr_set.fetch_or(bit, std::memory_order_release);
     }
     const uint32_t n = B.n, sms = (uint32_t)device_sm_count();
     const uint32_t chunks = (n + kSahChunk - 1) / kSahChunk;

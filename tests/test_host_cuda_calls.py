@@ -107,3 +107,14 @@ def test_shared_scene_creation_waits_for_its_copies(host):
     new = host.log()[at:]
     last_copy = max(k for k, line in enumerate(new) if line == "copy s0")
     assert "streamsync s0" in new[last_copy:]
+
+
+@pytest.mark.parametrize("flags", [rg.RG_BLAS_SAH, rg.RG_BLAS_SAH | rg.RG_MORTON63])
+def test_sah_builds_on_a_second_device(host, flags):
+    """The large shared memory of the SAH blocks is allowed per device."""
+    for dev in (0, 1, 0):
+        host.L.cudaSetDevice(dev)
+        h = host.scene()
+        for nt in (64, 2000):  # a block per segment; the levels above it in one block
+            assert host.blas(h, nt, flags) == 0, host.L.rg_last_error()
+    assert any("k_sah_rest" in line for line in host.log())
