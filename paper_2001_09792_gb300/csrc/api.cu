@@ -539,6 +539,11 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
     if (nt > (1u << 30)) return fail(RG_ERR_INVALID_ARG, "too many triangles");
     if ((r = set_device(s))) return r;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // a captured build would write the descriptor only when the graph is
+    // launched, while later calls on the scene take the BLAS as built
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    RG_CK(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return fail(RG_ERR_CUDA, "rg_blas_build on a capturing stream");
     const int bits = (flags & RG_MORTON63) ? 21 : 10;
     const bool wide = (flags & RG_COMPRESSED) || (s->desc.flags & RG_SCENE_COMPRESSED);
     const size_t n_int = nt > 1 ? nt - 1 : 1;

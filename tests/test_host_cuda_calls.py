@@ -118,3 +118,17 @@ def test_sah_builds_on_a_second_device(host, flags):
         for nt in (64, 2000):  # a block per segment; the levels above it in one block
             assert host.blas(h, nt, flags) == 0, host.L.rg_last_error()
     assert any("k_sah_rest" in line for line in host.log())
+
+
+@pytest.mark.parametrize("flags", [rg.RG_MORTON30, rg.RG_BLAS_SAH])
+def test_blas_build_is_refused_on_a_capturing_stream(host, flags):
+    """A captured build would leave the descriptor to the graph's first launch,
+    while the scene takes the BLAS as built; nothing is put into the graph."""
+    h, s = host.scene(), host.stream()
+    assert host.blas(h, stream=s) == 0
+    host.L.fake_set_capturing(s, 1)
+    at = len(host.log())
+    assert host.blas(h, flags=flags, stream=s) == rg.RG_ERR_CUDA
+    assert host.log()[at:] == []
+    host.L.fake_set_capturing(s, 0)
+    assert host.blas(h, flags=flags, stream=s) == 0
