@@ -1064,13 +1064,17 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         const uint32_t count = (uint32_t)((uint64_t)N * (band + 1) / n_bands) - first;
         const cudaStream_t bst = band ? s->band_stream[band - 1] : st;
         if (band) RG_CK(cudaStreamWaitEvent(bst, s->band_ev[0], 0));
-        if ((r = render_band(s, cd, w, h, max_depth, d_rgba, aligned, async, first, count, N, cap_q, cap_max,
-                             s->counters.p + n_counters * band, s->seg_count.p + (size_t)kShadowSplitMax * band, bst)))
-            return r;
-        if (band) {
-            RG_CK(cudaEventRecord(s->band_ev[band], bst));
-            RG_CK(cudaStreamWaitEvent(st, s->band_ev[band], 0));
+        r = render_band(s, cd, w, h, max_depth, d_rgba, aligned, async, first, count, N, cap_q, cap_max,
+                        s->counters.p + n_counters * band, s->seg_count.p + (size_t)kShadowSplitMax * band, bst);
+        if (band) {  // (a band that failed half-way as well: what it has queued uses the image and the queues)
+            cudaError_t e = cudaEventRecord(s->band_ev[band], bst);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->band_ev[band], 0);
+            if (e != cudaSuccess) {
+                cudaStreamSynchronize(bst);
+                if (!r) r = cuda_fail(e, "joining a band of the frame");
+            }
         }
+        if (r) return r;
     }
     return RG_OK;
 }

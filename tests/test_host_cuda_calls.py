@@ -62,6 +62,29 @@ class Host:
         return self.L.rg_blas_build(h, v.ctypes.data_as(ctypes.c_void_p), 8, i.ctypes.data_as(ctypes.c_void_p), nt, flags,
                                     ctypes.byref(bid), stream)
 
+    def renderable(self, flags=0):
+        """A scene of one mesh and instance with a material and a light."""
+        h = self.scene(flags)
+        assert self.blas(h) == 0
+        inst = np.zeros((1, 16), np.float32)
+        assert self.L.rg_tlas_build(h, inst.ctypes.data_as(ctypes.c_void_p), 1, None) == 0
+        mat = rg.rg_material(0, (ctypes.c_float * 3)(1, 1, 1), 1.0)
+        light = rg.rg_light((ctypes.c_float * 3)(0, 1, 0), (ctypes.c_float * 3)(1, 1, 1))
+        assert self.L.rg_scene_set_materials(h, ctypes.byref(mat), 1) == 0
+        assert self.L.rg_scene_set_lights(h, ctypes.byref(light), 1) == 0
+        return h
+
+    def render(self, h, stream=None, size=512, depth=2):
+        """The status of one frame, and what it put on the streams."""
+        at = len(self.log())
+        r = self.L.rg_render(h, ctypes.byref(rg.rg_camera()), size, size, depth, ctypes.c_void_p(1 << 20), stream)
+        return r, self.log()[at:]
+
+
+def launches(log):
+    """The streams of a log's kernel launches, in order."""
+    return [line.split()[2] for line in log if line.startswith("launch ")]
+
 
 @pytest.fixture
 def host(fake_lib):
@@ -132,3 +155,23 @@ def test_blas_build_is_refused_on_a_capturing_stream(host, flags):
     assert host.log()[at:] == []
     host.L.fake_set_capturing(s, 0)
     assert host.blas(h, flags=flags, stream=s) == 0
+
+
+def test_failed_frame_leaves_nothing_behind_the_callers_stream(host):
+    """When a launch of one band fails, the caller's stream still waits for
+    every band that has work queued."""
+    h, s = host.renderable(), host.stream()
+    own = f"s{s.value // 16}"
+    r, log = host.render(h, s)
+    assert r == 0 and len(set(launches(log))) == 4
+    host.L.fake_finish()
+    for k in range(1, len(launches(log)) + 1):
+        host.L.fake_fail_launch(k)
+        r, part = host.render(h, s)
+        host.L.fake_fail_launch(0)
+        host.L.fake_finish()
+        assert r == rg.RG_ERR_CUDA
+        for band in set(launches(part)) - {own}:
+            last = max(i for i, line in enumerate(part) if line.startswith("launch ") and line.split()[2] == band)
+            rec = next(i for i, line in enumerate(part) if i > last and line.startswith("record ") and line.endswith(band))
+            assert f"wait {own} {part[rec].split()[1]}" in part[rec:]
