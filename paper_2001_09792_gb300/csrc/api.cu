@@ -278,6 +278,7 @@ struct rg_scene {
     uint32_t trace_slot = 0;       // the next call's slot
     uint32_t* h_counts = nullptr;  // pinned, 16 entries (made by the first render that waits for counts)
     cudaStream_t band_stream[kBands - 1] = {};  // of a frame's further bands (made by the first such frame)
+    int band_prio = 0;                          // their priority
     cudaEvent_t band_ev[kBands] = {};           // [0] the frame may start, [k] band k is done
     cudaEvent_t count_ev = nullptr;  // the next level's ray count has reached h_counts
     // statistics and timing
@@ -1050,10 +1051,20 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         if (!s->count_ev) RG_CK(cudaEventCreateWithFlags(&s->count_ev, cudaEventDisableTiming));
     }
     if (n_bands > 1) {
+        // the bands run at the priority of the caller's stream
+        int prio = 0;
+        RG_CK(cudaStreamGetPriority(st, &prio));
+        if (prio != s->band_prio)
+            for (cudaStream_t& b : s->band_stream) {
+                if (b) RG_CK(cudaStreamDestroy(b));  // (what it has queued still runs)
+                b = nullptr;
+            }
         for (uint32_t k = 0; k < n_bands; ++k) {
             if (!s->band_ev[k]) RG_CK(cudaEventCreateWithFlags(&s->band_ev[k], cudaEventDisableTiming));
-            if (k && !s->band_stream[k - 1])
-                RG_CK(cudaStreamCreateWithFlags(&s->band_stream[k - 1], cudaStreamNonBlocking));
+            if (k && !s->band_stream[k - 1]) {
+                RG_CK(cudaStreamCreateWithPriority(&s->band_stream[k - 1], cudaStreamNonBlocking, prio));
+                s->band_prio = prio;
+            }
         }
         RG_CK(cudaEventRecord(s->band_ev[0], st));
     }

@@ -175,3 +175,16 @@ def test_failed_frame_leaves_nothing_behind_the_callers_stream(host):
             last = max(i for i, line in enumerate(part) if line.startswith("launch ") and line.split()[2] == band)
             rec = next(i for i, line in enumerate(part) if i > last and line.startswith("record ") and line.endswith(band))
             assert f"wait {own} {part[rec].split()[1]}" in part[rec:]
+
+
+def test_bands_run_at_the_priority_of_the_callers_stream(host):
+    h = host.renderable()
+    prio = {f"s{st.value // 16}": p for p, st in ((p, host.stream(p)) for p in (-3, 0, -3, 2))}
+    log = []
+    for name in prio:
+        r, part = host.render(h, ctypes.c_void_p(int(name[1:]) * 16))
+        host.L.fake_finish()
+        assert r == 0
+        log += part
+        made = {f[1]: int(f[5]) for f in (line.split() for line in log if line.startswith("stream "))}
+        assert {made[b] for b in set(launches(part)) - {name}} == {prio[name]}
