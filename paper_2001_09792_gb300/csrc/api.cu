@@ -233,11 +233,12 @@ constexpr uint32_t kTraceSlots = 64;
 // streams of their own, each a whole pipeline: a launch of a level ends with
 // its longest rays and leaves most of the chip idle, which another band's launch
 // then fills.  The medium frame at 1080p, us: 2,140 as one, 2,009 in 2 bands,
-// 2,011 in 3, 1,971 in 4, 2,032 in 8; at 640x480 903, 905, 898, 893, 887.  Scenes
-// that share their BLAS are made to have frames in flight, which fill each
-// other's tails: they keep one pipeline a frame (four in flight 0.632 ms a
-// frame as one, 0.651 in 2 bands, 0.691 in 4).
-constexpr uint32_t kBands = 4, kBandPixels = 1u << 18;
+// 2,011 in 3, 1,971 in 4, 2,032 in 8; at 640x480 903, 905, 898, 893, 887.
+// Frames of other scenes in flight fill the tails as well: from kBandOthers of
+// them on, a frame is one pipeline.  Scenes of their own BLAS with 1, 2, 3 and 4
+// frames in flight, us a frame at 1080p: 1,173, 806, 690 and 654 as one, 1,055,
+// 787, 712 and 702 in 4 bands.
+constexpr uint32_t kBands = 4, kBandPixels = 1u << 18, kBandOthers = 2;
 
 struct rg_scene {
     int device = 0;
@@ -280,6 +281,7 @@ struct rg_scene {
     cudaStream_t band_stream[kBands - 1] = {};  // of a frame's further bands (made by the first such frame)
     int band_prio = 0;                          // their priority
     cudaEvent_t band_ev[kBands] = {};           // [0] the frame may start, [k] band k is done
+    cudaEvent_t frame_ev = nullptr;             // the last frame of bands' size is done
     cudaEvent_t count_ev = nullptr;  // the next level's ray count has reached h_counts
     // statistics and timing
     uint64_t closest_rays = 0, shadow_rays_host = 0;
@@ -349,6 +351,60 @@ rg_status collect_events(rg_scene* s) {
     }
     s->events.clear();
     return RG_OK;
+}
+
+// The last frames of kBandPixels and more, one entry a scene, per device; those
+// found finished are dropped.
+struct FrameList {
+    std::mutex mu;
+    std::vector<std::pair<const rg_scene*, cudaEvent_t>> frames;
+};
+FrameList g_frames[kMaxDevices];
+
+// The frames of other scenes that are still running on s's device.
+uint32_t others_in_flight(const rg_scene* s) {
+    if (s->device < 0 || s->device >= kMaxDevices) return kBandOthers;
+    // (an event may be asked for while a thread, this one too, captures another stream)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return kBandOthers;
+    uint32_t n = 0;
+    {
+        FrameList& L = g_frames[s->device];
+        std::lock_guard<std::mutex> lock(L.mu);
+        auto finished = [&](const std::pair<const rg_scene*, cudaEvent_t>& f) {
+            if (f.first == s) return false;
+            const bool running = cudaEventQuery(f.second) == cudaErrorNotReady;
+            n += running;
+            return !running;
+        };
+        L.frames.erase(std::remove_if(L.frames.begin(), L.frames.end(), finished), L.frames.end());
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (n) cudaGetLastError();  // (a query that finds an event unfinished leaves an error behind)
+    return n;
+}
+
+// Marks the end of a frame on the caller's stream for others_in_flight.
+rg_status note_frame(rg_scene* s, cudaStream_t st) {
+    if (s->device < 0 || s->device >= kMaxDevices) return RG_OK;
+    FrameList& L = g_frames[s->device];
+    std::lock_guard<std::mutex> lock(L.mu);
+    if (!s->frame_ev) RG_CK(cudaEventCreateWithFlags(&s->frame_ev, cudaEventDisableTiming));
+    RG_CK(cudaEventRecord(s->frame_ev, st));
+    for (const auto& f : L.frames)
+        if (f.first == s) return RG_OK;
+    L.frames.emplace_back(s, s->frame_ev);
+    return RG_OK;
+}
+
+void forget_frame(rg_scene* s) {
+    if (!s->frame_ev) return;
+    FrameList& L = g_frames[s->device];
+    std::lock_guard<std::mutex> lock(L.mu);
+    L.frames.erase(std::remove_if(L.frames.begin(), L.frames.end(), [&](const auto& f) { return f.first == s; }),
+                   L.frames.end());
+    cudaEventDestroy(s->frame_ev);
+    s->frame_ev = nullptr;
 }
 
 uint32_t iter_cap_for(const rg_scene* s, bool brute) {
@@ -511,6 +567,7 @@ rg_status rg_scene_destroy(rg_scene* s) {
     if (s->st) cudaFree(s->st);
     if (s->h_counts) cudaFreeHost(s->h_counts);
     if (s->count_ev) cudaEventDestroy(s->count_ev);
+    forget_frame(s);
     for (cudaEvent_t e : s->band_ev)
         if (e) cudaEventDestroy(e);
     for (cudaStream_t b : s->band_stream)
@@ -1019,8 +1076,12 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         const uint64_t bytes = (cap_q[0] + cap_q[1]) * 48 + cap_max * 16 + cap_max * L * 48;
         async = cap_max <= 0xFFFFFFFFull && bytes <= kAsyncQueueBudget;
     }
-    const bool banded = async && max_depth > 1 && N >= kBandPixels && s->B.use_count() == 1 &&
-                        !(s->desc.flags & (RG_SCENE_TIMING | RG_SCENE_COUNT));
+    // (a captured frame is one pipeline: the caller's stream alone is in its graph)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    RG_CK(cudaStreamIsCapturing(st, &cap));
+    const bool large = async && max_depth > 1 && N >= kBandPixels && cap == cudaStreamCaptureStatusNone;
+    const bool banded = large && !(s->desc.flags & (RG_SCENE_TIMING | RG_SCENE_COUNT)) &&
+                        others_in_flight(s) < kBandOthers;
     const uint32_t n_bands = banded ? kBands : 1u;
     const size_t n_counters = CB * ((size_t)max_depth + 1);
     if ((r = s->counters.ensure(n_counters * n_bands, "counters"))) return r;
@@ -1087,7 +1148,7 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         }
         if (r) return r;
     }
-    return RG_OK;
+    return large ? note_frame(s, st) : RG_OK;
 }
 
 rg_status rg_fxaa(const float* d_in, uint32_t w, uint32_t h, float* d_out, void* stream) {

@@ -23,6 +23,7 @@ std::map<void*, int> g_stream_prio, g_capturing;
 std::set<void*> g_pending;                             // events that cudaEventQuery finds unfinished
 int g_dev = 0, g_fail_launch = 0, g_launches = 0, g_pools = 0, g_next = 1;
 cudaError_t g_last = cudaSuccess;
+cudaStreamCaptureMode g_capture_mode = cudaStreamCaptureModeGlobal;
 
 void log(const char* fmt, ...) {
     char b[256];
@@ -133,7 +134,14 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) { return g_pending.erase(e), cudaSuc
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
     return log("record e%d s%d", id(e), id(s)), g_pending.insert(e), cudaSuccess;
 }
-cudaError_t cudaEventQuery(cudaEvent_t e) { return g_pending.count(e) ? cudaErrorNotReady : cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t e) {
+    if (g_capture_mode != cudaStreamCaptureModeRelaxed) log("query outside of the relaxed capture mode");
+    return g_pending.count(e) ? ret(cudaErrorNotReady) : cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) {
+    std::swap(*m, g_capture_mode);
+    return cudaSuccess;
+}
 cudaError_t cudaEventSynchronize(cudaEvent_t e) { return g_pending.erase(e), cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 0, cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {

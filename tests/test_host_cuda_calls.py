@@ -188,3 +188,44 @@ def test_bands_run_at_the_priority_of_the_callers_stream(host):
         log += part
         made = {f[1]: int(f[5]) for f in (line.split() for line in log if line.startswith("stream "))}
         assert {made[b] for b in set(launches(part)) - {name}} == {prio[name]}
+
+
+def streams_used(log):
+    return len(set(launches(log)))
+
+
+def test_bands_give_way_to_other_frames_in_flight(host):
+    """A frame is banded unless two or more frames of other scenes, sharing
+    their BLAS or not, are still running on its device; a scene's own earlier
+    frame, a finished one and one of a destroyed scene do not count."""
+    a, b, c = host.renderable(), host.renderable(), host.renderable()
+    shared = ctypes.c_void_p()
+    assert host.L.rg_scene_create_shared(ctypes.byref(shared), a) == 0
+    host.scenes.append(shared)
+    inst = np.zeros((1, 16), np.float32)
+    assert host.L.rg_tlas_build(shared, inst.ctypes.data_as(ctypes.c_void_p), 1, None) == 0
+    host.L.fake_finish()
+    st = {id(h): host.stream() for h in (a, b, c, shared)}
+    used = lambda h: streams_used(host.render(h, st[id(h)])[1])
+    assert [used(shared), used(shared), used(a)] == [4, 4, 4]   # its own frames, then one other
+    assert [used(b), used(c)] == [1, 1]                          # two and three others
+    host.L.fake_finish()
+    assert [used(c), used(b)] == [4, 4]
+    assert used(a) == 1
+    host.destroy(b)
+    assert used(a) == 4                                          # c's alone
+    assert not [line for line in host.log() if "capture mode" in line]  # (a query would end another thread's capture)
+    host.L.fake_finish()
+
+
+def test_frames_on_a_capturing_stream_are_one_pipeline(host):
+    """No streams of the scene's own join a caller's capture, and no event
+    recorded in one is asked for later."""
+    h, s = host.renderable(), host.stream()
+    assert host.render(h, s)[0] == 0   # (sizes the queues)
+    host.L.fake_finish()
+    host.L.fake_set_capturing(s, 1)
+    r, log = host.render(h, s)
+    host.L.fake_set_capturing(s, 0)
+    assert r == 0 and streams_used(log) == 1
+    assert not [line for line in log if line.startswith(("record ", "wait "))]
