@@ -509,6 +509,7 @@ __device__ __forceinline__ float fxaa_luma(float4 c) {
 // image written by one kernel and read with the colours again by another.
 constexpr int kFxaaThreads = 256;
 constexpr uint64_t kFxaaManyTiles = 4800;
+constexpr uint32_t kFxaaRows = 65535;  // rows of tiles in the grid's y; further ones go on in z
 
 template <int T, int H>
 struct FxaaTile {
@@ -617,7 +618,8 @@ __global__ void __launch_bounds__(kFxaaThreads, BLOCKS) k_fxaa(const float4* __r
     __shared__ uint16_t list[T * T];
     __shared__ int n_list;
     const int t = threadIdx.x;
-    FxaaTile<T, H> I{in, s, w, h, (int)blockIdx.x * T - H, (int)blockIdx.y * T - H};
+    const int row = (int)(blockIdx.z * kFxaaRows + blockIdx.y);  // (the last z may run past the image)
+    FxaaTile<T, H> I{in, s, w, h, (int)blockIdx.x * T - H, row * T - H};
     if (t == 0) n_list = 0;
     float4 c[kPix];
 #pragma unroll
@@ -715,13 +717,16 @@ cudaError_t launch_fxaa(const float4* in, uint32_t w, uint32_t h, float4* out, c
     // against 58.5, 3200x1800 40.1 against 43.0, but 2880x1620 (4,590 tiles) 37.2
     // both and 1920x1080 23.6 against 21.9.
     const uint64_t tiles = (uint64_t)((w + 31) / 32) * ((h + 31) / 32);
-    const dim3 big((w + 31) / 32, (h + 31) / 32), small((w + 15) / 16, (h + 15) / 16);
-    if (tiles < (uint64_t)device_sm_count() || (h + 15) / 16 > 65535)
-        launch_chain(k_fxaa<16, 8, 4>, small, kFxaaThreads, 0, s, in, (int)w, (int)h, out);
+    const auto grid = [&](uint32_t T) {
+        const uint32_t rows = (h + T - 1) / T;
+        return dim3((w + T - 1) / T, min(rows, kFxaaRows), (rows + kFxaaRows - 1) / kFxaaRows);
+    };
+    if (tiles < (uint64_t)device_sm_count())
+        launch_chain(k_fxaa<16, 8, 4>, grid(16), kFxaaThreads, 0, s, in, (int)w, (int)h, out);
     else if (tiles < kFxaaManyTiles)
-        launch_chain(k_fxaa<32, 8, 4>, big, kFxaaThreads, 0, s, in, (int)w, (int)h, out);
+        launch_chain(k_fxaa<32, 8, 4>, grid(32), kFxaaThreads, 0, s, in, (int)w, (int)h, out);
     else
-        launch_chain(k_fxaa<32, 4, 5>, big, kFxaaThreads, 0, s, in, (int)w, (int)h, out);
+        launch_chain(k_fxaa<32, 4, 5>, grid(32), kFxaaThreads, 0, s, in, (int)w, (int)h, out);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -61,6 +61,12 @@ def test_long_edges_across_tiles(shape):
     assert_bitwise(gpu_fxaa(img), oracle.fxaa(img))
 
 
+def test_image_of_more_rows_of_tiles_than_one_grid_dimension():
+    rng = np.random.default_rng(3)
+    img = np.repeat(rng.uniform(0, 1, (2097120 // 8 + 5, 3, 4)).astype(np.float32), 8, 0)  # 2,097,160 rows
+    assert_bitwise(gpu_fxaa(img), oracle.fxaa(img))
+
+
 @pytest.mark.parametrize("which", ["tiny", "medium"])
 def test_rendered_frames(which):
     s = g.tiny_scene() if which == "tiny" else g.medium_scene()

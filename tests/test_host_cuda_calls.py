@@ -229,3 +229,10 @@ def test_frames_on_a_capturing_stream_are_one_pipeline(host):
     host.L.fake_set_capturing(s, 0)
     assert r == 0 and streams_used(log) == 1
     assert not [line for line in log if line.startswith(("record ", "wait "))]
+
+
+@pytest.mark.parametrize("w,h", [(3, 1048560), (3, 1048561), (1, 1 << 24), (33, 2097121), (1 << 24, 1)])
+def test_fxaa_of_long_images_fits_the_grid(host, w, h):
+    """Every size that rg_fxaa's argument check takes is launched."""
+    assert host.L.rg_fxaa(ctypes.c_void_p(1 << 20), w, h, ctypes.c_void_p(1 << 40), None) == 0
+    assert len(launches(host.log())) == 1
