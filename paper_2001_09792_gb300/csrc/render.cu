@@ -530,8 +530,23 @@ struct FxaaTile {
     __device__ __forceinline__ float luma_at(float px, float py) const {
         const float fx0 = floorf(px), fy0 = floorf(py);
         const float fx = px - fx0, fy = py - fy0;
-        const int x0 = (int)fx0, y0 = (int)fy0;
-        const float a = luma(x0, y0), b = luma(x0 + 1, y0), d = luma(x0, y0 + 1), e = luma(x0 + 1, y0 + 1);
+        const int x = (int)fx0, y = (int)fy0;
+        float a, b, d, e;
+        // one test for the four: an image that is edges everywhere (noise) is bound
+        // by these look-ups; at 3840x2160 305 us, against 379 with a test each
+        // and 348 from a luma image of its own
+        if ((unsigned)(x - x0) < (unsigned)(S - 1) && (unsigned)(y - y0) < (unsigned)(S - 1)) {
+            const float* m = s + (y - y0) * S + (x - x0);
+            a = m[0];
+            b = m[1];
+            d = m[S];
+            e = m[S + 1];
+        } else {
+            a = luma(x, y);
+            b = luma(x + 1, y);
+            d = luma(x, y + 1);
+            e = luma(x + 1, y + 1);
+        }
         const float top = a + fx * (b - a), bot = d + fx * (e - d);
         return top + fy * (bot - top);
     }
@@ -560,13 +575,13 @@ __constant__ float kFxaaStep[12] = {1.0f, 1.0f, 1.0f, 1.0f, 1.0f, 1.5f, 2.0f, 2.
 // Steps 3 to 7 for an edge pixel (x, y): its filtered colour.
 template <int T, int H>
 __device__ __forceinline__ float3 fxaa_edge(const FxaaTile<T, H>& I, int x, int y) {
-    const float lM = I.luma(x, y), lN = I.luma(x, y - 1), lS = I.luma(x, y + 1);
-    const float lW = I.luma(x - 1, y), lE = I.luma(x + 1, y);
+    constexpr int S = FxaaTile<T, H>::S;
+    const float* m = I.s + (y - I.y0) * S + (x - I.x0);  // (its neighbours are in the tile or its halo)
+    const float lM = m[0], lN = m[-S], lS = m[S], lW = m[-1], lE = m[1];
     const float lo = fminf(lM, fminf(fminf(lN, lS), fminf(lW, lE)));
     const float hi = fmaxf(lM, fmaxf(fmaxf(lN, lS), fmaxf(lW, lE)));
     const float range = hi - lo;
-            const float lNW = I.luma(x - 1, y - 1), lNE = I.luma(x + 1, y - 1);
-            const float lSW = I.luma(x - 1, y + 1), lSE = I.luma(x + 1, y + 1);
+            const float lNW = m[-S - 1], lNE = m[-S + 1], lSW = m[S - 1], lSE = m[S + 1];
             const float eH = (second_diff(lNW, lW, lSW) + 2.0f * second_diff(lN, lM, lS)) + second_diff(lNE, lE, lSE);
             const float eV = (second_diff(lNW, lN, lNE) + 2.0f * second_diff(lW, lM, lE)) + second_diff(lSW, lS, lSE);
             const bool horiz = eH >= eV;
