@@ -11,13 +11,17 @@ namespace rg {
 
 namespace {
 
-// The next k rays for this warp's idle lanes.  A query of no more rays than
-// the launch has threads has no work counter (and no launch that clears one):
-// each warp takes its own 32, once.
-template <int MODE>
+// The next k rays for this warp's idle lanes.  OWN: a query of no more rays than
+// the launch has threads comes without a work counter (and without a launch that
+// clears one), and each warp takes its own 32, once.  Larger queries have an
+// instantiation without that test, which cost any hits 0.5 to 1 % (1.76M rays
+// 522 -> 519 us, compressed 570 -> 563).  Small ones keep the test although
+// their counter is always null: without it the compiler splits the first claim
+// off the loop, and 64 compressed rays took 84 us instead of 69.
+template <bool OWN>
 __device__ __forceinline__ uint32_t claim_rays(const TraceArgs& a, uint32_t k, bool& exhausted) {
     uint32_t base = 0;
-    if ((MODE == kModeClosestAbi || MODE == kModeAnyAbi) && !a.work_counter) {
+    if (OWN && !a.work_counter) {
         base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u;
         exhausted = true;
     } else {
@@ -136,7 +140,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_trace_pair(TraceArgs sa
 // 11.36 ms, and runs of 2 or 4 without the pops 9.90 and 9.31 ms.  The visits
 // and their order per ray are unchanged.
 constexpr int kLeafBatch = 4, kLeafNodesMin = 8, kNodeRun = 4;
-template <int MODE, bool BRUTE, bool STATS, int BLOCK, int SD>
+template <int MODE, bool BRUTE, bool STATS, int BLOCK, int SD, bool OWN = false>
 __global__ void __launch_bounds__(BLOCK, (BRUTE || STATS) ? 1 : (MODE == kModeClosestBatch ? 896 : 1024) / BLOCK)
     k_trace_lane(TraceArgs a) {
     chain_wait();
@@ -178,7 +182,7 @@ __global__ void __launch_bounds__(BLOCK, (BRUTE || STATS) ? 1 : (MODE == kModeCl
         const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
         if (!exhausted && idle != 0u && (__popc(idle) >= (int)refill || idle == 0xFFFFFFFFu)) {
             const uint32_t k = (uint32_t)__popc(idle);
-            const uint32_t base = claim_rays<MODE>(a, k, exhausted);
+            const uint32_t base = claim_rays<OWN>(a, k, exhausted);
             if (base + k >= n) exhausted = true;
             if (!active) {
                 const uint32_t idx = base + (uint32_t)__popc(idle & ((1u << lane) - 1u));
@@ -661,7 +665,7 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
 // 2,009 with 8; 2,141 and 2,622 with runs of 2 and 4 nodes an iteration; 2,090
 // and 2,036 with a batch of 1 and 8; 2,156 with refill at 16 idle lanes.
 constexpr int kLeafBatch8 = 4, kLeafNodesMin8 = 8, kRefill8 = 8;
-template <int MODE, bool STATS>
+template <int MODE, bool STATS, bool OWN>
 __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(TraceArgs a) {
     chain_wait();
     const uint32_t iter_cap = a.iter_cap;
@@ -694,7 +698,7 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
         const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !active);
         if (!exhausted && idle != 0u && (__popc(idle) >= (int)refill || idle == 0xFFFFFFFFu)) {
             const uint32_t k = (uint32_t)__popc(idle);
-            const uint32_t base = claim_rays<MODE>(a, k, exhausted);
+            const uint32_t base = claim_rays<OWN>(a, k, exhausted);
             if (base + k >= n) exhausted = true;
             const uint32_t idx = base + (uint32_t)__popc(idle & ((1u << lane) - 1u));
             if (!active && idx < n) {
@@ -843,15 +847,18 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
     flush_counts<kAny, STATS>(a, c_nodes, c_tris, c_inst);
 }
 
-// Grid of a query on the per-lane kernels: as many blocks as its rays fill, up to
-// the resident ones; beyond those the warps share the work counter, cleared
-// here.
-cudaError_t query_grid(TraceArgs& a, int block, int& blocks, cudaStream_t s) {
+// A query on a per-lane kernel: as many blocks of `own` as its rays fill, up to
+// the `blocks` resident ones; beyond those the warps of `shared` take rays from
+// the work counter, cleared here.
+void launch_query(void (*own)(TraceArgs), void (*shared)(TraceArgs), TraceArgs a, int block, int blocks, size_t smem,
+                  cudaStream_t s) {
     const uint64_t need = ((uint64_t)a.n + block - 1) / block;
-    if (need > (uint64_t)blocks) return cudaMemsetAsync(a.work_counter, 0, 4, s);
-    a.work_counter = nullptr;
-    blocks = (int)need;
-    return cudaSuccess;
+    if (need <= (uint64_t)blocks) {
+        a.work_counter = nullptr;
+        launch_chain(own, (unsigned)need, block, smem, s, a);
+    } else if (cudaMemsetAsync(a.work_counter, 0, 4, s) == cudaSuccess) {  // (else the caller finds its error)
+        launch_chain(shared, blocks, block, smem, s, a);
+    }
 }
 
 // The queries of rg_trace_rays, whose rays are often incoherent, take the
@@ -865,7 +872,7 @@ cudaError_t launch_mode8(const TraceArgs& a0, cudaStream_t s) {
     a.refill = kRefill8;
     auto kernel = [] {
         if constexpr (kLane)
-            return k_trace8_lane<MODE, STATS>;
+            return k_trace8_lane<MODE, STATS, STATS>;
         else
             return k_trace8<MODE, STATS>;
     }();
@@ -878,11 +885,10 @@ cudaError_t launch_mode8(const TraceArgs& a0, cudaStream_t s) {
         blocks = device_sm_count() * (per_sm > 0 ? per_sm : 1);
         cached.store(blocks, std::memory_order_relaxed);
     }
-    if (kLane) {
-        const cudaError_t e = query_grid(a, kTraceBlock, blocks, s);
-        if (e != cudaSuccess) return e;
-    }
-    launch_chain(kernel, blocks, kTraceBlock, 0, s, a);
+    if constexpr (kLane)
+        launch_query(k_trace8_lane<MODE, STATS, true>, kernel, a, kTraceBlock, blocks, 0, s);
+    else
+        launch_chain(kernel, blocks, kTraceBlock, 0, s, a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -904,8 +910,7 @@ cudaError_t resident_blocks(K kernel, int block, size_t smem, std::atomic<int>& 
 }
 
 template <int MODE, bool BRUTE, bool STATS, int BLOCK, bool LANE, int SD>
-cudaError_t launch_block(const TraceArgs& a0, int blocks_per_sm, cudaStream_t s) {
-    TraceArgs a = a0;
+cudaError_t launch_block(const TraceArgs& a, int blocks_per_sm, cudaStream_t s) {
     static std::atomic<int> cached{0};
     constexpr size_t smem = (size_t)SD * BLOCK * sizeof(uint32_t);
     int per_sm = 0;
@@ -913,13 +918,15 @@ cudaError_t launch_block(const TraceArgs& a0, int blocks_per_sm, cudaStream_t s)
                          : resident_blocks(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, BLOCK, smem, cached, &per_sm);
     if (e != cudaSuccess) return e;
     const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
-    int blocks = device_sm_count() * b;
-    if (LANE && (MODE == kModeClosestAbi || MODE == kModeAnyAbi) && (e = query_grid(a, BLOCK, blocks, s)) != cudaSuccess)
-        return e;
-    if (LANE)
+    const int blocks = device_sm_count() * b;
+    if constexpr (LANE && (MODE == kModeClosestAbi || MODE == kModeAnyAbi)) {
+        launch_query(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD, true>,
+                     k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD, BRUTE || STATS>, a, BLOCK, blocks, smem, s);
+    } else if constexpr (LANE) {
         launch_chain(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD>, blocks, BLOCK, smem, s, a);
-    else
+    } else {
         launch_chain(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, blocks, BLOCK, smem, s, a);
+    }
     count_launches(1);
     return cudaGetLastError();
 }
