@@ -38,7 +38,8 @@ __device__ __forceinline__ uint32_t claim_rays(const TraceArgs& a, uint32_t k, b
 template <int MODE, bool BRUTE, bool STATS, int BLOCK, int SD>
 __global__ void __launch_bounds__(BLOCK) k_trace_warp(TraceArgs a) {
     chain_wait();
-    constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender || MODE == kModeShadowBatch);
+    static_assert(MODE != kModeClosestAbi && MODE != kModeAnyAbi, "queries take the per-lane kernels (launch_query)");
+    constexpr bool kAny = (MODE == kModeShadowRender || MODE == kModeShadowBatch);
     __shared__ uint32_t pre[kMaxLights + 1];
     const uint32_t n = ray_count<MODE == kModeShadowRender>(a, pre);
     count_closest<MODE>(a, n);
@@ -475,7 +476,8 @@ template <int MODE, bool STATS>
 __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
     chain_wait();
     const uint32_t iter_cap = a.iter_cap;
-    constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender);
+    static_assert(MODE == kModeClosestRender || MODE == kModeShadowRender, "queries take k_trace8_lane");
+    constexpr bool kAny = MODE == kModeShadowRender;
     __shared__ uint32_t pre[kMaxLights + 1];
     const uint32_t n = ray_count<MODE == kModeShadowRender>(a, pre);
     count_closest<MODE>(a, n);
@@ -500,10 +502,8 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
         uint32_t oct = oct_w;
         Shear sh;
 
-        constexpr bool kTies = MODE == kModeClosestAbi;
         Best2 best;
         best.reset(tmax);
-        float any_V = 0.f, any_W = 0.f, any_det = 1.f;
         bool found = false, ok = true, in_blas = false;
 
         uint2 stack[kStack8];
@@ -606,22 +606,15 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
                     const float4* tp = tri_rec(tris, item);
                     const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
                     if (STATS) ++c_tris;
-                    const float tlo =
-                        kAny ? tmax : (kTies && found ? fminf(__fmul_rn(best.t, kTieBand), tmax) : best.t);
-                    TriResult h = tri_test(sh, v0, v1, v2, tmin, tlo);
+                    const TriResult h = tri_test(sh, v0, v1, v2, tmin, kAny ? tmax : best.t);
                     if (h.hit) {
                         const uint32_t prim = __float_as_uint(v0.w);
                         if (kAny) {
-                            best.t = h.t; best.id = cur_id; best.prim = prim;
-                            best.il = cur_leaf; best.tl = item;
-                            any_V = h.V; any_W = h.W; any_det = h.det;
                             found = true;
                             done = true;
                             break;
                         }
-                        if (kTies) {
-                            if (best.offer(h.t, cur_id, prim)) found = true;
-                        } else if (h.t < best.t || cur_id < best.id || (cur_id == best.id && prim < best.prim)) {
+                        if (h.t < best.t || cur_id < best.id || (cur_id == best.id && prim < best.prim)) {
                             best.t = h.t; best.id = cur_id; best.prim = prim;
                             best.il = cur_leaf; best.tl = item;
                             found = true;
@@ -648,8 +641,7 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
             }
         }
         if (!ok) found = false;
-        emit<MODE>(a, i, j, found, ok, best.t, best.id, best.prim, best.il, best.tl, kTies ? best.tie_id() : kMiss,
-                   best.prim2, any_V, any_W, any_det);
+        emit<MODE>(a, i, j, found, ok, best.t, best.id, best.prim, best.il, best.tl);
     }
     flush_counts<kAny, STATS>(a, c_nodes, c_tris, c_inst);
 }
@@ -669,16 +661,14 @@ template <int MODE, bool STATS, bool OWN>
 __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(TraceArgs a) {
     chain_wait();
     const uint32_t iter_cap = a.iter_cap;
-    constexpr bool kAny = (MODE == kModeAnyAbi || MODE == kModeShadowRender);
-    constexpr bool kTies = MODE == kModeClosestAbi;
-    __shared__ uint32_t pre[kMaxLights + 1];
-    const uint32_t n = ray_count<MODE == kModeShadowRender>(a, pre);
-    count_closest<MODE>(a, n);
+    static_assert(MODE == kModeClosestAbi || MODE == kModeAnyAbi, "the renderer's rays take k_trace8");
+    constexpr bool kAny = MODE == kModeAnyAbi;
+    const uint32_t n = a.n;
     const uint32_t lane = threadIdx.x & 31u, refill = a.refill;
     unsigned long long c_nodes = 0, c_tris = 0, c_inst = 0;
 
     bool active = false, exhausted = false;
-    uint32_t i = 0, j = 0, iter = 0;
+    uint32_t i = 0, iter = 0;
     float tmin = 0.f, tmax = 0.f;
     SpaceRay wr, cr;
     uint32_t oct = 0;
@@ -703,8 +693,7 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
             const uint32_t idx = base + (uint32_t)__popc(idle & ((1u << lane) - 1u));
             if (!active && idx < n) {
                 i = idx;
-                j = sub_entry(a, pre, i);
-                const float4 r0 = __ldg(a.rays + 2 * (size_t)j), r1 = __ldg(a.rays + 2 * (size_t)j + 1);
+                const float4 r0 = __ldg(a.rays + 2 * (size_t)i), r1 = __ldg(a.rays + 2 * (size_t)i + 1);
                 tmin = r0.w;
                 tmax = r1.w;
                 wr.ox = r0.x; wr.oy = r0.y; wr.oz = r0.z;
@@ -772,7 +761,7 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
                 const float4 meta0 = __ldg(reinterpret_cast<const float4*>(&I->nodes));
                 const uint4 meta1 = __ldg(reinterpret_cast<const uint4*>(&I->root));
                 if (STATS) ++c_inst;
-                const float4 r1w = __ldg(a.rays + 2 * (size_t)j + 1);  // the world direction, read again
+                const float4 r1w = __ldg(a.rays + 2 * (size_t)i + 1);  // the world direction, read again
                 const float dx = r1w.x, dy = r1w.y, dz = r1w.z;
                 const float ox = fmaf(m0.x, wr.ox, fmaf(m0.y, wr.oy, fmaf(m0.z, wr.oz, m0.w)));
                 const float oy = fmaf(m1.x, wr.ox, fmaf(m1.y, wr.oy, fmaf(m1.z, wr.oz, m1.w)));
@@ -801,19 +790,17 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
             const float4* tp = tri_rec(tris, item);
             const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
             if (STATS) ++c_tris;
-            const float tlo = kAny ? tmax : (kTies && found ? fminf(__fmul_rn(best.t, kTieBand), tmax) : best.t);
+            const float tlo = kAny ? tmax : (found ? fminf(__fmul_rn(best.t, kTieBand), tmax) : best.t);
             const TriResult h = tri_test(sh, v0, v1, v2, tmin, tlo);
             if (h.hit) {
                 const uint32_t prim = __float_as_uint(v0.w);
-                if (kTies) {
-                    if (best.offer(h.t, cur_id, prim)) found = true;
-                } else if (kAny || h.t < best.t || cur_id < best.id || (cur_id == best.id && prim < best.prim)) {
+                if (kAny) {
                     best.t = h.t; best.id = cur_id; best.prim = prim;
-                    best.il = cur_leaf; best.tl = item;
                     any_V = h.V; any_W = h.W; any_det = h.det;
+                    found = finished = true;
+                } else if (best.offer(h.t, cur_id, prim)) {
                     found = true;
                 }
-                if (kAny) finished = true;
             }
         }
         // pop what the step left (the marker brings back the world-space ray)
@@ -839,8 +826,8 @@ __global__ void __launch_bounds__(kTraceBlock, STATS ? 1 : 6) k_trace8_lane(Trac
             }
         }
         if (finished) {
-            emit<MODE>(a, i, j, found && ok, ok, best.t, best.id, best.prim, best.il, best.tl,
-                       kTies ? best.tie_id() : kMiss, best.prim2, any_V, any_W, any_det);
+            emit<MODE>(a, i, i, found && ok, ok, best.t, best.id, best.prim, best.il, best.tl,
+                       kAny ? kMiss : best.tie_id(), best.prim2, any_V, any_W, any_det);
             active = false;
         }
     }
@@ -914,19 +901,21 @@ cudaError_t launch_block(const TraceArgs& a, int blocks_per_sm, cudaStream_t s) 
     static std::atomic<int> cached{0};
     constexpr size_t smem = (size_t)SD * BLOCK * sizeof(uint32_t);
     int per_sm = 0;
-    cudaError_t e = LANE ? resident_blocks(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD>, BLOCK, smem, cached, &per_sm)
-                         : resident_blocks(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, BLOCK, smem, cached, &per_sm);
+    constexpr bool kQuery = MODE == kModeClosestAbi || MODE == kModeAnyAbi;
+    auto kernel = [] {
+        if constexpr (LANE)
+            return k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD, kQuery && (BRUTE || STATS)>;
+        else
+            return k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>;
+    }();
+    const cudaError_t e = resident_blocks(kernel, BLOCK, smem, cached, &per_sm);
     if (e != cudaSuccess) return e;
     const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
     const int blocks = device_sm_count() * b;
-    if constexpr (LANE && (MODE == kModeClosestAbi || MODE == kModeAnyAbi)) {
-        launch_query(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD, true>,
-                     k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD, BRUTE || STATS>, a, BLOCK, blocks, smem, s);
-    } else if constexpr (LANE) {
-        launch_chain(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD>, blocks, BLOCK, smem, s, a);
-    } else {
-        launch_chain(k_trace_warp<MODE, BRUTE, STATS, BLOCK, SD>, blocks, BLOCK, smem, s, a);
-    }
+    if constexpr (kQuery)
+        launch_query(k_trace_lane<MODE, BRUTE, STATS, BLOCK, SD, true>, kernel, a, BLOCK, blocks, smem, s);
+    else
+        launch_chain(kernel, blocks, BLOCK, smem, s, a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -978,7 +967,8 @@ cudaError_t launch_mode(const TraceArgs& a0, cudaStream_t s, const TraceShape& s
     const int refill = (shape.refill >= 1 && shape.refill <= 32) ? shape.refill : default_refill<MODE>();
     a.refill = (uint32_t)refill;
     constexpr bool kTunable = !BRUTE && !STATS && MODE >= kModeClosestRender;
-    if (refill < 32) {
+    constexpr bool kQuery = MODE == kModeClosestAbi || MODE == kModeAnyAbi;
+    if (kQuery || refill < 32) {
         if constexpr (kTunable) {
             if (shape.block == 64) return launch_block<MODE, BRUTE, STATS, 64, true, 0>(a, shape.blocks_per_sm, s);
             if (shape.block == 256) return launch_block<MODE, BRUTE, STATS, 256, true, 0>(a, shape.blocks_per_sm, s);
@@ -989,7 +979,8 @@ cudaError_t launch_mode(const TraceArgs& a0, cudaStream_t s, const TraceShape& s
         if (shape.block == 64) return launch_block<MODE, BRUTE, STATS, 64, false, 0>(a, shape.blocks_per_sm, s);
         if (shape.block == 256) return launch_block<MODE, BRUTE, STATS, 256, false, 0>(a, shape.blocks_per_sm, s);
     }
-    return launch_block_128<MODE, BRUTE, STATS, false>(a, shape, s);
+    if constexpr (!kQuery) return launch_block_128<MODE, BRUTE, STATS, false>(a, shape, s);
+    return cudaErrorInvalidValue;
 }
 
 // Completes one provisional ABI hit record of a traversal launch (emit;

@@ -66,6 +66,12 @@ void* fake_stream(int prio) {
     return s;
 }
 void fake_set_capturing(void* s, int on) { g_capturing[s] = on; }
+const char* fake_kernels() {  // the names of the library's kernels
+    static std::string all;
+    all.clear();
+    for (const auto& k : g_kernels) all += k.second + '\n';
+    return all.c_str();
+}
 void fake_finish() { g_pending.clear(); }  // the device catches up
 
 // ---- the runtime

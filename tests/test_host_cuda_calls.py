@@ -26,7 +26,7 @@ def fake_lib(tmp_path_factory):
                     os.path.join(HERE, "fake_cudart.cpp"), *objs, "-o", out, "-Wl,-Bsymbolic", "-Wl,--no-undefined",
                     "-lpthread"], check=True)
     L = ctypes.CDLL(out)
-    L.fake_log.restype = ctypes.c_char_p
+    L.fake_log.restype = L.fake_kernels.restype = ctypes.c_char_p
     L.fake_stream.restype = ctypes.c_void_p
     L.rg_last_error.restype = ctypes.c_char_p
     return L
@@ -236,3 +236,12 @@ def test_fxaa_of_long_images_fits_the_grid(host, w, h):
     """Every size that rg_fxaa's argument check takes is launched."""
     assert host.L.rg_fxaa(ctypes.c_void_p(1 << 20), w, h, ctypes.c_void_p(1 << 40), None) == 0
     assert len(launches(host.log())) == 1
+
+
+def test_every_query_kernel_is_one_whose_counter_is_cleared(host):
+    """Queries clear their work counter where they launch the per-lane kernels;
+    no whole-warp instantiation of a query mode exists that could be reached
+    with a stale one."""
+    names = host.L.fake_kernels().decode().split()
+    query = [n for n in names if any(f"k_trace{k}ILi{m}E" in n for k in ("_lane", "_warp", "8_lane", "8") for m in (0, 1))]
+    assert query and all("_lane" in n for n in query), query
