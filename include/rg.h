@@ -27,6 +27,10 @@
  *  - All device geometry is float32.  float64 is used on the device only to
  *    invert instance transforms.
  *  - Calls on one scene must not run concurrently from several host threads.
+ *  - Temporaries of the calls come from a pool of the library's own, which keeps
+ *    up to 64 MiB per device between calls, and up to 16 MiB once the last scene
+ *    of the device is destroyed; an allocation of the library that runs out
+ *    of memory takes what it keeps first.
  *  - A scene lives on the CUDA device that was current when it was created.
  *    Every call on it makes that device current for the calling thread (and
  *    leaves it current); the device buffers and the stream passed to it must

@@ -65,13 +65,16 @@ uint32_t test_limit(const char* name) {
 // The pool of the calls' stream-ordered temporaries, one per device, made on
 // first use.  It keeps up to kPoolKeep bytes across synchronisations: the
 // device's default pool keeps none, so that the first temporary after each wait
-// for the GPU cost about 110 us of mapping.  What it keeps is given back
-// when a device allocation of the library runs out of memory.  (Null: the
-// default pool serves.)
-constexpr uint64_t kPoolKeep = 64ull << 20;
+// for the GPU cost about 110 us of mapping.  When the last scene of the device is
+// destroyed it gives back all but kPoolRest (loading a scene of 20,480 triangles
+// with no other one there: 500 us, 600 without the rest), and all that is unused
+// when a device allocation of the library runs out of memory.  (Null: the default
+// pool serves.)
+constexpr uint64_t kPoolKeep = 64ull << 20, kPoolRest = 16ull << 20;
 constexpr int kMaxDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pools[kMaxDevices] = {};
+std::atomic<int> g_scenes[kMaxDevices];  // scenes of each device
 
 cudaMemPool_t temp_pool() {
     int dev = 0;
@@ -95,12 +98,13 @@ cudaMemPool_t temp_pool() {
     return g_pools[dev];
 }
 
-// Gives back what the current device's pool holds unused; true if there is one.
-bool trim_pool() {
+// Gives back what the current device's pool holds unused above `rest` bytes;
+// true if there is a pool.
+bool trim_pool(uint64_t rest) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    return g_pools[dev] && cudaMemPoolTrimTo(g_pools[dev], 0) == cudaSuccess;
+    return g_pools[dev] && cudaMemPoolTrimTo(g_pools[dev], rest) == cudaSuccess;
 }
 
 rg_status dev_alloc(void** p, size_t bytes, const char* what) {
@@ -108,16 +112,8 @@ rg_status dev_alloc(void** p, size_t bytes, const char* what) {
     long k = ++g_alloc_count;
     if (fault_alloc_index() == k) return fail(RG_ERR_OOM, std::string("injected allocation failure: ") + what);
     if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation && trim_pool()) {
-        cudaGetLastError();
-        e = cudaMalloc(p, bytes);
-    }
-    if (e != cudaSuccess) {
-        *p = nullptr;
-        return cuda_fail(e, what);
-    }
-    return RG_OK;
+    const cudaError_t e = device_malloc(p, bytes);
+    return e == cudaSuccess ? RG_OK : cuda_fail(e, what);
 }
 
 // Parts of one allocation, each 256-byte aligned: the offset of the next part.
@@ -495,6 +491,7 @@ rg_status rg_scene_create(rg_scene** out, const rg_scene_desc* desc) {
         delete s;
         return cuda_fail(e, "scene setup");
     }
+    if (s->device < kMaxDevices) ++g_scenes[s->device];
     *out = s;
     return RG_OK;
 }
@@ -580,7 +577,9 @@ rg_status rg_scene_destroy(rg_scene* s) {
         cudaEventDestroy(ep.a);
         cudaEventDestroy(ep.b);
     }
+    const int device = s->device;
     delete s;
+    if (device < kMaxDevices && --g_scenes[device] == 0) trim_pool(kPoolRest);
     return RG_OK;
 }
 
@@ -1381,6 +1380,16 @@ rg_status scene_view(rg_scene* s, SceneView* v) {
 
 namespace rg {
 rg_status report_error(rg_status code, const char* msg) { return fail(code, msg); }
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && trim_pool(0)) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
+}
 
 static std::atomic<unsigned long long> g_launches{0};
 static thread_local bool g_capturing = false;

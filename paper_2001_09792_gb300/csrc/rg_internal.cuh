@@ -174,6 +174,8 @@ inline cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
 }
 
+// cudaMalloc that takes back what the pool of temporaries keeps before it gives up.
+cudaError_t device_malloc(void** p, size_t bytes);
 // Kernels launched by the library since process start (host counter).
 void count_launches(unsigned n);
 // While set (per host thread), count_launches ignores launches: they are

@@ -170,13 +170,8 @@ rg_status scuda(cudaError_t e, const char* what) {
 
 template <class T>
 rg_status salloc(T** p, size_t n, const char* what) {
-    *p = nullptr;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), (n ? n : 1) * sizeof(T));
-    if (e != cudaSuccess) {
-        *p = nullptr;
-        return scuda(e, what);
-    }
-    return RG_OK;
+    const cudaError_t e = device_malloc(reinterpret_cast<void**>(p), (n ? n : 1) * sizeof(T));
+    return e == cudaSuccess ? RG_OK : scuda(e, what);
 }
 
 struct SceneEntry {

@@ -21,7 +21,7 @@ std::map<const void*, std::string> g_kernels;
 std::map<std::pair<int, const void*>, size_t> g_smem;  // (device, kernel): dynamic shared memory allowed
 std::map<void*, int> g_stream_prio, g_capturing;
 std::set<void*> g_pending;                             // events that cudaEventQuery finds unfinished
-int g_dev = 0, g_fail_launch = 0, g_launches = 0, g_pools = 0, g_next = 1;
+int g_dev = 0, g_fail_launch = 0, g_launches = 0, g_mallocs = 0, g_fail_malloc = 0, g_next = 1;
 cudaError_t g_last = cudaSuccess;
 cudaStreamCaptureMode g_capture_mode = cudaStreamCaptureModeGlobal;
 
@@ -60,6 +60,7 @@ extern "C" {
 const char* fake_log() { return g_log.c_str(); }
 void fake_reset() { g_log.clear(), g_launches = g_fail_launch = 0; }
 void fake_fail_launch(int k) { g_launches = 0, g_fail_launch = k; }
+void fake_fail_malloc(int k) { g_mallocs = 0, g_fail_malloc = k; }
 void* fake_stream(int prio) {
     void* s = handle();
     g_stream_prio[s] = prio;
@@ -86,7 +87,7 @@ cudaError_t cudaSetDevice(int d) { return g_dev = d, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
 cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) { return memset(p, 0, sizeof *p), cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return log("devsync"), g_pending.clear(), cudaSuccess; }
-cudaError_t cudaMalloc(void** p, size_t n) { return get(p, n); }
+cudaError_t cudaMalloc(void** p, size_t n) { return ++g_mallocs == g_fail_malloc ? ret(cudaErrorMemoryAllocation) : get(p, n); }
 cudaError_t cudaMallocHost(void** p, size_t n) { return get(p, n); }
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return get(p, n); }
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) { return get(p, n); }
@@ -94,7 +95,7 @@ cudaError_t cudaFree(void* p) { return free(p), cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return free(p), cudaSuccess; }
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) {
-    return *p = reinterpret_cast<cudaMemPool_t>(handle()), ++g_pools, log("pool d%d", g_dev), cudaSuccess;
+    return *p = reinterpret_cast<cudaMemPool_t>(handle()), log("pool d%d", g_dev), cudaSuccess;
 }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t n) { return log("trim d%d %zu", g_dev, n), cudaSuccess; }

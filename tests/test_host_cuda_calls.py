@@ -245,3 +245,36 @@ def test_every_query_kernel_is_one_whose_counter_is_cleared(host):
     names = host.L.fake_kernels().decode().split()
     query = [n for n in names if any(f"k_trace{k}ILi{m}E" in n for k in ("_lane", "_warp", "8_lane", "8") for m in (0, 1))]
     assert query and all("_lane" in n for n in query), query
+
+
+def test_last_scene_of_a_device_gives_the_temporaries_back(host):
+    """What the pool of temporaries keeps goes back, down to 16 MiB, when the last
+    scene of its device is destroyed, not before, and not another device's."""
+    scenes = {}
+    for dev in (0, 0, 1):
+        host.L.cudaSetDevice(dev)
+        h = host.scene()
+        assert host.blas(h) == 0
+        scenes.setdefault(dev, []).append(h)
+    trims = lambda: [line for line in host.log() if line.startswith("trim ")]
+    host.destroy(scenes[0].pop())
+    assert trims() == []
+    host.destroy(scenes[0].pop())
+    assert trims() == ["trim d0 16777216"]
+    host.destroy(scenes[1].pop())
+    assert trims() == ["trim d0 16777216", "trim d1 16777216"]
+
+
+def test_allocations_take_the_kept_temporaries_before_they_fail(host):
+    h = host.scene()
+    assert host.blas(h) == 0
+    for k in range(1, 4):   # of a server: of a scene and of its queues the same function
+        host.L.fake_fail_malloc(k)
+        at = len(host.log())
+        srv = ctypes.c_void_p()
+        assert host.L.rg_server_create(ctypes.byref(srv), ctypes.byref(rg.rg_server_desc())) == 0
+        assert "trim d0 0" in host.log()[at:]
+        assert host.L.rg_server_destroy(srv) == 0
+    host.L.fake_fail_malloc(1)
+    host.scene()
+    host.L.fake_fail_malloc(0)
