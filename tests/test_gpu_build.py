@@ -112,6 +112,25 @@ def test_radix_sort_edges(n, key_bits, noalloc):
     assert np.array_equal(ko.cpu().numpy().view(keys.dtype), keys[order])
 
 
+@pytest.mark.parametrize("n", [819_199, 819_200, 819_201, 1_000_003, 4096 * 301 + 1])
+@pytest.mark.parametrize("key_bits", [32, 64])
+def test_radix_sort_large_tiles(n, key_bits):
+    """The tiles of 4,096 pairs (from 819,200 pairs on): both sides of the
+    switch, ragged ends, long runs of equal keys, the largest key among them;
+    exact, as every whole number is."""
+    rng = np.random.default_rng(n)
+    keys = rng.integers(0, 2 ** 63, n, dtype=np.uint64) >> np.uint64(64 - key_bits)
+    keys[rng.integers(0, n, n // 3)] = 12345
+    keys[rng.integers(0, n, n // 5)] = 2 ** key_bits - 1
+    keys[n // 2:n // 2 + 20_000] = 7
+    keys = keys.astype(np.uint32 if key_bits == 32 else np.uint64)
+    signed = torch.from_numpy(keys.view(np.int32 if key_bits == 32 else np.int64)).cuda()
+    ko, vo = rg.rg_radix_sort_pairs(signed, torch.arange(n, dtype=torch.int32).cuda())
+    order = np.argsort(keys, kind="stable")
+    assert np.array_equal(vo.cpu().numpy(), order)
+    assert np.array_equal(ko.cpu().numpy().view(keys.dtype), keys[order])
+
+
 @pytest.mark.parametrize("n,hi", [(2, 4), (3, 1), (17, 1), (1000, 8), (4097, 1 << 30), (50_000, 1 << 30), (9999, 64)])
 @pytest.mark.parametrize("key_bits", [32, 64])
 def test_karras_topology(n, hi, key_bits):
