@@ -902,9 +902,8 @@ static cudaError_t radix_sort_impl(const K* keys_in, const uint32_t* vals_in, ui
         K* kdst = to_out ? keys_out : kt;
         uint32_t* vdst = to_out ? vals_out : vt;
         auto* pass_kernel = large ? k_rs_pass<K, W, 2 * kSortItems> : k_rs_pass<K, W, kSortItems>;
-        launch_chain(pass_kernel, nb, kSortThreads, 0, s, 
-            ksrc, vsrc, n, 8 * pass, hist + 256 * pass, status[pass & 1],
-            pass + 1 < passes ? status[(pass + 1) & 1] : nullptr, ticket + pass, kdst, vdst);
+        launch_chain(pass_kernel, nb, kSortThreads, 0, s, ksrc, vsrc, n, 8 * pass, hist + 256 * pass, status[pass & 1],
+                     pass + 1 < passes ? status[(pass + 1) & 1] : nullptr, ticket + pass, kdst, vdst);
         ksrc = kdst;
         vsrc = vdst;
     }
@@ -927,11 +926,11 @@ cudaError_t launch_karras(const void* keys, uint32_t n, int key_bits, uint32_t* 
                           uint32_t* parents, cudaStream_t s, uint32_t* ranges) {
     if (n < 2) return cudaSuccess;
     if (key_bits == 64)
-        launch_chain(k_karras<uint64_t>, grid_for(n - 1), kBlock, 0, s, static_cast<const uint64_t*>(keys), n, child_base, stride,
-                                                              parents, ranges);
+        launch_chain(k_karras<uint64_t>, grid_for(n - 1), kBlock, 0, s, static_cast<const uint64_t*>(keys), n, child_base,
+                     stride, parents, ranges);
     else
-        launch_chain(k_karras<uint32_t>, grid_for(n - 1), kBlock, 0, s, static_cast<const uint32_t*>(keys), n, child_base, stride,
-                                                              parents, ranges);
+        launch_chain(k_karras<uint32_t>, grid_for(n - 1), kBlock, 0, s, static_cast<const uint32_t*>(keys), n, child_base,
+                     stride, parents, ranges);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -942,11 +941,11 @@ cudaError_t launch_karras_segments(const void* keys, int key_bits, const KarrasS
     if (n_segs == 0 || n_threads == 0) return cudaSuccess;
     uint32_t* child_base = reinterpret_cast<uint32_t*>(nodes) + 12;
     if (key_bits == 64)
-        launch_chain(k_karras_segments<uint64_t>, grid_for(n_threads), kBlock, 0, s, 
-            static_cast<const uint64_t*>(keys), segs, n_segs, n_threads, n_leaves, child_base, parents, ranges);
+        launch_chain(k_karras_segments<uint64_t>, grid_for(n_threads), kBlock, 0, s, static_cast<const uint64_t*>(keys), segs,
+                     n_segs, n_threads, n_leaves, child_base, parents, ranges);
     else
-        launch_chain(k_karras_segments<uint32_t>, grid_for(n_threads), kBlock, 0, s, 
-            static_cast<const uint32_t*>(keys), segs, n_segs, n_threads, n_leaves, child_base, parents, ranges);
+        launch_chain(k_karras_segments<uint32_t>, grid_for(n_threads), kBlock, 0, s, static_cast<const uint32_t*>(keys), segs,
+                     n_segs, n_threads, n_leaves, child_base, parents, ranges);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -981,8 +980,8 @@ cudaError_t launch_tlas_leaves_refit(const InstDev* tmp, const float* wbox, cons
                                      const uint32_t* parents, float4* nodes, uint32_t* flags, InstDev* inst_out,
                                      uint32_t* leaf_of_inst, DevStatus* st, cudaStream_t s,
                                      const uint32_t* boxes_done) {
-    launch_chain(k_tlas_leaves_refit, grid_for(n), kBlock, 0, s, tmp, wbox, perm, n, parents, nodes, flags, inst_out, leaf_of_inst, st,
-                                                       boxes_done);
+    launch_chain(k_tlas_leaves_refit, grid_for(n), kBlock, 0, s, tmp, wbox, perm, n, parents, nodes, flags,
+                 inst_out, leaf_of_inst, st, boxes_done);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -994,7 +993,7 @@ cudaError_t launch_tlas_small(const rg_instance* in, uint32_t n, const BlasDev* 
     if (n == 0 || n > kTlasSmallMax) return cudaErrorInvalidValue;
     const uint32_t threads = (n + 31u) & ~31u;
     launch_chain(k_tlas_small, 1, threads, 0, s, in, n, blas, nblas, tmp, wbox, refit, nodes, perm, parents, flags, ranges,
-inst_out, leaf_of_inst, st);
+                 inst_out, leaf_of_inst, st);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -581,51 +581,51 @@ __device__ __forceinline__ float3 fxaa_edge(const FxaaTile<T, H>& I, int x, int 
     const float lo = fminf(lM, fminf(fminf(lN, lS), fminf(lW, lE)));
     const float hi = fmaxf(lM, fmaxf(fmaxf(lN, lS), fmaxf(lW, lE)));
     const float range = hi - lo;
-            const float lNW = m[-S - 1], lNE = m[-S + 1], lSW = m[S - 1], lSE = m[S + 1];
-            const float eH = (second_diff(lNW, lW, lSW) + 2.0f * second_diff(lN, lM, lS)) + second_diff(lNE, lE, lSE);
-            const float eV = (second_diff(lNW, lN, lNE) + 2.0f * second_diff(lW, lM, lE)) + second_diff(lSW, lS, lSE);
-            const bool horiz = eH >= eV;
-            const float l1 = horiz ? lN : lW, l2 = horiz ? lS : lE;
-            const float g1 = l1 - lM, g2 = l2 - lM;
-            const bool neg = fabsf(g1) >= fabsf(g2);
-            const float gs = 0.25f * fmaxf(fabsf(g1), fabsf(g2));
-            const float edge = neg ? 0.5f * (l1 + lM) : 0.5f * (l2 + lM);
-            const float sgn = neg ? -1.0f : 1.0f;
-            const float fx = (float)x, fy = (float)y;
-            const float sx = horiz ? fx : fx + 0.5f * sgn, sy = horiz ? fy + 0.5f * sgn : fy;
-                float dist[2], endl[2];
-    #pragma unroll
-            for (int side = 0; side < 2; ++side) {
-                const float dir = side == 0 ? -1.0f : 1.0f;
-                float d = 0.0f, e = 0.0f;
-                for (int k = 0; k < 12; ++k) {
-                    d = d + kFxaaStep[k];
-                    const float px = horiz ? sx + dir * d : sx;
-                    const float py = horiz ? sy : sy + dir * d;
-                    e = I.luma_at(px, py) - edge;
-                    if (fabsf(e) >= gs) break;
-                }
-                dist[side] = d;
-                endl[side] = e;
-            }
-            const float len = dist[0] + dist[1];
-            const bool near0 = dist[0] < dist[1];
-            const float dmin = near0 ? dist[0] : dist[1];
-            const float e_near = near0 ? endl[0] : endl[1];
-            const float off = ((lM < edge) != (e_near < 0.0f)) ? 0.5f - __fdiv_rn(dmin, len) : 0.0f;
-            const float sum4 = (lN + lS) + (lW + lE);
-            const float sumc = (lNW + lNE) + (lSW + lSE);
-            const float avg = __fdiv_rn(2.0f * sum4 + sumc, 12.0f);
-            float sp = __fdiv_rn(fabsf(avg - lM), range);
-            if (sp > 1.0f) sp = 1.0f;
-            sp = ((3.0f - 2.0f * sp) * sp) * sp;
-            const float f = fmaxf(off, (sp * sp) * 0.75f);
-            return I.color_at(horiz ? fx : fx + f * sgn, horiz ? fy + f * sgn : fy);
+    const float lNW = m[-S - 1], lNE = m[-S + 1], lSW = m[S - 1], lSE = m[S + 1];
+    const float eH = (second_diff(lNW, lW, lSW) + 2.0f * second_diff(lN, lM, lS)) + second_diff(lNE, lE, lSE);
+    const float eV = (second_diff(lNW, lN, lNE) + 2.0f * second_diff(lW, lM, lE)) + second_diff(lSW, lS, lSE);
+    const bool horiz = eH >= eV;
+    const float l1 = horiz ? lN : lW, l2 = horiz ? lS : lE;
+    const float g1 = l1 - lM, g2 = l2 - lM;
+    const bool neg = fabsf(g1) >= fabsf(g2);
+    const float gs = 0.25f * fmaxf(fabsf(g1), fabsf(g2));
+    const float edge = neg ? 0.5f * (l1 + lM) : 0.5f * (l2 + lM);
+    const float sgn = neg ? -1.0f : 1.0f;
+    const float fx = (float)x, fy = (float)y;
+    const float sx = horiz ? fx : fx + 0.5f * sgn, sy = horiz ? fy + 0.5f * sgn : fy;
+    float dist[2], endl[2];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const float dir = side == 0 ? -1.0f : 1.0f;
+        float d = 0.0f, e = 0.0f;
+        for (int k = 0; k < 12; ++k) {
+            d = d + kFxaaStep[k];
+            const float px = horiz ? sx + dir * d : sx;
+            const float py = horiz ? sy : sy + dir * d;
+            e = I.luma_at(px, py) - edge;
+            if (fabsf(e) >= gs) break;
+        }
+        dist[side] = d;
+        endl[side] = e;
+    }
+    const float len = dist[0] + dist[1];
+    const bool near0 = dist[0] < dist[1];
+    const float dmin = near0 ? dist[0] : dist[1];
+    const float e_near = near0 ? endl[0] : endl[1];
+    const float off = ((lM < edge) != (e_near < 0.0f)) ? 0.5f - __fdiv_rn(dmin, len) : 0.0f;
+    const float sum4 = (lN + lS) + (lW + lE);
+    const float sumc = (lNW + lNE) + (lSW + lSE);
+    const float avg = __fdiv_rn(2.0f * sum4 + sumc, 12.0f);
+    float sp = __fdiv_rn(fabsf(avg - lM), range);
+    if (sp > 1.0f) sp = 1.0f;
+    sp = ((3.0f - 2.0f * sp) * sp) * sp;
+    const float f = fmaxf(off, (sp * sp) * 0.75f);
+    return I.color_at(horiz ? fx : fx + f * sgn, horiz ? fy + f * sgn : fy);
 }
 
 template <int T, int H, int BLOCKS>
 __global__ void __launch_bounds__(kFxaaThreads, BLOCKS) k_fxaa(const float4* __restrict__ in, int w, int h,
-                                                       float4* __restrict__ out) {
+                                                                float4* __restrict__ out) {
     chain_wait();
     constexpr int S = FxaaTile<T, H>::S, kPix = T * T / kFxaaThreads;
     constexpr int kRing = S * S - T * T;  // halo pixels: H rows above and below, then H columns left and right
@@ -711,7 +711,8 @@ cudaError_t launch_raygen_batch(const RaygenReq* reqs, const uint32_t* n_reqs, u
                                 const uint32_t* n_rays, const uint32_t* gen_base, uint32_t ring_mask, float4* rays,
                                 Payload* payload, cudaStream_t s) {
     const uint32_t blocks = (uint32_t)min((max_rays + 255u) / 256u, (uint32_t)device_sm_count() * 8u);
-    launch_chain(k_raygen_batch, blocks > 0 ? blocks : 1, 256, 0, s, reqs, n_reqs, n_rays, gen_base, ring_mask, rays, payload);
+    launch_chain(k_raygen_batch, blocks > 0 ? blocks : 1, 256, 0, s, reqs, n_reqs, n_rays, gen_base, ring_mask, rays,
+                 payload);
     count_launches(1);
     return cudaGetLastError();
 }

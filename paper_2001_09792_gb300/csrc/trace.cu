@@ -407,7 +407,7 @@ struct Groups {
 // Tests the eight children of the node at nd: the groups of those the ray meets.
 __device__ __forceinline__ void visit8(const float4* nd, const SpaceRay& cr, uint32_t oct, float tmin, float tlim,
                                        Groups& G) {
-        const float4 w0 = __ldg(nd);
+    const float4 w0 = __ldg(nd);
     const uint4 w1 = __ldg(reinterpret_cast<const uint4*>(nd + 1));
     const uint4 w2 = __ldg(reinterpret_cast<const uint4*>(nd + 2));
     const uint4 w3 = __ldg(reinterpret_cast<const uint4*>(nd + 3));
@@ -432,7 +432,7 @@ __device__ __forceinline__ void visit8(const float4* nd, const SpaceRay& cr, uin
     const uint32_t nx0 = nx ? w3.z : w2.x, nx1 = nx ? w3.w : w2.y, fx0 = nx ? w2.x : w3.z, fx1 = nx ? w2.y : w3.w;
     const uint32_t ny0 = ny ? w4.x : w2.z, ny1 = ny ? w4.y : w2.w, fy0 = ny ? w2.z : w4.x, fy1 = ny ? w2.w : w4.y;
     const uint32_t nz0 = nz ? w4.z : w3.x, nz1 = nz ? w4.w : w3.y, fz0 = nz ? w3.x : w4.z, fz1 = nz ? w3.y : w4.w;
-        const uint32_t meta_lo = w1.z, meta_hi = w1.w;
+    const uint32_t meta_lo = w1.z, meta_hi = w1.w;
     uint32_t hitmask = 0;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -528,27 +528,27 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
                     done = true;
                     break;
                 }
-                    const uint32_t b = 31 - __clz(g_hits);
-                    g_hits &= ~(1u << b);
-                    const uint32_t s = b ^ oct;
-                    const uint32_t node = g_base + __popc(g_imask & ((1u << s) - 1u));
-                    if (g_hits) {
-                        if (sp >= kStack8) {
-                            record_error(a.st, RG_ERR_STACK);
-                            ok = false;
-                            done = true;
-                            break;
-                        }
-                        stack[sp++] = make_uint2(g_base, g_hits | (g_imask << 8) | kKindNode);
+                const uint32_t b = 31 - __clz(g_hits);
+                g_hits &= ~(1u << b);
+                const uint32_t s = b ^ oct;
+                const uint32_t node = g_base + __popc(g_imask & ((1u << s) - 1u));
+                if (g_hits) {
+                    if (sp >= kStack8) {
+                        record_error(a.st, RG_ERR_STACK);
+                        ok = false;
+                        done = true;
+                        break;
                     }
-                    if (STATS) ++c_nodes;
-                    Groups G;
-                    visit8(nodes + 5 * (size_t)node, cr, oct, tmin, __fmul_rn(kAny ? tmax : best.t, kCullSlack), G);
-                    g_base = G.base;
-                    g_hits = G.hits;
-                    g_imask = G.imask;
-                    i_base = G.ibase;
-                    i_bits = G.ibits;
+                    stack[sp++] = make_uint2(g_base, g_hits | (g_imask << 8) | kKindNode);
+                }
+                if (STATS) ++c_nodes;
+                Groups G;
+                visit8(nodes + 5 * (size_t)node, cr, oct, tmin, __fmul_rn(kAny ? tmax : best.t, kCullSlack), G);
+                g_base = G.base;
+                g_hits = G.hits;
+                g_imask = G.imask;
+                i_base = G.ibase;
+                i_bits = G.ibits;
             }
             if (done) break;
             while (i_bits) {
@@ -558,68 +558,68 @@ __global__ void __launch_bounds__(kTraceBlock) k_trace8(TraceArgs a) {
                     done = true;
                     break;
                 }
-                    const uint32_t k = __ffs(i_bits) - 1;
-                    i_bits &= i_bits - 1;
-                    const uint32_t item = i_base + k;
-                    if (!in_blas) {
-                        // instance: save the TLAS groups, enter its BLAS
-                        if (sp + 3 > kStack8) {
-                            record_error(a.st, RG_ERR_STACK);
-                            ok = false;
-                            done = true;
-                            break;
-                        }
-                        if (g_hits) stack[sp++] = make_uint2(g_base, g_hits | (g_imask << 8) | kKindNode);
-                        if (i_bits) stack[sp++] = make_uint2(i_base, i_bits | kKindItem);
-                        stack[sp++] = make_uint2(0u, kKindMarker);
-                        const InstDev* I = a.inst8 + item;
-                        const float4 m0 = __ldg(&I->inv[0]), m1 = __ldg(&I->inv[1]), m2 = __ldg(&I->inv[2]);
-                        const float4 meta0 = __ldg(reinterpret_cast<const float4*>(&I->nodes));
-                        const uint4 meta1 = __ldg(reinterpret_cast<const uint4*>(&I->root));
-                        if (STATS) ++c_inst;
-                        const float dx = r1.x, dy = r1.y, dz = r1.z;
-                        float ox = fmaf(m0.x, wr.ox, fmaf(m0.y, wr.oy, fmaf(m0.z, wr.oz, m0.w)));
-                        float oy = fmaf(m1.x, wr.ox, fmaf(m1.y, wr.oy, fmaf(m1.z, wr.oz, m1.w)));
-                        float oz = fmaf(m2.x, wr.ox, fmaf(m2.y, wr.oy, fmaf(m2.z, wr.oz, m2.w)));
-                        float ddx = fmaf(m0.x, dx, fmaf(m0.y, dy, __fmul_rn(m0.z, dz)));
-                        float ddy = fmaf(m1.x, dx, fmaf(m1.y, dy, __fmul_rn(m1.z, dz)));
-                        float ddz = fmaf(m2.x, dx, fmaf(m2.y, dy, __fmul_rn(m2.z, dz)));
-                        cr.ox = ox; cr.oy = oy; cr.oz = oz;
-                        cr.ix = safe_rcp(ddx); cr.iy = safe_rcp(ddy); cr.iz = safe_rcp(ddz);
-                        oct = oct_of(cr);
-                        sh = make_shear(ox, oy, oz, ddx, ddy, ddz);
-                        const unsigned long long pn =
-                            ((unsigned long long)__float_as_uint(meta0.y) << 32) | __float_as_uint(meta0.x);
-                        const unsigned long long pt =
-                            ((unsigned long long)__float_as_uint(meta0.w) << 32) | __float_as_uint(meta0.z);
-                        nodes = reinterpret_cast<const float4*>(pn);
-                        tris = reinterpret_cast<const float4*>(pt) + 3 * sh.order;  // the ray's axis order
-                        cur_id = meta1.y;
-                        cur_leaf = item;
-                        in_blas = true;
-                        g_base = 0;
-                        g_hits = 1u << oct;
-                        g_imask = 1u;
-                        i_bits = 0;
-                        continue;
+                const uint32_t k = __ffs(i_bits) - 1;
+                i_bits &= i_bits - 1;
+                const uint32_t item = i_base + k;
+                if (!in_blas) {
+                    // instance: save the TLAS groups, enter its BLAS
+                    if (sp + 3 > kStack8) {
+                        record_error(a.st, RG_ERR_STACK);
+                        ok = false;
+                        done = true;
+                        break;
                     }
-                    const float4* tp = tri_rec(tris, item);
-                    const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
-                    if (STATS) ++c_tris;
-                    const TriResult h = tri_test(sh, v0, v1, v2, tmin, kAny ? tmax : best.t);
-                    if (h.hit) {
-                        const uint32_t prim = __float_as_uint(v0.w);
-                        if (kAny) {
-                            found = true;
-                            done = true;
-                            break;
-                        }
-                        if (h.t < best.t || cur_id < best.id || (cur_id == best.id && prim < best.prim)) {
-                            best.t = h.t; best.id = cur_id; best.prim = prim;
-                            best.il = cur_leaf; best.tl = item;
-                            found = true;
-                        }
+                    if (g_hits) stack[sp++] = make_uint2(g_base, g_hits | (g_imask << 8) | kKindNode);
+                    if (i_bits) stack[sp++] = make_uint2(i_base, i_bits | kKindItem);
+                    stack[sp++] = make_uint2(0u, kKindMarker);
+                    const InstDev* I = a.inst8 + item;
+                    const float4 m0 = __ldg(&I->inv[0]), m1 = __ldg(&I->inv[1]), m2 = __ldg(&I->inv[2]);
+                    const float4 meta0 = __ldg(reinterpret_cast<const float4*>(&I->nodes));
+                    const uint4 meta1 = __ldg(reinterpret_cast<const uint4*>(&I->root));
+                    if (STATS) ++c_inst;
+                    const float dx = r1.x, dy = r1.y, dz = r1.z;
+                    float ox = fmaf(m0.x, wr.ox, fmaf(m0.y, wr.oy, fmaf(m0.z, wr.oz, m0.w)));
+                    float oy = fmaf(m1.x, wr.ox, fmaf(m1.y, wr.oy, fmaf(m1.z, wr.oz, m1.w)));
+                    float oz = fmaf(m2.x, wr.ox, fmaf(m2.y, wr.oy, fmaf(m2.z, wr.oz, m2.w)));
+                    float ddx = fmaf(m0.x, dx, fmaf(m0.y, dy, __fmul_rn(m0.z, dz)));
+                    float ddy = fmaf(m1.x, dx, fmaf(m1.y, dy, __fmul_rn(m1.z, dz)));
+                    float ddz = fmaf(m2.x, dx, fmaf(m2.y, dy, __fmul_rn(m2.z, dz)));
+                    cr.ox = ox; cr.oy = oy; cr.oz = oz;
+                    cr.ix = safe_rcp(ddx); cr.iy = safe_rcp(ddy); cr.iz = safe_rcp(ddz);
+                    oct = oct_of(cr);
+                    sh = make_shear(ox, oy, oz, ddx, ddy, ddz);
+                    const unsigned long long pn =
+                        ((unsigned long long)__float_as_uint(meta0.y) << 32) | __float_as_uint(meta0.x);
+                    const unsigned long long pt =
+                        ((unsigned long long)__float_as_uint(meta0.w) << 32) | __float_as_uint(meta0.z);
+                    nodes = reinterpret_cast<const float4*>(pn);
+                    tris = reinterpret_cast<const float4*>(pt) + 3 * sh.order;  // the ray's axis order
+                    cur_id = meta1.y;
+                    cur_leaf = item;
+                    in_blas = true;
+                    g_base = 0;
+                    g_hits = 1u << oct;
+                    g_imask = 1u;
+                    i_bits = 0;
+                    continue;
+                }
+                const float4* tp = tri_rec(tris, item);
+                const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
+                if (STATS) ++c_tris;
+                const TriResult h = tri_test(sh, v0, v1, v2, tmin, kAny ? tmax : best.t);
+                if (h.hit) {
+                    const uint32_t prim = __float_as_uint(v0.w);
+                    if (kAny) {
+                        found = true;
+                        done = true;
+                        break;
                     }
+                    if (h.t < best.t || cur_id < best.id || (cur_id == best.id && prim < best.prim)) {
+                        best.t = h.t; best.id = cur_id; best.prim = prim;
+                        best.il = cur_leaf; best.tl = item;
+                        found = true;
+                    }
+                }
             }
             if (done) break;
             if (g_hits) continue;
