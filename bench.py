@@ -80,7 +80,7 @@ def parse(argv=None):
     p.add_argument("--lanes", type=int, default=0, help="serving: server lanes (0: the library's default)")
     p.add_argument("--no-serving", action="store_true", help="skip the serving measurement")
     p.add_argument("--tlas", default="sah", choices=["sah", "lbvh"],
-                   help="large workload: TLAS hierarchy, binned SAH in one block (RG_SCENE_SAH_TLAS) or LBVH")
+                   help="large workload: TLAS hierarchy, binned SAH (RG_SCENE_SAH_TLAS) or LBVH")
     p.add_argument("--blas", default="sah", choices=["sah", "lbvh"],
                    help="BLAS build of every scene: binned SAH (RG_BLAS_SAH, for trace speed) or LBVH (for build speed)")
     p.add_argument("--no-medium", action="store_true", help="large: skip the medium render frame")
@@ -1201,7 +1201,7 @@ def gpu_index(local):
 def blas_build_rate(scene, reps=3, sah=False):
     """BLAS builds of the scene's meshes (LBVH: boxes, Morton codes, radix
     sort, Karras hierarchy, refit, bounding sphere; with sah the binned-SAH
-    build, one host round trip per tree level), inputs already on the device,
+    build, usually with one host round trip), inputs already on the device,
     CUDA events around the builds; the median of `reps` builds."""
     import torch
     import paper_2001_09792_gb300 as rg

@@ -98,9 +98,9 @@ typedef struct { float pos[3]; float intensity[3]; } rg_light;
  * RG_SCENE_FRUGAL sizes rg_render's queues from each depth level's ray count
  * (the host waits once per level) instead of the frame's worst case.
  * RG_SCENE_SAH_TLAS builds a TLAS of 2 to 4,096 instances for trace speed:
- * the hierarchy of rg_blas_build's RG_BLAS_SAH, built in one single-block
- * launch without host round trips (larger TLAS keep the LBVH); the same hit
- * records, a slower build. */
+ * the hierarchy of rg_blas_build's RG_BLAS_SAH, built on the device without
+ * host round trips (larger TLAS keep the LBVH); the same hit records, a slower
+ * build. */
 enum {
     RG_SCENE_TIMING = 1u,
     RG_SCENE_COUNT = 2u,
@@ -165,9 +165,11 @@ enum { RG_MORTON30 = 0u, RG_MORTON63 = 1u, RG_COMPRESSED = 2u, RG_BLAS_SAH = 4u 
  * RG_BLAS_SAH to build for trace speed rather than build speed: every split
  * is chosen by the binned surface-area heuristic (16 bins per axis; below 40
  * levels the Karras hierarchy of the Morton codes takes over); same node
- * layout, any query gives the same results, and the build takes one host
- * round trip per tree level.  Writes the new
- * BLAS id to *blas_id.  nt >= 1;
+ * layout, any query gives the same results.  A SAH build of more than 4,096
+ * triangles waits for the stream, usually once; the others return without
+ * waiting (all wait for the device when the scene's table of BLAS grows).  A
+ * capturing stream is refused (RG_ERR_CUDA).  Writes the new BLAS id to
+ * *blas_id.  nt >= 1;
  * indices must be < nv (checked on the device: RG_ERR_INVALID_ARG at
  * rg_sync).  The mesh is copied; d_vtx/d_idx may be freed after the call
  * once the stream has passed it. */

@@ -714,7 +714,7 @@ rg_status rg_blas_build(rg_scene* s, const float* d_vtx, uint32_t nv, const uint
 static rg_status tlas_common(rg_scene* s, const rg_instance* d_inst, uint32_t n, cudaStream_t st, bool refit) {
     rg_status r;
     TempAlloc tmp(st);
-    // the SAH hierarchy (one block) when asked for, else the LBVH; a one-launch
+    // the SAH hierarchy when asked for, else the LBVH; a one-launch
     // build or refit of a small TLAS when its topology is the LBVH's or fixed
     const bool sah = (s->desc.flags & RG_SCENE_SAH_TLAS) && n >= 2 && n <= kSahOneMax;
     if (n <= kTlasSmallMax && !(sah && !refit)) {

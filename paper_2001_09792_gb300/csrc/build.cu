@@ -194,8 +194,8 @@ __global__ void k_morton(const float* __restrict__ lohi, uint32_t n, const int* 
 // Garland 2016, in the one-pass-per-digit form of Adinets & Merrill 2022) and
 // writes its pairs grouped by digit, so that the stores are runs.  Bound by
 // memory (12 B read and written per pair and pass) where the launch is large,
-// by the launches where it is small.  1,000,003 pairs of 32-bit keys: 78.7 us,
-// 304.7 us with a count, a one-block scan (50 us a pass) and a scatter per
+// by the launches where it is small.  1,000,003 pairs of 32-bit keys: 67.6 us,
+// 324.9 us with a count, a one-block scan (50 us a pass) and a scatter per
 // pass.
 //
 // The look-back waits on nothing: a tile takes its number from a counter, so
@@ -206,8 +206,11 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSpinMax = 1 << 14;
 constexpr uint32_t kLook = 8, kSortLargeTiles = 200;
 // Items per thread: 8 (tiles of kSortTilePairs), or 16 from kSortLargeTiles tiles
-// of those on: 1,000,003 pairs take 78.7 us with 16 and 88.9 with 8, 16M 615 and
-// 667, but 100,001 pairs 51.6 and 43.7 (few tiles, each longer).
+// of those on, 1.3 an SM of 152: with a tile and more on every SM the shorter
+// chain of look-backs outweighs the longer tile.  us with 8 and 16: 1,000,003 pairs 78.7
+// and 67.5 (64-bit keys 149.5, 131.9), 16M 654 and 605, 819,200 67.7 and 63.9; but
+// 311,297 41.9 and 45.4, and with 64-bit keys 100,001 60.4 and 75.7, 311,297 72.1
+// and 84.5.  Between 450,001 (50.2, 46.5) and the line 16 would be 4 to 8 % faster.
 constexpr int kSortItems = (int)kSortTilePairs / kSortThreads;
 
 // Ranks of a warp's ITEMS x 32 digits among its own: cnt (256 entries, this
@@ -326,8 +329,9 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_pass(const K* __restrict__ 
     const uint32_t first = scan256(hist[t], s_wsum);  // the digit's place over all tiles
     // the pairs of this digit in the tiles before
     // (kLook tiles are read at a time, for the chain of reads is what a pass waits
-    // on: 95.6 -> 88.9 us at 1,000,003 pairs; 16 and 32 at a time 86.0 and 98.4
-    // against 78.7 with the larger tiles)
+    // on: before the launches were chained 1,000,003 pairs took 95.6 us with one at a
+    // time, 88.9 with 8, and 78.7 with 8 and the larger tiles, 86.0 and 98.4 with 16
+    // and 32)
     uint32_t before = 0;
     for (uint32_t q = tile;; q -= kLook) {
         W v[kLook];

@@ -505,8 +505,9 @@ __device__ __forceinline__ float fxaa_luma(float4 c) {
 // in shared memory, are shared out over the block's threads, so that a few of
 // them do not hold the other lanes of their warps.  The edge search leaves
 // the halo only on long edges; there the luma comes from the colour.  Bound by
-// memory (32 B a pixel); 3840x2160: 50.3 us, 5.3 TB/s, against 101 us for a luma
-// image written by one kernel and read with the colours again by another.
+// memory (32 B a pixel); a rendered 3840x2160 frame: 49.4 us, 5.4 TB/s, against
+// 112 us for a luma image written by one kernel and read with the colours again
+// by another.
 constexpr int kFxaaThreads = 256;
 constexpr uint64_t kFxaaManyTiles = 4800;
 constexpr uint32_t kFxaaRows = 65535;  // rows of tiles in the grid's y; further ones go on in z
@@ -727,11 +728,11 @@ cudaError_t launch_fxaa(const float4* in, uint32_t w, uint32_t h, float4* out, c
     if (w == 0 || h == 0) return cudaSuccess;
     // 32 x 32 tiles with a halo of 8 read 2.25 pixels per pixel (the halo's from
     // L2), 16 x 16 tiles 4; the small ones where the large would not give every
-    // SM a block.  An image of many waves of tiles is bound by the reads rather
-    // than by the searches' chains, and takes a halo of 4 (1.56 pixels), which
-    // the searches leave sooner, and a fifth block per SM: 3840x2160 50.3 us
-    // against 58.5, 3200x1800 40.1 against 43.0, but 2880x1620 (4,590 tiles) 37.2
-    // both and 1920x1080 23.6 against 21.9.
+    // SM a block.  An image of many waves of tiles (kFxaaManyTiles: 8 waves of 4 blocks
+    // on 152 SMs) is bound by the reads rather than by the searches' chains, and takes
+    // a halo of 4 (1.56 pixels), which the searches leave sooner, and a fifth block
+    // per SM: 3840x2160 49.4 us against 57.9, 3200x1800 40.1 against 41.8, but
+    // 2880x1620 (4,590 tiles) 36.7 against 36.2 and 1920x1080 23.5 against 21.2.
     const uint64_t tiles = (uint64_t)((w + 31) / 32) * ((h + 31) / 32);
     const auto grid = [&](uint32_t T) {
         const uint32_t rows = (h + T - 1) / T;
