@@ -239,8 +239,8 @@ rg_status rg_trace_rays(rg_scene* scene, const rg_ray* d_rays, uint32_t n, uint3
  * scenes made with rg_scene_create_shared may render concurrently.  A frame
  * of 2^18 pixels or more is enqueued as four bands of pixels, three of them on
  * streams of the scene's own at the priority of `stream`, which goes on when
- * all are done; it is one pipeline on `stream` when two or more such frames
- * of other scenes are still running, when `stream` is being captured, and in
+ * all are done; it is one pipeline on `stream` when such frames of other
+ * scenes are still running on two or more other streams, when `stream` is being captured, and in
  * scenes with RG_SCENE_TIMING or RG_SCENE_COUNT, whose launches are timed or
  * counted one by one.  The image is the same either way up to the order in which a
  * pixel's contributions are added. */

@@ -230,8 +230,8 @@ constexpr uint32_t kTraceSlots = 64;
 // its longest rays and leaves most of the chip idle, which another band's launch
 // then fills.  The medium frame at 1080p, us: 2,140 as one, 2,009 in 2 bands,
 // 2,011 in 3, 1,971 in 4, 2,032 in 8; at 640x480 903, 905, 898, 893, 887.
-// Frames of other scenes in flight fill the tails as well: from kBandOthers of
-// them on, a frame is one pipeline.  Scenes of their own BLAS with 1, 2, 3 and 4
+// Frames of other scenes in flight on streams of their own fill the tails as
+// well: from kBandOthers of them on, a frame is one pipeline.  Scenes of their own BLAS with 1, 2, 3 and 4
 // frames in flight, us a frame at 1080p: 1,173, 806, 690 and 654 as one, 1,055,
 // 787, 712 and 702 in 4 bands.
 constexpr uint32_t kBands = 4, kBandPixels = 1u << 18, kBandOthers = 2;
@@ -349,16 +349,26 @@ rg_status collect_events(rg_scene* s) {
     return RG_OK;
 }
 
-// The last frames of kBandPixels and more, one entry a scene, per device; those
-// found finished are dropped.
+// The last frame of kBandPixels and more on each stream, per device (the frames
+// of one stream run one after another); those found finished are dropped.
 struct FrameList {
+    struct Frame {
+        const rg_scene* scene;
+        unsigned long long stream;  // cudaStreamGetId
+        cudaEvent_t done;           // the scene's
+    };
     std::mutex mu;
-    std::vector<std::pair<const rg_scene*, cudaEvent_t>> frames;
+    std::vector<Frame> frames;
+    template <class F>
+    void drop(F f) {
+        frames.erase(std::remove_if(frames.begin(), frames.end(), f), frames.end());
+    }
 };
 FrameList g_frames[kMaxDevices];
 
-// The frames of other scenes that are still running on s's device.
-uint32_t others_in_flight(const rg_scene* s) {
+// The streams other than that of id st on which frames of other scenes than s are still
+// running on s's device.
+uint32_t others_in_flight(const rg_scene* s, unsigned long long st) {
     if (s->device < 0 || s->device >= kMaxDevices) return kBandOthers;
     // (an event may be asked for while a thread, this one too, captures another stream)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -367,13 +377,12 @@ uint32_t others_in_flight(const rg_scene* s) {
     {
         FrameList& L = g_frames[s->device];
         std::lock_guard<std::mutex> lock(L.mu);
-        auto finished = [&](const std::pair<const rg_scene*, cudaEvent_t>& f) {
-            if (f.first == s) return false;
-            const bool running = cudaEventQuery(f.second) == cudaErrorNotReady;
+        L.drop([&](const FrameList::Frame& f) {
+            if (f.scene == s || f.stream == st) return false;
+            const bool running = cudaEventQuery(f.done) == cudaErrorNotReady;
             n += running;
             return !running;
-        };
-        L.frames.erase(std::remove_if(L.frames.begin(), L.frames.end(), finished), L.frames.end());
+        });
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (n) cudaGetLastError();  // (a query that finds an event unfinished leaves an error behind)
@@ -381,15 +390,14 @@ uint32_t others_in_flight(const rg_scene* s) {
 }
 
 // Marks the end of a frame on the caller's stream for others_in_flight.
-rg_status note_frame(rg_scene* s, cudaStream_t st) {
+rg_status note_frame(rg_scene* s, cudaStream_t stream, unsigned long long st) {
     if (s->device < 0 || s->device >= kMaxDevices) return RG_OK;
     FrameList& L = g_frames[s->device];
     std::lock_guard<std::mutex> lock(L.mu);
     if (!s->frame_ev) RG_CK(cudaEventCreateWithFlags(&s->frame_ev, cudaEventDisableTiming));
-    RG_CK(cudaEventRecord(s->frame_ev, st));
-    for (const auto& f : L.frames)
-        if (f.first == s) return RG_OK;
-    L.frames.emplace_back(s, s->frame_ev);
+    RG_CK(cudaEventRecord(s->frame_ev, stream));
+    L.drop([&](const FrameList::Frame& f) { return f.scene == s || f.stream == st; });
+    L.frames.push_back({s, st, s->frame_ev});
     return RG_OK;
 }
 
@@ -397,8 +405,7 @@ void forget_frame(rg_scene* s) {
     if (!s->frame_ev) return;
     FrameList& L = g_frames[s->device];
     std::lock_guard<std::mutex> lock(L.mu);
-    L.frames.erase(std::remove_if(L.frames.begin(), L.frames.end(), [&](const auto& f) { return f.first == s; }),
-                   L.frames.end());
+    L.drop([&](const FrameList::Frame& f) { return f.scene == s; });
     cudaEventDestroy(s->frame_ev);
     s->frame_ev = nullptr;
 }
@@ -1079,8 +1086,10 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     RG_CK(cudaStreamIsCapturing(st, &cap));
     const bool large = async && max_depth > 1 && N >= kBandPixels && cap == cudaStreamCaptureStatusNone;
+    unsigned long long st_id = 0;
+    if (large) RG_CK(cudaStreamGetId(st, &st_id));
     const bool banded = large && !(s->desc.flags & (RG_SCENE_TIMING | RG_SCENE_COUNT)) &&
-                        others_in_flight(s) < kBandOthers;
+                        others_in_flight(s, st_id) < kBandOthers;
     const uint32_t n_bands = banded ? kBands : 1u;
     const size_t n_counters = CB * ((size_t)max_depth + 1);
     if ((r = s->counters.ensure(n_counters * n_bands, "counters"))) return r;
@@ -1147,7 +1156,7 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, uint32_t w, uint32_t h, u
         }
         if (r) return r;
     }
-    return large ? note_frame(s, st) : RG_OK;
+    return large ? note_frame(s, st, st_id) : RG_OK;
 }
 
 rg_status rg_fxaa(const float* d_in, uint32_t w, uint32_t h, float* d_out, void* stream) {

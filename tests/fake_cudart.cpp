@@ -117,6 +117,7 @@ cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned flags, int pr
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned f) { return cudaStreamCreateWithPriority(s, f, 0); }
 cudaError_t cudaStreamGetPriority(cudaStream_t s, int* p) { return *p = g_stream_prio[s], cudaSuccess; }
+cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long* n) { return *n = (size_t)s, cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { return log("destroy s%d", id(s)), cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
     return g_capturing[s] ? ret(cudaErrorStreamCaptureUnsupported) : (log("streamsync s%d", id(s)), cudaSuccess);

@@ -278,3 +278,14 @@ def test_allocations_take_the_kept_temporaries_before_they_fail(host):
     host.L.fake_fail_malloc(1)
     host.scene()
     host.L.fake_fail_malloc(0)
+
+
+def test_frames_queued_on_one_stream_are_not_in_flight_together(host):
+    """Frames of several scenes on one stream run one after another: each is
+    banded, and together they count as one frame for the other streams."""
+    scenes, s, t = [host.renderable() for _ in range(4)], host.stream(), host.stream()
+    host.L.fake_finish()
+    assert [streams_used(host.render(h, s)[1]) for h in scenes[:3]] == [4, 4, 4]
+    assert streams_used(host.render(scenes[3], t)[1]) == 4     # one other stream
+    assert streams_used(host.render(scenes[0], s)[1]) == 4
+    host.L.fake_finish()
