@@ -301,6 +301,11 @@ rg_status set_device(rg_scene* s) {
     return RG_OK;
 }
 
+// Waits for a clear or copy just queued on the default stream, which neither a
+// memset nor a small copy from pageable memory does, and which the streams of
+// later calls may not wait for.
+cudaError_t settle() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 rg_status event_begin(rg_scene* s, int kind, cudaStream_t st, EventPair** out) {
     *out = nullptr;
     if (!(s->desc.flags & RG_SCENE_TIMING)) return RG_OK;
@@ -490,9 +495,8 @@ rg_status rg_scene_create(rg_scene** out, const rg_scene_desc* desc) {
         return r;
     }
     s->trace_ctr = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(s->st) + kCtrAt);
-    // (the clear goes to the default stream, which the streams of later calls may not wait for)
     cudaError_t e = cudaMemset(s->st, 0, sizeof(DevStatus));
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e == cudaSuccess) e = settle();
     if (e != cudaSuccess) {
         cudaFree(s->st);
         delete s;
@@ -536,8 +540,7 @@ rg_status rg_scene_create_shared(rg_scene** out, rg_scene* src) {
             return cuda_fail(e, "copying lights");
         }
     }
-    // (copies between device buffers do not wait on the host)
-    if (cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy); e != cudaSuccess) {
+    if (cudaError_t e = settle(); e != cudaSuccess) {
         rg_scene_destroy(s);
         return cuda_fail(e, "copying materials and lights");
     }
@@ -846,6 +849,7 @@ rg_status rg_scene_set_materials(rg_scene* s, const rg_material* h, uint32_t n) 
     if ((r = set_device(s))) return r;
     if ((r = s->mats.ensure(n, "materials"))) return r;
     RG_CK(cudaMemcpy(s->mats.p, h, n * sizeof(rg_material), cudaMemcpyHostToDevice));
+    RG_CK(settle());
     s->n_mats = n;
     return RG_OK;
 }
@@ -858,6 +862,7 @@ rg_status rg_scene_set_lights(rg_scene* s, const rg_light* h, uint32_t n) {
     if ((r = set_device(s))) return r;
     if ((r = s->lights.ensure(n ? n : 1, "lights"))) return r;
     if (n) RG_CK(cudaMemcpy(s->lights.p, h, n * sizeof(rg_light), cudaMemcpyHostToDevice));
+    RG_CK(settle());
     s->n_lights = n;
     return RG_OK;
 }
@@ -1181,6 +1186,7 @@ rg_status rg_sync(rg_scene* s) {
     RG_CK(cudaMemcpy(&err, &s->st->error, sizeof(int), cudaMemcpyDeviceToHost));
     if (err) {
         RG_CK(cudaMemset(&s->st->error, 0, sizeof(int)));
+        RG_CK(settle());
         const char* what = err == RG_ERR_STACK       ? "traversal stack overflow"
                            : err == RG_ERR_TIMEOUT   ? "device loop iteration cap reached"
                            : err == RG_ERR_SINGULAR  ? "singular instance transform"
@@ -1232,6 +1238,7 @@ rg_status rg_reset_stats(rg_scene* s) {
     s->launch_base = launches_so_far();
     RG_CK(cudaMemset(reinterpret_cast<char*>(s->st) + offsetof(DevStatus, closest_rays), 0,
                      sizeof(DevStatus) - offsetof(DevStatus, closest_rays)));
+    RG_CK(settle());
     return RG_OK;
 }
 

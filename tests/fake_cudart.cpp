@@ -21,6 +21,7 @@ std::map<const void*, std::string> g_kernels;
 std::map<std::pair<int, const void*>, size_t> g_smem;  // (device, kernel): dynamic shared memory allowed
 std::map<void*, int> g_stream_prio, g_capturing;
 std::set<void*> g_pending;                             // events that cudaEventQuery finds unfinished
+void* g_cleared = nullptr;                             // by the last cudaMemset
 int g_dev = 0, g_fail_launch = 0, g_launches = 0, g_mallocs = 0, g_fail_malloc = 0, g_next = 1;
 cudaError_t g_last = cudaSuccess;
 cudaStreamCaptureMode g_capture_mode = cudaStreamCaptureModeGlobal;
@@ -73,6 +74,7 @@ const char* fake_kernels() {  // the names of the library's kernels
     for (const auto& k : g_kernels) all += k.second + '\n';
     return all.c_str();
 }
+void* fake_cleared() { return g_cleared; }
 void fake_finish() { g_pending.clear(); }  // the device catches up
 
 // ---- the runtime
@@ -99,7 +101,7 @@ cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) {
 }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t n) { return log("trim d%d %zu", g_dev, n), cudaSuccess; }
-cudaError_t cudaMemset(void* p, int v, size_t n) { return log("memset s0"), memset(p, v, n), cudaSuccess; }
+cudaError_t cudaMemset(void* p, int v, size_t n) { return log("memset s0"), memset(g_cleared = p, v, n), cudaSuccess; }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) {
     return log("memset s%d", id(s)), memset(p, v, n), cudaSuccess;
 }

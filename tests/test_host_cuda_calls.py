@@ -27,7 +27,7 @@ def fake_lib(tmp_path_factory):
                     "-lpthread"], check=True)
     L = ctypes.CDLL(out)
     L.fake_log.restype = L.fake_kernels.restype = ctypes.c_char_p
-    L.fake_stream.restype = ctypes.c_void_p
+    L.fake_stream.restype = L.fake_cleared.restype = ctypes.c_void_p
     L.rg_last_error.restype = ctypes.c_char_p
     return L
 
@@ -130,6 +130,30 @@ def test_shared_scene_creation_waits_for_its_copies(host):
     new = host.log()[at:]
     last_copy = max(k for k, line in enumerate(new) if line == "copy s0")
     assert "streamsync s0" in new[last_copy:]
+
+
+@pytest.mark.parametrize("call", ["materials", "lights", "sync", "reset"])
+def test_calls_wait_for_their_copies_and_clears(host, call):
+    """What a call writes to the scene through the default stream is in place
+    when it returns: the next one may come on a stream that does not wait."""
+    h = host.scene()
+    status = host.L.fake_cleared()   # (the scene's status word, its error code first)
+    mat = rg.rg_material(0, (ctypes.c_float * 3)(1, 1, 1), 1.0)
+    light = rg.rg_light((ctypes.c_float * 3)(0, 1, 0), (ctypes.c_float * 3)(1, 1, 1))
+    at = len(host.log())
+    if call == "materials":
+        assert host.L.rg_scene_set_materials(h, ctypes.byref(mat), 1) == 0
+    elif call == "lights":
+        assert host.L.rg_scene_set_lights(h, ctypes.byref(light), 1) == 0
+    elif call == "sync":
+        ctypes.c_int.from_address(status).value = rg.RG_ERR_STACK
+        assert host.L.rg_sync(h) == rg.RG_ERR_STACK and host.L.rg_sync(h) == 0
+    else:
+        assert host.L.rg_reset_stats(h) == 0
+    new = host.log()[at:]
+    write = "memset s0" if call in ("sync", "reset") else "copy s0"
+    last = max(k for k, line in enumerate(new) if line == write)
+    assert "streamsync s0" in new[last:]
 
 
 @pytest.mark.parametrize("flags", [rg.RG_BLAS_SAH, rg.RG_BLAS_SAH | rg.RG_MORTON63])
