@@ -143,12 +143,13 @@ rg_status sfail(rg_status code, const std::string& msg) { return report_error(co
 // free-running 32-bit counters (ring entries are positions masked by the
 // capacity, sizes are differences of positions), so any start is valid; the
 // tests start near 2^32 to make a run wrap the counters (RG_TEST_RING_START,
-// read when a server is created; 0 otherwise).
-cudaError_t reset_ring(RingState* d_rs, uint32_t start) {
+// read when a server is created; 0 otherwise).  On the lane's stream, which waits
+// for no other.
+cudaError_t reset_ring(RingState* d_rs, uint32_t start, cudaStream_t stream) {
     RingState rs;
     std::memset(&rs, 0, sizeof rs);
     rs.head = rs.tail = rs.gen_base = rs.next_base = rs.cons = start;
-    return cudaMemcpy(d_rs, &rs, sizeof rs, cudaMemcpyHostToDevice);
+    return cudaMemcpyAsync(d_rs, &rs, sizeof rs, cudaMemcpyHostToDevice, stream);
 }
 
 uint32_t ring_start_for_tests() {
@@ -627,7 +628,7 @@ rg_status finish_step(rg_server* s, Lane& L, uint32_t* n_completed) {
     if (n_completed) *n_completed += completed;
     if (O.error) {
         // the step completed (a ray that failed counts as a miss); report it
-        SV_CK(cudaMemset(&L.st->error, 0, sizeof(int)));
+        SV_CK(cudaMemsetAsync(&L.st->error, 0, sizeof(int), L.stream));
         return sfail(O.error, std::string("render server step: ") + device_error_text(O.error));
     }
     if (live_sum != (int64_t)L.ring_rays_now) return sfail(RG_ERR_CUDA, "render server: ring count mismatch");
@@ -803,8 +804,9 @@ rg_status rg_server_create(rg_server** out, const rg_server_desc* desc) {
             return bail(sfail(RG_ERR_OOM, "pinned host buffers"));
         std::memset(L.h_hdr, 0, sizeof(StepHdr));
         std::memset(L.h_out, 0, sizeof(StepOut));
-        if (cudaMemset(L.st, 0, sizeof(DevStatus)) != cudaSuccess || reset_ring(L.d_rs, s->ring_start) != cudaSuccess ||
-            cudaMemset(L.d_hdr, 0, sizeof(StepHdr)) != cudaSuccess)
+        if (cudaMemsetAsync(L.st, 0, sizeof(DevStatus), L.stream) != cudaSuccess ||
+            reset_ring(L.d_rs, s->ring_start, L.stream) != cudaSuccess ||
+            cudaMemsetAsync(L.d_hdr, 0, sizeof(StepHdr), L.stream) != cudaSuccess)
             return bail(scuda(cudaGetLastError(), "cudaMemset"));
     }
     *out = s;
@@ -1131,8 +1133,8 @@ rg_status rg_server_autotune(rg_server* s, const rg_request* sample, const char*
         SV_CK(cudaStreamSynchronize(L.stream));
         int err = 0;
         SV_CK(cudaMemcpy(&err, &L.st->error, sizeof(int), cudaMemcpyDeviceToHost));
-        SV_CK(reset_ring(L.d_rs, s->ring_start));
-        SV_CK(cudaMemset(&L.st->error, 0, sizeof(int)));
+        SV_CK(reset_ring(L.d_rs, s->ring_start, L.stream));
+        SV_CK(cudaMemsetAsync(&L.st->error, 0, sizeof(int), L.stream));
         L.ring_rays_now = 0;
         L.admitted = 0;
         for (Active& a : L.active) a = Active();

@@ -156,6 +156,19 @@ def test_calls_wait_for_their_copies_and_clears(host, call):
     assert "streamsync s0" in new[last:]
 
 
+def test_server_lanes_are_set_up_on_their_own_streams(host):
+    """A lane's stream waits for no other, so its first step finds the lane's
+    status, ring and header only if they were written there."""
+    srv = ctypes.c_void_p()
+    at = len(host.log())
+    assert host.L.rg_server_create(ctypes.byref(srv), ctypes.byref(rg.rg_server_desc())) == 0
+    new = host.log()[at:]
+    assert host.L.rg_server_destroy(srv) == 0
+    lanes = {line.split()[1] for line in new if line.startswith("stream ")}
+    writes = [line.split()[1] for line in new if line.startswith(("memset ", "copy "))]
+    assert lanes and len(writes) >= 3 * len(lanes) and set(writes) == lanes
+
+
 @pytest.mark.parametrize("flags", [rg.RG_BLAS_SAH, rg.RG_BLAS_SAH | rg.RG_MORTON63])
 def test_sah_builds_on_a_second_device(host, flags):
     """The large shared memory of the SAH blocks is allowed per device."""
