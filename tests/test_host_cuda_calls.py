@@ -103,7 +103,8 @@ def test_growing_the_blas_table_waits_for_builds_on_other_streams(host):
     stream writes its descriptor and root box there, so the copy comes after
     it."""
     h, a, b = host.scene(), host.stream(), host.stream()
-    assert host.blas(h, stream=a) == 0 and host.blas(h, stream=a) == 0
+    assert [host.blas(h, stream=a) for _ in range(16)] == [0] * 16
+    assert "devsync" not in host.log()   # (the first table holds 16)
     at = len(host.log())
     assert host.blas(h, stream=b) == 0
     new = host.log()[at:]
